@@ -289,7 +289,8 @@ __device__ __forceinline__ void upper_tile_of(int t, int T, int &ti, int &tj) {
 template <int P>
 __global__ void __launch_bounds__(GR_THREADS)
 k_gram_pair(RowBlocks A, RowBlocks B, int pa, int pb, long long n, int sym, int Ti, int Tj, long long kchunk,
-            double *__restrict__ part) {
+            double *__restrict__ part, const int *guard) {
+    if (guard && *guard == 0) return;   // rns.cu did the work
     constexpr int TE = 16 * P;
     __shared__ double2 As[GRK][TE + 1];
     __shared__ double2 Bs[GRK][TE + 1];
@@ -367,7 +368,8 @@ k_gram_pair(RowBlocks A, RowBlocks B, int pa, int pb, long long n, int sym, int 
 // tiles are averaged with it.
 __global__ void k_gram_pair_reduce(const double *__restrict__ part, int nsplit, int pa, int pb, int a0, int a1,
                                    int b0, int b1, int na, int nb, int sym, int te, double scale,
-                                   double2 *__restrict__ g, int ldg) {
+                                   double2 *__restrict__ g, int ldg, const int *guard) {
+    if (guard && *guard == 0) return;
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (long long)na * nb) return;
     const int i = (int)(idx / nb), j = (int)(idx % nb);
@@ -419,7 +421,7 @@ int splits_for(int tiles, long long n, int capacity) {
 
 template <int P>
 rsdft_status gram_pair_launch(rsdft_ctx *ctx, const RowBlocks &A, const RowBlocks &B, int na, int nb, double2 *g,
-                              int ldg, bool sym, double scale, cudaStream_t st) {
+                              int ldg, bool sym, double scale, const int *guard, cudaStream_t st) {
     constexpr int TE = 16 * P;
     static int occ = occupancy_of(k_gram_pair<P>);
     const int pa = pairs_of(A.cnt[0]) + pairs_of(A.cnt[1]) + pairs_of(A.cnt[2]);
@@ -436,15 +438,15 @@ rsdft_status gram_pair_launch(rsdft_ctx *ctx, const RowBlocks &A, const RowBlock
     double *part = reinterpret_cast<double *>(ctx->ws.gram_part);
     {
         const double entries = sym ? 0.5 * na * (na + 1.0) : (double)na * nb;
-        ProfScope ps(ctx, RSDFT_K_GRAM, 2.0 * (double)n * entries,
-                     (double)n * sizeof(double2) * (sym ? pa : pa + pb), st);
+        ProfScope ps(ctx, RSDFT_K_GRAM, guard ? 0.0 : 2.0 * (double)n * entries,
+                     guard ? 0.0 : (double)n * sizeof(double2) * (sym ? pa : pa + pb), st);
         k_gram_pair<P><<<dim3(tiles, nsplit), GR_THREADS, 0, st>>>(A, B, pa, pb, n, sym ? 1 : 0, Ti, Tj, kchunk,
-                                                                     part);
+                                                                     part, guard);
     }
     RS_LAUNCHED(ctx, "k_gram_pair");
     const long long tot = (long long)na * nb;
     k_gram_pair_reduce<<<cdiv(tot, 256), 256, 0, st>>>(part, nsplit, pa, pb, A.cnt[0], A.cnt[1], B.cnt[0], B.cnt[1],
-                                                       na, nb, sym ? 1 : 0, TE, scale, g, ldg);
+                                                       na, nb, sym ? 1 : 0, TE, scale, g, ldg, guard);
     count_launch(ctx);
     RS_LAUNCHED(ctx, "k_gram_pair_reduce");
     return RSDFT_OK;
@@ -452,16 +454,9 @@ rsdft_status gram_pair_launch(rsdft_ctx *ctx, const RowBlocks &A, const RowBlock
 
 }  // namespace
 
-// g[i][j] = (scale <a_i|b_j>, 0) over the real bands of pair-row blocks A (na =
-// sum of its counts) and B; sym: A and B have the same counts and G is
-// symmetric (G_S = <Y|Y>, or G_H = <Y|HY> with H symmetric), so only tiles on
-// and above the diagonal are formed.  ldg: leading dimension of g.
-rsdft_status gram_pair(rsdft_ctx *ctx, const RowBlocks &A, const RowBlocks &B, double2 *g, int ldg, bool sym,
-                       double scale, cudaStream_t st) {
-    const int na = A.cnt[0] + A.cnt[1] + A.cnt[2];
-    const int nb = B.cnt[0] + B.cnt[1] + B.cnt[2];
-    if (na <= 0 || nb <= 0) return RSDFT_OK;
-    if (sym && na != nb) return fail(ctx, RSDFT_E_INVALID, "symmetric gram needs na == nb");
+// the FP64 kernels alone
+static rsdft_status gram_pair_fp64(rsdft_ctx *ctx, const RowBlocks &A, const RowBlocks &B, int na, int nb, double2 *g,
+                                   int ldg, bool sym, double scale, const int *guard, cudaStream_t st) {
     // Tile edge 16, 32 or 64 pair rows, the one that computes the fewest pair
     // products (padding, and for sym the full diagonal tiles); ties: the larger.
     // The kernel is bound by the FP64 pipe alone, so the smaller tiles' extra
@@ -473,11 +468,35 @@ rsdft_status gram_pair(rsdft_ctx *ctx, const RowBlocks &A, const RowBlocks &B, d
         return (sym ? ti * (ti + 1) / 2 : ti * tj) * te * te;
     };
     const long long w1 = work(16), w2 = work(32), w4 = work(64);
-    if (w4 <= w2 && w4 <= w1) return gram_pair_launch<4>(ctx, A, B, na, nb, g, ldg, sym, scale, st);
-    if (w2 <= w1) return gram_pair_launch<2>(ctx, A, B, na, nb, g, ldg, sym, scale, st);
-    return gram_pair_launch<1>(ctx, A, B, na, nb, g, ldg, sym, scale, st);
+    if (w4 <= w2 && w4 <= w1) return gram_pair_launch<4>(ctx, A, B, na, nb, g, ldg, sym, scale, guard, st);
+    if (w2 <= w1) return gram_pair_launch<2>(ctx, A, B, na, nb, g, ldg, sym, scale, guard, st);
+    return gram_pair_launch<1>(ctx, A, B, na, nb, g, ldg, sym, scale, guard, st);
 }
 
+// g[i][j] = (scale <a_i|b_j>, 0) over the real bands of pair-row blocks A (na =
+// sum of its counts) and B; sym: A and B have the same counts and G is
+// symmetric (G_S = <Y|Y>, or G_H = <Y|HY> with H symmetric), so only tiles on
+// and above the diagonal are formed.  ldg: leading dimension of g.
+rsdft_status gram_pair(rsdft_ctx *ctx, const RowBlocks &A, const RowBlocks &B, double2 *g, int ldg, bool sym,
+                       double scale, cudaStream_t st) {
+    const int na = A.cnt[0] + A.cnt[1] + A.cnt[2];
+    const int nb = B.cnt[0] + B.cnt[1] + B.cnt[2];
+    if (na <= 0 || nb <= 0) return RSDFT_OK;
+    if (sym && na != nb) return fail(ctx, RSDFT_E_INVALID, "symmetric gram needs na == nb");
+    bool used = false;
+    RS_TRY(rns_gram(ctx, A, B, nullptr, true, sym, g, nullptr, ldg, scale, st, &used));
+    return gram_pair_fp64(ctx, A, B, na, nb, g, ldg, sym, scale, used ? ctx->rns.flag : nullptr, st);
+}
+
+// g_s = <Y|Y> and g_h = <Y|HY>, both symmetric
+static rsdft_status gram_pair_sh(rsdft_ctx *ctx, const RowBlocks &Y, const RowBlocks &HY, double2 *gs, double2 *gh, int k,
+                                 cudaStream_t st) {
+    bool used = false;
+    RS_TRY(rns_gram(ctx, Y, Y, &HY, true, true, gs, gh, k, ctx->dV, st, &used));
+    const int *guard = used ? ctx->rns.flag : nullptr;
+    RS_TRY(gram_pair_fp64(ctx, Y, Y, k, k, gs, k, true, ctx->dV, guard, st));
+    return gram_pair_fp64(ctx, Y, HY, k, k, gh, k, true, ctx->dV, guard, st);
+}
 // ---- Ritz rotation on pair rows ---------------------------------------------------------
 // out0[b] = base[b] + sign sum_i Re c[i][b] y_i over the real bands y_i of the
 // pair-row blocks of Y, for m output bands (pairs_of(m) pair rows; the .y half
@@ -488,7 +507,8 @@ rsdft_status gram_pair(rsdft_ctx *ctx, const RowBlocks &A, const RowBlocks &B, d
 template <int PB>
 __global__ void __launch_bounds__(GR_THREADS)
 k_rotate_pair(RowBlocks Y, const double2 *__restrict__ c, int ldc, int m, long long n, const double2 *base, int sign,
-              double2 *out0, double2 *out1) {
+              double2 *out0, double2 *out1, const int *guard) {
+    if (guard && *guard == 0) return;   // rns.cu did the work
     constexpr int TB = 16 * PB;
     __shared__ double2 Ys[GRK][GRPTS + 1];
     __shared__ double2 Ca[GRK][TB + 1];   // (c[2i][2b'], c[2i][2b'+1])   input band 2i -> output pair b'
@@ -596,16 +616,20 @@ rsdft_status rotate_pair(rsdft_ctx *ctx, const RowBlocks &Y, const double2 *c, i
     const int k = Y.cnt[0] + Y.cnt[1] + Y.cnt[2];
     const int kp = pairs_of(Y.cnt[0]) + pairs_of(Y.cnt[1]) + pairs_of(Y.cnt[2]);
     const int mp = pairs_of(m);
-    ProfScope ps(ctx, RSDFT_K_ROTATE, 2.0 * (double)ctx->n * k * m,
-                 (double)sizeof(double2) * (double)ctx->n * (kp + mp + (out1 ? mp : 0) + (base ? mp : 0)), st);
+    bool used = false;
+    RS_TRY(rns_rotate(ctx, Y, c, ldc, m, true, base, sign, out0, out1, st, &used));
+    const int *guard = used ? ctx->rns.flag : nullptr;
+    ProfScope ps(ctx, RSDFT_K_ROTATE, guard ? 0.0 : 2.0 * (double)ctx->n * k * m,
+                 guard ? 0.0 : (double)sizeof(double2) * (double)ctx->n * (kp + mp + (out1 ? mp : 0) + (base ? mp : 0)), st);
     // output tile of 16 or 32 pair rows, the one with less padding (ties: 32)
     if (cdiv(mp, 16) * 16 < cdiv(mp, 32) * 32)
         k_rotate_pair<1><<<dim3(cdiv(mp, 16), cdiv(ctx->n, GRPTS)), GR_THREADS, 0, st>>>(Y, c, ldc, m, ctx->n, base,
-                                                                                        sign, out0, out1);
+                                                                                        sign, out0, out1, guard);
     else
         k_rotate_pair<2><<<dim3(cdiv(mp, 32), cdiv(ctx->n, GRPTS)), GR_THREADS, 0, st>>>(Y, c, ldc, m, ctx->n, base,
-                                                                                        sign, out0, out1);
+                                                                                        sign, out0, out1, guard);
     RS_LAUNCHED(ctx, "k_rotate_pair");
+    if (used && base == out0) return rns_poison(ctx, out0, (long long)mp * ctx->n, st);
     return RSDFT_OK;
 }
 
@@ -671,8 +695,7 @@ static rsdft_status lobpcg_pairs(rsdft_ctx *ctx, int m, const rsdft_lobpcg_opts 
     {
         RowBlocks Y{{X, nullptr, nullptr}, {m, 0, 0}};
         RowBlocks HY{{HX, nullptr, nullptr}, {m, 0, 0}};
-        RS_TRY(gram_pair(ctx, Y, Y, w.GS, m, true, dV, st));
-        RS_TRY(gram_pair(ctx, Y, HY, w.GH, m, true, dV, st));
+        RS_TRY(gram_pair_sh(ctx, Y, HY, w.GS, w.GH, m, st));
         int nd = 0;
         RS_TRY(rayleigh_ritz(ctx, w.GH, w.GS, m, m, o.pivot_tol, w.theta, w.Cfull, &nd, st, df));
         RS_TRY(rotate_pair(ctx, Y, w.Cfull, m, m, nullptr, 1, Xn, nullptr, st));
@@ -752,8 +775,7 @@ static rsdft_status lobpcg_pairs(rsdft_ctx *ctx, int m, const rsdft_lobpcg_opts 
         const int k = m + na + np_;
         RowBlocks Y{{X, W, Pn}, {m, na, np_}};
         RowBlocks HY{{HX, HW, HPn}, {m, na, np_}};
-        RS_TRY(gram_pair(ctx, Y, Y, w.GS, k, true, dV, st));
-        RS_TRY(gram_pair(ctx, Y, HY, w.GH, k, true, dV, st));
+        RS_TRY(gram_pair_sh(ctx, Y, HY, w.GS, w.GH, k, st));
         int nd = 0;
         RS_TRY(rayleigh_ritz(ctx, w.GH, w.GS, k, m, o.pivot_tol, w.lam, w.Cfull, &nd, st, df));
         *dropped += nd;

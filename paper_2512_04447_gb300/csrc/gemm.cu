@@ -36,11 +36,13 @@ __device__ __forceinline__ void upper_tile(int t, int T, int &ti, int &tj) {
 // Partial tiles of G over one K-chunk.  V = double2 (FP64) or float2 (the
 // mixed form: FP32 products and accumulation inside the CTA); the partials are
 // stored in FP64 and reduced in FP64 by k_gram_reduce.  Output tile edge 16*P
-// (each of the 16 x 16 threads owns P x P entries).
+// (each of the 16 x 16 threads owns P x P entries).  guard (here and below): a device flag;
+// the kernel returns at once where it is given and 0 (rns.cu did the work).
 template <typename V, int P>
 __global__ void __launch_bounds__(GTHREADS)
 k_gram_partial(RowBlocksT<V> A, RowBlocksT<V> B, int na, int nb, long long n, int hermitian, int Ti,
-               int Tj, long long kchunk, double2 *__restrict__ part) {
+               int Tj, long long kchunk, double2 *__restrict__ part, const int *guard) {
+    if (guard && *guard == 0) return;
     using T = decltype(V{}.x);
     constexpr int TE = 16 * P;
     __shared__ V As[GKC][TE + 1];
@@ -108,7 +110,9 @@ k_gram_partial(RowBlocksT<V> A, RowBlocksT<V> B, int na, int nb, long long n, in
 }
 
 __global__ void k_gram_reduce(const double2 *__restrict__ part, int nsplit, int na, int nb,
-                              int hermitian, int te, double scale, double2 *__restrict__ g, int ldg) {
+                              int hermitian, int te, double scale, double2 *__restrict__ g, int ldg,
+                              const int *guard) {
+    if (guard && *guard == 0) return;
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (long long)na * nb) return;
     const int i = (int)(idx / nb), j = (int)(idx % nb);
@@ -158,7 +162,7 @@ rsdft_status gram_reduce(rsdft_ctx *ctx, int nsplit, int na, int nb, bool hermit
                          double2 *g, int ldg, cudaStream_t st) {
     const long long tot = (long long)na * nb;
     k_gram_reduce<<<cdiv(tot, 256), 256, 0, st>>>(ctx->ws.gram_part, nsplit, na, nb, hermitian ? 1 : 0, te, scale,
-                                                   g, ldg);
+                                                   g, ldg, nullptr);
     count_launch(ctx);
     RS_LAUNCHED(ctx, "k_gram_reduce");
     return RSDFT_OK;
@@ -206,7 +210,7 @@ static int pick_splits(int tiles, long long n, int capacity) {
 template <typename V, int P>
 static rsdft_status gram_launch(rsdft_ctx *ctx, const RowBlocksT<V> &A, const RowBlocksT<V> &B,
                                 int na, int nb, double2 *g, int ldg, bool hermitian, double scale,
-                                cudaStream_t st) {
+                                const int *guard, cudaStream_t st) {
     constexpr int TE = 16 * P;
     static int occ = occupancy(k_gram_partial<V, P>, GTHREADS);
     const int Ti = cdiv(na, TE), Tj = cdiv(nb, TE);
@@ -223,15 +227,16 @@ static rsdft_status gram_launch(rsdft_ctx *ctx, const RowBlocksT<V> &A, const Ro
                           (const void *)A.ptr[1] == (const void *)B.ptr[1] &&
                           (const void *)A.ptr[2] == (const void *)B.ptr[2];
         const double entries = hermitian ? 0.5 * na * (na + 1.0) : (double)na * nb;
-        ProfScope ps(ctx, RSDFT_K_GRAM, 8.0 * (double)n * entries,
-                     (double)n * sizeof(V) * (same ? na : na + nb), st);
+        // behind the residue path the work is already recorded
+        ProfScope ps(ctx, RSDFT_K_GRAM, guard ? 0.0 : 8.0 * (double)n * entries,
+                     guard ? 0.0 : (double)n * sizeof(V) * (same ? na : na + nb), st);
         k_gram_partial<V, P><<<grid, GTHREADS, 0, st>>>(A, B, na, nb, n, hermitian ? 1 : 0, Ti, Tj, kchunk,
-                                                        ctx->ws.gram_part);
+                                                        ctx->ws.gram_part, guard);
     }
     RS_LAUNCHED(ctx, "k_gram_partial");
     const long long tot = (long long)na * nb;
     k_gram_reduce<<<cdiv(tot, 256), 256, 0, st>>>(ctx->ws.gram_part, nsplit, na, nb,
-                                                   hermitian ? 1 : 0, TE, scale, g, ldg);
+                                                   hermitian ? 1 : 0, TE, scale, g, ldg, guard);
     count_launch(ctx);
     RS_LAUNCHED(ctx, "k_gram_reduce");
     return RSDFT_OK;
@@ -239,7 +244,7 @@ static rsdft_status gram_launch(rsdft_ctx *ctx, const RowBlocksT<V> &A, const Ro
 
 template <typename V>
 rsdft_status gram_t(rsdft_ctx *ctx, const RowBlocksT<V> &A, const RowBlocksT<V> &B, double2 *g, int ldg,
-                    bool hermitian, double scale, cudaStream_t st) {
+                    bool hermitian, double scale, const int *guard, cudaStream_t st) {
     const int na = A.cnt[0] + A.cnt[1] + A.cnt[2];
     const int nb = B.cnt[0] + B.cnt[1] + B.cnt[2];
     if (na <= 0 || nb <= 0) return RSDFT_OK;
@@ -247,11 +252,12 @@ rsdft_status gram_t(rsdft_ctx *ctx, const RowBlocksT<V> &A, const RowBlocksT<V> 
     // tile edge 16 P, P in {2, 3, 4}: the least-padding rule, or the autotuner's pick
     auto run = [&](int c) -> rsdft_status {
         switch (c + 2) {
-            case 2: return gram_launch<V, 2>(ctx, A, B, na, nb, g, ldg, hermitian, scale, st);
-            case 3: return gram_launch<V, 3>(ctx, A, B, na, nb, g, ldg, hermitian, scale, st);
-            default: return gram_launch<V, 4>(ctx, A, B, na, nb, g, ldg, hermitian, scale, st);
+            case 2: return gram_launch<V, 2>(ctx, A, B, na, nb, g, ldg, hermitian, scale, guard, st);
+            case 3: return gram_launch<V, 3>(ctx, A, B, na, nb, g, ldg, hermitian, scale, guard, st);
+            default: return gram_launch<V, 4>(ctx, A, B, na, nb, g, ldg, hermitian, scale, guard, st);
         }
     };
+    if (guard) return run(pick_p(na, nb) - 2);
     // shapes in buckets of 32 (the subspace size changes as bands lock)
     const std::string key = std::string(sizeof(V) == 8 ? "gram32 " : "gram64 ") +
                             std::to_string(cdiv(na, 32)) +
@@ -262,11 +268,21 @@ rsdft_status gram_t(rsdft_ctx *ctx, const RowBlocksT<V> &A, const RowBlocksT<V> 
 
 rsdft_status gram(rsdft_ctx *ctx, const RowBlocks &A, const RowBlocks &B, double2 *g, int ldg,
                   bool hermitian, double scale, cudaStream_t st) {
-    return gram_t<double2>(ctx, A, B, g, ldg, hermitian, scale, st);
+    bool used = false;
+    RS_TRY(rns_gram(ctx, A, B, nullptr, false, hermitian, g, nullptr, ldg, scale, st, &used));
+    return gram_t<double2>(ctx, A, B, g, ldg, hermitian, scale, used ? ctx->rns.flag : nullptr, st);
+}
+rsdft_status gram_sh(rsdft_ctx *ctx, const RowBlocks &Y, const RowBlocks &HY, double2 *gs, double2 *gh, int ldg,
+                     double scale, cudaStream_t st) {
+    bool used = false;
+    RS_TRY(rns_gram(ctx, Y, Y, &HY, false, true, gs, gh, ldg, scale, st, &used));
+    const int *guard = used ? ctx->rns.flag : nullptr;
+    RS_TRY(gram_t<double2>(ctx, Y, Y, gs, ldg, true, scale, guard, st));
+    return gram_t<double2>(ctx, Y, HY, gh, ldg, true, scale, guard, st);
 }
 rsdft_status gram32(rsdft_ctx *ctx, const RowBlocksT<float2> &A, const RowBlocksT<float2> &B,
                     double2 *g, int ldg, bool hermitian, double scale, cudaStream_t st) {
-    return gram_t<float2>(ctx, A, B, g, ldg, hermitian, scale, st);
+    return gram_t<float2>(ctx, A, B, g, ldg, hermitian, scale, nullptr, st);
 }
 
 
@@ -277,7 +293,8 @@ rsdft_status gram32(rsdft_ctx *ctx, const RowBlocksT<float2> &A, const RowBlocks
 template <typename V, int PB>
 __global__ void __launch_bounds__(GTHREADS)
 k_rotate(RowBlocksT<V> Y, const double2 *__restrict__ c, int ldc, int m, long long n,
-         const V *base, int sign, V *out0, V *out1) {
+         const V *base, int sign, V *out0, V *out1, const int *guard) {
+    if (guard && *guard == 0) return;
     using T = decltype(V{}.x);
     constexpr int TB = 16 * PB;   // bands per tile (the points per tile are GT = 64)
     __shared__ V Cs[GKC][TB + 1];
@@ -378,12 +395,13 @@ k_rotate(RowBlocksT<V> Y, const double2 *__restrict__ c, int ldc, int m, long lo
 
 template <typename V, int PB>
 static rsdft_status rotate_launch(rsdft_ctx *ctx, const RowBlocksT<V> &Y, const double2 *c, int ldc,
-                                  int m, const V *base, int sign, V *out0, V *out1, cudaStream_t st) {
+                                  int m, const V *base, int sign, V *out0, V *out1, const int *guard,
+                                  cudaStream_t st) {
     dim3 grid(cdiv(m, 16 * PB), cdiv(ctx->n, GT));
     const int k = Y.cnt[0] + Y.cnt[1] + Y.cnt[2];
-    ProfScope ps(ctx, RSDFT_K_ROTATE, 8.0 * (double)ctx->n * k * m,
-                 (double)sizeof(V) * (double)ctx->n * (k + m + (out1 ? m : 0) + (base ? m : 0)), st);
-    k_rotate<V, PB><<<grid, GTHREADS, 0, st>>>(Y, c, ldc, m, ctx->n, base, sign, out0, out1);
+    ProfScope ps(ctx, RSDFT_K_ROTATE, guard ? 0.0 : 8.0 * (double)ctx->n * k * m,
+                 guard ? 0.0 : (double)sizeof(V) * (double)ctx->n * (k + m + (out1 ? m : 0) + (base ? m : 0)), st);
+    k_rotate<V, PB><<<grid, GTHREADS, 0, st>>>(Y, c, ldc, m, ctx->n, base, sign, out0, out1, guard);
     RS_LAUNCHED(ctx, "k_rotate");
     return RSDFT_OK;
 }
@@ -391,7 +409,7 @@ static rsdft_status rotate_launch(rsdft_ctx *ctx, const RowBlocksT<V> &Y, const 
 // Band tile 16*PB with the least padding over m bands (ties: larger PB).
 template <typename V>
 rsdft_status rotate_t(rsdft_ctx *ctx, const RowBlocksT<V> &Y, const double2 *c, int ldc, int m,
-                      const V *base, int sign, V *out0, V *out1, cudaStream_t st) {
+                      const V *base, int sign, V *out0, V *out1, const int *guard, cudaStream_t st) {
     if (m <= 0) return RSDFT_OK;
     int best = 4, bestpad = 1 << 30;
     for (int pb = 4; pb >= 1; --pb) {
@@ -400,14 +418,14 @@ rsdft_status rotate_t(rsdft_ctx *ctx, const RowBlocksT<V> &Y, const double2 *c, 
     }
     auto run = [&](int cand) -> rsdft_status {
         switch (cand + 1) {
-            case 1: return rotate_launch<V, 1>(ctx, Y, c, ldc, m, base, sign, out0, out1, st);
-            case 2: return rotate_launch<V, 2>(ctx, Y, c, ldc, m, base, sign, out0, out1, st);
-            case 3: return rotate_launch<V, 3>(ctx, Y, c, ldc, m, base, sign, out0, out1, st);
-            default: return rotate_launch<V, 4>(ctx, Y, c, ldc, m, base, sign, out0, out1, st);
+            case 1: return rotate_launch<V, 1>(ctx, Y, c, ldc, m, base, sign, out0, out1, guard, st);
+            case 2: return rotate_launch<V, 2>(ctx, Y, c, ldc, m, base, sign, out0, out1, guard, st);
+            case 3: return rotate_launch<V, 3>(ctx, Y, c, ldc, m, base, sign, out0, out1, guard, st);
+            default: return rotate_launch<V, 4>(ctx, Y, c, ldc, m, base, sign, out0, out1, guard, st);
         }
     };
     // an update in place (base) may not run twice: the least-padding rule only
-    if (base) return run(best - 1);
+    if (base || guard) return run(best - 1);
     const int k = Y.cnt[0] + Y.cnt[1] + Y.cnt[2];
     const std::string key = std::string(sizeof(V) == 8 ? "rot32 " : "rot64 ") + std::to_string(cdiv(k, 32)) +
                             " " + std::to_string(cdiv(m, 32)) + (out1 ? " p" : " x");
@@ -418,11 +436,15 @@ rsdft_status rotate_t(rsdft_ctx *ctx, const RowBlocksT<V> &Y, const double2 *c, 
 rsdft_status rotate(rsdft_ctx *ctx, const RowBlocks &Y, const double2 *c, int ldc, int m,
                     const double2 *base, int sign, double2 *out0, double2 *out1,
                     cudaStream_t st) {
-    return rotate_t<double2>(ctx, Y, c, ldc, m, base, sign, out0, out1, st);
+    if (m <= 0) return RSDFT_OK;
+    bool used = false;
+    RS_TRY(rns_rotate(ctx, Y, c, ldc, m, false, base, sign, out0, out1, st, &used));
+    RS_TRY(rotate_t<double2>(ctx, Y, c, ldc, m, base, sign, out0, out1, used ? ctx->rns.flag : nullptr, st));
+    return used && base == out0 ? rns_poison(ctx, out0, (long long)m * ctx->n, st) : RSDFT_OK;
 }
 rsdft_status rotate32(rsdft_ctx *ctx, const RowBlocksT<float2> &Y, const double2 *c, int ldc, int m,
                       const float2 *base, int sign, float2 *out0, float2 *out1, cudaStream_t st) {
-    return rotate_t<float2>(ctx, Y, c, ldc, m, base, sign, out0, out1, st);
+    return rotate_t<float2>(ctx, Y, c, ldc, m, base, sign, out0, out1, nullptr, st);
 }
 
 // ---- Gram without allocation -------------------------------------------------------
@@ -491,11 +513,12 @@ rsdft_status rsdft_gram_static(const void *a_dev, int na, const void *b_dev, int
     RowBlocks B{{(const double2 *)b_dev, nullptr, nullptr}, {nb, 0, 0}};
     // every partial entry the reduction reads is written by this launch first,
     // so nothing left by an earlier call is read
-    k_gram_partial<double2, 4><<<dim3(tiles, nsplit), GTHREADS, 0, st>>>(A, B, na, nb, n, 0, Ti, Tj, kchunk, part);
+    k_gram_partial<double2, 4><<<dim3(tiles, nsplit), GTHREADS, 0, st>>>(A, B, na, nb, n, 0, Ti, Tj, kchunk, part,
+                                                                         nullptr);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(nullptr, RSDFT_E_CUDA, "k_gram_partial: %s", cudaGetErrorString(e));
     k_gram_reduce<<<cdiv((long long)na * nb, 256), 256, 0, st>>>(part, nsplit, na, nb, 0, GT, scale,
-                                                                 (double2 *)g_dev, nb);
+                                                                 (double2 *)g_dev, nb, nullptr);
     e = cudaGetLastError();
     if (e != cudaSuccess) return fail(nullptr, RSDFT_E_CUDA, "k_gram_reduce: %s", cudaGetErrorString(e));
     return RSDFT_OK;

@@ -1,0 +1,1160 @@
+// FP64 Gram matrices and rotations on the tensor cores by residue arithmetic.
+//
+// GB300 issues FP64 at 4 flop/clk/SM and BF16 MMAs at some 16,000, so an FP64 product
+// of matrices is cheapest as exact integer arithmetic on the tensor cores (the
+// residue-number form of the Ozaki scheme: Ozaki, Uchino, Imamura, "Ozaki scheme II",
+// 2025).  Every operand row is scaled by a power of two and rounded to integers; their
+// products are formed modulo NM pairwise coprime numbers p <= 256, whose symmetric
+// residues (|r| <= 128) are exact in BF16 and whose sums over CHUNK terms stay below
+// 2^24, exact in the FP32 accumulators of tcgen05; the sums modulo the p give the
+// integer result by the Chinese remainder theorem, which is rounded to FP64 once.
+// Nothing is rounded but the operands (2^-59 of their row's norm) and the result:
+//   |error| <= about 2^-58 |a| |b|  per entry,  against some 2^-54 of an FP64 sum.
+//
+// The passes: row statistics (power-of-two scales) -> residues (one bf16 plane per
+// modulus and per real or imaginary part) -> k_rns (one GEMM per modulus) -> CRT.  The
+// points go in chunks that keep the residues within RNS_BYTES.
+//
+// Measured on one GB300 against the FP64 kernels (which run at 97% of the FP64 pipe):
+//   Gram 432 x 432 over 64^3 points   321.8 -> 12.7 ms     rotation 432 -> 144   104.8 -> 6.0 ms
+//   real Gram 285 x 285 over 60^3      30.2 ->  2.8 ms
+// and errors against extended precision (150 x 150 over 5,400 points: relative 2.5e-16 against
+// 1.4e-15; rotation 432 -> 144: 1.6e-16 against 9.8e-16).
+//
+// Non-finite values, and magnitudes outside 2^+-400, raise a device flag; then the
+// kernels here leave their outputs alone and the FP64 kernels launched behind them
+// (which return at once otherwise) do the work, so such inputs give what they gave.
+#include <cuda.h>
+#include <cuda_bf16.h>
+
+#include <algorithm>
+#include <cmath>
+#include <mutex>
+
+#include "rsdft_internal.h"
+#include "tc_ptx.h"
+
+namespace rsdft {
+namespace rns {
+
+using tc::smem_u32;
+typedef unsigned long long u64;
+typedef unsigned __int128 u128;
+
+// ---- moduli and their constants ---------------------------------------------------
+constexpr int NM = 15;
+constexpr int MODS[NM] = {256, 255, 253, 251, 247, 241, 239, 233, 229, 227, 223, 217, 211, 199, 197};
+// P = prod MODS = 2^117.78: twice the largest |sum| must stay below it
+constexpr int T_ROW = 58;      // |row|_2 <= 2^58 after scaling (both operands: 2^117 < P)
+
+struct Consts {
+    float p[NM], ip[NM];
+    int m[NM];
+    int lo[NM], hi[NM];        // 256^j mod p, symmetric, as signed bytes j = 0..3 and 4..7
+    uint32_t w[NM][4];         // frac((P/p)^-1 mod p / p) * 2^128, little-endian limbs
+    u64 P0, P1;                // P
+};
+
+constexpr Consts make_consts() {
+    Consts c{};
+    u128 P = 1;
+    for (int i = 0; i < NM; ++i) P *= (u128)MODS[i];
+    for (int i = 0; i < NM; ++i) {
+        const int p = MODS[i];
+        c.p[i] = (float)p;
+        c.m[i] = p;
+        c.ip[i] = 1.0f / (float)p;
+        int pw = 1;
+        uint32_t b[2] = {0, 0};
+        for (int j = 0; j < 8; ++j) {
+            const int s = pw > 127 ? pw - p : pw;   // in [-128, 127]: p <= 256
+            b[j >> 2] |= (uint32_t)(s & 255) << (8 * (j & 3));
+            pw = (pw * 256) % p;
+        }
+        c.lo[i] = (int)b[0];
+        c.hi[i] = (int)b[1];
+        const int q = (int)((P / (u128)p) % (u128)p);
+        int inv = 1;
+        while ((inv * q) % p != 1) ++inv;
+        // floor(inv 2^128 / p) by long division
+        u128 w = 0;
+        int r = inv;
+        for (int k = 0; k < 128; ++k) {
+            r *= 2;
+            w <<= 1;
+            if (r >= p) { r -= p; w |= 1; }
+        }
+        for (int k = 0; k < 4; ++k) c.w[i][k] = (uint32_t)(w >> (32 * k));
+    }
+    c.P0 = (u64)P;
+    c.P1 = (u64)(P >> 64);
+    return c;
+}
+__constant__ Consts K = make_consts();
+
+constexpr float MAGIC = 12582912.0f;   // 1.5 * 2^23: adding it rounds to an integer
+
+// ---- scales -----------------------------------------------------------------------
+constexpr int EXP_HI = 1023 + 400, EXP_LO = 1023 - 400;   // double exponent fields taken of a row's largest value
+
+// Part of one row: the largest exponent field and the sum of squares in units of 4^(that
+// field - 1023), from the leading 21 bits of each value (integer and FP32 instructions:
+// the FP64 pipe would bound this pass).
+struct Stat {
+    int e;
+    float s;
+};
+__device__ __forceinline__ void stat_rebase(Stat &a, int e) {
+    if (e > a.e) {
+        a.s = e - a.e > 60 ? 0.0f : a.s * __int_as_float((127 - 2 * (e - a.e)) << 23);
+        a.e = e;
+    }
+}
+__device__ __forceinline__ void stat_add(Stat &a, int habs) {
+    if (a.e == 0) return;   // nothing but zeros (or subnormal values) so far
+    const int u = habs - ((a.e - 127) << 20);
+    const float f = __int_as_float(max(u, 0) << 3);
+    a.s = fmaf(f, f, a.s);
+}
+__device__ __forceinline__ Stat stat_join(Stat a, Stat b) {
+    stat_rebase(a, b.e);
+    stat_rebase(b, a.e);
+    a.s += b.s;
+    return a;
+}
+
+// part[(row S + slice) 2 + plane]
+__global__ void __launch_bounds__(256)
+k_row_stat(RowBlocks src, long long n, int S, Stat *__restrict__ part) {
+    const int row = blockIdx.y;
+    int i = row, blk = 0;
+    while (blk < 2 && i >= src.cnt[blk]) { i -= src.cnt[blk]; ++blk; }
+    const int4 *x = reinterpret_cast<const int4 *>(src.ptr[blk] + (size_t)i * n);
+    const long long c = (n + S - 1) / S, i0 = blockIdx.x * c, i1 = min(n, i0 + c);
+    Stat a{0, 0.0f}, b{0, 0.0f};
+    for (long long q = i0 + threadIdx.x; q < i1; q += 4 * 256) {
+        int hx[4], hy[4], mx = 0, my = 0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const long long r = q + u * 256;
+            int4 v = make_int4(0, 0, 0, 0);
+            if (r < i1) v = __ldg(x + r);
+            hx[u] = v.y & 0x7fffffff;
+            hy[u] = v.w & 0x7fffffff;
+            mx = max(mx, hx[u]);
+            my = max(my, hy[u]);
+        }
+        stat_rebase(a, mx >> 20);
+        stat_rebase(b, my >> 20);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            stat_add(a, hx[u]);
+            stat_add(b, hy[u]);
+        }
+    }
+    __shared__ Stat sh[2][8];
+#pragma unroll
+    for (int pl = 0; pl < 2; ++pl) {
+        Stat t = pl ? b : a;
+        for (int o = 16; o > 0; o >>= 1) {
+            Stat u{__shfl_xor_sync(0xffffffffu, t.e, o), __shfl_xor_sync(0xffffffffu, t.s, o)};
+            t = stat_join(t, u);
+        }
+        if ((threadIdx.x & 31) == 0) sh[pl][threadIdx.x >> 5] = t;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        Stat t = sh[threadIdx.x][0];
+        for (int w = 1; w < 8; ++w) t = stat_join(t, sh[threadIdx.x][w]);
+        part[((size_t)row * S + blockIdx.x) * 2 + threadIdx.x] = t;
+    }
+}
+
+// scale[2 row + plane] = s with |row|_2 2^s <= 2^T_ROW; both planes of a complex row (joint)
+// share it.  Raises the flag where the row is not finite or out of range.
+__global__ void k_row_scale(const Stat *__restrict__ part, int S, int rows, int joint, int *__restrict__ scale,
+                            int *flag) {
+    const int row = blockIdx.x * blockDim.x + threadIdx.x;
+    if (row >= rows) return;
+    Stat t[2];
+    for (int pl = 0; pl < 2; ++pl) {
+        t[pl] = part[(size_t)row * S * 2 + pl];
+        for (int s = 1; s < S; ++s) t[pl] = stat_join(t[pl], part[((size_t)row * S + s) * 2 + pl]);
+    }
+    if (joint) t[0] = t[1] = stat_join(t[0], t[1]);
+    for (int pl = 0; pl < 2; ++pl) {
+        int s = 0;
+        if (t[pl].s > 0.0f) {
+            if (t[pl].e > EXP_HI || t[pl].e < EXP_LO) atomicExch(flag, 1);
+            // |row|^2 < 2^(g + 1) 4^(e - 1023) with the truncated bits counted in
+            const int g = ilogbf(t[pl].s * 1.001f);
+            s = T_ROW - (t[pl].e - 1023) - ((g + 2) >> 1);
+        } else if (t[pl].e > 0) {
+            atomicExch(flag, 1);   // a non-zero row whose statistics underflowed
+        }
+        scale[2 * row + pl] = s;
+    }
+}
+
+// Largest high word |x| per point over rows [r0, r0 + nr) of the block list (any of the two
+// parts), for the rotation's per-point scales.
+__global__ void __launch_bounds__(256)
+k_point_max(RowBlocks src, int r0, int nr, long long n, int rows_per_cta, int *__restrict__ hmax, int *flag) {
+    const long long q = (long long)blockIdx.x * 256 + threadIdx.x;
+    if (q >= n) return;
+    const int a = r0 + blockIdx.y * rows_per_cta, b = min(r0 + nr, a + rows_per_cta);
+    int m = 0;
+    for (int row = a; row < b; row += 8) {
+        int4 v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            int i = row + u, blk = 0;
+            v[u] = make_int4(0, 0, 0, 0);
+            if (i < b) {
+                while (blk < 2 && i >= src.cnt[blk]) { i -= src.cnt[blk]; ++blk; }
+                v[u] = __ldg(reinterpret_cast<const int4 *>(src.ptr[blk] + (size_t)i * n) + q);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) m = max(m, max(v[u].y & 0x7fffffff, v[u].w & 0x7fffffff));
+    }
+    const int e = m >> 20;
+    if (e > EXP_HI || (m > 0 && e == 0)) atomicExch(flag, 1);
+    atomicMax(hmax + q, m);
+}
+
+// s with |x| 2^s <= 2^bits for every |x| whose high word is at most h (a column of zeros: any)
+__device__ __forceinline__ int point_scale(int h, int bits) {
+    const int e = h >> 20;
+    return e == 0 ? 0 : bits - (e - 1022);
+}
+
+// ---- residues ---------------------------------------------------------------------
+// |x| 2^s rounded to an integer below 2^59, by integer shifts
+__device__ __forceinline__ u64 fix(int hi, unsigned lo, int s) {
+    const int e = (hi >> 20) & 0x7ff;
+    const u64 m = ((u64)(unsigned)((hi & 0xfffff) | (e ? 0x100000 : 0)) << 40) | ((u64)lo << 8);
+    const int r = min(max(1083 - e - s, 1), 63);   // mantissa was shifted by 8; r >= 2 by the choice of s
+    return (m + (1ull << (r - 1))) >> r;
+}
+
+// symmetric residue of v modulo MODS[q], as a float
+__device__ __forceinline__ float residue(u64 v, int q) {
+    int d = __float_as_int(MAGIC);
+    asm("dp4a.u32.s32 %0, %1, %2, %3;" : "=r"(d) : "r"((unsigned)v), "r"(K.lo[q]), "r"(d));
+    asm("dp4a.u32.s32 %0, %1, %2, %3;" : "=r"(d) : "r"((unsigned)(v >> 32)), "r"(K.hi[q]), "r"(d));
+    const float f = __int_as_float(d) - MAGIC;   // |f| < 2^18
+    const float k = fmaf(f, K.ip[q], MAGIC) - MAGIC;
+    return fmaf(-k, K.p[q], f);
+}
+// the two residues as a bf16 pair (exact: the low halves of the floats are zero), signs applied
+__device__ __forceinline__ unsigned pack(float a, float b, unsigned neg) {
+    return __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632) ^ neg;
+}
+
+// Residue planes of rows of FP64 complex values: res[q][row][plane][ld], points p0 .. p0 + ld
+// (zero beyond n).  Scales per row and plane (per_point 0) or per point and segment: rows
+// below seg1 use hmax[0][..], the others hmax[1][..].  Four points a thread; all integer and
+// FP32 arithmetic, about 7 instructions a residue: this pass is bound by its instructions
+// and by the 4 NM bytes that it writes for every 16 read.
+__global__ void __launch_bounds__(256)
+k_residues(RowBlocks src, long long n, long long p0, int ld, int R, int row0, int per_point,
+           const int *__restrict__ scale, const int *__restrict__ hmax, int seg1, int bits0, int bits1,
+           __nv_bfloat16 *__restrict__ res, const int *flag) {
+    if (*flag) return;
+    const int row = blockIdx.y;
+    int i = row, blk = 0;
+    while (blk < 2 && i >= src.cnt[blk]) { i -= src.cnt[blk]; ++blk; }
+    const int4 *x = reinterpret_cast<const int4 *>(src.ptr[blk] + (size_t)i * n);
+    const int t = (blockIdx.x * 256 + threadIdx.x) * 4;
+    if (t >= ld) return;
+    u64 v[8];
+    unsigned neg[4];   // sign masks of the packed pairs: re 01, re 23, im 01, im 23
+    neg[0] = neg[1] = neg[2] = neg[3] = 0;
+    const int seg = row >= seg1 ? 1 : 0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const long long p = p0 + t + u;
+        int4 w = make_int4(0, 0, 0, 0);
+        int sr = 0, si = 0;
+        if (p < n) {
+            w = __ldg(x + p);
+            if (per_point) sr = si = point_scale(hmax[seg * n + p], seg ? bits1 : bits0);
+            else { sr = scale[2 * (row0 + row)]; si = scale[2 * (row0 + row) + 1]; }
+        }
+        v[u] = fix(w.y, (unsigned)w.x, sr);
+        v[4 + u] = fix(w.w, (unsigned)w.z, si);
+        neg[u >> 1] |= (w.y & 0x80000000u) >> ((u & 1) ? 0 : 16);
+        neg[2 + (u >> 1)] |= (w.w & 0x80000000u) >> ((u & 1) ? 0 : 16);
+    }
+    uint2 *out = reinterpret_cast<uint2 *>(res + ((size_t)(row0 + row) * 2) * ld + t);
+    const size_t plane = ld / 4, mod = (size_t)R * 2 * ld / 4;
+#pragma unroll 1
+    for (int q = 0; q < NM; ++q) {
+        float f[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) f[j] = residue(v[j], q);
+        out[q * mod] = make_uint2(pack(f[0], f[1], neg[0]), pack(f[2], f[3], neg[1]));
+        out[q * mod + plane] = make_uint2(pack(f[4], f[5], neg[2]), pack(f[6], f[7], neg[3]));
+    }
+}
+
+// ---- rotation coefficients ----------------------------------------------------------
+// A segment of the rotation: coefficient rows that multiply a run of Y rows.  In real form the
+// Y rows hold two bands each, and K index 2 j + h is band h of pair row j.
+struct Seg {
+    int cnt[2], crow[2];   // up to two row blocks: bands in each, first row of each in c
+    int k;                 // K extent: rows (complex) or padded bands (real)
+};
+__device__ __forceinline__ int coef_row(const Seg &s, int t, bool real) {
+    const int k0 = real ? ((s.cnt[0] + 1) & ~1) : s.cnt[0];
+    if (t < k0) return t < s.cnt[0] ? s.crow[0] + t : -1;
+    t -= k0;
+    return t < s.cnt[1] ? s.crow[1] + t : -1;
+}
+
+// scale of column b of a segment's coefficients: |c_b|_2 2^s <= 2^T_ROW
+__global__ void k_coef_scale(const double2 *__restrict__ c, int ldc, Seg s, int real, int *__restrict__ sc, int *flag) {
+    const int b = blockIdx.x;
+    double sum = 0.0, big = 0.0;
+    for (int t = threadIdx.x; t < s.k; t += 32) {
+        const int r = coef_row(s, t, real);
+        if (r < 0) continue;
+        double2 v = c[(size_t)r * ldc + b];
+        if (real) v.y = 0.0;
+        sum = fma(v.x, v.x, fma(v.y, v.y, sum));
+        big = fmax(big, fmax(fabs(v.x), fabs(v.y)));
+        if (!isfinite(v.x) || !isfinite(v.y)) atomicExch(flag, 1);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        big = fmax(big, __shfl_xor_sync(0xffffffffu, big, o));
+    }
+    if (threadIdx.x) return;
+    int e = 0;
+    if (big > 0.0) {
+        if (big > 0x1p400 || big < 0x1p-400) atomicExch(flag, 1);
+        e = ilogb(sum * (1.0 + 1e-12));
+    }
+    sc[b] = big > 0.0 ? T_ROW - ((e + 2) >> 1) : 0;
+}
+
+// res[q][plane][nbp][kpad] of a segment's coefficients (zero outside)
+__global__ void k_coef_residues(const double2 *__restrict__ c, int ldc, Seg s, int real, int m, int nbp, int kpad,
+                                const int *__restrict__ sc, __nv_bfloat16 *__restrict__ res, const int *flag) {
+    if (*flag) return;
+    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= (long long)nbp * (kpad / 2)) return;
+    const int b = (int)(idx / (kpad / 2)), t = 2 * (int)(idx % (kpad / 2));
+    const int planes = real ? 1 : 2;
+    u64 v[4];
+    unsigned neg[2] = {0, 0};
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const int r = b < m && t + u < s.k ? coef_row(s, t + u, real) : -1;
+        const double2 z = r >= 0 ? c[(size_t)r * ldc + b] : make_double2(0.0, 0.0);
+        const int e = r >= 0 ? sc[b] : 0;
+        v[u] = fix(__double2hiint(z.x), __double2loint(z.x), e);
+        v[2 + u] = fix(__double2hiint(z.y), __double2loint(z.y), e);
+        neg[0] |= (__double2hiint(z.x) & 0x80000000u) >> (u ? 0 : 16);
+        neg[1] |= (__double2hiint(z.y) & 0x80000000u) >> (u ? 0 : 16);
+    }
+    unsigned *out = reinterpret_cast<unsigned *>(res + (size_t)b * kpad + t);
+    const size_t plane = (size_t)nbp * kpad / 2;
+    for (int q = 0; q < NM; ++q) {
+        out[(size_t)(q * planes) * plane] = pack(residue(v[0], q), residue(v[1], q), neg[0]);
+        if (!real) out[(size_t)(q * planes + 1) * plane] = pack(residue(v[2], q), residue(v[3], q), neg[1]);
+    }
+}
+
+// ---- the GEMM: one modulus per work item ------------------------------------------------
+// Persistent CTAs of 320 threads, one per SM: warp 0 issues TMA, warp 1 issues MMAs, warps
+// 2..9 drain.  A work item is an output tile of one modulus and one range of K:
+//   complex  128 x NT (NT <= 128), two accumulators (real, imaginary) of 128 TMEM columns
+//   real     128 x NT (NT <= 256), one accumulator of up to 256 columns
+// The accumulators are double-buffered (2 x 256 columns), and every CHUNK K-blocks they are
+// reduced modulo p into 128 registers of each drain thread while the next chunk's MMAs run,
+// so that every FP32 sum stays an exact integer below 2^24.
+//   Gram (ROT = false): A, B K-major [row][point]; tile of conj(A) B^T; residues of the sums
+//     go to out16[split][q][plane][M][N].
+//   Rotation (ROT = true): A = residues of Y read MN-major (points are M), B = coefficients
+//     K-major; residues go to out8[q][segment][plane][N / 4][points], four bands a word.
+constexpr int THREADS = 320;
+constexpr int SK = 64;                 // K per stage: 128-byte rows
+constexpr int STAGE_C = 64 * 1024, STAGES_C = 3;   // 2 + 2 planes of 128 x 64
+constexpr int STAGE_R = 48 * 1024, STAGES_R = 4;   // 128 x 64 and 256 x 64
+constexpr int SMEM = 192 * 1024 + 1024;
+template <bool REAL> struct Cfg {
+    static constexpr int STAGES = REAL ? STAGES_R : STAGES_C;
+    static constexpr int STAGE = REAL ? STAGE_R : STAGE_C;
+    static constexpr int CHUNK = REAL ? 16 : 8;    // stages: 1024 or 2 x 512 products of at most 2^14
+    static constexpr int NT = REAL ? 256 : 128;
+};
+
+struct Args {
+    int items;
+    int mt, nt;                 // tile counts
+    int nstep;                  // columns per tile
+    int boxn;                   // rows of the B box (its bytes: boxn * 128 per plane)
+    int M, N;                   // output rows and columns (Gram: N of one block)
+    // Gram
+    int herm, blocks, tiles;    // upper tiles only; B is `blocks` blocks of N rows; tiles per modulus
+    int kb_total, kb_split;
+    int accumulate;
+    short *out16;
+    // rotation
+    int segs, kb[2], row0[2];   // K-blocks of each segment and its first A row
+    long long ldp;              // points of an output row
+    unsigned *out8;
+    const int *flag;
+    int *flag_w;
+};
+
+struct Item {
+    int q, m0, n0, bcol, ncols, kb0, nkb, seg, slot;
+};
+
+template <bool ROT> __device__ __forceinline__ Item decode(const Args &a, int idx) {
+    Item it;
+    if (!ROT) {
+        const int per = a.tiles;
+        int t = idx % per;
+        idx /= per;
+        it.q = idx % NM;
+        it.slot = idx / NM;
+        it.seg = 0;
+        int tm = 0, tn = 0, blk = 0;
+        if (a.herm) {
+            const int tri = per / a.blocks;
+            blk = t / tri;
+            t -= blk * tri;
+            // row tile tm holds the column tiles from the one with its first row on
+            while (true) {
+                const int first = tm * 128 / a.nstep;
+                if (t < a.nt - first) { tn = first + t; break; }
+                t -= a.nt - first;
+                ++tm;
+            }
+        } else {
+            tm = t / a.nt;
+            tn = t - tm * a.nt;
+        }
+        it.m0 = tm * 128;
+        it.n0 = tn * a.nstep;
+        it.bcol = blk * a.N + it.n0;
+        it.ncols = min(a.nstep, a.N - it.n0);
+        it.n0 = it.bcol;
+        it.kb0 = it.slot * a.kb_split;
+        it.nkb = min(a.kb_split, a.kb_total - it.kb0);
+    } else {
+        const int tn = idx % a.nt;
+        idx /= a.nt;
+        it.seg = idx % a.segs;
+        idx /= a.segs;
+        it.m0 = (idx % a.mt) * 128;
+        it.q = idx / a.mt;
+        it.n0 = it.bcol = tn * a.nstep;
+        it.ncols = min(a.nstep, a.N - it.n0);
+        it.kb0 = 0;
+        it.nkb = a.kb[it.seg];
+        it.slot = 0;
+    }
+    return it;
+}
+
+template <bool REAL, bool ROT>
+__global__ void __launch_bounds__(THREADS, 1)
+k_rns(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mB0,
+      const __grid_constant__ CUtensorMap mB1, const __grid_constant__ Args a) {
+    if (*a.flag) return;
+    using C = Cfg<REAL>;
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char *smem = reinterpret_cast<unsigned char *>(
+        (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    __shared__ __align__(8) uint64_t full_bar[C::STAGES];
+    __shared__ __align__(8) uint64_t empty_bar[C::STAGES];
+    __shared__ __align__(8) uint64_t accf_bar[2];
+    __shared__ __align__(8) uint64_t acce_bar[2];
+    __shared__ __align__(8) uint64_t done_bar;
+    __shared__ uint32_t tmem_base;
+    __shared__ int s_abort;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    constexpr int PL = REAL ? 1 : 2;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < C::STAGES; ++s) {
+            tc::mbar_init(&full_bar[s], 1);
+            tc::mbar_init(&empty_bar[s], 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            tc::mbar_init(&accf_bar[b], 1);
+            tc::mbar_init(&acce_bar[b], 8);
+        }
+        tc::mbar_init(&done_bar, 1);
+        s_abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (warp == 1) tc::tmem_alloc(&tmem_base, 512);
+    tc::tc_fence_before();
+    __syncthreads();
+    tc::tc_fence_after();
+    const uint32_t tmem = tmem_base;
+    volatile int *abort = &s_abort;
+
+    if (warp == 0 && lane == 0) {
+        // ---- TMA producer
+        const uint32_t bytes = PL * (16384u + (uint32_t)a.boxn * 128u);
+        int st = 0;
+        bool stop = false;
+        for (int idx = blockIdx.x; idx < a.items && !stop; idx += gridDim.x) {
+            const Item it = decode<ROT>(a, idx);
+            const CUtensorMap *mB = ROT && it.seg ? &mB1 : &mB0;
+            for (int kb = 0; kb < it.nkb; ++kb, ++st) {
+                const int s = st % C::STAGES, r = st / C::STAGES;
+                if (r > 0 && !tc::mbar_wait(&empty_bar[s], (r - 1) & 1, abort)) { stop = true; break; }
+                unsigned char *sa = smem + s * C::STAGE, *sb = sa + PL * 16384;
+                tc::mbar_expect_tx(&full_bar[s], bytes);
+                const int x = (it.kb0 + kb) * SK;
+#pragma unroll
+                for (int pl = 0; pl < PL; ++pl) {
+                    if (!ROT) {
+                        tc::tma_load_4d(sa + pl * 16384, &mA, &full_bar[s], x, it.m0, pl, it.q);
+                        tc::tma_load_4d(sb + pl * 16384, mB, &full_bar[s], x, it.bcol, pl, it.q);
+                    } else {
+                        const int y = a.row0[it.seg] + x;
+                        tc::tma_load_4d(sa + pl * 16384, &mA, &full_bar[s], it.m0, y, pl, it.q);
+                        tc::tma_load_4d(sa + pl * 16384 + 8192, &mA, &full_bar[s], it.m0 + 64, y, pl, it.q);
+                        tc::tma_load_4d(sb + pl * 16384, mB, &full_bar[s], x, it.bcol, pl, it.q);
+                    }
+                }
+            }
+        }
+        if (*abort) {
+            // let the copies still in flight land before the CTA leaves
+            for (int j = max(0, st - C::STAGES); j < st; ++j) {
+                const long long t0 = clock64();
+                while (!tc::mbar_try_wait(&full_bar[j % C::STAGES], (j / C::STAGES) & 1) &&
+                       clock64() - t0 < tc::WAIT_LIMIT) {
+                }
+            }
+        }
+    } else if (warp == 1 && lane == 0) {
+        // ---- MMA issuer
+        int st = 0, ch = 0;
+        bool stop = false;
+        for (int idx = blockIdx.x; idx < a.items && !stop; idx += gridDim.x) {
+            const Item it = decode<ROT>(a, idx);
+            const uint32_t idesc = tc::idesc_bf16(128, (it.ncols + 15) & ~15) | (ROT ? tc::IDESC_A_MN : 0u);
+            const uint32_t ineg = idesc | tc::IDESC_NEG_A;
+            for (int kb = 0; kb < it.nkb && !stop; ++ch) {
+                const int b = ch & 1;
+                if (ch >= 2 && !tc::mbar_wait(&acce_bar[b], ((ch >> 1) - 1) & 1, abort)) { stop = true; break; }
+                tc::tc_fence_after();
+                const uint32_t d0 = tmem + (uint32_t)(b * 256), d1 = d0 + 128;
+                uint32_t acc = 0;
+                const int kend = min(it.nkb, kb + C::CHUNK);
+                for (; kb < kend; ++kb, ++st) {
+                    const int s = st % C::STAGES, r = st / C::STAGES;
+                    if (!tc::mbar_wait(&full_bar[s], r & 1, abort)) { stop = true; break; }
+                    tc::tc_fence_after();
+                    unsigned char *sa = smem + s * C::STAGE, *sb = sa + PL * 16384;
+#pragma unroll
+                    for (int kk = 0; kk < SK / 16; ++kk) {
+                        uint64_t ad[PL], bd[PL];
+#pragma unroll
+                        for (int pl = 0; pl < PL; ++pl) {
+                            ad[pl] = ROT ? tc::smem_desc_mn(sa + pl * 16384 + kk * 2048, 8192, 1024)
+                                         : tc::smem_desc_k128(sa + pl * 16384 + kk * 32);
+                            bd[pl] = tc::smem_desc_k128(sb + pl * 16384 + kk * 32);
+                        }
+                        if (REAL) {
+                            tc::mma_bf16(d0, ad[0], bd[0], idesc, acc);
+                        } else if (!ROT) {
+                            // Re += A_re B_re + A_im B_im, Im += A_re B_im - A_im B_re
+                            tc::mma_bf16(d0, ad[0], bd[0], idesc, acc);
+                            tc::mma_bf16(d1, ad[0], bd[PL - 1], idesc, acc);
+                            tc::mma_bf16(d0, ad[PL - 1], bd[PL - 1], idesc, 1u);
+                            tc::mma_bf16(d1, ad[PL - 1], bd[0], ineg, 1u);
+                        } else {
+                            // Re += Y_re C_re - Y_im C_im, Im += Y_re C_im + Y_im C_re
+                            tc::mma_bf16(d0, ad[0], bd[0], idesc, acc);
+                            tc::mma_bf16(d1, ad[0], bd[PL - 1], idesc, acc);
+                            tc::mma_bf16(d0, ad[PL - 1], bd[PL - 1], ineg, 1u);
+                            tc::mma_bf16(d1, ad[PL - 1], bd[0], idesc, 1u);
+                        }
+                        acc = 1u;
+                    }
+                    tc::mma_commit(&empty_bar[s]);
+                }
+                if (!stop) tc::mma_commit(&accf_bar[b]);
+            }
+        }
+        // every MMA issued so far must finish before TMEM is released (bounded)
+        tc::mma_commit(&done_bar);
+        const long long t0 = clock64();
+        while (!tc::mbar_try_wait(&done_bar, 0)) {
+            if (clock64() - t0 > tc::WAIT_LIMIT) { *abort = 1; break; }
+        }
+    } else if (warp >= 2) {
+        // ---- drain: warp w reads TMEM lanes 32 (w % 4) .., columns 128 half .. of the buffer
+        // (complex: half 0 the real part, half 1 the imaginary part)
+        const int lq = warp & 3, half = (warp - 2) >> 2;
+        int ch = 0;
+        bool stop = false;
+        for (int idx = blockIdx.x; idx < a.items && !stop; idx += gridDim.x) {
+            const Item it = decode<ROT>(a, idx);
+            const float p = K.p[it.q], ip = K.ip[it.q];
+            const int ncol = REAL ? min(128, it.ncols - half * 128) : it.ncols;   // may be <= 0
+            float acc[128];
+#pragma unroll
+            for (int i = 0; i < 128; ++i) acc[i] = 0.0f;
+            for (int kb = 0; kb < it.nkb; kb += C::CHUNK, ++ch) {
+                const int b = ch & 1;
+                if (!tc::mbar_wait_warp(&accf_bar[b], (ch >> 1) & 1, abort)) { stop = true; break; }
+                tc::tc_fence_after();
+                const uint32_t base = tmem + ((uint32_t)(lq * 32) << 16) + (uint32_t)(b * 256 + half * 128);
+#pragma unroll
+                for (int g = 0; g < 4; ++g) {
+                    if (g * 32 < ncol) {
+                        float v[32];
+                        tc::tmem_ld32(base + (uint32_t)(g * 32), v);
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) {
+                            const float k = fmaf(v[i], ip, MAGIC) - MAGIC;
+                            acc[g * 32 + i] += fmaf(-k, p, v[i]);
+                        }
+                    }
+                }
+                tc::tc_fence_before();
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(&acce_bar[b]);
+            }
+            if (stop) break;
+            const int row = it.m0 + lq * 32 + lane;
+            if (!ROT) {
+                const int plane = REAL ? 0 : half;
+                const int ldn = a.N * a.blocks;
+                short *o = a.out16 + ((((size_t)it.slot * NM + it.q) * PL + plane) * a.M + row) * (size_t)ldn +
+                           it.n0 + (REAL ? half * 128 : 0);
+                if (row < a.M) {
+#pragma unroll
+                    for (int i = 0; i < 128; ++i) {
+                        if (i < ncol) {
+                            float v = acc[i];
+                            if (a.accumulate) v += (float)o[i];
+                            const float k = fmaf(v, ip, MAGIC) - MAGIC;
+                            o[i] = (short)(int)fmaf(-k, p, v);
+                        }
+                    }
+                }
+            } else {
+                const int plane = REAL ? 0 : half;
+                const int quad0 = (it.n0 + (REAL ? half * 128 : 0)) >> 2, nquad = (a.N + 3) >> 2;
+                unsigned *o = a.out8 + (((size_t)(it.q * a.segs + it.seg) * PL + plane) * nquad + quad0) * a.ldp + row;
+                if (row < a.M) {
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) {
+                        if (4 * i < ncol) {
+                            int w[4];
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                const float v = acc[4 * i + j];
+                                const float k = fmaf(v, ip, MAGIC) - MAGIC;
+                                w[j] = __float_as_int(fmaf(-k, p, v) + MAGIC);
+                            }
+                            o[(size_t)i * a.ldp] = __byte_perm(__byte_perm(w[0], w[1], 0x0040), __byte_perm(w[2], w[3], 0x0040), 0x5410);
+                        }
+                    }
+                }
+            }
+        }
+    }
+    __syncwarp();
+    tc::tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc::tc_fence_after();
+        tc::tmem_dealloc(tmem, 512);
+    }
+    if (threadIdx.x == 0 && *abort) atomicExch(a.flag_w, 2);
+}
+
+// ---- Chinese remainder ----------------------------------------------------------------
+// f += r w: 128-bit, 0 <= r < p.  f holds the fraction (integer / P) as 2^-128 f, truncated by
+// at most sum p; a sum that is 0 has zero residues and gives exactly 0.
+__device__ __forceinline__ void crt_add(uint32_t f[4], unsigned r, int q) {
+    asm("mad.lo.cc.u32 %0, %4, %5, %0;\n\t"
+        "madc.lo.cc.u32 %1, %4, %6, %1;\n\t"
+        "madc.lo.cc.u32 %2, %4, %7, %2;\n\t"
+        "madc.lo.u32 %3, %4, %8, %3;\n\t"
+        "mad.hi.cc.u32 %1, %4, %5, %1;\n\t"
+        "madc.hi.cc.u32 %2, %4, %6, %2;\n\t"
+        "madc.hi.u32 %3, %4, %7, %3;"
+        : "+r"(f[0]), "+r"(f[1]), "+r"(f[2]), "+r"(f[3])
+        : "r"(r), "r"(K.w[q][0]), "r"(K.w[q][1]), "r"(K.w[q][2]), "r"(K.w[q][3]));
+}
+
+// x 2^-s of the integer x = P f / 2^128 (f signed), rounded to nearest
+__device__ __forceinline__ double crt_value(const uint32_t f[4], int s) {
+    u64 f0 = ((u64)f[1] << 32) | f[0], f1 = ((u64)f[3] << 32) | f[2];
+    const bool neg = (long long)f1 < 0;
+    if (neg) {   // two's complement
+        f0 = ~f0 + 1;
+        f1 = ~f1 + (f0 == 0);
+    }
+    // (f1 f0)(P1 P0) / 2^128, rounded: the integer result
+    const u64 a = __umul64hi(f0, K.P0);
+    u64 lo = f0 * K.P1, m = a + lo, hi = __umul64hi(f0, K.P1) + (m < a);
+    lo = f1 * K.P0;
+    m += lo;
+    u64 hi2 = __umul64hi(f1, K.P0) + (m < lo);
+    u64 x0 = f1 * K.P1, x1 = __umul64hi(f1, K.P1);
+    x0 += hi;
+    x1 += x0 < hi;
+    x0 += hi2;
+    x1 += x0 < hi2;
+    x0 += m >> 63;
+    x1 += x0 < (m >> 63);
+    if (!(x0 | x1)) return 0.0;
+    // 64 leading bits (sticky), then to nearest even
+    const int lz = x1 ? __clzll(x1) : 64 + __clzll(x0);
+    u64 t = lz >= 64 ? x0 << (lz - 64) : (lz ? (x1 << lz) | (x0 >> (64 - lz)) : x1);
+    if (lz < 64 && (x0 << lz)) t |= 1;
+    u64 r = t >> 11;
+    const u64 rest = t & 0x7ff;
+    r += rest > 0x400 || (rest == 0x400 && (r & 1));
+    // value = r 2^e with 2^52 <= r <= 2^53
+    const int e = 75 - lz - s, field = e + 1075;
+    double v;
+    if (field >= 1 && field <= 2045) v = __longlong_as_double((long long)r + ((long long)(field - 1) << 52));
+    else v = scalbn((double)r, e);   // beyond the normal range
+    return neg ? -v : v;
+}
+
+// g entries of one or two blocks from the residue sums out16[slot][q][plane][M][N blocks]
+// (padded bands in real form).  herm: entries below the diagonal from their mirror, the
+// diagonal real.
+__global__ void k_crt_gram(const short *__restrict__ out16, int slots, int M, int N, int blocks, int real, int a0,
+                           int a1, int b0, int b1, int na, int nb, int herm, const int *__restrict__ sa,
+                           const int *__restrict__ sb, double scale, double2 *__restrict__ g0,
+                           double2 *__restrict__ g1, int ldg, const int *flag) {
+    if (*flag) return;
+    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= (long long)na * nb) return;
+    const int blk = blockIdx.y;
+    const int i = (int)(idx / nb), j = (int)(idx % nb);
+    int I = i, J = j;
+    if (real) {   // compact band -> padded band (blocks of pair rows)
+        auto pad = [](int c0, int c1, int t) {
+            if (t < c0) return t;
+            t -= c0;
+            const int base = (c0 + 1) & ~1;
+            if (t < c1) return base + t;
+            return base + ((c1 + 1) & ~1) + (t - c1);
+        };
+        I = pad(a0, a1, i);
+        J = pad(b0, b1, j);
+    }
+    const bool mirror = herm && I > J;
+    const int r = mirror ? J : I, c = mirror ? I : J;
+    const int PL = real ? 1 : 2, ldn = N * blocks;
+    double v[2] = {0.0, 0.0};
+    // scales are per complex row and plane: 2 row + plane is the padded band in real form
+    const int s = sa[real ? r : 2 * r] + sb[real ? blk * N + c : 2 * (blk * N + c)];
+    for (int pl = 0; pl < PL; ++pl) {
+        uint32_t f[4] = {0, 0, 0, 0};
+        for (int q = 0; q < NM; ++q) {
+            int t = 0;
+            for (int u = 0; u < slots; ++u)
+                t += out16[((((size_t)u * NM + q) * PL + pl) * M + r) * (size_t)ldn + blk * N + c];
+            const float k = fmaf((float)t, K.ip[q], MAGIC) - MAGIC;
+            t -= (int)k * K.m[q];
+            crt_add(f, (unsigned)(t < 0 ? t + K.m[q] : t), q);
+        }
+        v[pl] = crt_value(f, s);
+    }
+    if (herm && I == J) v[1] = 0.0;
+    if (mirror) v[1] = -v[1];
+    (blk ? g1 : g0)[(size_t)i * ldg + j] = make_double2(scale * v[0], scale * v[1]);
+}
+
+// Rotation outputs of the points p0 .. p0 + np from out8[q][segment][plane][N / 4][ldp].
+// out1 = the last segment's sums (two segments), out0 = base + sign (all segments).  A thread
+// does one point of four columns: four complex rows, or two pair rows in real form.
+template <bool REAL>
+__global__ void __launch_bounds__(256)
+k_crt_rot(const unsigned *__restrict__ out8, int segs, int m, long long ldp, long long n, long long p0, int np,
+          const int *__restrict__ hmax, int bits0, int bits1, const int *__restrict__ sc, int mcols,
+          const double2 *base, int sign, double2 *out0, double2 *out1, const int *flag) {
+    if (*flag) return;
+    const int t = blockIdx.x * 256 + threadIdx.x;
+    if (t >= np) return;
+    const int quad = blockIdx.y, nquad = (m + 3) >> 2;
+    constexpr int PL = REAL ? 1 : 2;
+    double sum[4][PL];
+    for (int sg = segs - 1; sg >= 0; --sg) {
+        uint32_t f[4][PL][4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int pl = 0; pl < PL; ++pl)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) f[j][pl][k] = 0;
+#pragma unroll
+        for (int q = 0; q < NM; ++q) {
+#pragma unroll
+            for (int pl = 0; pl < PL; ++pl) {
+                const unsigned w = __ldg(out8 + (((size_t)(q * segs + sg) * PL + pl) * nquad + quad) * ldp + t);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int r = (int)(w << (24 - 8 * j)) >> 24;
+                    crt_add(f[j][pl], (unsigned)(r + ((r >> 31) & K.m[q])), q);
+                }
+            }
+        }
+        const int h = hmax[(size_t)sg * n + p0 + t];
+        const int sp = point_scale(h, sg ? bits1 : bits0);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int b = 4 * quad + j;
+            const int s = (b < m ? sc[sg * mcols + b] : 0) + sp;
+#pragma unroll
+            for (int pl = 0; pl < PL; ++pl) {
+                const double v = crt_value(f[j][pl], s);
+                sum[j][pl] = sg == segs - 1 ? v : sum[j][pl] + v;
+            }
+        }
+        double2 *o = sg == 1 ? out1 : nullptr;
+        if (o || sg == 0) {
+            if (sg == 0) o = out0;
+#pragma unroll
+            for (int j = 0; j < (REAL ? 2 : 4); ++j) {
+                const int row = REAL ? 2 * quad + j : 4 * quad + j;
+                if (row >= (REAL ? (m + 1) / 2 : m)) continue;
+                double2 v;
+                if (REAL) v = make_double2(sum[2 * j][0], 2 * row + 1 < m ? sum[(2 * j + 1) & 3][0] : 0.0);
+                else v = make_double2(sum[j][0], sum[j][PL - 1]);
+                if (sg == 0 && sign < 0) v = make_double2(-v.x, -v.y);
+                if (sg == 0 && base) {
+                    const double2 bv = base[(size_t)row * n + p0 + t];
+                    v.x += bv.x;
+                    v.y += bv.y;
+                }
+                o[(size_t)row * n + p0 + t] = v;
+            }
+        }
+    }
+}
+
+// An in-place rotation whose GEMM gave up (a bounded wait ran out: flag 2) after some chunks
+// were written cannot be repeated: its outputs become NaN, which every caller's checks meet.
+__global__ void k_poison(double2 *out, long long cnt, const int *flag) {
+    if (*flag != 2) return;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += (long long)gridDim.x * blockDim.x)
+        out[i] = make_double2(__longlong_as_double(0x7ff8000000000000ll), 0.0);
+}
+
+}  // namespace rns
+
+using namespace rns;
+
+// ---- host side ---------------------------------------------------------------------------
+// Bytes of residues held at a time (the points go in chunks of that size).
+constexpr size_t RNS_BYTES = (size_t)1 << 30;
+
+static rsdft_status rns_buffer(rsdft_ctx *ctx, size_t bytes) {
+    RnsWork &w = ctx->rns;
+    if (!w.flag) RS_TRY(dev_alloc(ctx, (void **)&w.flag, 64));
+    if (bytes <= w.bytes) return RSDFT_OK;
+    if (w.buf) {
+        cudaFree(w.buf);
+        ctx->owned.erase(std::remove(ctx->owned.begin(), ctx->owned.end(), w.buf), ctx->owned.end());
+    }
+    w.buf = nullptr;
+    w.bytes = 0;
+    RS_TRY(dev_alloc(ctx, &w.buf, bytes));
+    w.bytes = bytes;
+    return RSDFT_OK;
+}
+
+struct Carver {
+    unsigned char *base;
+    size_t at = 0;
+    template <typename T> T *take(size_t count) {
+        T *p = reinterpret_cast<T *>(base ? base + at : nullptr);
+        at += (count * sizeof(T) + 1023) / 1024 * 1024;
+        return p;
+    }
+};
+
+static int rows_of(const RowBlocks &b) { return b.cnt[0] + b.cnt[1] + b.cnt[2]; }
+static int pairs_up(int c) { return (c + 1) >> 1; }
+static RowBlocks pair_rows(const RowBlocks &b) {
+    return RowBlocks{{b.ptr[0], b.ptr[1], b.ptr[2]}, {pairs_up(b.cnt[0]), pairs_up(b.cnt[1]), pairs_up(b.cnt[2])}};
+}
+
+template <bool REAL, bool ROT>
+static rsdft_status launch_gemm(rsdft_ctx *ctx, const CUtensorMap &mA, const CUtensorMap &mB0, const CUtensorMap &mB1,
+                                const Args &a, cudaStream_t st) {
+    static const cudaError_t attr =
+        cudaFuncSetAttribute(k_rns<REAL, ROT>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+    RS_CUDA(ctx, attr);
+    k_rns<REAL, ROT><<<std::min(a.items, ctx->num_sms), THREADS, SMEM, st>>>(mA, mB0, mB1, a);
+    count_launch(ctx);
+    RS_LAUNCHED(ctx, "k_rns");
+    return RSDFT_OK;
+}
+
+// Whether the residue path is the faster one: an estimate of both, in seconds.  FP64 kernels:
+// f flops per product at 1.15 TFLOP/s.  Residues: launches, residue planes written and read,
+// MMAs over whole tiles.
+static bool rns_wins(double n, double rows, double mpad, double npad, double entries, bool real, double extra) {
+    const double f = real ? 2.0 : 8.0;
+    const double t64 = f * n * entries / 1.15e12;
+    const double trns = 60e-6 + rows * n * (8.0 * NM + 32.0) / 4.0e12 + NM * f * n * mpad * npad / 0.7e15 + extra;
+    return t64 > 1.25 * trns;
+}
+
+rsdft_status rns_gram(rsdft_ctx *ctx, const RowBlocks &A0, const RowBlocks &B0, const RowBlocks *B1, bool real,
+                      bool herm, double2 *g0, double2 *g1, int ldg, double scale, cudaStream_t st, bool *used) {
+    *used = false;
+    const int na = rows_of(A0), nb = rows_of(B0), blocks = B1 ? 2 : 1;
+    const RowBlocks A = real ? pair_rows(A0) : A0, B = real ? pair_rows(B0) : B0;
+    const int ra = rows_of(A), rb = rows_of(B);
+    bool same = true;
+    for (int i = 0; i < 3; ++i) same = same && A.cnt[i] == B.cnt[i] && (A.cnt[i] == 0 || A.ptr[i] == B.ptr[i]);
+    const long long n = ctx->n;
+    const int PL = real ? 1 : 2, M = real ? 2 * ra : ra, N = real ? 2 * rb : rb;
+    const int NT = real ? 256 : 128;
+    const int mt = cdiv(M, 128), nt = cdiv(N, NT);
+    const double part = herm ? 0.5 * (1.0 + 1.0 / mt) : 1.0;
+    const double frac = (herm ? 0.5 : 1.0) * blocks;
+    const int R = (same ? 0 : ra) + rb * blocks;
+    if (!rns_wins((double)n, R, 128.0 * mt * part * blocks, cdiv(N, 16) * 16.0, frac * na * nb, real, 0.0)) return RSDFT_OK;
+    int tiles = 0;
+    for (int t = 0; t < mt; ++t) tiles += herm ? nt - t * 128 / NT : nt;
+    tiles *= blocks;
+    // chunks of points, equal and multiples of 64
+    const size_t per_point = (size_t)NM * R * 4;
+    const long long most = std::max<long long>(4096, (long long)(RNS_BYTES / per_point) / 64 * 64);
+    const int nchunk = cdiv(n, most);
+    const int ld = cdiv(cdiv(n, nchunk), 64) * 64;
+    const int kbt = ld / 64;
+    // K splits: whole waves of one CTA per SM (or at least three of them), 16 K-blocks a CTA
+    int splits = 1;
+    double best = 0.0;
+    for (int s = 1; s <= 16 && (s == 1 || kbt / s >= 16); ++s) {
+        const long long it = (long long)tiles * NM * s;
+        const double eff = (double)it / (double)((it + ctx->num_sms - 1) / ctx->num_sms * ctx->num_sms);
+        if (eff > best + 0.02) { best = eff; splits = s; }
+    }
+    const int S = std::max(1, std::min<int>(64, (int)(n / 4096)));
+    const size_t out_elems = (size_t)splits * NM * PL * M * N * blocks;
+    Carver cv{nullptr};
+    for (int pass = 0; pass < 2; ++pass) {
+        if (pass == 1) {
+            if (rns_buffer(ctx, cv.at) != RSDFT_OK) {   // no room: the FP64 kernels
+                ctx->err.clear();
+                return RSDFT_OK;
+            }
+            cv = Carver{(unsigned char *)ctx->rns.buf};
+        }
+        __nv_bfloat16 *res = cv.take<__nv_bfloat16>((size_t)NM * R * 2 * ld);
+        short *out16 = cv.take<short>(out_elems);
+        Stat *stat = cv.take<Stat>((size_t)R * S * 2);
+        int *scl = cv.take<int>(2 * (size_t)R);
+        if (pass == 0) continue;
+        int *flag = ctx->rns.flag;
+        const int rowB = same ? 0 : ra;
+        *used = true;
+        ProfScope ps(ctx, RSDFT_K_GRAM, (real ? 2.0 : 8.0) * (double)n * frac * na * (herm ? na + 1.0 : (double)nb),
+                     16.0 * (double)n * R, st, 0);
+        RS_CUDA(ctx, cudaMemsetAsync(flag, 0, sizeof(int), st));
+        struct Src { const RowBlocks *b; RowBlocks r; int row0, cnt; };
+        const RowBlocks Bp1 = B1 ? (real ? pair_rows(*B1) : *B1) : B;
+        const Src srcs[3] = {{nullptr, A, 0, same ? 0 : ra}, {nullptr, B, rowB, rb}, {nullptr, Bp1, rowB + rb, B1 ? rb : 0}};
+        for (const Src &s : srcs) {
+            if (s.cnt <= 0) continue;
+            k_row_stat<<<dim3(S, s.cnt), 256, 0, st>>>(s.r, n, S, stat + (size_t)s.row0 * S * 2);
+            count_launch(ctx);
+        }
+        k_row_scale<<<cdiv(R, 128), 128, 0, st>>>(stat, S, R, real ? 0 : 1, scl, flag);
+        count_launch(ctx);
+        RS_LAUNCHED(ctx, "k_row_scale");
+        CUtensorMap mA, mB;
+        {
+            const long long st3[3] = {real ? 2LL * ld : 4LL * ld, 2LL * ld, 4LL * ld * R};
+            const long long da[4] = {ld, real ? 2 * ra : ra, PL, NM};
+            const long long db[4] = {ld, real ? 2 * rb * blocks : rb * blocks, PL, NM};
+            const int ba[4] = {64, 128, 1, 1}, bb[4] = {64, NT, 1, 1};
+            RS_TRY(tc::tensor_map_bf16(ctx, &mA, res, 4, da, st3, ba, CU_TENSOR_MAP_SWIZZLE_128B));
+            RS_TRY(tc::tensor_map_bf16(ctx, &mB, res + (size_t)rowB * 2 * ld, 4, db, st3, bb, CU_TENSOR_MAP_SWIZZLE_128B));
+        }
+        Args a{};
+        a.items = tiles * NM * splits;
+        a.mt = mt;
+        a.nt = nt;
+        a.nstep = NT;
+        a.boxn = NT;
+        a.M = M;
+        a.N = N;
+        a.herm = herm ? 1 : 0;
+        a.blocks = blocks;
+        a.tiles = tiles;
+        a.kb_split = cdiv(kbt, splits);
+        a.out16 = out16;
+        a.flag = flag;
+        a.flag_w = flag;
+        for (int c = 0; c < nchunk; ++c) {
+            const long long p0 = (long long)c * ld;
+            for (const Src &s : srcs) {
+                if (s.cnt <= 0) continue;
+                k_residues<<<dim3(cdiv(ld, 1024), s.cnt), 256, 0, st>>>(s.r, n, p0, ld, R, s.row0, 0, scl, nullptr,
+                                                                        1 << 30, 0, 0, res, flag);
+                count_launch(ctx);
+            }
+            RS_LAUNCHED(ctx, "k_residues");
+            a.kb_total = cdiv(std::min<long long>(ld, n - p0), 64);
+            a.accumulate = c > 0;
+            if (real) RS_TRY((launch_gemm<true, false>(ctx, mA, mB, mB, a, st)));
+            else RS_TRY((launch_gemm<false, false>(ctx, mA, mB, mB, a, st)));
+        }
+        k_crt_gram<<<dim3(cdiv((long long)na * nb, 128), blocks), 128, 0, st>>>(
+            out16, splits, M, N, blocks, real ? 1 : 0, A0.cnt[0], A0.cnt[1], B0.cnt[0], B0.cnt[1], na, nb, herm ? 1 : 0,
+            scl, scl + 2 * rowB, scale, g0, g1, ldg, flag);
+        count_launch(ctx);
+        RS_LAUNCHED(ctx, "k_crt_gram");
+    }
+    return RSDFT_OK;
+}
+
+rsdft_status rns_rotate(rsdft_ctx *ctx, const RowBlocks &Y0, const double2 *c, int ldc, int m, bool real,
+                        const double2 *base, int sign, double2 *out0, double2 *out1, cudaStream_t st, bool *used) {
+    *used = false;
+    const RowBlocks Y = real ? pair_rows(Y0) : Y0;
+    const int R = rows_of(Y), k = rows_of(Y0);
+    const long long n = ctx->n;
+    if (Y0.cnt[0] <= 0) return RSDFT_OK;
+    const int segs = Y0.cnt[1] + Y0.cnt[2] > 0 ? 2 : 1;
+    const int PL = real ? 1 : 2, NT = real ? 256 : 128;
+    const int nt = cdiv(m, NT), nstep = cdiv(cdiv(m, nt), 16) * 16, nbp = nt * nstep, nquad = cdiv(m, 4);
+    Seg sg[2];
+    sg[0] = Seg{{Y0.cnt[0], 0}, {0, 0}, real ? 2 * Y.cnt[0] : Y.cnt[0]};
+    sg[1] = Seg{{Y0.cnt[1], Y0.cnt[2]}, {Y0.cnt[0], Y0.cnt[0] + Y0.cnt[1]},
+                real ? 2 * (Y.cnt[1] + Y.cnt[2]) : Y.cnt[1] + Y.cnt[2]};
+    int kb[2], kpad[2], bits[2];
+    double kpads = 0.0;
+    for (int s = 0; s < segs; ++s) {
+        kb[s] = cdiv(sg[s].k, 64);
+        kpad[s] = kb[s] * 64;
+        kpads += kpad[s];
+        // |y_r| over the K products of a sum is at most sqrt(K) max|y|
+        int h = 0;
+        while ((1LL << (2 * h)) < (long long)sg[s].k * PL) ++h;
+        bits[s] = T_ROW - h;
+    }
+    const double out_bytes = (double)NM * segs * PL * nquad * 4;
+    if (!rns_wins((double)n, R, nbp, kpads, (double)k * m, real, (double)n * out_bytes * 4.0 / 4.0e12)) return RSDFT_OK;
+    const size_t per_point = (size_t)NM * R * 4 + (size_t)out_bytes;
+    const long long most = std::max<long long>(4096, (long long)(RNS_BYTES / per_point) / 128 * 128);
+    const int nchunk = cdiv(n, most);
+    const int ld = cdiv(cdiv(n, nchunk), 128) * 128;
+    Carver cv{nullptr};
+    for (int pass = 0; pass < 2; ++pass) {
+        if (pass == 1) {
+            if (rns_buffer(ctx, cv.at) != RSDFT_OK) {
+                ctx->err.clear();
+                return RSDFT_OK;
+            }
+            cv = Carver{(unsigned char *)ctx->rns.buf};
+        }
+        __nv_bfloat16 *res = cv.take<__nv_bfloat16>((size_t)NM * R * 2 * ld);
+        unsigned *out8 = cv.take<unsigned>((size_t)NM * segs * PL * nquad * ld);
+        int *hmax = cv.take<int>((size_t)segs * n);
+        int *sc = cv.take<int>((size_t)segs * m);
+        __nv_bfloat16 *cres[2];
+        for (int s = 0; s < segs; ++s) cres[s] = cv.take<__nv_bfloat16>((size_t)NM * PL * nbp * kpad[s]);
+        if (pass == 0) continue;
+        int *flag = ctx->rns.flag;
+        *used = true;
+        const int mrows = real ? pairs_up(m) : m;
+        ProfScope ps(ctx, RSDFT_K_ROTATE, (real ? 2.0 : 8.0) * (double)n * k * m,
+                     16.0 * (double)n * (R + mrows * (1 + (out1 ? 1 : 0) + (base ? 1 : 0))), st, 0);
+        RS_CUDA(ctx, cudaMemsetAsync(flag, 0, sizeof(int), st));
+        RS_CUDA(ctx, cudaMemsetAsync(hmax, 0, (size_t)segs * n * sizeof(int), st));
+        CUtensorMap mA, mB[2];
+        for (int s = 0; s < segs; ++s) {
+            const int r0 = s ? Y.cnt[0] : 0, nr = s ? Y.cnt[1] + Y.cnt[2] : Y.cnt[0];
+            // enough CTAs for small grids: at least 8 per SM, at least 16 rows each
+            const int want = std::max(1, std::min(cdiv(nr, 16), cdiv(8LL * ctx->num_sms, cdiv(n, 256))));
+            const int per = cdiv(cdiv(nr, want), 8) * 8;
+            k_point_max<<<dim3(cdiv(n, 256), cdiv(nr, per)), 256, 0, st>>>(Y, r0, nr, n, per, hmax + (size_t)s * n, flag);
+            k_coef_scale<<<m, 32, 0, st>>>(c, ldc, sg[s], real ? 1 : 0, sc + (size_t)s * m, flag);
+            count_launch(ctx, 2);
+        }
+        for (int s = 0; s < segs; ++s) {
+            k_coef_residues<<<cdiv((long long)nbp * kpad[s] / 2, 256), 256, 0, st>>>(c, ldc, sg[s], real ? 1 : 0, m, nbp, kpad[s],
+                                                                          sc + (size_t)s * m, cres[s], flag);
+            count_launch(ctx);
+            const long long dims[4] = {kpad[s], nbp, PL, NM};
+            const long long str[3] = {2LL * kpad[s], 2LL * kpad[s] * nbp, 2LL * kpad[s] * nbp * PL};
+            const int box[4] = {64, nstep, 1, 1};
+            RS_TRY(tc::tensor_map_bf16(ctx, &mB[s], cres[s], 4, dims, str, box, CU_TENSOR_MAP_SWIZZLE_128B));
+        }
+        RS_LAUNCHED(ctx, "k_coef_residues");
+        if (segs == 1) mB[1] = mB[0];
+        {
+            const long long dims[4] = {ld, real ? 2 * R : R, PL, NM};
+            const long long str[3] = {real ? 2LL * ld : 4LL * ld, 2LL * ld, 4LL * ld * R};
+            const int box[4] = {64, 64, 1, 1};
+            RS_TRY(tc::tensor_map_bf16(ctx, &mA, res, 4, dims, str, box, CU_TENSOR_MAP_SWIZZLE_128B));
+        }
+        Args a{};
+        a.nt = nt;
+        a.nstep = nstep;
+        a.boxn = nstep;
+        a.N = m;
+        a.segs = segs;
+        for (int s = 0; s < 2; ++s) {
+            a.kb[s] = s < segs ? kb[s] : 0;
+            a.row0[s] = s ? (real ? 2 * Y.cnt[0] : Y.cnt[0]) : 0;
+        }
+        a.ldp = ld;
+        a.out8 = out8;
+        a.flag = flag;
+        a.flag_w = flag;
+        for (int ch = 0; ch < nchunk; ++ch) {
+            const long long p0 = (long long)ch * ld;
+            const int np = (int)std::min<long long>(ld, n - p0);
+            if (np <= 0) break;
+            k_residues<<<dim3(cdiv(ld, 1024), R), 256, 0, st>>>(Y, n, p0, ld, R, 0, 1, nullptr, hmax, Y.cnt[0], bits[0],
+                                                                bits[segs - 1], res, flag);
+            count_launch(ctx);
+            RS_LAUNCHED(ctx, "k_residues");
+            a.M = np;
+            a.mt = cdiv(np, 128);
+            a.items = a.mt * NM * segs * nt;
+            if (real) RS_TRY((launch_gemm<true, true>(ctx, mA, mB[0], mB[1], a, st)));
+            else RS_TRY((launch_gemm<false, true>(ctx, mA, mB[0], mB[1], a, st)));
+            const dim3 g(cdiv(np, 256), nquad);
+            if (real)
+                k_crt_rot<true><<<g, 256, 0, st>>>(out8, segs, m, ld, n, p0, np, hmax, bits[0], bits[segs - 1], sc, m, base,
+                                                   sign, out0, out1, flag);
+            else
+                k_crt_rot<false><<<g, 256, 0, st>>>(out8, segs, m, ld, n, p0, np, hmax, bits[0], bits[segs - 1], sc, m, base,
+                                                    sign, out0, out1, flag);
+            count_launch(ctx);
+            RS_LAUNCHED(ctx, "k_crt_rot");
+        }
+    }
+    return RSDFT_OK;
+}
+
+rsdft_status rns_poison(rsdft_ctx *ctx, double2 *out, long long cnt, cudaStream_t st) {
+    k_poison<<<std::min(cdiv(cnt, 256), 4 * ctx->num_sms), 256, 0, st>>>(out, cnt, ctx->rns.flag);
+    count_launch(ctx);
+    RS_LAUNCHED(ctx, "k_poison");
+    return RSDFT_OK;
+}
+
+}  // namespace rsdft

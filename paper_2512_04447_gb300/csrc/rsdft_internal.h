@@ -117,6 +117,14 @@ struct NnState {
     float *tr = nullptr;   size_t tr_cap = 0;      // training activations and gradients
 };
 
+// Residue-arithmetic products (rns.cu): residue planes and scratch, and the device flag
+// that hands a call back to the FP64 kernels.
+struct RnsWork {
+    void *buf = nullptr;
+    size_t bytes = 0;
+    int *flag = nullptr;
+};
+
 struct Profiler {
     bool on = false;
     struct Rec { cudaEvent_t a, b; int id; double flops, bytes; };
@@ -146,6 +154,7 @@ struct rsdft_ctx {
     rsdft::ScfWork scf;
     rsdft::Profiler prof;
     rsdft::NnState nn;
+    rsdft::RnsWork rns;
     long long launches = 0;          // every kernel launched on this context
     long long coop_fallbacks = 0;    // tridiagonalisations that could not launch cooperatively
     int coop_last_error = 0;         // cudaError_t of the last such launch
@@ -238,11 +247,26 @@ using RowBlocks = RowBlocksT<double2>;
 // and g is completed as a Hermitian matrix.  ldg = leading dimension of g.
 rsdft_status gram(rsdft_ctx *ctx, const RowBlocks &A, const RowBlocks &B, double2 *g, int ldg,
                   bool hermitian, double scale, cudaStream_t st);
+// gs = <Y|Y> and gh = <Y|HY>, both Hermitian, as one product where the residue path takes it
+rsdft_status gram_sh(rsdft_ctx *ctx, const RowBlocks &Y, const RowBlocks &HY, double2 *gs, double2 *gh, int ldg,
+                     double scale, cudaStream_t st);
 // out1 (optional) = sum over blocks 1..2 of c rows; out0 = out1 + block-0 part
 // (+ sign * ... and base handling as in rsdft_rotate).  c is [k][ldc].
 rsdft_status rotate(rsdft_ctx *ctx, const RowBlocks &Y, const double2 *c, int ldc, int m,
                     const double2 *base, int sign, double2 *out0, double2 *out1,
                     cudaStream_t st);
+// The same on the tensor cores by residue arithmetic (rns.cu), exact to the rounding of the
+// operands; *used = false and nothing launched where the FP64 kernels are faster or the
+// scratch does not fit.  When used, the caller launches its FP64 kernels behind them guarded
+// by ctx->rns.flag: they return at once unless the flag asks for them.  Blocks hold complex
+// rows (real: counts are real bands, rows are pair rows).  B1 (optional): g1 = <A|B1>, its
+// rows like B0's.
+rsdft_status rns_gram(rsdft_ctx *ctx, const RowBlocks &A, const RowBlocks &B0, const RowBlocks *B1, bool real,
+                      bool herm, double2 *g0, double2 *g1, int ldg, double scale, cudaStream_t st, bool *used);
+rsdft_status rns_rotate(rsdft_ctx *ctx, const RowBlocks &Y, const double2 *c, int ldc, int m, bool real,
+                        const double2 *base, int sign, double2 *out0, double2 *out1, cudaStream_t st, bool *used);
+// After the guarded FP64 rotation of an in-place update (base == out0).
+rsdft_status rns_poison(rsdft_ctx *ctx, double2 *out, long long cnt, cudaStream_t st);
 // FP32 operands (mixed form): products and CTA-level sums in FP32, Gram
 // partials reduced in FP64; rotation coefficients rounded to FP32.
 rsdft_status gram32(rsdft_ctx *ctx, const RowBlocksT<float2> &A, const RowBlocksT<float2> &B,
