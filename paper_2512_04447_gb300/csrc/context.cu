@@ -4,6 +4,7 @@
 #include <cstdarg>
 #include <algorithm>
 
+#include "fix_fft.h"
 #include "rsdft_internal.h"
 
 namespace rsdft {
@@ -129,6 +130,52 @@ static rsdft_status build_fft_tables(rsdft_ctx *ctx) {
         ctx->fft.tw32[a] = d_twf;
         ctx->fft.g2pos[a] = d_g2;
         ctx->fft.g2pos32[a] = d_g2f;
+    }
+    return RSDFT_OK;
+}
+
+// Tables of the fixed-point transforms, from the same twiddles, frequencies and G^2.
+static rsdft_status build_fix_tables(rsdft_ctx *ctx) {
+    const long double two_pi = 6.283185307179586476925286766559005768L;
+    FixFft &f = ctx->fix;
+    double total = 0.0;
+    for (int a = 0; a < 3; ++a) {
+        const double g = M_PI * ctx->N[a] / ctx->L[a];
+        total += g * g;
+    }
+    f.kexp = 59 - std::ilogb(0.5 * total / (double)ctx->n);   // the sum of the three stays below 2^60
+    for (int a = 0; a < 3; ++a) {
+        const AxisPlan &p = ctx->fft.ax[a];
+        const int N = p.N;
+        std::vector<fix::W4> tw(N);
+        std::vector<long long> kin(N);
+        std::vector<double> g2abs(N / 2 + 1);
+        std::vector<unsigned char> fabs(N);
+        const double gunit = 2.0 * M_PI / ctx->L[a];
+        for (int k = 0; k < N; ++k) {
+            const long double ang = two_pi * (long double)k / (long double)N;
+            const long long c = llroundl(cosl(ang) * 0x1p62L), s = llroundl(-sinl(ang) * 0x1p62L);
+            tw[k] = fix::W4{fix::hi_of(c), fix::lo_of(c), fix::hi_of(s), fix::lo_of(s)};
+        }
+        for (int pos = 0; pos < N; ++pos) {
+            const int k = position_to_freq(p, pos), ka = std::min(k, N - k);
+            const double g = gunit * ka;
+            fabs[pos] = (unsigned char)ka;
+            g2abs[ka] = g * g;
+            kin[pos] = llroundl(ldexpl(0.5L * (long double)(g * g) / (long double)ctx->n, f.kexp));
+        }
+        fix::W4 *d_tw;
+        long long *d_kin;
+        double *d_g2;
+        unsigned char *d_f;
+        RS_TRY(upload(ctx, &d_tw, tw.data(), N));
+        RS_TRY(upload(ctx, &d_kin, kin.data(), N));
+        RS_TRY(upload(ctx, &d_g2, g2abs.data(), g2abs.size()));
+        RS_TRY(upload(ctx, &d_f, fabs.data(), N));
+        f.tw[a] = d_tw;
+        f.kin[a] = d_kin;
+        f.g2abs[a] = d_g2;
+        f.fabs[a] = d_f;
     }
     return RSDFT_OK;
 }
@@ -399,6 +446,7 @@ rsdft_status rsdft_create(const rsdft_cell *cell, const rsdft_grid *grid, const 
     ctx->n = (long long)grid->n[0] * grid->n[1] * grid->n[2];
     ctx->dV = L[0] * L[1] * L[2] / (double)ctx->n;
     rsdft_status st = build_fft_tables(ctx);
+    if (st == RSDFT_OK) st = build_fix_tables(ctx);
     if (st == RSDFT_OK) st = upload(ctx, &ctx->vloc, v_loc_host, (size_t)ctx->n);
     if (st == RSDFT_OK) st = upload(ctx, &ctx->v, v_loc_host, (size_t)ctx->n);
     if (st == RSDFT_OK) st = dev_alloc(ctx, (void **)&ctx->v32, (size_t)ctx->n * sizeof(float));

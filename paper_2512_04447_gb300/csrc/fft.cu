@@ -1,4 +1,5 @@
-// Batched 3D FFT kernels and H psi (SCF tasks (1) and (4)).
+// Batched 3D FFT kernels of the FP32 data path, the projector gather and H psi (SCF tasks (1)
+// and (4)).  The FP64 passes, of the same shape, are in fft_fix.cu.
 //
 // Layout: orbital block [band][z][y][x] complex, x fastest.  A 3D transform is
 // three shared-memory passes over HBM:
@@ -16,11 +17,12 @@
 #include <mutex>
 #include <vector>
 
+#include "fft_common.h"
 #include "rsdft_internal.h"
 
 namespace rsdft {
 
-// ---- complex helpers (double2 / float2) ---------------------------------------
+// ---- complex helpers ---------------------------------------
 template <typename V> struct Sc;
 template <> struct Sc<double2> { using T = double; };
 template <> struct Sc<float2> { using T = float; };
@@ -144,16 +146,6 @@ __device__ __forceinline__ void bfly(V *s, int base, int step, int j, int twstep
 // Element e of line l sits at s[l * lstride + e * es].  lines_fast selects the
 // thread mapping: consecutive threads take consecutive lines (use when es > 1
 // and lstride == 1), else consecutive butterflies of one line.
-// x / d for x < 2^16 from the multiply-high divisor of d (mag = 0 means d = 1).
-__device__ __forceinline__ int qdiv(int x, unsigned mag) { return mag ? (int)__umulhi((unsigned)x, mag) : x; }
-
-// xy planes live in shared memory with an odd row stride RS = Nx | 1 (complex
-// values): the lines of both transform directions are then read by consecutive
-// threads without bank conflicts (successive rows start two banks apart).
-__device__ __forceinline__ int plane_rs(int Nx) { return Nx | 1; }
-// shared-memory index of plane element i = y Nx + x
-__device__ __forceinline__ int pidx(int i, int Nx, int RS, unsigned nxmag) { return i + qdiv(i, nxmag) * (RS - Nx); }
-
 // nlmag: multiply-high divisor of nlines.  Quotients and remainders of the
 // index decomposition use it instead of integer division (total < 2^16).
 template <typename V, bool INV>
@@ -194,65 +186,28 @@ template <typename V> struct FftTabs {
     AxisPlan ax[3];
     const V *tw[3];
     const typename Sc<V>::T *g2[3];
-    const double *g1[3];   // G_a (first derivatives; FP64 real fields only)
     double inv_n;   // 1 / (Nx Ny Nz), formed on the host
 };
 
-static FftTabs<double2> tabs_of(const rsdft_ctx *ctx, double2 *) {
-    FftTabs<double2> t;
-    for (int a = 0; a < 3; ++a) {
-        t.ax[a] = ctx->fft.ax[a];
-        t.tw[a] = ctx->fft.tw64[a];
-        t.g2[a] = ctx->fft.g2pos[a];
-        t.g1[a] = ctx->fft.gpos[a];
-    }
-    t.inv_n = 1.0 / (double)ctx->n;
-    return t;
-}
 static FftTabs<float2> tabs_of(const rsdft_ctx *ctx, float2 *) {
     FftTabs<float2> t;
     for (int a = 0; a < 3; ++a) {
         t.ax[a] = ctx->fft.ax[a];
         t.tw[a] = ctx->fft.tw32[a];
         t.g2[a] = ctx->fft.g2pos32[a];
-        t.g1[a] = ctx->fft.gpos[a];
     }
     t.inv_n = 1.0 / (double)ctx->n;
     return t;
 }
 static const ProjT<double> &proj_of(const rsdft_ctx *ctx, double2 *) { return ctx->pt; }
 static const ProjT<float> &proj_of(const rsdft_ctx *ctx, float2 *) { return ctx->pt32; }
-static const double *v_of(const rsdft_ctx *ctx, double2 *) { return ctx->v; }
 static const float *v_of(const rsdft_ctx *ctx, float2 *) { return ctx->v32; }
-
-// Global -> shared copy of a plane or slab with several loads in flight per thread:
-// each batch issues its loads (src(i)) before any of its stores (dst(i, v)); the
-// plain loop would leave one load per thread in flight, and the passes stalled on
-// load latency well below the HBM rate.
-template <typename V, typename SrcF, typename DstF>
-__device__ __forceinline__ void stage_in(int tot, SrcF src, DstF dst) {
-    constexpr int U = sizeof(V) == 8 ? 8 : 2;
-    for (int i0 = threadIdx.x; i0 < tot; i0 += U * blockDim.x) {
-        V r[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int i = i0 + u * blockDim.x;
-            if (i < tot) r[u] = src(i);
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int i = i0 + u * blockDim.x;
-            if (i < tot) dst(i, r[u]);
-        }
-    }
-}
 
 // ---- xy forward pass ------------------------------------------------------------
 template <typename V, Src SRC>
 __global__ void __launch_bounds__(FFT_THREADS, sizeof(V) == 8 ? 3 : 1)
 k_xy_forward(FftTabs<V> tb, const V *__restrict__ src, const V *__restrict__ src2,
-             const double *__restrict__ theta, const int *__restrict__ act,
-             const double *__restrict__ rsrc, V *__restrict__ dst) {
+             const double *__restrict__ theta, const int *__restrict__ act, V *__restrict__ dst) {
     using T = typename Sc<V>::T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V *s_plane = reinterpret_cast<V *>(smem_raw);
@@ -276,9 +231,6 @@ k_xy_forward(FftTabs<V> tb, const V *__restrict__ src, const V *__restrict__ src
             const V h = hx[i], v = x[i];
             return mk<V>(h.x - th * v.x, h.y - th * v.y);
         }, put);
-    } else {
-        const double *in = rsrc + off;
-        stage_in<V>((int)plane, [&](int i) { return mk<V>((T)in[i], (T)0); }, put);
     }
     __syncthreads();
     fft_lines<V, false>(s_plane, tb.ax[0], tb.tw[0], Ny, tb.ax[1].nmag, RS, 1, true);
@@ -319,66 +271,30 @@ k_z_mid(FftTabs<V> tb, V *__restrict__ buf, const double *__restrict__ tkin) {
         if (!(t >= 1e-12)) t = 1.0;
         tk = (T)t;
     }
-    if constexpr (MID == Mid::GradX || MID == Mid::GradY || MID == Mid::GradZ) {
-        // i G_a / n: (re, im) -> (-f im, f re)
-        for (int i = threadIdx.x; i < tot; i += blockDim.x) {
-            const int z = qdiv(i, tb.ax[0].nmag), x = i - z * Nx;
-            const T ga = (T)(MID == Mid::GradX ? tb.g1[0][x] : (MID == Mid::GradY ? tb.g1[1][y] : tb.g1[2][z]));
-            const T f = ga * inv_n;
-            s_slab[i] = mk<V>(-f * s_slab[i].y, f * s_slab[i].x);
-        }
-        __syncthreads();
-        fft_lines<V, true>(s_slab, tb.ax[2], tb.tw[2], Nx, tb.ax[0].nmag, 1, Nx, true);
-        for (int i = threadIdx.x; i < tot; i += blockDim.x) {
-            const int z = qdiv(i, tb.ax[0].nmag), x = i - z * Nx;
-            base[z * zstride + x] = s_slab[i];
-        }
-    } else {
-        for (int i = threadIdx.x; i < tot; i += blockDim.x) {
-            const int z = qdiv(i, tb.ax[0].nmag), x = i - z * Nx;
-            T g2 = tb.g2[0][x] + gy2 + tb.g2[2][z];
-            T f;
-            if (MID == Mid::Kinetic) f = (T)0.5 * g2 * inv_n;
-            else if (MID == Mid::Tpa) f = tpa_k<T>((T)0.5 * g2 / tk) * inv_n;
-            else if (MID == Mid::Hartree) f = g2 > (T)0 ? (T)(4.0 * M_PI) / g2 * inv_n : (T)0;
-            else f = inv_n;
-            s_slab[i] = mk<V>(s_slab[i].x * f, s_slab[i].y * f);
-        }
-        __syncthreads();
-        fft_lines<V, true>(s_slab, tb.ax[2], tb.tw[2], Nx, tb.ax[0].nmag, 1, Nx, true);
-        for (int i = threadIdx.x; i < tot; i += blockDim.x) {
-            const int z = qdiv(i, tb.ax[0].nmag), x = i - z * Nx;
-            base[z * zstride + x] = s_slab[i];
-        }
+    for (int i = threadIdx.x; i < tot; i += blockDim.x) {
+        const int z = qdiv(i, tb.ax[0].nmag), x = i - z * Nx;
+        T g2 = tb.g2[0][x] + gy2 + tb.g2[2][z];
+        T f;
+        if (MID == Mid::Kinetic) f = (T)0.5 * g2 * inv_n;
+        else f = tpa_k<T>((T)0.5 * g2 / tk) * inv_n;
+        s_slab[i] = mk<V>(s_slab[i].x * f, s_slab[i].y * f);
+    }
+    __syncthreads();
+    fft_lines<V, true>(s_slab, tb.ax[2], tb.tw[2], Nx, tb.ax[0].nmag, 1, Nx, true);
+    for (int i = threadIdx.x; i < tot; i += blockDim.x) {
+        const int z = qdiv(i, tb.ax[0].nmag), x = i - z * Nx;
+        base[z * zstride + x] = s_slab[i];
     }
 }
 
-// The four beta values of one projector-table entry (16- or 32-byte aligned: the
-// tables are [nent][4]) in one 16-byte load (FP32) or two (FP64), instead of four
-// scalar loads that each cost the L1 a wavefront per thread.
-__device__ __forceinline__ void beta4(const float *bt, float b[4]) {
-    const float4 q = *reinterpret_cast<const float4 *>(bt);
-    b[0] = q.x;
-    b[1] = q.y;
-    b[2] = q.z;
-    b[3] = q.w;
-}
-__device__ __forceinline__ void beta4(const double *bt, double b[4]) {
-    const double2 q0 = reinterpret_cast<const double2 *>(bt)[0], q1 = reinterpret_cast<const double2 *>(bt)[1];
-    b[0] = q0.x;
-    b[1] = q0.y;
-    b[2] = q1.x;
-    b[3] = q1.y;
-}
-
 // ---- xy inverse pass + epilogue ------------------------------------------------------
-enum class Epi { Plain, Hpsi, Real };
+enum class Epi { Plain, Hpsi };
 
 template <typename V, Epi EPI>
 __global__ void __launch_bounds__(FFT_THREADS, sizeof(V) == 8 ? 3 : 1)
 k_xy_inverse(FftTabs<V> tb, const V *__restrict__ buf, const V *__restrict__ psi,
              const typename Sc<V>::T *__restrict__ v, ProjT<typename Sc<V>::T> pt,
-             const V *__restrict__ p, V *__restrict__ out, double *__restrict__ rout, int stage_pe) {
+             const V *__restrict__ p, V *__restrict__ out, int stage_pe) {
     using T = typename Sc<V>::T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V *s_plane = reinterpret_cast<V *>(smem_raw);
@@ -397,9 +313,6 @@ k_xy_inverse(FftTabs<V> tb, const V *__restrict__ buf, const V *__restrict__ psi
     if (EPI == Epi::Plain) {
         V *o = out + band * n + off;
         for (int i = threadIdx.x; i < (int)plane; i += blockDim.x) o[i] = s_plane[pidx(i, Nx, RS, nxm)];
-    } else if (EPI == Epi::Real) {
-        double *o = rout + off;
-        for (int i = threadIdx.x; i < (int)plane; i += blockDim.x) o[i] = (double)s_plane[pidx(i, Nx, RS, nxm)].x;
     } else {
         const V *ps = psi + band * n + off;
         const T *vv = v + off;
@@ -522,51 +435,25 @@ template <typename V> static size_t slab_bytes(const rsdft_ctx *ctx) {
     return (size_t)ctx->N[0] * ctx->N[2] * sizeof(V);
 }
 
-constexpr size_t MAX_DYN_SMEM = 227 * 1024;   // largest dynamic shared memory of one CTA
-
-// The attribute is per function and process-wide, so it is raised once to the
-// largest size (occupancy follows each launch's own dynamic size); lowering it
-// per launch would race with launches of other contexts on other threads.
-template <typename K> static rsdft_status set_smem(rsdft_ctx *ctx, K kernel, size_t bytes) {
-    if (bytes <= 48 * 1024) return RSDFT_OK;
-    if (bytes > MAX_DYN_SMEM) return fail(ctx, RSDFT_E_INVALID, "plane needs %zu B of shared memory", bytes);
-    static std::mutex mu;
-    static std::vector<const void *> done;
-    std::lock_guard<std::mutex> g(mu);
-    const void *key = reinterpret_cast<const void *>(kernel);
-    if (std::find(done.begin(), done.end(), key) == done.end()) {
-        RS_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MAX_DYN_SMEM));
-        done.push_back(key);
-    }
-    return RSDFT_OK;
-}
-
 template <typename V>
 rsdft_status fft_xy_forward_t(rsdft_ctx *ctx, Src kind, const V *src, const V *src2,
-                              const double *theta, const int *act, const double *rsrc, V *dst,
+                              const double *theta, const int *act, V *dst,
                               int nb, cudaStream_t st) {
     if (nb <= 0) return RSDFT_OK;
     const size_t sm = plane_bytes<V>(ctx);
     dim3 grid(ctx->N[2], nb);
     const double nxy = (double)ctx->N[0] * ctx->N[1];
     const double e = (double)sizeof(V);
-    const double bpp = kind == Src::Plain ? 2 * e : (kind == Src::Residual ? 3 * e : 8.0 + e);
+    const double bpp = kind == Src::Plain ? 2 * e : 3 * e;
     ProfScope ps(ctx, RSDFT_K_FFT_XY_FWD, 5.0 * nxy * std::log2(nxy) * ctx->N[2] * nb,
                  bpp * (double)ctx->n * nb, st);
     const FftTabs<V> tb = tabs_of(ctx, (V *)nullptr);
-    switch (kind) {
-        case Src::Plain:
-            RS_TRY(set_smem(ctx, k_xy_forward<V, Src::Plain>, sm));
-            k_xy_forward<V, Src::Plain><<<grid, FFT_THREADS, sm, st>>>(tb, src, src2, theta, act, rsrc, dst);
-            break;
-        case Src::Residual:
-            RS_TRY(set_smem(ctx, k_xy_forward<V, Src::Residual>, sm));
-            k_xy_forward<V, Src::Residual><<<grid, FFT_THREADS, sm, st>>>(tb, src, src2, theta, act, rsrc, dst);
-            break;
-        case Src::RealField:
-            RS_TRY(set_smem(ctx, k_xy_forward<V, Src::RealField>, sm));
-            k_xy_forward<V, Src::RealField><<<grid, FFT_THREADS, sm, st>>>(tb, src, src2, theta, act, rsrc, dst);
-            break;
+    if (kind == Src::Plain) {
+        RS_TRY(set_smem(ctx, k_xy_forward<V, Src::Plain>, sm));
+        k_xy_forward<V, Src::Plain><<<grid, FFT_THREADS, sm, st>>>(tb, src, src2, theta, act, dst);
+    } else {
+        RS_TRY(set_smem(ctx, k_xy_forward<V, Src::Residual>, sm));
+        k_xy_forward<V, Src::Residual><<<grid, FFT_THREADS, sm, st>>>(tb, src, src2, theta, act, dst);
     }
     RS_LAUNCHED(ctx, "k_xy_forward");
     return RSDFT_OK;
@@ -581,67 +468,41 @@ rsdft_status fft_z_mid_t(rsdft_ctx *ctx, Mid mid, V *buf, const double *tkin, in
     ProfScope ps(ctx, RSDFT_K_FFT_Z, 10.0 * (double)ctx->n * std::log2((double)ctx->N[2]) * nb,
                  2.0 * sizeof(V) * (double)ctx->n * nb, st);
     const FftTabs<V> tb = tabs_of(ctx, (V *)nullptr);
-    switch (mid) {
-        case Mid::Kinetic:
-            RS_TRY(set_smem(ctx, k_z_mid<V, Mid::Kinetic>, sm));
-            k_z_mid<V, Mid::Kinetic><<<grid, FFT_THREADS, sm, st>>>(tb, buf, tkin);
-            break;
-        case Mid::Tpa:
-            RS_TRY(set_smem(ctx, k_z_mid<V, Mid::Tpa>, sm));
-            k_z_mid<V, Mid::Tpa><<<grid, FFT_THREADS, sm, st>>>(tb, buf, tkin);
-            break;
-        case Mid::Hartree:
-            RS_TRY(set_smem(ctx, k_z_mid<V, Mid::Hartree>, sm));
-            k_z_mid<V, Mid::Hartree><<<grid, FFT_THREADS, sm, st>>>(tb, buf, tkin);
-            break;
-        case Mid::Scale:
-            RS_TRY(set_smem(ctx, k_z_mid<V, Mid::Scale>, sm));
-            k_z_mid<V, Mid::Scale><<<grid, FFT_THREADS, sm, st>>>(tb, buf, tkin);
-            break;
-        case Mid::GradX:
-            RS_TRY(set_smem(ctx, k_z_mid<V, Mid::GradX>, sm));
-            k_z_mid<V, Mid::GradX><<<grid, FFT_THREADS, sm, st>>>(tb, buf, tkin);
-            break;
-        case Mid::GradY:
-            RS_TRY(set_smem(ctx, k_z_mid<V, Mid::GradY>, sm));
-            k_z_mid<V, Mid::GradY><<<grid, FFT_THREADS, sm, st>>>(tb, buf, tkin);
-            break;
-        case Mid::GradZ:
-            RS_TRY(set_smem(ctx, k_z_mid<V, Mid::GradZ>, sm));
-            k_z_mid<V, Mid::GradZ><<<grid, FFT_THREADS, sm, st>>>(tb, buf, tkin);
-            break;
+    if (mid == Mid::Kinetic) {
+        RS_TRY(set_smem(ctx, k_z_mid<V, Mid::Kinetic>, sm));
+        k_z_mid<V, Mid::Kinetic><<<grid, FFT_THREADS, sm, st>>>(tb, buf, tkin);
+    } else {
+        RS_TRY(set_smem(ctx, k_z_mid<V, Mid::Tpa>, sm));
+        k_z_mid<V, Mid::Tpa><<<grid, FFT_THREADS, sm, st>>>(tb, buf, tkin);
     }
     RS_LAUNCHED(ctx, "k_z_mid");
     return RSDFT_OK;
 }
 
 template <typename V>
-rsdft_status fft_xy_inverse_t(rsdft_ctx *ctx, const V *buf, const V *psi, const V *p, V *out,
-                              double *rout, int nb, cudaStream_t st) {
+rsdft_status fft_xy_inverse_t(rsdft_ctx *ctx, const V *buf, const V *psi, const V *p, V *out, int nb,
+                              cudaStream_t st) {
     if (nb <= 0) return RSDFT_OK;
     const size_t sm = plane_bytes<V>(ctx);
     dim3 grid(ctx->N[2], nb);
     const double nxy = (double)ctx->N[0] * ctx->N[1];
     const double e = (double)sizeof(V);
-    const double bpp = rout ? e + 8.0 : (psi ? 3 * e : 2 * e);
+    const double bpp = psi ? 3 * e : 2 * e;
     ProfScope ps(ctx, RSDFT_K_FFT_XY_INV, 5.0 * nxy * std::log2(nxy) * ctx->N[2] * nb,
                  bpp * (double)ctx->n * nb + (psi ? 0.5 * e * (double)ctx->n : 0.0), st);
     const FftTabs<V> tb = tabs_of(ctx, (V *)nullptr);
     const auto &pt = proj_of(ctx, (V *)nullptr);
     const auto *v = v_of(ctx, (V *)nullptr);
-    if (rout) {
-        RS_TRY(set_smem(ctx, k_xy_inverse<V, Epi::Real>, sm));
-        k_xy_inverse<V, Epi::Real><<<grid, FFT_THREADS, sm, st>>>(tb, buf, psi, v, pt, p, out, rout, 0);
-    } else if (psi) {
+    if (psi) {
         // the plane plus, when it fits, the band's E_aj <beta_aj|psi> after it
         const size_t smh = sm + (size_t)pt.natom * pt.nproj * sizeof(V);
         const int stage = smh <= MAX_DYN_SMEM ? 1 : 0;
         const size_t smu = stage ? smh : sm;
         RS_TRY(set_smem(ctx, k_xy_inverse<V, Epi::Hpsi>, smu));
-        k_xy_inverse<V, Epi::Hpsi><<<grid, FFT_THREADS, smu, st>>>(tb, buf, psi, v, pt, p, out, rout, stage);
+        k_xy_inverse<V, Epi::Hpsi><<<grid, FFT_THREADS, smu, st>>>(tb, buf, psi, v, pt, p, out, stage);
     } else {
         RS_TRY(set_smem(ctx, k_xy_inverse<V, Epi::Plain>, sm));
-        k_xy_inverse<V, Epi::Plain><<<grid, FFT_THREADS, sm, st>>>(tb, buf, psi, v, pt, p, out, rout, 0);
+        k_xy_inverse<V, Epi::Plain><<<grid, FFT_THREADS, sm, st>>>(tb, buf, psi, v, pt, p, out, 0);
     }
     RS_LAUNCHED(ctx, "k_xy_inverse");
     return RSDFT_OK;
@@ -659,32 +520,18 @@ rsdft_status project_t(rsdft_ctx *ctx, const V *psi, V *p, int nb, cudaStream_t 
     return RSDFT_OK;
 }
 
-rsdft_status fft_xy_forward(rsdft_ctx *ctx, Src kind, const double2 *src, const double2 *src2,
-                            const double *theta, const int *act, const double *rsrc,
-                            double2 *dst, int nb, cudaStream_t st) {
-    return fft_xy_forward_t<double2>(ctx, kind, src, src2, theta, act, rsrc, dst, nb, st);
-}
 rsdft_status fft_xy_forward32(rsdft_ctx *ctx, Src kind, const float2 *src, const float2 *src2,
                               const double *theta, const int *act, float2 *dst, int nb,
                               cudaStream_t st) {
-    return fft_xy_forward_t<float2>(ctx, kind, src, src2, theta, act, nullptr, dst, nb, st);
-}
-rsdft_status fft_z_mid(rsdft_ctx *ctx, Mid mid, double2 *buf, const double *tkin, int nb,
-                       cudaStream_t st) {
-    return fft_z_mid_t<double2>(ctx, mid, buf, tkin, nb, st);
+    return fft_xy_forward_t<float2>(ctx, kind, src, src2, theta, act, dst, nb, st);
 }
 rsdft_status fft_z_mid32(rsdft_ctx *ctx, Mid mid, float2 *buf, const double *tkin, int nb,
                          cudaStream_t st) {
     return fft_z_mid_t<float2>(ctx, mid, buf, tkin, nb, st);
 }
-rsdft_status fft_xy_inverse(rsdft_ctx *ctx, const double2 *buf, const double2 *psi,
-                            const double2 *p, double2 *out, double *rout, int nb,
-                            cudaStream_t st) {
-    return fft_xy_inverse_t<double2>(ctx, buf, psi, p, out, rout, nb, st);
-}
 rsdft_status fft_xy_inverse32(rsdft_ctx *ctx, const float2 *buf, const float2 *psi,
                               const float2 *p, float2 *out, int nb, cudaStream_t st) {
-    return fft_xy_inverse_t<float2>(ctx, buf, psi, p, out, nullptr, nb, st);
+    return fft_xy_inverse_t<float2>(ctx, buf, psi, p, out, nb, st);
 }
 rsdft_status project(rsdft_ctx *ctx, const double2 *psi, double2 *p, int nb, cudaStream_t st) {
     return project_t<double2>(ctx, psi, p, nb, st);

@@ -1,0 +1,81 @@
+// Pieces shared by the FP32 passes (fft.cu) and the fixed-point passes (fft_fix.cu).
+#pragma once
+
+#include <algorithm>
+#include <mutex>
+#include <vector>
+
+#include "rsdft_internal.h"
+
+namespace rsdft {
+
+// x / d for x < 2^16 from the multiply-high divisor of d (mag = 0 means d = 1).
+__device__ __forceinline__ int qdiv(int x, unsigned mag) { return mag ? (int)__umulhi((unsigned)x, mag) : x; }
+
+// xy planes live in shared memory with an odd row stride RS = Nx | 1 (complex
+// values): the lines of both transform directions are then read by consecutive
+// threads without bank conflicts (successive rows start two banks apart).
+__device__ __forceinline__ int plane_rs(int Nx) { return Nx | 1; }
+// shared-memory index of plane element i = y Nx + x
+__device__ __forceinline__ int pidx(int i, int Nx, int RS, unsigned nxmag) { return i + qdiv(i, nxmag) * (RS - Nx); }
+
+// Global -> shared copy of a plane or slab with several loads in flight per thread:
+// each batch issues its loads (src(i)) before any of its stores (dst(i, v)); the
+// plain loop would leave one load per thread in flight, and the passes stalled on
+// load latency well below the HBM rate.
+template <typename V, typename SrcF, typename DstF>
+__device__ __forceinline__ void stage_in(int tot, SrcF src, DstF dst) {
+    constexpr int U = sizeof(V) == 8 ? 8 : 4;
+    for (int i0 = threadIdx.x; i0 < tot; i0 += U * blockDim.x) {
+        V r[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int i = i0 + u * blockDim.x;
+            if (i < tot) r[u] = src(i);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int i = i0 + u * blockDim.x;
+            if (i < tot) dst(i, r[u]);
+        }
+    }
+}
+
+// The four beta values of one projector-table entry (16- or 32-byte aligned: the
+// tables are [nent][4]) in one 16-byte load (FP32) or two (FP64), instead of four
+// scalar loads that each cost the L1 a wavefront per thread.
+__device__ __forceinline__ void beta4(const float *bt, float b[4]) {
+    const float4 q = *reinterpret_cast<const float4 *>(bt);
+    b[0] = q.x;
+    b[1] = q.y;
+    b[2] = q.z;
+    b[3] = q.w;
+}
+__device__ __forceinline__ void beta4(const double *bt, double b[4]) {
+    const double2 q0 = reinterpret_cast<const double2 *>(bt)[0], q1 = reinterpret_cast<const double2 *>(bt)[1];
+    b[0] = q0.x;
+    b[1] = q0.y;
+    b[2] = q1.x;
+    b[3] = q1.y;
+}
+
+constexpr size_t MAX_DYN_SMEM = 227 * 1024;   // largest dynamic shared memory of one CTA
+
+// The attribute is per function and process-wide, so it is raised once to the
+// largest size (occupancy follows each launch's own dynamic size); lowering it
+// per launch would race with launches of other contexts on other threads.
+template <typename K> static rsdft_status set_smem(rsdft_ctx *ctx, K kernel, size_t bytes) {
+    if (bytes <= 48 * 1024) return RSDFT_OK;
+    if (bytes > MAX_DYN_SMEM) return fail(ctx, RSDFT_E_INVALID, "plane needs %zu B of shared memory", bytes);
+    static std::mutex mu;
+    static std::vector<const void *> done;
+    std::lock_guard<std::mutex> g(mu);
+    const void *key = reinterpret_cast<const void *>(kernel);
+    if (std::find(done.begin(), done.end(), key) == done.end()) {
+        RS_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MAX_DYN_SMEM));
+        done.push_back(key);
+    }
+    return RSDFT_OK;
+}
+
+}  // namespace rsdft

@@ -1,0 +1,647 @@
+// FP64 3D FFT passes of H psi, TPA and the field solvers in 64-bit fixed point (fix_fft.h).
+//
+// The passes are those of fft.cu (xy planes, z slabs with the per-G factor, xy planes with the
+// epilogue; digit-reversed spectrum in between), FP64 in and out.  A block (an xy plane, or the
+// slab of one y) is scaled to integers by its largest value; between the passes the buffer
+// holds integers, and (exponent, bits) of every block says what they are worth, so that the
+// next pass brings its rows to one exponent.  The per-G factor keeps full precision: products
+// are formed with a normalised factor and shifted to the largest one of the slab.
+//
+// What bounds it: the FP64 passes ran at some 80% of the FP64 pipe; the integer instructions on
+// 64-bit values bound these.  144 bands on 64^3, one GB300: forward 3.23 -> 0.68 ms, z 3.66 ->
+// 0.84 ms, inverse 5.9 -> 3.6 ms (with the FP64 projector scatter, now its larger part); TPA of 53
+// bands on 45^3 1.94 -> 0.55 ms.  Errors against 64-bit FFTs are those of the reference itself:
+// relative 4.4e-16 (FP64 passes 4.8e-16) for TPA, 7.1e-16 (8.4e-16) for H psi.
+//
+// Non-finite values make a block's exponent BAD, which every following pass hands on, and the
+// outputs of that band NaN.
+#include <algorithm>
+#include <cmath>
+
+#include "fft_common.h"
+#include "fix_fft.h"
+#include "rsdft_internal.h"
+
+namespace rsdft {
+
+using fix::I2;
+using fix::i64;
+using fix::u64;
+using fix::W4;
+
+namespace {
+
+constexpr int BAD = 0x40000000;        // exponent of a block with non-finite values
+constexpr int EMPTY = -0x10000000;     // exponent of a block of zeros
+constexpr int MAX_THREADS = 768;       // 85 registers: three CTAs of 256 threads on a 64 x 64 plane
+constexpr int HEAD = 32;               // reduction words ahead of the plane
+constexpr int SHIFTS = MAX_N * 4;      // row shifts behind it (xy planes with padded rows keep them in the padding)
+
+struct FixTabs {
+    AxisPlan ax[3];
+    const W4 *tw[3];
+    const i64 *kin[3];                 // G_a^2 / (2 n) in units of 2^-kexp, by position
+    int kexp;
+    const double *g2[3], *g1[3];       // by position
+    const double *g2abs[3];            // G_a^2 by |frequency index|
+    const unsigned char *fabs[3];      // |frequency index| by position
+    double inv_n;
+    int fexp;                          // other factors: |f| < 2^(61 - fexp)
+};
+
+struct Meta { int e, bits; };          // block values are integers below 2^bits times 2^e
+
+__device__ __forceinline__ unsigned mag_hi(I2 v) {
+    const int hx = (int)(v.x >> 32), hy = (int)(v.y >> 32);
+    return (unsigned)(hx ^ (hx >> 31)) | (unsigned)(hy ^ (hy >> 31));
+}
+__device__ __forceinline__ int bits_hi(unsigned m) { return 64 - __clz((int)m); }   // 32 for m = 0
+
+// Every thread's word joined over the block (or / max); red: a zeroed word of shared memory
+__device__ __forceinline__ unsigned block_or(unsigned v, unsigned *red) {
+    v = __reduce_or_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0) atomicOr(red, v);
+    __syncthreads();
+    return *red;
+}
+__device__ __forceinline__ int block_max(int v, int *red) {
+    v = __reduce_max_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0) atomicMax(red, v);
+    __syncthreads();
+    return *red;
+}
+
+// State of one transform: every component is below 2^bits, in units of 2^e; stage counter.
+struct Scale { int bits, e, n; };
+
+// sh: right shift of the inputs (left where negative)
+template <int R, bool INV, bool RAW>
+__device__ __forceinline__ unsigned bfly(I2 *s, int base, int step, int j, int twstep, const W4 *tw, int sh, int s0,
+                                         bool twiddle) {
+    I2 v[R];
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+        v[q] = s[base + q * step];
+        if (RAW) {
+            v[q].x = fix::from_double((int)(v[q].x >> 32), (unsigned)v[q].x, s0);
+            v[q].y = fix::from_double((int)(v[q].y >> 32), (unsigned)v[q].y, s0);
+        }
+    }
+    if (!RAW) {
+        if (sh > 0) {
+#pragma unroll
+            for (int q = 0; q < R; ++q) v[q] = fix::rshift(v[q], sh);
+        } else if (sh < 0) {
+#pragma unroll
+            for (int q = 0; q < R; ++q) v[q] = I2{v[q].x << -sh, v[q].y << -sh};
+        }
+    }
+    // times w^(j p) / 4; j = 0 (a whole warp's lines share j) is a shift
+    auto turn = [&] {
+        v[0] = fix::rshift(v[0], 2);
+        if (j == 0) {
+#pragma unroll
+            for (int p = 1; p < R; ++p) v[p] = fix::rshift(v[p], 2);
+            return;
+        }
+#pragma unroll
+        for (int p = 1; p < R; ++p) {
+            const int4 w = __ldg(reinterpret_cast<const int4 *>(tw + j * p * twstep));
+            v[p] = fix::mul_w<INV>(v[p], W4{w.x, w.y, w.z, w.w});
+        }
+    };
+    if (INV && twiddle) turn();
+    fix::dft<R, INV>(v);
+    if (!INV && twiddle) turn();
+    unsigned m = 0;
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+        s[base + q * step] = v[q];
+        m |= mag_hi(v[q]);
+    }
+    return m;
+}
+
+template <int R, bool INV, bool RAW>
+__device__ __forceinline__ unsigned stage(I2 *s, const AxisPlan &ax, int st, const W4 *tw, int nlines, unsigned nlmag,
+                                          int lstride, int es, int sh, int s0) {
+    const int N = ax.N, len = ax.len[st], sub = ax.sub[st];
+    const unsigned smag = ax.submag[st];
+    const int total = N / R * nlines, twstep = N / len, step = sub * es;
+    unsigned m = 0;
+    for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
+        const int bf = qdiv(idx, nlmag), line = idx - bf * nlines;   // consecutive threads: consecutive lines
+        const int b = qdiv(bf, smag), j = bf - b * sub;
+        m |= bfly<R, INV, RAW>(s, line * lstride + (b * len + j) * es, step, j, twstep, tw, sh, s0, sub > 1);
+    }
+    return m;
+}
+
+// bits that the first stage of a transform provides for
+__device__ __forceinline__ int first_growth(const AxisPlan &ax, bool inv) {
+    return fix::growth(ax.radix[inv ? ax.nstage - 1 : 0]);
+}
+
+// All stages of nlines transforms in shared memory (fft.cu's fft_lines).  Each stage brings its
+// inputs to the largest scale at which its sums cannot overflow, from the bits that the stage
+// before left (slot: three words in turn, so that one can be cleared while the others are in use).
+// RAW: the first stage reads doubles, scaled by 2^s0 to sc.bits as it reads them.
+template <bool INV, bool RAW>
+__device__ void lines(I2 *s, const AxisPlan &ax, const W4 *tw, int nlines, unsigned nlmag, int lstride, int es, Scale &sc,
+                      int s0, unsigned *slot) {
+    for (int t = 0; t < ax.nstage; ++t) {
+        const int st = INV ? ax.nstage - 1 - t : t;
+        const int r = ax.radix[st];
+        const bool twiddle = ax.sub[st] > 1;
+        const int sh = sc.bits - (INV && twiddle ? 2 : 0) - (fix::TOP - fix::growth(r));
+        sc.e += sh + (twiddle ? 2 : 0);
+        const int now = sc.n % 3;
+        if (threadIdx.x == 0) slot[(now + 1) % 3] = 0;
+        unsigned m;
+        if (RAW && t == 0) {
+            switch (r) {
+                case 2: m = stage<2, INV, RAW>(s, ax, st, tw, nlines, nlmag, lstride, es, sh, s0); break;
+                case 3: m = stage<3, INV, RAW>(s, ax, st, tw, nlines, nlmag, lstride, es, sh, s0); break;
+                case 4: m = stage<4, INV, RAW>(s, ax, st, tw, nlines, nlmag, lstride, es, sh, s0); break;
+                case 5: m = stage<5, INV, RAW>(s, ax, st, tw, nlines, nlmag, lstride, es, sh, s0); break;
+                default: m = stage<8, INV, RAW>(s, ax, st, tw, nlines, nlmag, lstride, es, sh, s0); break;
+            }
+        } else {
+            switch (r) {
+                case 2: m = stage<2, INV, false>(s, ax, st, tw, nlines, nlmag, lstride, es, sh, s0); break;
+                case 3: m = stage<3, INV, false>(s, ax, st, tw, nlines, nlmag, lstride, es, sh, s0); break;
+                case 4: m = stage<4, INV, false>(s, ax, st, tw, nlines, nlmag, lstride, es, sh, s0); break;
+                case 5: m = stage<5, INV, false>(s, ax, st, tw, nlines, nlmag, lstride, es, sh, s0); break;
+                default: m = stage<8, INV, false>(s, ax, st, tw, nlines, nlmag, lstride, es, sh, s0); break;
+            }
+        }
+        sc.bits = bits_hi(block_or(m, slot + now));
+        ++sc.n;
+    }
+}
+
+// shifts that bring rows of the given blocks to one exponent, the largest value just below
+// 2^bits: row r is read as rshift(v, shift[r]) (left for negative shifts) in units of 2^(return value);
+// BAD if a block is.
+__device__ __forceinline__ int row_shifts(const Meta *meta, int rows, int bits, int *shift, int stride, int *red) {
+    int top = EMPTY, bad = 0;
+    Meta m{EMPTY, 0};
+    if ((int)threadIdx.x < rows) {
+        m = meta[threadIdx.x];
+        bad = m.e == BAD;
+        top = bad ? EMPTY : m.e + m.bits;
+    }
+    const int any = __syncthreads_or(bad);
+    if ((int)threadIdx.x == 0) *red = EMPTY;
+    __syncthreads();
+    const int e = block_max(top, red) - bits;
+    if ((int)threadIdx.x < rows) shift[threadIdx.x * stride] = min(max(e - m.e, -62), 63);
+    __syncthreads();
+    return any ? BAD : (e < EMPTY / 2 ? 0 : e);
+}
+__device__ __forceinline__ i64 shifted(i64 v, int s) {
+    if (s < 0) return v << -s;
+    return s > 62 ? 0 : fix::rshift(v, s);
+}
+
+__device__ __forceinline__ double value(i64 v, int e) {
+    bool odd;
+    const u64 b = fix::to_double_bits(v, e, &odd);
+    return odd ? scalbn((double)v, e) : __longlong_as_double((long long)b);
+}
+
+}  // namespace
+
+// ---- xy forward pass ------------------------------------------------------------
+template <Src SRC>
+__global__ void __launch_bounds__(MAX_THREADS)
+k_xy_forward_fix(FixTabs tb, const double2 *__restrict__ src, const double2 *__restrict__ src2,
+                 const double *__restrict__ theta, const int *__restrict__ act, const double *__restrict__ rsrc, int RS,
+                 I2 *__restrict__ dst, Meta *__restrict__ meta) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    int *red = reinterpret_cast<int *>(smem_raw);
+    I2 *s_plane = reinterpret_cast<I2 *>(smem_raw + HEAD);
+    const int Nx = tb.ax[0].N, Ny = tb.ax[1].N, Nz = tb.ax[2].N;
+    const int z = blockIdx.x, band = blockIdx.y;
+    const int plane = Nx * Ny;
+    const size_t n = (size_t)plane * Nz, off = (size_t)z * plane;
+    const unsigned nxm = tb.ax[0].nmag;
+    unsigned *slot = reinterpret_cast<unsigned *>(red + 4);
+    if (threadIdx.x < 8) red[threadIdx.x] = 0;
+    int hmax = 0;
+    auto put = [&](int i, double2 v) {
+        const int hx = __double2hiint(v.x), hy = __double2hiint(v.y);
+        hmax = max(hmax, max(hx & 0x7fffffff, hy & 0x7fffffff));
+        s_plane[pidx(i, Nx, RS, nxm)] = I2{__double_as_longlong(v.x), __double_as_longlong(v.y)};
+    };
+    if (SRC == Src::Plain) {
+        const double2 *in = src + band * n + off;
+        stage_in<double2>(plane, [&](int i) { return in[i]; }, put);
+    } else if (SRC == Src::Residual) {
+        const int b = act[band];
+        const double th = theta[b];
+        const double2 *hx = src + b * n + off, *x = src2 + b * n + off;
+        stage_in<double2>(plane, [&](int i) {
+            const double2 h = hx[i], v = x[i];
+            return make_double2(h.x - th * v.x, h.y - th * v.y);
+        }, put);
+    } else {
+        const double *in = rsrc + off;
+        stage_in<double2>(plane, [&](int i) { return make_double2(in[i], 0.0); }, put);
+    }
+    __syncthreads();
+    const int top = block_max(hmax, red) >> 20;
+    Meta *m = meta + (size_t)band * Nz + z;
+    if (top == 0x7ff) {
+        if (threadIdx.x == 0) *m = Meta{BAD, 0};
+        return;
+    }
+    const int bits0 = fix::TOP - first_growth(tb.ax[0], false), s0 = bits0 - (top - 1022);
+    Scale sc{bits0, -s0, 0};
+    lines<false, true>(s_plane, tb.ax[0], tb.tw[0], Ny, tb.ax[1].nmag, RS, 1, sc, s0, slot);
+    lines<false, false>(s_plane, tb.ax[1], tb.tw[1], Nx, tb.ax[0].nmag, 1, RS, sc, 0, slot);
+    I2 *out = dst + band * n + off;
+    for (int i = threadIdx.x; i < plane; i += blockDim.x) out[i] = s_plane[pidx(i, Nx, RS, nxm)];
+    if (threadIdx.x == 0) *m = Meta{top == 0 ? EMPTY : sc.e, sc.bits};
+}
+
+// ---- z pass with the per-G factor ------------------------------------------------
+template <Mid MID> __device__ __forceinline__ double factor(const FixTabs &tb, int x, int y, int z) {
+    if constexpr (MID == Mid::GradX) return tb.g1[0][x] * tb.inv_n;
+    if constexpr (MID == Mid::GradY) return tb.g1[1][y] * tb.inv_n;
+    if constexpr (MID == Mid::GradZ) return tb.g1[2][z] * tb.inv_n;
+    const double g2 = tb.g2[0][x] + tb.g2[1][y] + tb.g2[2][z];   // Hartree
+    return g2 > 0.0 ? 4.0 * M_PI / g2 * tb.inv_n : 0.0;
+}
+__device__ __forceinline__ double tpa_factor(double x) {
+    const double num = 27.0 + x * (18.0 + x * (12.0 + 8.0 * x));
+    return num / (num + 16.0 * x * x * x * x);
+}
+__device__ __forceinline__ i64 fixed_factor(double f, int s) {
+    return fix::from_double(__double2hiint(f), (unsigned)__double2loint(f), s);
+}
+
+// tab: TPA's factor depends on |k| of each axis only, so a slab evaluates it once per (|kz|, |kx|),
+// into shared memory after the slab (table != 0), a quarter of the FP64 divisions; slabs too large
+// for that evaluate it per point.
+template <Mid MID>
+__global__ void __launch_bounds__(MAX_THREADS)
+k_z_mid_fix(FixTabs tb, I2 *__restrict__ buf, const double *__restrict__ tkin, const Meta *__restrict__ min,
+            Meta *__restrict__ mout, int table) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    int *red = reinterpret_cast<int *>(smem_raw);
+    I2 *s_slab = reinterpret_cast<I2 *>(smem_raw + HEAD);
+    const int Nx = tb.ax[0].N, Ny = tb.ax[1].N, Nz = tb.ax[2].N;
+    const int y = blockIdx.x, band = blockIdx.y;
+    const size_t zstride = (size_t)Nx * Ny;
+    I2 *base = buf + band * zstride * Nz + (size_t)y * Nx;
+    const int tot = Nx * Nz;
+    const unsigned nxm = tb.ax[0].nmag;
+    int *shift = reinterpret_cast<int *>(s_slab + tot);
+    i64 *tab = reinterpret_cast<i64 *>(shift + SHIFTS / 4);
+    const int hx = Nx / 2 + 1, hz = Nz / 2 + 1;
+    double tk = 1.0;
+    if (MID == Mid::Tpa) {
+        const double t = tkin[band];
+        if (t >= 1e-12) tk = t;
+    }
+    unsigned *slot = reinterpret_cast<unsigned *>(red + 4);
+    if (threadIdx.x > 0 && threadIdx.x < 8) red[threadIdx.x] = threadIdx.x == 1 ? EMPTY : 0;
+    const int bits0 = fix::TOP - first_growth(tb.ax[2], false);
+    Meta *m = mout + (size_t)band * Ny + y;
+    const int e0 = row_shifts(min + (size_t)band * Nz, Nz, bits0, shift, 1, red);
+    if (e0 == BAD) {
+        if (threadIdx.x == 0) *m = Meta{BAD, 0};
+        return;
+    }
+    stage_in<I2>(tot, [&](int i) {
+        const int z = qdiv(i, nxm), x = i - z * Nx;
+        return base[z * zstride + x];
+    }, [&](int i, I2 v) {
+        const int s = shift[qdiv(i, nxm)];
+        s_slab[i] = I2{shifted(v.x, s), shifted(v.y, s)};
+    });
+    if (MID == Mid::Tpa && table) {
+        const double gy = tb.g2[1][y];
+        for (int i = threadIdx.x; i < hx * hz; i += blockDim.x) {
+            const int z = i / hx, x = i - z * hx;
+            const double g2 = tb.g2abs[0][x] + gy + tb.g2abs[2][z];
+            tab[i] = fixed_factor(tpa_factor(0.5 * g2 / tk) * tb.inv_n, tb.fexp);
+        }
+    }
+    __syncthreads();
+    Scale sc{bits0, e0, 0};
+    lines<false, false>(s_slab, tb.ax[2], tb.tw[2], Nx, nxm, 1, Nx, sc, 0, slot);
+    const i64 ky = MID == Mid::Kinetic ? tb.kin[1][y] : 0;
+    auto f_of = [&](int i, bool &neg) -> i64 {
+        const int z = qdiv(i, nxm), x = i - z * Nx;
+        if constexpr (MID == Mid::Kinetic) {
+            return tb.kin[0][x] + ky + tb.kin[2][z];
+        } else if constexpr (MID == Mid::Tpa) {
+            if (table) return tab[(int)tb.fabs[2][z] * hx + tb.fabs[0][x]];
+            const double g2 = tb.g2[0][x] + tb.g2[1][y] + tb.g2[2][z];
+            return fixed_factor(tpa_factor(0.5 * g2 / tk) * tb.inv_n, tb.fexp);
+        } else {
+            const double f = factor<MID>(tb, x, y, z);
+            neg = f < 0.0;
+            return fixed_factor(fabs(f), tb.fexp);
+        }
+    };
+    // bits of the largest product v F 2^-62, then the products shifted to it
+    int big = EMPTY;
+    bool neg = false;
+    for (int i = threadIdx.x; i < tot; i += blockDim.x) {
+        const i64 f = f_of(i, neg);
+        if (f) big = max(big, bits_hi(mag_hi(s_slab[i])) - __clzll(f));
+    }
+    big = block_max(big, red + 1);
+    const int g = big <= EMPTY / 2 ? 0 : fix::TOP - big;   // normalising by clz - 2 gives the 2 of pr's bound back
+    constexpr bool GRAD = MID == Mid::GradX || MID == Mid::GradY || MID == Mid::GradZ;
+    for (int i = threadIdx.x; i < tot; i += blockDim.x) {
+        bool ng = false;
+        const i64 f = f_of(i, ng);
+        I2 v{0, 0};
+        if (f) {
+            const int nf = __clzll(f) - 2;
+            const i64 w = f << nf;                                // in [2^61, 2^62)
+            v = fix::mul_w<false>(s_slab[i], W4{fix::hi_of(w), fix::lo_of(w), 0, 0});   // v w 2^-64
+            const int d = g - nf;
+            v = I2{shifted(v.x, -d), shifted(v.y, -d)};
+            if (GRAD) v = ng ? fix::rot<false>(v) : fix::rot<true>(v);   // i f v
+        }
+        s_slab[i] = v;
+    }
+    __syncthreads();
+    sc.bits = fix::TOP;
+    sc.e += 64 - (MID == Mid::Kinetic ? tb.kexp : tb.fexp) - g;
+    lines<true, false>(s_slab, tb.ax[2], tb.tw[2], Nx, nxm, 1, Nx, sc, 0, slot);
+    for (int i = threadIdx.x; i < tot; i += blockDim.x) {
+        const int z = qdiv(i, nxm), x = i - z * Nx;
+        base[z * zstride + x] = s_slab[i];
+    }
+    if (threadIdx.x == 0) *m = Meta{big <= EMPTY / 2 ? EMPTY : sc.e, sc.bits};
+}
+
+// ---- xy inverse pass + epilogue ------------------------------------------------------
+enum class FixEpi { Plain, Hpsi, Real };
+
+template <FixEpi EPI>
+__global__ void __launch_bounds__(MAX_THREADS)
+k_xy_inverse_fix(FixTabs tb, const I2 *__restrict__ buf, const Meta *__restrict__ meta, const double2 *__restrict__ psi,
+                 const double *__restrict__ vloc, ProjTables pt, const double2 *__restrict__ p, int RS,
+                 double2 *__restrict__ out, double *__restrict__ rout, int stage_pe) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    int *red = reinterpret_cast<int *>(smem_raw);
+    I2 *s_plane = reinterpret_cast<I2 *>(smem_raw + HEAD);
+    const int Nx = tb.ax[0].N, Ny = tb.ax[1].N, Nz = tb.ax[2].N;
+    int *shift = reinterpret_cast<int *>(RS > Nx ? s_plane + Nx : s_plane + (size_t)Ny * RS);
+    const int sst = RS > Nx ? 4 * RS : 1;
+    const int z = blockIdx.x, band = blockIdx.y;
+    const int plane = Nx * Ny;
+    const size_t n = (size_t)plane * Nz, off = (size_t)z * plane;
+    const I2 *in = buf + band * n + off;
+    const unsigned nxm = tb.ax[0].nmag;
+    unsigned *slot = reinterpret_cast<unsigned *>(red + 4);
+    if (threadIdx.x > 0 && threadIdx.x < 8) red[threadIdx.x] = 0;
+    const int bits0 = fix::TOP + (tb.ax[1].sub[tb.ax[1].nstage - 1] > 1 ? 2 : 0) - first_growth(tb.ax[1], true);
+    const int e0 = row_shifts(meta + (size_t)band * Ny, Ny, bits0, shift, sst, red);
+    Scale sc{bits0, e0, 0};
+    if (e0 != BAD) {
+        stage_in<I2>(plane, [&](int i) { return in[i]; }, [&](int i, I2 v) {
+            const int s = shift[qdiv(i, nxm) * sst];
+            s_plane[pidx(i, Nx, RS, nxm)] = I2{shifted(v.x, s), shifted(v.y, s)};
+        });
+        __syncthreads();
+        lines<true, false>(s_plane, tb.ax[1], tb.tw[1], Nx, nxm, 1, RS, sc, 0, slot);
+        lines<true, false>(s_plane, tb.ax[0], tb.tw[0], Ny, tb.ax[1].nmag, RS, 1, sc, 0, slot);
+    }
+    const double nan = __longlong_as_double(0x7ff8000000000000ll);
+    auto at = [&](int i) {
+        if (e0 == BAD) return make_double2(nan, nan);
+        const I2 v = s_plane[pidx(i, Nx, RS, nxm)];
+        return make_double2(value(v.x, sc.e), value(v.y, sc.e));
+    };
+    if (EPI == FixEpi::Plain) {
+        double2 *o = out + band * n + off;
+        for (int i = threadIdx.x; i < plane; i += blockDim.x) o[i] = at(i);
+    } else if (EPI == FixEpi::Real) {
+        double *o = rout + off;
+        for (int i = threadIdx.x; i < plane; i += blockDim.x) o[i] = at(i).x;
+    } else {
+        const double2 *ps = psi + band * n + off;
+        const double *vv = vloc + off;
+        const int np = pt.natom * pt.nproj;
+        const double2 *pb = p + (size_t)band * np;
+        // E_aj <beta_aj|psi> of this band, staged once per CTA after the plane
+        // (when it fits; else read from global memory)
+        double2 *s_pe = reinterpret_cast<double2 *>(s_plane + (size_t)Ny * RS + (RS > Nx ? 0 : SHIFTS / 16));
+        if (stage_pe) {
+            for (int q = threadIdx.x; q < np; q += blockDim.x) {
+                const double2 c = pb[q];
+                const double e = pt.e_kb[q];
+                s_pe[q] = make_double2(e * c.x, e * c.y);
+            }
+            __syncthreads();
+        }
+        double2 *o = out + band * n + off;
+        for (int i = threadIdx.x; i < plane; i += blockDim.x) {
+            const double2 t = at(i);
+            const double2 y = ps[i];
+            const double vi = vv[i];
+            double ax = t.x + vi * y.x, ay = t.y + vi * y.y;
+            const int g = (int)off + i;
+            const int e0_ = pt.c_rowptr[g], e1 = pt.c_rowptr[g + 1];
+            for (int e = e0_; e < e1; ++e) {
+                const int a0 = pt.c_atom[e] * pt.nproj;
+                double bt[4];
+                beta4(pt.c_beta + 4 * (size_t)e, bt);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (j >= pt.nproj) break;
+                    double2 q;
+                    if (stage_pe) {
+                        q = s_pe[a0 + j];
+                    } else {
+                        const double2 c = pb[a0 + j];
+                        const double ek = pt.e_kb[a0 + j];
+                        q = make_double2(ek * c.x, ek * c.y);
+                    }
+                    ax += bt[j] * q.x;
+                    ay += bt[j] * q.y;
+                }
+            }
+            o[i] = make_double2(ax, ay);
+        }
+    }
+}
+
+// ---- host side -------------------------------------------------------------------------
+namespace {
+
+// An xy plane: rows padded to an odd stride, or as they are with the shifts behind them
+int plane_stride(const rsdft_ctx *ctx) { return ctx->N[0] | 1; }
+size_t plane_smem(const rsdft_ctx *ctx) {
+    return HEAD + (size_t)(ctx->N[0] | 1) * ctx->N[1] * sizeof(I2) + (ctx->N[0] & 1 ? SHIFTS : 0);
+}
+
+// what the passes take: planes and slabs of at most 227 KB with an odd stride
+rsdft_status check_plane(rsdft_ctx *ctx) {
+    const size_t odd = (size_t)(ctx->N[0] | 1) * ctx->N[1] * sizeof(I2), slab = (size_t)ctx->N[0] * ctx->N[2] * sizeof(I2);
+    if (std::max(odd, slab) > MAX_DYN_SMEM)
+        return fail(ctx, RSDFT_E_INVALID, "plane needs %zu B of shared memory", std::max(odd, slab));
+    return RSDFT_OK;
+}
+
+// A radix-8 butterfly a thread, 256 threads where three CTAs share an SM, else enough to fill it
+// alone or in pairs (and at least one thread a row)
+int threads_for(size_t smem, int points) {
+    if (smem <= 75 * 1024) return std::max(128, std::min(256, cdiv(points, 256) * 32));
+    return smem <= 113 * 1024 ? 384 : 768;
+}
+
+rsdft_status ensure_meta(rsdft_ctx *ctx, int nb, Meta **planes, Meta **slabs) {
+    FixFft &f = ctx->fix;
+    if (nb > f.cap_band) {
+        if (f.meta) {
+            cudaFree(f.meta);
+            ctx->owned.erase(std::remove(ctx->owned.begin(), ctx->owned.end(), f.meta), ctx->owned.end());
+        }
+        f.meta = nullptr;
+        f.cap_band = 0;
+        RS_TRY(dev_alloc(ctx, &f.meta, (size_t)nb * (ctx->N[1] + ctx->N[2]) * sizeof(Meta)));
+        f.cap_band = nb;
+    }
+    *planes = static_cast<Meta *>(f.meta);
+    *slabs = *planes + (size_t)nb * ctx->N[2];
+    return RSDFT_OK;
+}
+
+FixTabs tabs_of(const rsdft_ctx *ctx) {
+    FixTabs t;
+    for (int a = 0; a < 3; ++a) {
+        t.ax[a] = ctx->fft.ax[a];
+        t.tw[a] = static_cast<const W4 *>(ctx->fix.tw[a]);
+        t.kin[a] = ctx->fix.kin[a];
+        t.g2[a] = ctx->fft.g2pos[a];
+        t.g1[a] = ctx->fft.gpos[a];
+        t.g2abs[a] = ctx->fix.g2abs[a];
+        t.fabs[a] = ctx->fix.fabs[a];
+    }
+    t.kexp = ctx->fix.kexp;
+    t.inv_n = 1.0 / (double)ctx->n;
+    t.fexp = 0;
+    return t;
+}
+
+}  // namespace
+
+rsdft_status fft_xy_forward(rsdft_ctx *ctx, Src kind, const double2 *src, const double2 *src2, const double *theta,
+                            const int *act, const double *rsrc, double2 *dst, int nb, cudaStream_t st) {
+    if (nb <= 0) return RSDFT_OK;
+    RS_TRY(check_plane(ctx));
+    Meta *mp, *ms;
+    RS_TRY(ensure_meta(ctx, nb, &mp, &ms));
+    const int RS = plane_stride(ctx);
+    const size_t sm = HEAD + (size_t)RS * ctx->N[1] * sizeof(I2);
+    const dim3 grid(ctx->N[2], nb);
+    const int th = threads_for(sm, ctx->N[0] * ctx->N[1]);
+    const double nxy = (double)ctx->N[0] * ctx->N[1];
+    const double bpp = kind == Src::Plain ? 32.0 : (kind == Src::Residual ? 48.0 : 24.0);
+    ProfScope ps(ctx, RSDFT_K_FFT_XY_FWD, 5.0 * nxy * std::log2(nxy) * ctx->N[2] * nb, bpp * (double)ctx->n * nb, st);
+    const FixTabs tb = tabs_of(ctx);
+    I2 *o = reinterpret_cast<I2 *>(dst);
+    switch (kind) {
+        case Src::Plain:
+            RS_TRY(set_smem(ctx, k_xy_forward_fix<Src::Plain>, sm));
+            k_xy_forward_fix<Src::Plain><<<grid, th, sm, st>>>(tb, src, src2, theta, act, rsrc, RS, o, mp);
+            break;
+        case Src::Residual:
+            RS_TRY(set_smem(ctx, k_xy_forward_fix<Src::Residual>, sm));
+            k_xy_forward_fix<Src::Residual><<<grid, th, sm, st>>>(tb, src, src2, theta, act, rsrc, RS, o, mp);
+            break;
+        case Src::RealField:
+            RS_TRY(set_smem(ctx, k_xy_forward_fix<Src::RealField>, sm));
+            k_xy_forward_fix<Src::RealField><<<grid, th, sm, st>>>(tb, src, src2, theta, act, rsrc, RS, o, mp);
+            break;
+    }
+    RS_LAUNCHED(ctx, "k_xy_forward_fix");
+    return RSDFT_OK;
+}
+
+rsdft_status fft_z_mid(rsdft_ctx *ctx, Mid mid, double2 *buf, const double *tkin, int nb, cudaStream_t st) {
+    if (nb <= 0) return RSDFT_OK;
+    RS_TRY(check_plane(ctx));
+    Meta *mp, *ms;
+    RS_TRY(ensure_meta(ctx, nb, &mp, &ms));
+    size_t sm = HEAD + (size_t)ctx->N[0] * ctx->N[2] * sizeof(I2) + SHIFTS;
+    const size_t tabb = (size_t)(ctx->N[0] / 2 + 1) * (ctx->N[2] / 2 + 1) * sizeof(i64);
+    int table = 0;
+    if (mid == Mid::Tpa && sm + tabb <= MAX_DYN_SMEM) {
+        table = 1;
+        sm += tabb;
+    }
+    const dim3 grid(ctx->N[1], nb);
+    const int th = threads_for(sm, ctx->N[0] * ctx->N[2]);
+    ProfScope ps(ctx, RSDFT_K_FFT_Z, 10.0 * (double)ctx->n * std::log2((double)ctx->N[2]) * nb, 32.0 * (double)ctx->n * nb, st);
+    FixTabs tb = tabs_of(ctx);
+    // bound of the factor: 1 (TPA), 4 pi / min G^2, max |G|; all divided by n
+    double fmax = 1.0;
+    const double gmin = 2.0 * M_PI / std::max(ctx->L[0], std::max(ctx->L[1], ctx->L[2]));
+    if (mid == Mid::Hartree) fmax = 4.0 * M_PI / (gmin * gmin);
+    else if (mid == Mid::GradX) fmax = M_PI * ctx->N[0] / ctx->L[0];
+    else if (mid == Mid::GradY) fmax = M_PI * ctx->N[1] / ctx->L[1];
+    else if (mid == Mid::GradZ) fmax = M_PI * ctx->N[2] / ctx->L[2];
+    tb.fexp = 59 - std::ilogb(fmax * tb.inv_n);   // |f| 2^fexp < 2^60
+    I2 *b = reinterpret_cast<I2 *>(buf);
+#define RS_Z(M)                                                              \
+    case M:                                                                  \
+        RS_TRY(set_smem(ctx, k_z_mid_fix<M>, sm));                           \
+        k_z_mid_fix<M><<<grid, th, sm, st>>>(tb, b, tkin, mp, ms, table);    \
+        break;
+    switch (mid) {
+        RS_Z(Mid::Kinetic)
+        RS_Z(Mid::Tpa)
+        RS_Z(Mid::Hartree)
+        RS_Z(Mid::GradX)
+        RS_Z(Mid::GradY)
+        RS_Z(Mid::GradZ)
+    }
+#undef RS_Z
+    RS_LAUNCHED(ctx, "k_z_mid_fix");
+    return RSDFT_OK;
+}
+
+rsdft_status fft_xy_inverse(rsdft_ctx *ctx, const double2 *buf, const double2 *psi, const double2 *p, double2 *out,
+                            double *rout, int nb, cudaStream_t st) {
+    if (nb <= 0) return RSDFT_OK;
+    RS_TRY(check_plane(ctx));
+    Meta *mp, *ms;
+    RS_TRY(ensure_meta(ctx, nb, &mp, &ms));
+    // the plane plus, when it fits, the band's E_aj <beta_aj|psi> after it
+    const size_t pe = psi ? (size_t)ctx->pt.natom * ctx->pt.nproj * sizeof(double2) : 0;
+    const int RS = plane_stride(ctx);
+    const int stage = psi && plane_smem(ctx) + pe <= MAX_DYN_SMEM ? 1 : 0;
+    const size_t sm = plane_smem(ctx) + (stage ? pe : 0);
+    const dim3 grid(ctx->N[2], nb);
+    const int th = threads_for(sm, ctx->N[0] * ctx->N[1]);
+    const double nxy = (double)ctx->N[0] * ctx->N[1];
+    const double bpp = rout ? 24.0 : (psi ? 48.0 : 32.0);
+    ProfScope ps(ctx, RSDFT_K_FFT_XY_INV, 5.0 * nxy * std::log2(nxy) * ctx->N[2] * nb,
+                 bpp * (double)ctx->n * nb + (psi ? 8.0 * (double)ctx->n : 0.0), st);
+    const FixTabs tb = tabs_of(ctx);
+    const I2 *b = reinterpret_cast<const I2 *>(buf);
+    if (rout) {
+        RS_TRY(set_smem(ctx, k_xy_inverse_fix<FixEpi::Real>, sm));
+        k_xy_inverse_fix<FixEpi::Real><<<grid, th, sm, st>>>(tb, b, ms, psi, ctx->v, ctx->pt, p, RS, out, rout, 0);
+    } else if (psi) {
+        RS_TRY(set_smem(ctx, k_xy_inverse_fix<FixEpi::Hpsi>, sm));
+        k_xy_inverse_fix<FixEpi::Hpsi><<<grid, th, sm, st>>>(tb, b, ms, psi, ctx->v, ctx->pt, p, RS, out, rout, stage);
+    } else {
+        RS_TRY(set_smem(ctx, k_xy_inverse_fix<FixEpi::Plain>, sm));
+        k_xy_inverse_fix<FixEpi::Plain><<<grid, th, sm, st>>>(tb, b, ms, psi, ctx->v, ctx->pt, p, RS, out, rout, 0);
+    }
+    RS_LAUNCHED(ctx, "k_xy_inverse_fix");
+    return RSDFT_OK;
+}
+
+}  // namespace rsdft

@@ -117,6 +117,17 @@ struct NnState {
     float *tr = nullptr;   size_t tr_cap = 0;      // training activations and gradients
 };
 
+// Tables and block exponents of the fixed-point FP64 transforms (fft_fix.cu).
+struct FixFft {
+    const void *tw[3] = {};                  // [N] exp(-2 pi i k / N) as fix::W4
+    const long long *kin[3] = {};            // G_a^2 / (2 n) 2^kexp by position
+    int kexp = 0;
+    const double *g2abs[3] = {};             // G_a^2 by |frequency index|
+    const unsigned char *fabs[3] = {};       // |frequency index| by position
+    void *meta = nullptr;                    // exponents of the planes and slabs in flight
+    int cap_band = 0;
+};
+
 // Residue-arithmetic products (rns.cu): residue planes and scratch, and the device flag
 // that hands a call back to the FP64 kernels.
 struct RnsWork {
@@ -155,6 +166,7 @@ struct rsdft_ctx {
     rsdft::Profiler prof;
     rsdft::NnState nn;
     rsdft::RnsWork rns;
+    rsdft::FixFft fix;
     long long launches = 0;          // every kernel launched on this context
     long long coop_fallbacks = 0;    // tridiagonalisations that could not launch cooperatively
     int coop_last_error = 0;         // cudaError_t of the last such launch
@@ -203,9 +215,11 @@ rsdft_status ensure_workspace(rsdft_ctx *ctx, int nband);
 inline cudaStream_t as_stream(void *s) { return reinterpret_cast<cudaStream_t>(s); }
 inline int cdiv(long long a, long long b) { return (int)((a + b - 1) / b); }
 
-// ---- FFT / H psi (fft.cu) ---------------------------------------------------
-enum class Mid { Kinetic, Tpa, Hartree, Scale, GradX, GradY, GradZ };
+// ---- FFT / H psi (fft.cu, fft_fix.cu) ---------------------------------------------------
+enum class Mid { Kinetic, Tpa, Hartree, GradX, GradY, GradZ };   // FP32: Kinetic and Tpa
 enum class Src { Plain, Residual, RealField };
+// FP64 passes (fft_fix.cu).  Between them the buffer holds fixed-point values whose exponents are kept
+// in the context, so the three passes of a transform follow one another on one stream.
 // Forward xy-plane pass: src -> dst ([nb][n] complex).  Src::Residual reads
 // hx[act[b]] - theta[act[b]] x[act[b]]; Src::RealField reads a real [n] field
 // (nb must be 1).
