@@ -46,23 +46,7 @@ static rsdft_status upload(rsdft_ctx *ctx, T **dst, const T *src, size_t count) 
     return RSDFT_OK;
 }
 
-// N = 2^a 3^b 5^c, 2 <= N <= MAX_N.  Radices: 8s and 4s for the power of two
-// (fewer stages), then 3s, then 5s.
-static bool make_axis_plan(int N, AxisPlan &p) {
-    if (N < 2 || N > MAX_N) return false;
-    int n = N, p2 = 0, p3 = 0, p5 = 0;
-    while (n % 2 == 0) { n /= 2; ++p2; }
-    while (n % 3 == 0) { n /= 3; ++p3; }
-    while (n % 5 == 0) { n /= 5; ++p5; }
-    if (n != 1) return false;
-    std::vector<int> r;
-    if (p2 % 3 == 0) { for (int i = 0; i < p2 / 3; ++i) r.push_back(8); }
-    else if (p2 % 3 == 1) {
-        if (p2 >= 4) { r.push_back(4); r.push_back(4); for (int i = 0; i < (p2 - 4) / 3; ++i) r.push_back(8); }
-        else r.push_back(2);
-    } else { r.push_back(4); for (int i = 0; i < (p2 - 2) / 3; ++i) r.push_back(8); }
-    for (int i = 0; i < p3; ++i) r.push_back(3);
-    for (int i = 0; i < p5; ++i) r.push_back(5);
+static bool fill_axis_plan(int N, const std::vector<int> &r, AxisPlan &p) {
     if ((int)r.size() > MAX_STAGES) return false;
     p.N = N;
     p.nstage = (int)r.size();
@@ -81,6 +65,41 @@ static bool make_axis_plan(int N, AxisPlan &p) {
         p.bfmag[s] = mag(N / r[s]);
     }
     return true;
+}
+
+// N = 2^a 3^b 5^c, 2 <= N <= MAX_N.  Radices: 8s and 4s for the power of two
+// (fewer stages), then 3s, then 5s.
+static bool make_axis_plan(int N, AxisPlan &p) {
+    if (N < 2 || N > MAX_N) return false;
+    int n = N, p2 = 0, p3 = 0, p5 = 0;
+    while (n % 2 == 0) { n /= 2; ++p2; }
+    while (n % 3 == 0) { n /= 3; ++p3; }
+    while (n % 5 == 0) { n /= 5; ++p5; }
+    if (n != 1) return false;
+    std::vector<int> r;
+    if (p2 % 3 == 0) { for (int i = 0; i < p2 / 3; ++i) r.push_back(8); }
+    else if (p2 % 3 == 1) {
+        if (p2 >= 4) { r.push_back(4); r.push_back(4); for (int i = 0; i < (p2 - 4) / 3; ++i) r.push_back(8); }
+        else r.push_back(2);
+    } else { r.push_back(4); for (int i = 0; i < (p2 - 2) / 3; ++i) r.push_back(8); }
+    for (int i = 0; i < p3; ++i) r.push_back(3);
+    for (int i = 0; i < p5; ++i) r.push_back(5);
+    return fill_axis_plan(N, r, p);
+}
+
+// The FP32 passes hold up to 16 points in registers: two balanced stages where N has them (the largest
+// radix as small as it can be), else the radices above.
+static void make_axis_plan32(int N, const AxisPlan &base, AxisPlan &p) {
+    static const int R[] = {2, 3, 4, 5, 6, 8, 9, 10, 12, 16};
+    std::vector<int> best;
+    for (int a : R) {
+        if (a == N) best = {a};
+        for (int b : R)
+            if (a * b == N && a >= b && (best.empty() || (best.size() == 2 && a < best[0]) || (best.size() == 1 && best[0] > 8)))
+                best = {a, b};
+    }
+    if (best.empty()) p = base;
+    else fill_axis_plan(N, best, p);
 }
 
 // Frequency index held at a digit-reversed position after the forward stages.
@@ -107,7 +126,9 @@ static rsdft_status build_fft_tables(rsdft_ctx *ctx) {
             tw[k] = make_double2(c, s);
             twf[k] = make_float2((float)c, (float)s);
         }
+        make_axis_plan32(N, p, ctx->fft.ax32[a]);
         std::vector<double> g2(N), g1(N);
+        std::vector<float> g2f(N);
         double gunit = 2.0 * M_PI / ctx->L[a];
         for (int pos = 0; pos < N; ++pos) {
             int k = position_to_freq(p, pos);
@@ -118,7 +139,11 @@ static rsdft_status build_fft_tables(rsdft_ctx *ctx) {
             // real field its derivative is imaginary, i.e. 0 in the real part)
             g1[pos] = (N % 2 == 0 && k == N / 2) ? 0.0 : g;
         }
-        std::vector<float> g2f(g2.begin(), g2.end());
+        for (int pos = 0; pos < N; ++pos) {
+            const int k = position_to_freq(ctx->fft.ax32[a], pos);
+            const double g = gunit * (k < (N + 1) / 2 ? k : k - N);
+            g2f[pos] = (float)(g * g);
+        }
         double2 *d_tw; float2 *d_twf; double *d_g2; float *d_g2f; double *d_g1;
         RS_TRY(upload(ctx, &d_g1, g1.data(), N));
         ctx->fft.gpos[a] = d_g1;
@@ -182,94 +207,192 @@ static rsdft_status build_fix_tables(rsdft_ctx *ctx) {
 
 static inline double min_image(double d, double L) { return d - L * std::floor(d / L + 0.5); }
 
-// Per axis: the grid indices whose minimal-image displacement from R lies
-// strictly inside (-rcut, rcut), with those displacements.
+// Per axis: the grid indices whose minimal-image displacement from R lies strictly inside
+// (-rcut, rcut), by increasing displacement (consecutive modulo N, as rcut < L / 2).
 static void axis_window(int N, double L, double R, double rcut, std::vector<int> &idx,
                         std::vector<double> &disp) {
+    std::vector<std::pair<double, int>> w;
+    const double h = L / N;
+    for (int i = 0; i < N; ++i) {
+        const double d = min_image(i * h - R, L);
+        if (std::fabs(d) < rcut) w.emplace_back(d, i);
+    }
+    std::sort(w.begin(), w.end());
     idx.clear();
     disp.clear();
-    double h = L / N;
-    for (int i = 0; i < N; ++i) {
-        double d = min_image(i * h - R, L);
-        if (std::fabs(d) < rcut) { idx.push_back(i); disp.push_back(d); }
+    for (const auto &p : w) {
+        disp.push_back(p.first);
+        idx.push_back(p.second);
     }
 }
 
+// v in units of 2^-62 as high and (signed) low words; exact, |v| <= 1
+static void split62(double v, int &hi, int &lo) {
+    const long long q = (long long)std::nearbyint(std::ldexp(v, 62));
+    hi = fix::hi_of(q);
+    lo = fix::lo_of(q);
+}
+
+// The projectors as discs (proj.h): per atom its windows and factors, per plane its rows.
 static rsdft_status build_projectors(rsdft_ctx *ctx, const rsdft_projectors *pj) {
     const int natom = pj->natom, nproj = pj->nproj;
     const double rc = pj->rc, rcut = pj->rcut;
     const int Nx = ctx->N[0], Ny = ctx->N[1], Nz = ctx->N[2];
-    std::vector<int> a_start(natom + 1, 0), a_idx;
-    std::vector<double> a_beta;
-    std::vector<int> ix, iy, iz;
-    std::vector<double> dx, dy, dz;
+    struct Atom { std::vector<int> i[3]; std::vector<double> g[3], h[3], d[3]; };
+    std::vector<Atom> at(natom);
     for (int a = 0; a < natom; ++a) {
-        const double *R = pj->pos + 3 * a;
-        axis_window(Nx, ctx->L[0], R[0], rcut, ix, dx);
-        axis_window(Ny, ctx->L[1], R[1], rcut, iy, dy);
-        axis_window(Nz, ctx->L[2], R[2], rcut, iz, dz);
-        size_t first = a_idx.size();
-        // points in increasing linear index order (z, then y, then x)
-        std::vector<int> oz(iz.size()), oy(iy.size()), ox(ix.size());
-        for (size_t i = 0; i < oz.size(); ++i) oz[i] = (int)i;
-        for (size_t i = 0; i < oy.size(); ++i) oy[i] = (int)i;
-        for (size_t i = 0; i < ox.size(); ++i) ox[i] = (int)i;
-        std::sort(oz.begin(), oz.end(), [&](int p, int q) { return iz[p] < iz[q]; });
-        std::sort(oy.begin(), oy.end(), [&](int p, int q) { return iy[p] < iy[q]; });
-        std::sort(ox.begin(), ox.end(), [&](int p, int q) { return ix[p] < ix[q]; });
-        for (int kz : oz)
-            for (int ky : oy)
-                for (int kx : ox) {
-                    double d2 = dx[kx] * dx[kx] + dy[ky] * dy[ky] + dz[kz] * dz[kz];
-                    if (!(d2 < rcut * rcut)) continue;
-                    double g = std::exp(-d2 / (2.0 * rc * rc));
-                    a_idx.push_back((iz[kz] * Ny + iy[ky]) * Nx + ix[kx]);
-                    a_beta.push_back(g);
-                    a_beta.push_back(nproj == 4 ? dx[kx] / rc * g : 0.0);
-                    a_beta.push_back(nproj == 4 ? dy[ky] / rc * g : 0.0);
-                    a_beta.push_back(nproj == 4 ? dz[kz] / rc * g : 0.0);
-                }
-        // grid normalisation: sum beta^2 dV = 1
-        for (int j = 0; j < nproj; ++j) {
-            double s = 0.0;
-            for (size_t e = first; e < a_idx.size(); ++e) s += a_beta[4 * e + j] * a_beta[4 * e + j];
-            double c = s > 0.0 ? 1.0 / std::sqrt(s * ctx->dV) : 0.0;
-            for (size_t e = first; e < a_idx.size(); ++e) a_beta[4 * e + j] *= c;
+        const int N[3] = {Nx, Ny, Nz};
+        for (int k = 0; k < 3; ++k) {
+            axis_window(N[k], ctx->L[k], pj->pos[3 * a + k], rcut, at[a].i[k], at[a].d[k]);
+            for (double d : at[a].d[k]) {
+                const double g = std::exp(-d * d / (2.0 * rc * rc));
+                at[a].g[k].push_back(g);
+                at[a].h[k].push_back(d / rc * g);
+            }
         }
-        a_start[a + 1] = (int)a_idx.size();
     }
-    const long long nent = (long long)a_idx.size();
-    if (nent > 0x7fffffffLL) return fail(ctx, RSDFT_E_INVALID, "projector table too large");
-    // point-major CSR (entries of a point ordered by atom)
-    std::vector<int> rowptr(ctx->n + 1, 0), c_atom(nent);
-    std::vector<double> c_beta(4 * nent);
-    for (long long e = 0; e < nent; ++e) rowptr[a_idx[e] + 1]++;
-    for (long long i = 0; i < ctx->n; ++i) rowptr[i + 1] += rowptr[i];
-    std::vector<int> fillp(rowptr.begin(), rowptr.end() - 1);
+    // per plane its discs with their rows by increasing dy (and the sums of beta^2 per atom), then in the
+    // order of their colours
+    std::vector<std::vector<int>> zpos(natom, std::vector<int>(Nz, -1));
     for (int a = 0; a < natom; ++a)
-        for (int e = a_start[a]; e < a_start[a + 1]; ++e) {
-            int slot = fillp[a_idx[e]]++;
-            c_atom[slot] = a;
-            for (int j = 0; j < 4; ++j) c_beta[4 * slot + j] = a_beta[4 * e + j];
+        for (size_t t = 0; t < at[a].i[2].size(); ++t) zpos[a][at[a].i[2][t]] = (int)t;
+    struct Row { int y, t0, cnt; double g, h; };
+    struct Disc { int atom, tz, xa, xn; std::vector<Row> rows; };
+    std::vector<std::vector<Disc>> planes(Nz);
+    std::vector<double> sq(4 * (size_t)natom, 0.0);
+    long long nent = 0;
+    int mrows = 1, mdiscs = 1, wmax = 1;
+    for (int z = 0; z < Nz; ++z) {
+        for (int a = 0; a < natom; ++a) {
+            const int tz = zpos[a][z];
+            if (tz < 0) continue;
+            const Atom &A = at[a];
+            const double dz = A.d[2][tz], g_z = A.g[2][tz], h_z = A.h[2][tz];
+            Disc D{a, tz, 255, 0, {}};
+            int xb = 0;
+            for (size_t ty = 0; ty < A.i[1].size(); ++ty) {
+                const double dy = A.d[1][ty];
+                int t0 = -1, cnt = 0;
+                for (size_t tx = 0; tx < A.i[0].size(); ++tx) {
+                    const double dx = A.d[0][tx];
+                    if (!(dx * dx + dy * dy + dz * dz < rcut * rcut)) continue;
+                    if (t0 < 0) t0 = (int)tx;
+                    ++cnt;
+                    const double gg = A.g[0][tx] * A.g[1][ty] * g_z;
+                    const double b[4] = {gg, A.h[0][tx] * A.g[1][ty] * g_z, A.g[0][tx] * A.h[1][ty] * g_z,
+                                         A.g[0][tx] * A.g[1][ty] * h_z};
+                    for (int j = 0; j < 4; ++j) sq[4 * a + j] += b[j] * b[j];
+                }
+                if (cnt == 0) continue;
+                D.rows.push_back(Row{A.i[1][ty], t0, cnt, A.g[1][ty], A.h[1][ty]});
+                D.xa = std::min(D.xa, t0);
+                xb = std::max(xb, t0 + cnt);
+                nent += cnt;
+            }
+            if (D.rows.empty()) continue;
+            D.xn = xb - D.xa;
+            mrows = std::max(mrows, (int)D.rows.size());
+            wmax = std::max(wmax, D.xn);
+            planes[z].push_back(std::move(D));
         }
-    std::vector<double> ekb(pj->e_kb, pj->e_kb + (size_t)natom * nproj);
-    int *d_as, *d_ai, *d_rp, *d_ca;
-    double *d_ab, *d_cb, *d_e;
-    RS_TRY(upload(ctx, &d_as, a_start.data(), a_start.size()));
-    RS_TRY(upload(ctx, &d_ai, a_idx.data(), a_idx.size()));
-    RS_TRY(upload(ctx, &d_ab, a_beta.data(), a_beta.size()));
-    RS_TRY(upload(ctx, &d_rp, rowptr.data(), rowptr.size()));
-    RS_TRY(upload(ctx, &d_ca, c_atom.data(), c_atom.size()));
-    RS_TRY(upload(ctx, &d_cb, c_beta.data(), c_beta.size()));
-    RS_TRY(upload(ctx, &d_e, ekb.data(), ekb.size()));
-    ctx->pt = ProjTables{natom, nproj, d_as, d_ai, d_ab, d_rp, d_ca, d_cb, d_e};
-    std::vector<float> abf(a_beta.begin(), a_beta.end()), cbf(c_beta.begin(), c_beta.end()),
-        ekf(ekb.begin(), ekb.end());
-    float *d_abf, *d_cbf, *d_ef;
-    RS_TRY(upload(ctx, &d_abf, abf.data(), abf.size()));
-    RS_TRY(upload(ctx, &d_cbf, cbf.data(), cbf.size()));
-    RS_TRY(upload(ctx, &d_ef, ekf.data(), ekf.size()));
-    ctx->pt32 = ProjT<float>{natom, nproj, d_as, d_ai, d_abf, d_rp, d_ca, d_cbf, d_ef};
+        mdiscs = std::max(mdiscs, (int)planes[z].size());
+    }
+    std::vector<int> plane_start(Nz + 1, 0), color_ptr(Nz + 1, 0), color_start, datom;
+    std::vector<DiscMeta> meta;
+    std::vector<DiscRow> row;
+    std::vector<DiscRowFix> rowfix;
+    std::vector<float2> gx;
+    std::vector<int4> gxfix;
+    std::vector<double2> gz;
+    for (int z = 0; z < Nz; ++z) {
+        // greedy colouring: a disc takes the first colour none of whose points (bits of the plane) it has
+        std::vector<std::vector<int>> colors;
+        std::vector<std::vector<char>> used;
+        for (int k = 0; k < (int)planes[z].size(); ++k) {
+            const Disc &D = planes[z][k];
+            const int x0 = at[D.atom].i[0][0];
+            auto each = [&](auto f) {
+                for (const Row &r : D.rows)
+                    for (int i = 0; i < r.cnt; ++i)
+                        if (!f((size_t)r.y * Nx + (x0 + r.t0 + i) % Nx)) return false;
+                return true;
+            };
+            size_t col = 0;
+            while (col < colors.size() && !each([&](size_t p) { return !used[col][p]; })) ++col;
+            if (col == colors.size()) {
+                colors.emplace_back();
+                used.emplace_back((size_t)Nx * Ny, 0);
+            }
+            colors[col].push_back(k);
+            each([&](size_t p) { used[col][p] = 1; return true; });
+        }
+        for (const auto &col : colors) {
+            color_start.push_back((int)meta.size());
+            for (int k : col) {
+                const Disc &D = planes[z][k];
+                const Atom &A = at[D.atom];
+                meta.push_back(DiscMeta{(int)row.size(), (unsigned)D.rows.size() | (unsigned)D.xn << 8 |
+                                                             (unsigned)((A.i[0][0] + D.xa) % Nx) << 16});
+                datom.push_back(D.atom);
+                gz.push_back(make_double2(A.g[2][D.tz], A.h[2][D.tz]));
+                for (const Row &r : D.rows) {
+                    const int packed = r.y | (r.t0 - D.xa) << 8 | r.cnt << 16;
+                    row.push_back(DiscRow{packed, (float)r.g, (float)r.h, 0});
+                    DiscRowFix f{};
+                    f.packed = packed;
+                    split62(r.g, f.gh, f.gl);
+                    split62(r.h, f.hh, f.hl);
+                    rowfix.push_back(f);
+                }
+                for (int t = 0; t < wmax; ++t) {
+                    const double g = t < D.xn ? A.g[0][D.xa + t] : 0.0, h = t < D.xn ? A.h[0][D.xa + t] : 0.0;
+                    gx.push_back(make_float2((float)g, (float)h));
+                    int4 f;
+                    split62(g, f.x, f.y);
+                    split62(h, f.z, f.w);
+                    gxfix.push_back(f);
+                }
+            }
+        }
+        plane_start[z + 1] = (int)meta.size();
+        color_ptr[z + 1] = (int)color_start.size();
+    }
+    color_start.push_back((int)meta.size());
+    if (nent > 0x7fffffffLL) return fail(ctx, RSDFT_E_INVALID, "projector table too large");
+    // grid normalisation: sum beta^2 dV = 1
+    std::vector<double> cnorm(4 * (size_t)natom, 0.0), ekb(pj->e_kb, pj->e_kb + (size_t)natom * nproj);
+    for (int a = 0; a < natom; ++a)
+        for (int j = 0; j < nproj; ++j)
+            if (sq[4 * a + j] > 0.0) cnorm[4 * a + j] = 1.0 / std::sqrt(sq[4 * a + j] * ctx->dV);
+    std::vector<int> atom_start(natom + 1, 0), atom_disc(datom.size());
+    for (int a : datom) atom_start[a + 1]++;
+    for (int a = 0; a < natom; ++a) atom_start[a + 1] += atom_start[a];
+    std::vector<int> at_fill(atom_start.begin(), atom_start.end() - 1);
+    for (size_t d = 0; d < datom.size(); ++d) atom_disc[at_fill[datom[d]]++] = (int)d;
+    int *d_ps, *d_as, *d_ad, *d_cp, *d_cs;
+    DiscMeta *d_meta;
+    DiscRow *d_row;
+    DiscRowFix *d_rowf;
+    float2 *d_gx;
+    int4 *d_gxf;
+    double2 *d_gz;
+    double *d_cn, *d_ek;
+    RS_TRY(upload(ctx, &d_ps, plane_start.data(), plane_start.size()));
+    RS_TRY(upload(ctx, &d_as, atom_start.data(), atom_start.size()));
+    RS_TRY(upload(ctx, &d_ad, atom_disc.data(), atom_disc.size()));
+    RS_TRY(upload(ctx, &d_meta, meta.data(), meta.size()));
+    RS_TRY(upload(ctx, &d_row, row.data(), row.size()));
+    RS_TRY(upload(ctx, &d_rowf, rowfix.data(), rowfix.size()));
+    RS_TRY(upload(ctx, &d_cp, color_ptr.data(), color_ptr.size()));
+    RS_TRY(upload(ctx, &d_cs, color_start.data(), color_start.size()));
+    RS_TRY(upload(ctx, &d_gx, gx.data(), gx.size()));
+    RS_TRY(upload(ctx, &d_gxf, gxfix.data(), gxfix.size()));
+    RS_TRY(upload(ctx, &d_gz, gz.data(), gz.size()));
+    RS_TRY(upload(ctx, &d_cn, cnorm.data(), cnorm.size()));
+    RS_TRY(upload(ctx, &d_ek, ekb.data(), ekb.size()));
+    ctx->pt = ProjTables{natom, nproj, d_ek};
+    ctx->discs = Discs{natom, nproj, (int)datom.size(), wmax, mrows, mdiscs, d_ps, d_cp, d_cs, d_meta, d_row, d_rowf,
+                       d_gx, d_gxf, d_as, d_ad, d_gz, d_cn, d_ek};
     ctx->nent = nent;
     return RSDFT_OK;
 }

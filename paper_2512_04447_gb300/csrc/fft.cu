@@ -1,6 +1,11 @@
 // Batched 3D FFT kernels of the FP32 data path, the projector gather and H psi (SCF tasks (1)
 // and (4)).  The FP64 passes, of the same shape, are in fft_fix.cu.
 //
+// What bounds the passes is their instructions (72% of the issue slots), most of them around the
+// butterflies: addresses, shared-memory accesses, twiddle loads.  So a thread holds up to 16 points
+// and an axis has two stages where its length allows (96 = 12 x 8 instead of 8 x 4 x 3): the
+// z pass of 160 bands on 96^3 went from 1.04 to 0.78 ms, its instructions from 0.96 to 0.60 billion.
+//
 // Layout: orbital block [band][z][y][x] complex, x fastest.  A 3D transform is
 // three shared-memory passes over HBM:
 //   xy-forward  (one CTA per (band, z) plane: x lines then y lines, DIF)
@@ -18,15 +23,12 @@
 #include <vector>
 
 #include "fft_common.h"
+#include "proj.h"
 #include "rsdft_internal.h"
 
 namespace rsdft {
 
 // ---- complex helpers ---------------------------------------
-template <typename V> struct Sc;
-template <> struct Sc<double2> { using T = double; };
-template <> struct Sc<float2> { using T = float; };
-
 template <typename V> __device__ __forceinline__ V mk(typename Sc<V>::T x, typename Sc<V>::T y) {
     V r; r.x = x; r.y = y; return r;
 }
@@ -111,74 +113,145 @@ template <typename V, bool INV> __device__ __forceinline__ void dft8(V *v) {
     }
 }
 
+// Composite radices: R = A B as A transforms over B.  Coprime factors need no twiddles (Good and
+// Thomas: input q = (B q1 + A q2) mod R, output p with p mod A = p1 and p mod B = p2 and the inner
+// exponents as in a two-dimensional transform of A x B points); 9 and 16 have theirs.
+template <typename V, int R, bool INV> __device__ __forceinline__ void dftR(V *v);
+template <typename V, int A, int B, bool INV> __device__ __forceinline__ void dft_coprime(V *v) {
+    constexpr int R = A * B;
+    V t[B][A];
+#pragma unroll
+    for (int q2 = 0; q2 < B; ++q2) {
+#pragma unroll
+        for (int q1 = 0; q1 < A; ++q1) t[q2][q1] = v[(B * q1 + A * q2) % R];
+        dftR<V, A, INV>(t[q2]);
+    }
+#pragma unroll
+    for (int p1 = 0; p1 < A; ++p1) {
+        V c[B];
+#pragma unroll
+        for (int q2 = 0; q2 < B; ++q2) c[q2] = t[q2][p1];
+        dftR<V, B, INV>(c);
+        // exp(2 pi i (B q1 + A q2) p / R) = exp(2 pi i q1 p / A) exp(2 pi i q2 p / B): p = (p1, p2)
+#pragma unroll
+        for (int p = 0; p < R; ++p)
+            if (p % A == p1) v[p] = c[p % B];
+    }
+}
+// exp(-2 pi i k / R) of the inner twiddles of R = 9 and 16
+template <int R> __device__ __forceinline__ constexpr double inner_cos(int k) {
+    constexpr double c9[5] = {1.0, 0.766044443118978035202392650555, 0.173648177666930348851716626769, -0.5,
+                              -0.939692620785908384054109277325};
+    constexpr double c16[10] = {1.0, 0.923879532511286756128183189397, 0.707106781186547524400844362105,
+                                0.382683432365089771728459984030, 0.0, -0.382683432365089771728459984030,
+                                -0.707106781186547524400844362105, -0.923879532511286756128183189397, -1.0,
+                                -0.923879532511286756128183189397};
+    return R == 9 ? c9[k] : c16[k];
+}
+template <int R> __device__ __forceinline__ constexpr double inner_sin(int k) {
+    constexpr double s9[5] = {0.0, 0.642787609686539326322643409907, 0.984807753012208059366743024590,
+                              0.866025403784438646763723170753, 0.342020143325668733044099614682};
+    constexpr double s16[10] = {0.0, 0.382683432365089771728459984030, 0.707106781186547524400844362105,
+                                0.923879532511286756128183189397, 1.0, 0.923879532511286756128183189397,
+                                0.707106781186547524400844362105, 0.382683432365089771728459984030, 0.0,
+                                -0.382683432365089771728459984030};
+    return R == 9 ? s9[k] : s16[k];
+}
+template <typename V, int A, bool INV> __device__ __forceinline__ void dft_square(V *v) {   // R = A A
+    using T = typename Sc<V>::T;
+    constexpr int R = A * A;
+    V t[A][A];
+#pragma unroll
+    for (int q2 = 0; q2 < A; ++q2) {
+#pragma unroll
+        for (int q1 = 0; q1 < A; ++q1) t[q2][q1] = v[A * q1 + q2];
+        dftR<V, A, INV>(t[q2]);
+    }
+#pragma unroll
+    for (int p1 = 0; p1 < A; ++p1) {
+        V c[A];
+#pragma unroll
+        for (int q2 = 0; q2 < A; ++q2) {
+            const V w = mk<V>((T)inner_cos<R>(p1 * q2), (T)(-inner_sin<R>(p1 * q2)));
+            c[q2] = p1 * q2 == 0 ? t[q2][p1] : (INV ? cmulconj(t[q2][p1], w) : cmul(t[q2][p1], w));
+        }
+        dftR<V, A, INV>(c);
+#pragma unroll
+        for (int p2 = 0; p2 < A; ++p2) v[p1 + A * p2] = c[p2];
+    }
+}
+
 template <typename V, int R, bool INV> __device__ __forceinline__ void dftR(V *v) {
     if constexpr (R == 2) dft2<V, INV>(v);
     else if constexpr (R == 3) dft3<V, INV>(v);
     else if constexpr (R == 4) dft4<V, INV>(v);
     else if constexpr (R == 5) dft5<V, INV>(v);
-    else dft8<V, INV>(v);
+    else if constexpr (R == 6) dft_coprime<V, 2, 3, INV>(v);
+    else if constexpr (R == 8) dft8<V, INV>(v);
+    else if constexpr (R == 9) dft_square<V, 3, INV>(v);
+    else if constexpr (R == 10) dft_coprime<V, 2, 5, INV>(v);
+    else if constexpr (R == 12) dft_coprime<V, 3, 4, INV>(v);
+    else dft_square<V, 4, INV>(v);
 }
 
 template <typename V> __device__ __forceinline__ V ldtw(const V *tw, int k) { return __ldg(tw + k); }
 
-// One radix-R butterfly of a stage, in place in shared memory.
+// One radix-R butterfly of a stage, in place in shared memory (j = 0: unit twiddles).
 template <typename V, int R, bool INV>
-__device__ __forceinline__ void bfly(V *s, int base, int step, int j, int twstep, const V *tw) {
+__device__ __forceinline__ void bfly(V *s, int step, int j, int twstep, const V *tw) {
     V v[R];
-    if (!INV) {
 #pragma unroll
-        for (int q = 0; q < R; ++q) v[q] = s[base + q * step];
-        dftR<V, R, false>(v);
-#pragma unroll
-        for (int p = 1; p < R; ++p) v[p] = cmul(v[p], ldtw(tw, j * p * twstep));
-    } else {
-#pragma unroll
-        for (int p = 0; p < R; ++p) v[p] = s[base + p * step];
+    for (int q = 0; q < R; ++q) v[q] = s[q * step];
+    if (INV && j) {
 #pragma unroll
         for (int p = 1; p < R; ++p) v[p] = cmulconj(v[p], ldtw(tw, j * p * twstep));
-        dftR<V, R, true>(v);
+    }
+    dftR<V, R, INV>(v);
+    if (!INV && j) {
+#pragma unroll
+        for (int p = 1; p < R; ++p) v[p] = cmul(v[p], ldtw(tw, j * p * twstep));
     }
 #pragma unroll
-    for (int q = 0; q < R; ++q) s[base + q * step] = v[q];
+    for (int q = 0; q < R; ++q) s[q * step] = v[q];
 }
 
-// All stages of nlines 1D transforms of length ax.N in shared memory.
-// Element e of line l sits at s[l * lstride + e * es].  lines_fast selects the
-// thread mapping: consecutive threads take consecutive lines (use when es > 1
-// and lstride == 1), else consecutive butterflies of one line.
-// nlmag: multiply-high divisor of nlines.  Quotients and remainders of the
-// index decomposition use it instead of integer division (total < 2^16).
+template <typename V, int R, bool INV>
+__device__ __forceinline__ void stage(V *s, const AxisPlan &ax, int st, const V *tw, int nlines, unsigned nlmag,
+                                      int lstride, int es) {
+    const int N = ax.N, len = ax.len[st], sub = ax.sub[st];
+    const unsigned smag = ax.submag[st];
+    const int total = N / R * nlines, twstep = N / len, step = sub * es;
+    for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
+        const int bf = qdiv(idx, nlmag), line = idx - bf * nlines;   // consecutive threads: consecutive lines
+        const int b = qdiv(bf, smag), j = bf - b * sub;
+        bfly<V, R, INV>(s + line * lstride + (b * len + j) * es, step, j, twstep, tw);
+    }
+}
+
+// All stages of nlines 1D transforms of length ax.N in shared memory: element e of line l at
+// s[l * lstride + e * es] (nlmag: multiply-high divisor of nlines, total < 2^16).
 template <typename V, bool INV>
-__device__ void fft_lines(V *s, const AxisPlan &ax, const V *tw, int nlines, unsigned nlmag, int lstride,
-                          int es, bool lines_fast) {
-    const int N = ax.N;
+__device__ void fft_lines(V *s, const AxisPlan &ax, const V *tw, int nlines, unsigned nlmag, int lstride, int es) {
     for (int t = 0; t < ax.nstage; ++t) {
         const int st = INV ? ax.nstage - 1 - t : t;
-        const int r = ax.radix[st], len = ax.len[st], sub = ax.sub[st];
-        const unsigned smag = ax.submag[st], bmag = ax.bfmag[st];
-        const int nbf = N / r;
-        const int total = nbf * nlines;
-        const int twstep = N / len;
-        for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
-            int line, bf;
-            if (lines_fast) { bf = qdiv(idx, nlmag); line = idx - bf * nlines; }
-            else { line = qdiv(idx, bmag); bf = idx - line * nbf; }
-            const int b = qdiv(bf, smag), j = bf - b * sub;
-            const int base = line * lstride + (b * len + j) * es;
-            const int step = sub * es;
-            switch (r) {
-                case 2: bfly<V, 2, INV>(s, base, step, j, twstep, tw); break;
-                case 3: bfly<V, 3, INV>(s, base, step, j, twstep, tw); break;
-                case 4: bfly<V, 4, INV>(s, base, step, j, twstep, tw); break;
-                case 5: bfly<V, 5, INV>(s, base, step, j, twstep, tw); break;
-                default: bfly<V, 8, INV>(s, base, step, j, twstep, tw); break;
-            }
+        switch (ax.radix[st]) {
+            case 2: stage<V, 2, INV>(s, ax, st, tw, nlines, nlmag, lstride, es); break;
+            case 3: stage<V, 3, INV>(s, ax, st, tw, nlines, nlmag, lstride, es); break;
+            case 4: stage<V, 4, INV>(s, ax, st, tw, nlines, nlmag, lstride, es); break;
+            case 5: stage<V, 5, INV>(s, ax, st, tw, nlines, nlmag, lstride, es); break;
+            case 6: stage<V, 6, INV>(s, ax, st, tw, nlines, nlmag, lstride, es); break;
+            case 8: stage<V, 8, INV>(s, ax, st, tw, nlines, nlmag, lstride, es); break;
+            case 9: stage<V, 9, INV>(s, ax, st, tw, nlines, nlmag, lstride, es); break;
+            case 10: stage<V, 10, INV>(s, ax, st, tw, nlines, nlmag, lstride, es); break;
+            case 12: stage<V, 12, INV>(s, ax, st, tw, nlines, nlmag, lstride, es); break;
+            default: stage<V, 16, INV>(s, ax, st, tw, nlines, nlmag, lstride, es); break;
         }
         __syncthreads();
     }
 }
 
-constexpr int FFT_THREADS = 512;
+// 80 registers: a radix-16 butterfly without spills
+constexpr int FFT_THREADS = 768;   // at most (fft_threads)
 
 // Tables of one precision: twiddles exp(-2 pi i k/N) and G_a^2 at each
 // digit-reversed position.
@@ -192,22 +265,66 @@ template <typename V> struct FftTabs {
 static FftTabs<float2> tabs_of(const rsdft_ctx *ctx, float2 *) {
     FftTabs<float2> t;
     for (int a = 0; a < 3; ++a) {
-        t.ax[a] = ctx->fft.ax[a];
+        t.ax[a] = ctx->fft.ax32[a];
         t.tw[a] = ctx->fft.tw32[a];
         t.g2[a] = ctx->fft.g2pos32[a];
     }
     t.inv_n = 1.0 / (double)ctx->n;
     return t;
 }
-static const ProjT<double> &proj_of(const rsdft_ctx *ctx, double2 *) { return ctx->pt; }
-static const ProjT<float> &proj_of(const rsdft_ctx *ctx, float2 *) { return ctx->pt32; }
 static const float *v_of(const rsdft_ctx *ctx, float2 *) { return ctx->v32; }
+
+// part[disc][3] = sums of gx gy v, hx gy v, gx hy v over each disc of plane z (row stride RS)
+__device__ __forceinline__ void gather_plane(const float2 *plane, int RS, const Discs &t, int z, int Nx,
+                                             float2 *__restrict__ part) {
+    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    const int d1 = t.plane_start[z + 1];
+    for (int d = t.plane_start[z] + (threadIdx.x >> 5); d < d1; d += nw) {
+        const int2 m = __ldg(reinterpret_cast<const int2 *>(t.meta + d));
+        const int rows = disc_rows(m.y), w = disc_width(m.y);
+        const float2 *gx = t.gx + (size_t)d * t.wmax;
+        float s[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        for (int r0 = 0; r0 < rows; r0 += 32) {
+            int4 q = make_int4(0, 0, 0, 0);
+            if (r0 + lane < rows) q = __ldg(reinterpret_cast<const int4 *>(t.row + m.x + r0 + lane));
+            const float2 *row = plane + (q.x & 255) * RS;
+            int x = disc_x0(m.y);
+            float ux = 0.f, uy = 0.f, vx = 0.f, vy = 0.f;   // sums of gx v, hx v along the row
+#pragma unroll 4
+            for (int j = 0; j < w; ++j) {
+                const float2 k = __ldg(gx + j);
+                const float2 v = row[x];
+                const bool in = in_row(q.x, j);   // a select, not a branch
+                const float g = in ? k.x : 0.f, h = in ? k.y : 0.f;
+                ux = fmaf(g, v.x, ux);
+                uy = fmaf(g, v.y, uy);
+                vx = fmaf(h, v.x, vx);
+                vy = fmaf(h, v.y, vy);
+                x = x + 1 == Nx ? 0 : x + 1;
+            }
+            const float g = __int_as_float(q.y), h = __int_as_float(q.z);
+            s[0] += g * ux;
+            s[1] += g * uy;
+            s[2] += g * vx;
+            s[3] += g * vy;
+            s[4] += h * ux;
+            s[5] += h * uy;
+        }
+#pragma unroll
+        for (int k = 0; k < 6; ++k)
+            for (int o = 16; o > 0; o >>= 1) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
+        if (lane < 3)
+            part[(size_t)d * 3 + lane] = make_float2(lane == 0 ? s[0] : (lane == 1 ? s[2] : s[4]),
+                                                     lane == 0 ? s[1] : (lane == 1 ? s[3] : s[5]));
+    }
+}
 
 // ---- xy forward pass ------------------------------------------------------------
 template <typename V, Src SRC>
-__global__ void __launch_bounds__(FFT_THREADS, sizeof(V) == 8 ? 3 : 1)
+__global__ void __launch_bounds__(FFT_THREADS)
 k_xy_forward(FftTabs<V> tb, const V *__restrict__ src, const V *__restrict__ src2,
-             const double *__restrict__ theta, const int *__restrict__ act, V *__restrict__ dst) {
+             const double *__restrict__ theta, const int *__restrict__ act, V *__restrict__ dst,
+             Discs discs, V *__restrict__ part) {
     using T = typename Sc<V>::T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V *s_plane = reinterpret_cast<V *>(smem_raw);
@@ -233,8 +350,12 @@ k_xy_forward(FftTabs<V> tb, const V *__restrict__ src, const V *__restrict__ src
         }, put);
     }
     __syncthreads();
-    fft_lines<V, false>(s_plane, tb.ax[0], tb.tw[0], Ny, tb.ax[1].nmag, RS, 1, true);
-    fft_lines<V, false>(s_plane, tb.ax[1], tb.tw[1], Nx, tb.ax[0].nmag, 1, RS, true);
+    if (SRC == Src::Plain && part) {
+        gather_plane(s_plane, RS, discs, z, Nx, part + (size_t)band * discs.ndisc * 3);
+        __syncthreads();
+    }
+    fft_lines<V, false>(s_plane, tb.ax[0], tb.tw[0], Ny, tb.ax[1].nmag, RS, 1);
+    fft_lines<V, false>(s_plane, tb.ax[1], tb.tw[1], Nx, tb.ax[0].nmag, 1, RS);
     V *out = dst + band * n + off;
     for (int i = threadIdx.x; i < (int)plane; i += blockDim.x) out[i] = s_plane[pidx(i, Nx, RS, nxm)];
 }
@@ -246,7 +367,7 @@ template <typename T> __device__ __forceinline__ T tpa_k(T x) {
 }
 
 template <typename V, Mid MID>
-__global__ void __launch_bounds__(FFT_THREADS, sizeof(V) == 8 ? 3 : 1)
+__global__ void __launch_bounds__(FFT_THREADS)
 k_z_mid(FftTabs<V> tb, V *__restrict__ buf, const double *__restrict__ tkin) {
     using T = typename Sc<V>::T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -262,7 +383,7 @@ k_z_mid(FftTabs<V> tb, V *__restrict__ buf, const double *__restrict__ tkin) {
         return base[z * zstride + x];
     }, [&](int i, V v) { s_slab[i] = v; });
     __syncthreads();
-    fft_lines<V, false>(s_slab, tb.ax[2], tb.tw[2], Nx, tb.ax[0].nmag, 1, Nx, true);
+    fft_lines<V, false>(s_slab, tb.ax[2], tb.tw[2], Nx, tb.ax[0].nmag, 1, Nx);
     const T inv_n = (T)tb.inv_n;
     const T gy2 = tb.g2[1][y];
     T tk = (T)1;
@@ -280,21 +401,60 @@ k_z_mid(FftTabs<V> tb, V *__restrict__ buf, const double *__restrict__ tkin) {
         s_slab[i] = mk<V>(s_slab[i].x * f, s_slab[i].y * f);
     }
     __syncthreads();
-    fft_lines<V, true>(s_slab, tb.ax[2], tb.tw[2], Nx, tb.ax[0].nmag, 1, Nx, true);
+    fft_lines<V, true>(s_slab, tb.ax[2], tb.tw[2], Nx, tb.ax[0].nmag, 1, Nx);
     for (int i = threadIdx.x; i < tot; i += blockDim.x) {
         const int z = qdiv(i, tb.ax[0].nmag), x = i - z * Nx;
         base[z * zstride + x] = s_slab[i];
     }
 }
 
+// plane += sum over its discs of gx (gy A + hy By) + hx gy Bx, ab[disc] = (A, Bx, By); uw: room discs
+__device__ __forceinline__ void scatter_plane(float2 *s_plane, int RS, const Discs &t, int z, int Nx,
+                                              const float2 *__restrict__ ab, float4 *uw, int room) {
+    const int lane = threadIdx.x & 31, d0 = t.plane_start[z];
+    int base = 0;
+    for_discs(t, z, room, [&](int c0, int n) {
+        base = d0 + c0;
+        for (int i = threadIdx.x; i < n * t.wmax; i += blockDim.x) {
+            const int d = base + i / t.wmax;
+            const float2 k = __ldg(t.gx + (size_t)base * t.wmax + i);
+            const float2 A = __ldg(ab + 3 * (size_t)d), Bx = __ldg(ab + 3 * (size_t)d + 1), By = __ldg(ab + 3 * (size_t)d + 2);
+            uw[i] = make_float4(k.x * A.x + k.y * Bx.x, k.x * A.y + k.y * Bx.y, k.x * By.x, k.x * By.y);
+        }
+    }, [&](int d, int ja, int jb) {
+        const int2 m = __ldg(reinterpret_cast<const int2 *>(t.meta + d));
+        const int rows = disc_rows(m.y);
+        const float4 *ue = uw + (d - base) * t.wmax;
+        for (int r0 = 0; r0 < rows; r0 += 32) {
+            int4 q = make_int4(0, 0, 0, 0);
+            if (r0 + lane < rows) q = __ldg(reinterpret_cast<const int4 *>(t.row + m.x + r0 + lane));
+            const float g = __int_as_float(q.y), h = __int_as_float(q.z);
+            float2 *row = s_plane + (q.x & 255) * RS;
+            int x = disc_x0(m.y) + ja;
+            if (x >= Nx) x -= Nx;
+#pragma unroll 4
+            for (int j = ja; j < jb; ++j) {
+                const float4 k = ue[j];
+                if (in_row(q.x, j)) {
+                    float2 o = row[x];
+                    o.x += g * k.x + h * k.z;
+                    o.y += g * k.y + h * k.w;
+                    row[x] = o;
+                }
+                x = x + 1 == Nx ? 0 : x + 1;
+            }
+        }
+    });
+}
+
 // ---- xy inverse pass + epilogue ------------------------------------------------------
 enum class Epi { Plain, Hpsi };
 
 template <typename V, Epi EPI>
-__global__ void __launch_bounds__(FFT_THREADS, sizeof(V) == 8 ? 3 : 1)
+__global__ void __launch_bounds__(FFT_THREADS)
 k_xy_inverse(FftTabs<V> tb, const V *__restrict__ buf, const V *__restrict__ psi,
-             const typename Sc<V>::T *__restrict__ v, ProjT<typename Sc<V>::T> pt,
-             const V *__restrict__ p, V *__restrict__ out, int stage_pe) {
+             const typename Sc<V>::T *__restrict__ v, Discs discs, int room,
+             const V *__restrict__ ab, V *__restrict__ out) {
     using T = typename Sc<V>::T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V *s_plane = reinterpret_cast<V *>(smem_raw);
@@ -306,118 +466,156 @@ k_xy_inverse(FftTabs<V> tb, const V *__restrict__ buf, const V *__restrict__ psi
     const V *in = buf + band * n + off;
     const int RS = plane_rs(Nx);
     const unsigned nxm = tb.ax[0].nmag;
+    const bool scatter = EPI == Epi::Hpsi && ab;
+    const V *abb = ab + (size_t)band * discs.ndisc * 3;
+    float4 *uw = reinterpret_cast<float4 *>(s_plane + (((size_t)Ny * RS + 1) & ~(size_t)1));
     stage_in<V>((int)plane, [&](int i) { return in[i]; }, [&](int i, V v) { s_plane[pidx(i, Nx, RS, nxm)] = v; });
     __syncthreads();
-    fft_lines<V, true>(s_plane, tb.ax[1], tb.tw[1], Nx, tb.ax[0].nmag, 1, RS, true);
-    fft_lines<V, true>(s_plane, tb.ax[0], tb.tw[0], Ny, tb.ax[1].nmag, RS, 1, true);
+    fft_lines<V, true>(s_plane, tb.ax[1], tb.tw[1], Nx, tb.ax[0].nmag, 1, RS);
+    fft_lines<V, true>(s_plane, tb.ax[0], tb.tw[0], Ny, tb.ax[1].nmag, RS, 1);
     if (EPI == Epi::Plain) {
         V *o = out + band * n + off;
         for (int i = threadIdx.x; i < (int)plane; i += blockDim.x) o[i] = s_plane[pidx(i, Nx, RS, nxm)];
     } else {
         const V *ps = psi + band * n + off;
         const T *vv = v + off;
-        const int np = pt.natom * pt.nproj;
-        const V *pb = p + (size_t)band * np;
-        // E_aj <beta_aj|psi> of this band, staged once per CTA after the plane
-        // (when it fits; else read from global memory)
-        V *s_pe = s_plane + (size_t)Ny * RS;
-        if (stage_pe) {
-            for (int q = threadIdx.x; q < np; q += blockDim.x) {
-                const V c = pb[q];
-                const T e = pt.e_kb[q];
-                s_pe[q] = mk<V>(e * c.x, e * c.y);
-            }
-            __syncthreads();
+        if (scatter) {
+            scatter_plane(s_plane, RS, discs, z, Nx, abb, uw, room);
         }
         V *o = out + band * n + off;
         for (int i = threadIdx.x; i < (int)plane; i += blockDim.x) {
-            V t = s_plane[pidx(i, Nx, RS, nxm)];
-            V y = ps[i];
-            T vi = vv[i];
-            T ax = t.x + vi * y.x, ay = t.y + vi * y.y;
-            const int g = (int)off + i;
-            const int e0 = pt.c_rowptr[g], e1 = pt.c_rowptr[g + 1];
-            for (int e = e0; e < e1; ++e) {
-                const int a0 = pt.c_atom[e] * pt.nproj;
-                T bt[4];
-                beta4(pt.c_beta + 4 * (size_t)e, bt);
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    if (j >= pt.nproj) break;
-                    V q;
-                    if (stage_pe) {
-                        q = s_pe[a0 + j];
-                    } else {
-                        const V c = pb[a0 + j];
-                        const T ek = pt.e_kb[a0 + j];
-                        q = mk<V>(ek * c.x, ek * c.y);
-                    }
-                    const T c = bt[j];
-                    ax += c * q.x;
-                    ay += c * q.y;
-                }
-            }
-            o[i] = mk<V>(ax, ay);
+            const V t = s_plane[pidx(i, Nx, RS, nxm)];
+            const V y = ps[i];
+            const T vi = vv[i];
+            o[i] = mk<V>(t.x + vi * y.x, t.y + vi * y.y);
         }
     }
 }
 
-// ---- projection <beta|psi> (atom-major gather) ------------------------------------------
+// ---- projectors --------------------------------------------------------------------------
+// The gather alone, on planes in global memory (lane = x; FP64 takes the fixed-point factors).
 constexpr int PROJ_THREADS = 256;
-constexpr int PROJ_BANDS = 4;
+
+__device__ __forceinline__ double unfix(int h, int l) { return ((double)h * 4294967296.0 + (double)l) * 0x1p-62; }
 
 template <typename V>
 __global__ void __launch_bounds__(PROJ_THREADS)
-k_project(ProjT<typename Sc<V>::T> pt, const V *__restrict__ psi, V *__restrict__ p, int nb,
-          long long n, double dV) {
+k_gather(Discs t, const V *__restrict__ psi, int Nx, int Ny, long long n, V *__restrict__ part) {
     using T = typename Sc<V>::T;
-    const int a = blockIdx.x;
-    const int b0 = blockIdx.y * PROJ_BANDS;
-    const int e0 = pt.a_start[a], e1 = pt.a_start[a + 1];
-    T acc[PROJ_BANDS][4][2];
-#pragma unroll
-    for (int bb = 0; bb < PROJ_BANDS; ++bb)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[bb][j][0] = acc[bb][j][1] = (T)0;
-    for (int e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
-        const int g = pt.a_idx[e];
-        T be[4];
-        beta4(pt.a_beta + 4 * (size_t)e, be);
-#pragma unroll
-        for (int bb = 0; bb < PROJ_BANDS; ++bb) {
-            const int band = b0 + bb;
-            if (band >= nb) break;
-            const V v = psi[(size_t)band * n + g];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                acc[bb][j][0] += be[j] * v.x;
-                acc[bb][j][1] += be[j] * v.y;
+    const int z = blockIdx.x, band = blockIdx.y;
+    const V *plane = psi + (size_t)band * n + (size_t)z * Nx * Ny;
+    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    const int d1 = t.plane_start[z + 1];
+    for (int d = t.plane_start[z] + (threadIdx.x >> 5); d < d1; d += nw) {
+        const DiscMeta m = t.meta[d];
+        const int rows = disc_rows(m.packed), w = disc_width(m.packed);
+        T s[6] = {(T)0, (T)0, (T)0, (T)0, (T)0, (T)0};
+        for (int c = 0; c < w; c += 32) {
+            const int l = c + lane;
+            int x = disc_x0(m.packed) + l;
+            if (x >= Nx) x -= Nx;
+            T ax = (T)0, ay = (T)0, bx = (T)0, by = (T)0;
+#pragma unroll 4
+            for (int r = 0; r < rows; ++r) {
+                int pk;
+                T g, h;
+                if constexpr (sizeof(T) == 4) {
+                    const int4 k = __ldg(reinterpret_cast<const int4 *>(t.row + m.row0 + r));
+                    pk = k.x;
+                    g = __int_as_float(k.y);
+                    h = __int_as_float(k.z);
+                } else {
+                    const int4 k = __ldg(reinterpret_cast<const int4 *>(t.rowfix + m.row0 + r));
+                    pk = k.x;
+                    g = unfix(k.y, k.z);
+                    h = unfix(k.w, __ldg(&t.rowfix[m.row0 + r].hl));
+                }
+                if (in_row(pk, l)) {
+                    const V v = plane[(pk & 255) * Nx + x];
+                    ax += g * v.x;
+                    ay += g * v.y;
+                    bx += h * v.x;
+                    by += h * v.y;
+                }
             }
+            T gx = (T)0, hx = (T)0;
+            if (l < w) {
+                if constexpr (sizeof(T) == 4) {
+                    const float2 k = __ldg(t.gx + (size_t)d * t.wmax + l);
+                    gx = k.x;
+                    hx = k.y;
+                } else {
+                    const int4 k = __ldg(t.gxfix + (size_t)d * t.wmax + l);
+                    gx = unfix(k.x, k.y);
+                    hx = unfix(k.z, k.w);
+                }
+            }
+            s[0] += gx * ax;
+            s[1] += gx * ay;
+            s[2] += hx * ax;
+            s[3] += hx * ay;
+            s[4] += gx * bx;
+            s[5] += gx * by;
         }
+#pragma unroll
+        for (int k = 0; k < 6; ++k)
+            for (int o = 16; o > 0; o >>= 1) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
+        if (lane < 3)
+            part[((size_t)band * t.ndisc + d) * 3 + lane] = mk<V>(lane == 0 ? s[0] : (lane == 1 ? s[2] : s[4]),
+                                                                 lane == 0 ? s[1] : (lane == 1 ? s[3] : s[5]));
     }
-    // block reduction, fixed order
-    __shared__ T red[PROJ_THREADS / 32][PROJ_BANDS * 8];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+}
+
+// One warp per (band, atom): the disc sums joined with their z factors, p[band][atom nproj + j] =
+// <beta_j|psi> (p may be null) and the scatter coefficients of every disc, ab[band][disc] =
+// (gz q_s + hz q_z, gz q_x, gz q_y) with q_j = c_j E_j <beta_j|psi> (ab may be null).
+template <typename V>
+__global__ void __launch_bounds__(PROJ_THREADS)
+k_disc_fin(Discs t, const V *__restrict__ part, int nb, typename Sc<V>::T dV, V *__restrict__ p,
+           V *__restrict__ ab) {
+    using T = typename Sc<V>::T;
+    const int w = (blockIdx.x * PROJ_THREADS + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    const int band = w / t.natom, a = w - band * t.natom;
+    if (band >= nb) return;
+    const int i0 = t.atom_start[a], i1 = t.atom_start[a + 1];
+    T s[8];
 #pragma unroll
-    for (int bb = 0; bb < PROJ_BANDS; ++bb)
+    for (int k = 0; k < 8; ++k) s[k] = (T)0;
+    const V *pb = part + (size_t)band * t.ndisc * 3;
+    for (int i = i0 + lane; i < i1; i += 32) {
+        const int d = t.atom_disc[i];
+        const double2 gd = t.gz[d];
+        const V g = mk<V>((T)gd.x, (T)gd.y), v0 = pb[3 * (size_t)d], v1 = pb[3 * (size_t)d + 1], v2 = pb[3 * (size_t)d + 2];
+        s[0] += g.x * v0.x;
+        s[1] += g.x * v0.y;
+        s[2] += g.x * v1.x;
+        s[3] += g.x * v1.y;
+        s[4] += g.x * v2.x;
+        s[5] += g.x * v2.y;
+        s[6] += g.y * v0.x;
+        s[7] += g.y * v0.y;
+    }
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
+    for (int k = 0; k < 8; ++k)
+        for (int o = 16; o > 0; o >>= 1) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
+    V q[4];
 #pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                T s = acc[bb][j][c];
-                for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-                if (lane == 0) red[warp][(bb * 4 + j) * 2 + c] = s;
-            }
-    __syncthreads();
-    if (threadIdx.x < PROJ_BANDS * 8) {
-        T s = (T)0;
-        for (int w = 0; w < PROJ_THREADS / 32; ++w) s += red[w][threadIdx.x];
-        const int bb = threadIdx.x / 8, j = (threadIdx.x / 2) % 4, c = threadIdx.x % 2;
-        const int band = b0 + bb;
-        if (band < nb && j < pt.nproj) {
-            T *dst = reinterpret_cast<T *>(p + (size_t)band * pt.natom * pt.nproj + a * pt.nproj + j);
-            dst[c] = s * (T)dV;
-        }
+    for (int j = 0; j < 4; ++j) {
+        const T c = (T)t.cnorm[4 * a + j];   // 0 for projectors that are not there
+        q[j] = mk<V>(c * dV * s[2 * j], c * dV * s[2 * j + 1]);
+        if (p && lane == 0 && j < t.nproj) p[(size_t)band * t.natom * t.nproj + a * t.nproj + j] = q[j];
+        const T e = j < t.nproj ? c * (T)t.e_kb[a * t.nproj + j] : (T)0;
+        q[j] = mk<V>(e * q[j].x, e * q[j].y);
+    }
+    if (!ab) return;
+    V *ob = ab + (size_t)band * t.ndisc * 3;
+    for (int i = i0 + lane; i < i1; i += 32) {
+        const int d = t.atom_disc[i];
+        const double2 gd = t.gz[d];
+        const V g = mk<V>((T)gd.x, (T)gd.y);
+        ob[3 * (size_t)d] = mk<V>(g.x * q[0].x + g.y * q[3].x, g.x * q[0].y + g.y * q[3].y);
+        ob[3 * (size_t)d + 1] = mk<V>(g.x * q[1].x, g.x * q[1].y);
+        ob[3 * (size_t)d + 2] = mk<V>(g.x * q[2].x, g.x * q[2].y);
     }
 }
 
@@ -431,29 +629,45 @@ __global__ void k_to_float(const double *__restrict__ in, long long n, float *__
 template <typename V> static size_t plane_bytes(const rsdft_ctx *ctx) {
     return (size_t)(ctx->N[0] | 1) * ctx->N[1] * sizeof(V);   // odd row stride
 }
+// 256 threads where three CTAs share an SM (fewer for small planes), else enough to fill it
+static int fft_threads(size_t smem, int points) {
+    if (smem <= 75 * 1024) return std::max(64, std::min(256, cdiv(points, 256) * 32));
+    return smem <= 113 * 1024 ? 384 : 768;
+}
 template <typename V> static size_t slab_bytes(const rsdft_ctx *ctx) {
     return (size_t)ctx->N[0] * ctx->N[2] * sizeof(V);
+}
+
+// shared memory of a plane with the scatter table of its discs beside it
+static rsdft_status disc_smem(rsdft_ctx *ctx, size_t *sm, int *room) {
+    const size_t base = (*sm + 15) / 16 * 16, per = (size_t)ctx->discs.wmax * sizeof(float4);
+    *room = disc_room(base, per, ctx->discs.maxdiscs, MAX_DYN_SMEM);
+    if (*room < 1) return fail(ctx, RSDFT_E_INVALID, "no shared memory for the projectors beside a plane");
+    *sm = base + *room * per;
+    return RSDFT_OK;
 }
 
 template <typename V>
 rsdft_status fft_xy_forward_t(rsdft_ctx *ctx, Src kind, const V *src, const V *src2,
                               const double *theta, const int *act, V *dst,
-                              int nb, cudaStream_t st) {
+                              int nb, cudaStream_t st, V *part) {
     if (nb <= 0) return RSDFT_OK;
     const size_t sm = plane_bytes<V>(ctx);
     dim3 grid(ctx->N[2], nb);
+    const int pts = ctx->N[0] * ctx->N[1];
     const double nxy = (double)ctx->N[0] * ctx->N[1];
     const double e = (double)sizeof(V);
     const double bpp = kind == Src::Plain ? 2 * e : 3 * e;
     ProfScope ps(ctx, RSDFT_K_FFT_XY_FWD, 5.0 * nxy * std::log2(nxy) * ctx->N[2] * nb,
                  bpp * (double)ctx->n * nb, st);
     const FftTabs<V> tb = tabs_of(ctx, (V *)nullptr);
+    const Discs &discs = ctx->discs;
     if (kind == Src::Plain) {
         RS_TRY(set_smem(ctx, k_xy_forward<V, Src::Plain>, sm));
-        k_xy_forward<V, Src::Plain><<<grid, FFT_THREADS, sm, st>>>(tb, src, src2, theta, act, dst);
+        k_xy_forward<V, Src::Plain><<<grid, fft_threads(sm, pts), sm, st>>>(tb, src, src2, theta, act, dst, discs, part);
     } else {
         RS_TRY(set_smem(ctx, k_xy_forward<V, Src::Residual>, sm));
-        k_xy_forward<V, Src::Residual><<<grid, FFT_THREADS, sm, st>>>(tb, src, src2, theta, act, dst);
+        k_xy_forward<V, Src::Residual><<<grid, fft_threads(sm, pts), sm, st>>>(tb, src, src2, theta, act, dst, discs, part);
     }
     RS_LAUNCHED(ctx, "k_xy_forward");
     return RSDFT_OK;
@@ -465,73 +679,107 @@ rsdft_status fft_z_mid_t(rsdft_ctx *ctx, Mid mid, V *buf, const double *tkin, in
     if (nb <= 0) return RSDFT_OK;
     const size_t sm = slab_bytes<V>(ctx);
     dim3 grid(ctx->N[1], nb);
+    const int pts = ctx->N[0] * ctx->N[2];
     ProfScope ps(ctx, RSDFT_K_FFT_Z, 10.0 * (double)ctx->n * std::log2((double)ctx->N[2]) * nb,
                  2.0 * sizeof(V) * (double)ctx->n * nb, st);
     const FftTabs<V> tb = tabs_of(ctx, (V *)nullptr);
     if (mid == Mid::Kinetic) {
         RS_TRY(set_smem(ctx, k_z_mid<V, Mid::Kinetic>, sm));
-        k_z_mid<V, Mid::Kinetic><<<grid, FFT_THREADS, sm, st>>>(tb, buf, tkin);
+        k_z_mid<V, Mid::Kinetic><<<grid, fft_threads(sm, pts), sm, st>>>(tb, buf, tkin);
     } else {
         RS_TRY(set_smem(ctx, k_z_mid<V, Mid::Tpa>, sm));
-        k_z_mid<V, Mid::Tpa><<<grid, FFT_THREADS, sm, st>>>(tb, buf, tkin);
+        k_z_mid<V, Mid::Tpa><<<grid, fft_threads(sm, pts), sm, st>>>(tb, buf, tkin);
     }
     RS_LAUNCHED(ctx, "k_z_mid");
     return RSDFT_OK;
 }
 
 template <typename V>
-rsdft_status fft_xy_inverse_t(rsdft_ctx *ctx, const V *buf, const V *psi, const V *p, V *out, int nb,
+rsdft_status fft_xy_inverse_t(rsdft_ctx *ctx, const V *buf, const V *psi, const V *ab, V *out, int nb,
                               cudaStream_t st) {
     if (nb <= 0) return RSDFT_OK;
-    const size_t sm = plane_bytes<V>(ctx);
+    size_t sm = plane_bytes<V>(ctx);
+    int room = 0;
+    if (ab) RS_TRY(disc_smem(ctx, &sm, &room));
     dim3 grid(ctx->N[2], nb);
+    const int pts = ctx->N[0] * ctx->N[1];
     const double nxy = (double)ctx->N[0] * ctx->N[1];
     const double e = (double)sizeof(V);
     const double bpp = psi ? 3 * e : 2 * e;
     ProfScope ps(ctx, RSDFT_K_FFT_XY_INV, 5.0 * nxy * std::log2(nxy) * ctx->N[2] * nb,
                  bpp * (double)ctx->n * nb + (psi ? 0.5 * e * (double)ctx->n : 0.0), st);
     const FftTabs<V> tb = tabs_of(ctx, (V *)nullptr);
-    const auto &pt = proj_of(ctx, (V *)nullptr);
+    const Discs &discs = ctx->discs;
     const auto *v = v_of(ctx, (V *)nullptr);
     if (psi) {
-        // the plane plus, when it fits, the band's E_aj <beta_aj|psi> after it
-        const size_t smh = sm + (size_t)pt.natom * pt.nproj * sizeof(V);
-        const int stage = smh <= MAX_DYN_SMEM ? 1 : 0;
-        const size_t smu = stage ? smh : sm;
-        RS_TRY(set_smem(ctx, k_xy_inverse<V, Epi::Hpsi>, smu));
-        k_xy_inverse<V, Epi::Hpsi><<<grid, FFT_THREADS, smu, st>>>(tb, buf, psi, v, pt, p, out, stage);
+        RS_TRY(set_smem(ctx, k_xy_inverse<V, Epi::Hpsi>, sm));
+        k_xy_inverse<V, Epi::Hpsi><<<grid, fft_threads(sm, pts), sm, st>>>(tb, buf, psi, v, discs, room, ab, out);
     } else {
         RS_TRY(set_smem(ctx, k_xy_inverse<V, Epi::Plain>, sm));
-        k_xy_inverse<V, Epi::Plain><<<grid, FFT_THREADS, sm, st>>>(tb, buf, psi, v, pt, p, out, 0);
+        k_xy_inverse<V, Epi::Plain><<<grid, fft_threads(sm, pts), sm, st>>>(tb, buf, psi, v, discs, room, ab, out);
     }
     RS_LAUNCHED(ctx, "k_xy_inverse");
     return RSDFT_OK;
 }
 
+rsdft_status disc_buffers(rsdft_ctx *ctx, int nb, double2 **part, double2 **ab) {
+    const size_t per = (size_t)ctx->discs.ndisc * 3;
+    if (nb > ctx->disc_cap) {
+        if (ctx->discbuf) {
+            cudaFree(ctx->discbuf);
+            ctx->owned.erase(std::remove(ctx->owned.begin(), ctx->owned.end(), ctx->discbuf), ctx->owned.end());
+        }
+        ctx->discbuf = nullptr;
+        ctx->disc_cap = 0;
+        RS_TRY(dev_alloc(ctx, &ctx->discbuf, 2 * per * nb * sizeof(double2)));
+        ctx->disc_cap = nb;
+    }
+    *part = static_cast<double2 *>(ctx->discbuf);
+    *ab = *part + per * nb;
+    return RSDFT_OK;
+}
+
+template <typename V>
+static rsdft_status disc_finish_t(rsdft_ctx *ctx, const V *part, int nb, V *p, V *ab, cudaStream_t st) {
+    using T = typename Sc<V>::T;
+    k_disc_fin<V><<<cdiv((long long)nb * ctx->pt.natom * 32, PROJ_THREADS), PROJ_THREADS, 0, st>>>(
+        ctx->discs, part, nb, (T)ctx->dV, p, ab);
+    count_launch(ctx);
+    RS_LAUNCHED(ctx, "k_disc_fin");
+    return RSDFT_OK;
+}
+rsdft_status disc_finish(rsdft_ctx *ctx, const double2 *part, int nb, double2 *p, double2 *ab, cudaStream_t st) {
+    return disc_finish_t<double2>(ctx, part, nb, p, ab, st);
+}
+
 template <typename V>
 rsdft_status project_t(rsdft_ctx *ctx, const V *psi, V *p, int nb, cudaStream_t st) {
     if (nb <= 0 || ctx->pt.natom == 0) return RSDFT_OK;
-    dim3 grid(ctx->pt.natom, cdiv(nb, PROJ_BANDS));
+    double2 *part, *ab;
+    RS_TRY(disc_buffers(ctx, nb, &part, &ab));
     const double ne = (double)ctx->nent;
     const double e = (double)sizeof(V);
-    ProfScope ps(ctx, RSDFT_K_PROJECT, 4.0 * ctx->pt.nproj * ne * nb, e * ne * nb + (4 + 2 * e) * ne, st);
-    k_project<V><<<grid, PROJ_THREADS, 0, st>>>(proj_of(ctx, (V *)nullptr), psi, p, nb, ctx->n, ctx->dV);
-    RS_LAUNCHED(ctx, "k_project");
-    return RSDFT_OK;
+    {
+        ProfScope ps(ctx, RSDFT_K_PROJECT, 4.0 * ctx->pt.nproj * ne * nb, e * ne * nb, st);
+        k_gather<V><<<dim3(ctx->N[2], nb), PROJ_THREADS, 0, st>>>(ctx->discs, psi, ctx->N[0], ctx->N[1], ctx->n,
+                                                                reinterpret_cast<V *>(part));
+    }
+    RS_LAUNCHED(ctx, "k_gather");
+    return disc_finish_t<V>(ctx, reinterpret_cast<const V *>(part), nb, p, (V *)nullptr, st);
 }
 
 rsdft_status fft_xy_forward32(rsdft_ctx *ctx, Src kind, const float2 *src, const float2 *src2,
                               const double *theta, const int *act, float2 *dst, int nb,
-                              cudaStream_t st) {
-    return fft_xy_forward_t<float2>(ctx, kind, src, src2, theta, act, dst, nb, st);
+                              cudaStream_t st, float2 *part) {
+    return fft_xy_forward_t<float2>(ctx, kind, src, src2, theta, act, dst, nb, st, part);
 }
 rsdft_status fft_z_mid32(rsdft_ctx *ctx, Mid mid, float2 *buf, const double *tkin, int nb,
                          cudaStream_t st) {
     return fft_z_mid_t<float2>(ctx, mid, buf, tkin, nb, st);
 }
 rsdft_status fft_xy_inverse32(rsdft_ctx *ctx, const float2 *buf, const float2 *psi,
-                              const float2 *p, float2 *out, int nb, cudaStream_t st) {
-    return fft_xy_inverse_t<float2>(ctx, buf, psi, p, out, nb, st);
+                              const float2 *ab, float2 *out, int nb, cudaStream_t st) {
+    return fft_xy_inverse_t<float2>(ctx, buf, psi, ab, out, nb, st);
 }
 rsdft_status project(rsdft_ctx *ctx, const double2 *psi, double2 *p, int nb, cudaStream_t st) {
     return project_t<double2>(ctx, psi, p, nb, st);
@@ -547,13 +795,17 @@ rsdft_status refresh_v32(rsdft_ctx *ctx, cudaStream_t st) {
     return RSDFT_OK;
 }
 
+// H psi: the forward pass gathers the projections of its planes, the inverse pass scatters them.
 rsdft_status apply_h64(rsdft_ctx *ctx, const double2 *psi, double2 *hpsi, int nb, cudaStream_t st) {
     if (nb <= 0) return RSDFT_OK;
     RS_TRY(ensure_workspace(ctx, nb));
-    RS_TRY(project(ctx, psi, ctx->ws.proj, nb, st));
-    RS_TRY(fft_xy_forward(ctx, Src::Plain, psi, nullptr, nullptr, nullptr, nullptr, ctx->ws.T1, nb, st));
+    double2 *part = nullptr, *ab = nullptr;
+    const bool nl = ctx->discs.ndisc > 0;
+    if (nl) RS_TRY(disc_buffers(ctx, nb, &part, &ab));
+    RS_TRY(fft_xy_forward(ctx, Src::Plain, psi, nullptr, nullptr, nullptr, nullptr, ctx->ws.T1, nb, st, part));
+    if (nl) RS_TRY(disc_finish(ctx, part, nb, nullptr, ab, st));
     RS_TRY(fft_z_mid(ctx, Mid::Kinetic, ctx->ws.T1, nullptr, nb, st));
-    RS_TRY(fft_xy_inverse(ctx, ctx->ws.T1, psi, ctx->ws.proj, hpsi, nullptr, nb, st));
+    RS_TRY(fft_xy_inverse(ctx, ctx->ws.T1, psi, ab, hpsi, nullptr, nb, st));
     return RSDFT_OK;
 }
 
@@ -561,12 +813,15 @@ rsdft_status apply_h64(rsdft_ctx *ctx, const double2 *psi, double2 *hpsi, int nb
 rsdft_status apply_h32(rsdft_ctx *ctx, const float2 *psi, float2 *hpsi, int nb, cudaStream_t st) {
     if (nb <= 0) return RSDFT_OK;
     RS_TRY(ensure_workspace(ctx, nb));
-    float2 *proj = reinterpret_cast<float2 *>(ctx->ws.proj);
+    double2 *part = nullptr, *ab = nullptr;
+    const bool nl = ctx->discs.ndisc > 0;
+    if (nl) RS_TRY(disc_buffers(ctx, nb, &part, &ab));
+    float2 *part32 = reinterpret_cast<float2 *>(part), *ab32 = reinterpret_cast<float2 *>(ab);
     float2 *t1 = reinterpret_cast<float2 *>(ctx->ws.T1);
-    RS_TRY(project32(ctx, psi, proj, nb, st));
-    RS_TRY(fft_xy_forward32(ctx, Src::Plain, psi, nullptr, nullptr, nullptr, t1, nb, st));
+    RS_TRY(fft_xy_forward32(ctx, Src::Plain, psi, nullptr, nullptr, nullptr, t1, nb, st, part32));
+    if (nl) RS_TRY(disc_finish_t<float2>(ctx, part32, nb, nullptr, ab32, st));
     RS_TRY(fft_z_mid32(ctx, Mid::Kinetic, t1, nullptr, nb, st));
-    RS_TRY(fft_xy_inverse32(ctx, t1, psi, proj, hpsi, nb, st));
+    RS_TRY(fft_xy_inverse32(ctx, t1, psi, ab32, hpsi, nb, st));
     return RSDFT_OK;
 }
 

@@ -41,24 +41,6 @@ __device__ __forceinline__ void stage_in(int tot, SrcF src, DstF dst) {
     }
 }
 
-// The four beta values of one projector-table entry (16- or 32-byte aligned: the
-// tables are [nent][4]) in one 16-byte load (FP32) or two (FP64), instead of four
-// scalar loads that each cost the L1 a wavefront per thread.
-__device__ __forceinline__ void beta4(const float *bt, float b[4]) {
-    const float4 q = *reinterpret_cast<const float4 *>(bt);
-    b[0] = q.x;
-    b[1] = q.y;
-    b[2] = q.z;
-    b[3] = q.w;
-}
-__device__ __forceinline__ void beta4(const double *bt, double b[4]) {
-    const double2 q0 = reinterpret_cast<const double2 *>(bt)[0], q1 = reinterpret_cast<const double2 *>(bt)[1];
-    b[0] = q0.x;
-    b[1] = q0.y;
-    b[2] = q1.x;
-    b[3] = q1.y;
-}
-
 constexpr size_t MAX_DYN_SMEM = 227 * 1024;   // largest dynamic shared memory of one CTA
 
 // The attribute is per function and process-wide, so it is raised once to the

@@ -8,8 +8,9 @@
 // are formed with a normalised factor and shifted to the largest one of the slab.
 //
 // What bounds it: the FP64 passes ran at some 80% of the FP64 pipe; the integer instructions on
-// 64-bit values bound these.  144 bands on 64^3, one GB300: forward 3.23 -> 0.68 ms, z 3.66 ->
-// 0.84 ms, inverse 5.9 -> 3.6 ms (with the FP64 projector scatter, now its larger part); TPA of 53
+// 64-bit values bound these.  144 bands on 64^3, one GB300: forward 3.23 -> 0.68 ms (1.46 with
+// the projector gather, then 1.77 on its own), z 3.66 -> 0.81 ms, inverse 5.9 -> 2.1 ms with the
+// projector scatter; TPA of 53
 // bands on 45^3 1.94 -> 0.55 ms.  Errors against 64-bit FFTs are those of the reference itself:
 // relative 4.4e-16 (FP64 passes 4.8e-16) for TPA, 7.1e-16 (8.4e-16) for H psi.
 //
@@ -20,6 +21,7 @@
 
 #include "fft_common.h"
 #include "fix_fft.h"
+#include "proj.h"
 #include "rsdft_internal.h"
 
 namespace rsdft {
@@ -153,7 +155,8 @@ __device__ void lines(I2 *s, const AxisPlan &ax, const W4 *tw, int nlines, unsig
         const int st = INV ? ax.nstage - 1 - t : t;
         const int r = ax.radix[st];
         const bool twiddle = ax.sub[st] > 1;
-        const int sh = sc.bits - (INV && twiddle ? 2 : 0) - (fix::TOP - fix::growth(r));
+        // (an inverse stage turns before it sums, at 2^62 at most)
+        const int room = fix::TOP - fix::growth(r), sh = sc.bits - (INV && twiddle ? min(room + 2, 62) : room);
         sc.e += sh + (twiddle ? 2 : 0);
         const int now = sc.n % 3;
         if (threadIdx.x == 0) slot[(now + 1) % 3] = 0;
@@ -210,6 +213,144 @@ __device__ __forceinline__ double value(i64 v, int e) {
     return odd ? scalbn((double)v, e) : __longlong_as_double((long long)b);
 }
 
+// v w 2^-64 for w given as (h, l) with |w| < 2^62 (half: rounds)
+__device__ __forceinline__ i64 mul_hl(i64 v, int h, int l) {
+    const int vl = fix::lo_of(v), vh = fix::hi_of(v);
+    return fix::mw(vh, h, fix::mw(vl, h, fix::mw(vh, l, 0x80000000ll)) >> 32);
+}
+// (v w + u z) 2^-64
+__device__ __forceinline__ i64 mul2_hl(i64 v, int wh, int wl, i64 u, int zh, int zl) {
+    const int vl = fix::lo_of(v), vh = fix::hi_of(v), ul = fix::lo_of(u), uh = fix::hi_of(u);
+    const i64 mid = fix::mw(vl, wh, fix::mw(vh, wl, 0x80000000ll)) + fix::mw(ul, zh, fix::mw(uh, zl, 0));
+    return fix::mw(vh, wh, fix::mw(uh, zh, mid >> 32));
+}
+
+// fft.cu's gather on an integer plane in units of 2^e, with the factors in units of 2^-62: the values
+// leave room for the sum over the widest disc
+__device__ __forceinline__ void gather_plane_fix(const I2 *plane, int RS, const Discs &t, int z, int Nx, int e,
+                                                 double2 *__restrict__ part) {
+    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    const int d1 = t.plane_start[z + 1];
+    for (int d = t.plane_start[z] + (threadIdx.x >> 5); d < d1; d += nw) {
+        const int2 m = __ldg(reinterpret_cast<const int2 *>(t.meta + d));
+        const int rows = disc_rows(m.y), w = disc_width(m.y);
+        const int4 *gx = t.gxfix + (size_t)d * t.wmax;
+        i64 s[6] = {0, 0, 0, 0, 0, 0};
+        for (int r0 = 0; r0 < rows; r0 += 32) {
+            int4 q = make_int4(0, 0, 0, 0);
+            int hl = 0;
+            if (r0 + lane < rows) {
+                const DiscRowFix *rp = t.rowfix + m.x + r0 + lane;
+                q = __ldg(reinterpret_cast<const int4 *>(rp));
+                hl = __ldg(&rp->hl);
+            }
+            const I2 *row = plane + (q.x & 255) * RS;
+            int x = disc_x0(m.y);
+            I2 U{0, 0}, V{0, 0};   // sums of gx v, hx v along the row
+#pragma unroll 2
+            for (int j = 0; j < w; ++j) {
+                const int4 k = __ldg(gx + j);
+                I2 v = row[x];
+                if (!in_row(q.x, j)) v = I2{0, 0};
+                U.x += mul_hl(v.x, k.x, k.y);
+                U.y += mul_hl(v.y, k.x, k.y);
+                V.x += mul_hl(v.x, k.z, k.w);
+                V.y += mul_hl(v.y, k.z, k.w);
+                x = x + 1 == Nx ? 0 : x + 1;
+            }
+            U = fix::rshift(U, 5);   // room for the 128 rows' sum
+            V = fix::rshift(V, 5);
+            s[0] += mul_hl(U.x, q.y, q.z);
+            s[1] += mul_hl(U.y, q.y, q.z);
+            s[2] += mul_hl(V.x, q.y, q.z);
+            s[3] += mul_hl(V.y, q.y, q.z);
+            s[4] += mul_hl(U.x, q.w, hl);
+            s[5] += mul_hl(U.y, q.w, hl);
+        }
+#pragma unroll
+        for (int k = 0; k < 6; ++k)
+            for (int o = 16; o > 0; o >>= 1) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
+        if (lane < 3) {
+            const i64 re = lane == 0 ? s[0] : (lane == 1 ? s[2] : s[4]), im = lane == 0 ? s[1] : (lane == 1 ? s[3] : s[5]);
+            part[(size_t)d * 3 + lane] = make_double2(value(re, e + 9), value(im, e + 9));
+        }
+    }
+}
+
+// fft.cu's scatter into an integer plane of sc: the coefficients go to the plane's unit, or the plane
+// to the coefficients' where those are larger.  Returns false where a coefficient is not finite.
+__device__ __forceinline__ bool scatter_plane_fix(I2 *plane, int RS, const Discs &t, int z, int Nx, int Ny,
+                                                  const double2 *__restrict__ ab, I2 *uw, int room, Scale &sc, int *red) {
+    const int lane = threadIdx.x & 31;
+    const int d0 = t.plane_start[z], nd = t.plane_start[z + 1] - d0;
+    if (nd == 0) return true;
+    const double *a = reinterpret_cast<const double *>(ab + 3 * (size_t)d0);
+    int hmax = 0;
+    for (int i = threadIdx.x; i < 6 * nd; i += blockDim.x) hmax = max(hmax, __double2hiint(a[i]) & 0x7fffffff);
+    const int top = block_max(hmax, red) >> 20;
+    if (top == 0x7ff) return false;
+    // a point gets at most nd times 2.3 of the largest coefficient: below 2^59 units of 2^e
+    const int e = max(sc.e, top - 1022 + 3 + (32 - __clz(nd)) - 60);
+    if (e > sc.e) {
+        const int sh = min(e - sc.e, 63);
+        for (int i = threadIdx.x; i < Ny * RS; i += blockDim.x) {
+            const I2 v = plane[i];
+            plane[i] = I2{shifted(v.x, sh), shifted(v.y, sh)};
+        }
+        sc.e = e;
+    }
+    auto in = [&](double v) { return fix::from_double(__double2hiint(v), (unsigned)__double2loint(v), 4 - e); };
+    // U and W of disc d at x offset l
+    auto make_uw = [&](int d, int l, I2 &U, I2 &W) {
+        const int4 g = __ldg(t.gxfix + (size_t)d * t.wmax + l);
+        const double2 A = __ldg(ab + 3 * (size_t)d), Bx = __ldg(ab + 3 * (size_t)d + 1), By = __ldg(ab + 3 * (size_t)d + 2);
+        U = I2{mul2_hl(in(A.x), g.x, g.y, in(Bx.x), g.z, g.w), mul2_hl(in(A.y), g.x, g.y, in(Bx.y), g.z, g.w)};
+        W = I2{mul_hl(in(By.x), g.x, g.y), mul_hl(in(By.y), g.x, g.y)};
+    };
+    int base = d0;
+    for_discs(t, z, room ? room : nd, [&](int c0, int n) {
+        base = d0 + c0;
+        if (room == 0) return;   // no room beside the plane: U and W where they are used
+        for (int i = threadIdx.x; i < n * t.wmax; i += blockDim.x) {
+            const int d = i / t.wmax;
+            make_uw(base + d, i - d * t.wmax, uw[2 * i], uw[2 * i + 1]);
+        }
+    }, [&](int d, int ja, int jb) {
+        const int2 m = __ldg(reinterpret_cast<const int2 *>(t.meta + d));
+        const int rows = disc_rows(m.y);
+        const I2 *ue = uw + 2 * (size_t)(d - base) * t.wmax;
+        for (int r0 = 0; r0 < rows; r0 += 32) {
+            int4 q = make_int4(0, 0, 0, 0);
+            int hl = 0;
+            if (r0 + lane < rows) {
+                const DiscRowFix *rp = t.rowfix + m.x + r0 + lane;
+                q = __ldg(reinterpret_cast<const int4 *>(rp));
+                hl = __ldg(&rp->hl);
+            }
+            I2 *row = plane + (q.x & 255) * RS;
+            int x = disc_x0(m.y) + ja;
+            if (x >= Nx) x -= Nx;
+            for (int j = ja; j < jb; ++j) {
+                I2 U, W;
+                if (room) {
+                    U = ue[2 * j];
+                    W = ue[2 * j + 1];
+                } else {
+                    make_uw(d, j, U, W);
+                }
+                if (in_row(q.x, j)) {
+                    I2 o = row[x];
+                    o.x += mul2_hl(U.x, q.y, q.z, W.x, q.w, hl);
+                    o.y += mul2_hl(U.y, q.y, q.z, W.y, q.w, hl);
+                    row[x] = o;
+                }
+                x = x + 1 == Nx ? 0 : x + 1;
+            }
+        }
+    });
+    return true;
+}
+
 }  // namespace
 
 // ---- xy forward pass ------------------------------------------------------------
@@ -217,7 +358,7 @@ template <Src SRC>
 __global__ void __launch_bounds__(MAX_THREADS)
 k_xy_forward_fix(FixTabs tb, const double2 *__restrict__ src, const double2 *__restrict__ src2,
                  const double *__restrict__ theta, const int *__restrict__ act, const double *__restrict__ rsrc, int RS,
-                 I2 *__restrict__ dst, Meta *__restrict__ meta) {
+                 I2 *__restrict__ dst, Meta *__restrict__ meta, Discs discs, int disc_bits, double2 *__restrict__ part) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     int *red = reinterpret_cast<int *>(smem_raw);
     I2 *s_plane = reinterpret_cast<I2 *>(smem_raw + HEAD);
@@ -234,6 +375,7 @@ k_xy_forward_fix(FixTabs tb, const double2 *__restrict__ src, const double2 *__r
         hmax = max(hmax, max(hx & 0x7fffffff, hy & 0x7fffffff));
         s_plane[pidx(i, Nx, RS, nxm)] = I2{__double_as_longlong(v.x), __double_as_longlong(v.y)};
     };
+    const bool gather = SRC == Src::Plain && part;
     if (SRC == Src::Plain) {
         const double2 *in = src + band * n + off;
         stage_in<double2>(plane, [&](int i) { return in[i]; }, put);
@@ -254,11 +396,30 @@ k_xy_forward_fix(FixTabs tb, const double2 *__restrict__ src, const double2 *__r
     Meta *m = meta + (size_t)band * Nz + z;
     if (top == 0x7ff) {
         if (threadIdx.x == 0) *m = Meta{BAD, 0};
+        if (gather) {
+            const double nan = __longlong_as_double(0x7ff8000000000000ll);
+            for (int i = 3 * discs.plane_start[z] + threadIdx.x; i < 3 * discs.plane_start[z + 1]; i += blockDim.x)
+                part[(size_t)band * discs.ndisc * 3 + i] = make_double2(nan, nan);
+        }
         return;
     }
-    const int bits0 = fix::TOP - first_growth(tb.ax[0], false), s0 = bits0 - (top - 1022);
+    int bits0 = fix::TOP - first_growth(tb.ax[0], false);
+    if (gather) bits0 = min(bits0, disc_bits);
+    const int s0 = bits0 - (top - 1022);
     Scale sc{bits0, -s0, 0};
-    lines<false, true>(s_plane, tb.ax[0], tb.tw[0], Ny, tb.ax[1].nmag, RS, 1, sc, s0, slot);
+    if (gather) {
+        for (int i = threadIdx.x; i < Ny * RS; i += blockDim.x) {
+            const I2 v = s_plane[i];
+            s_plane[i] = I2{fix::from_double((int)(v.x >> 32), (unsigned)v.x, s0),
+                            fix::from_double((int)(v.y >> 32), (unsigned)v.y, s0)};
+        }
+        __syncthreads();
+        gather_plane_fix(s_plane, RS, discs, z, Nx, -s0, part + (size_t)band * discs.ndisc * 3);
+        __syncthreads();
+        lines<false, false>(s_plane, tb.ax[0], tb.tw[0], Ny, tb.ax[1].nmag, RS, 1, sc, 0, slot);
+    } else {
+        lines<false, true>(s_plane, tb.ax[0], tb.tw[0], Ny, tb.ax[1].nmag, RS, 1, sc, s0, slot);
+    }
     lines<false, false>(s_plane, tb.ax[1], tb.tw[1], Nx, tb.ax[0].nmag, 1, RS, sc, 0, slot);
     I2 *out = dst + band * n + off;
     for (int i = threadIdx.x; i < plane; i += blockDim.x) out[i] = s_plane[pidx(i, Nx, RS, nxm)];
@@ -388,8 +549,8 @@ enum class FixEpi { Plain, Hpsi, Real };
 template <FixEpi EPI>
 __global__ void __launch_bounds__(MAX_THREADS)
 k_xy_inverse_fix(FixTabs tb, const I2 *__restrict__ buf, const Meta *__restrict__ meta, const double2 *__restrict__ psi,
-                 const double *__restrict__ vloc, ProjTables pt, const double2 *__restrict__ p, int RS,
-                 double2 *__restrict__ out, double *__restrict__ rout, int stage_pe) {
+                 const double *__restrict__ vloc, Discs discs, const double2 *__restrict__ ab, int room, int RS,
+                 double2 *__restrict__ out, double *__restrict__ rout) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     int *red = reinterpret_cast<int *>(smem_raw);
     I2 *s_plane = reinterpret_cast<I2 *>(smem_raw + HEAD);
@@ -403,7 +564,7 @@ k_xy_inverse_fix(FixTabs tb, const I2 *__restrict__ buf, const Meta *__restrict_
     const unsigned nxm = tb.ax[0].nmag;
     unsigned *slot = reinterpret_cast<unsigned *>(red + 4);
     if (threadIdx.x > 0 && threadIdx.x < 8) red[threadIdx.x] = 0;
-    const int bits0 = fix::TOP + (tb.ax[1].sub[tb.ax[1].nstage - 1] > 1 ? 2 : 0) - first_growth(tb.ax[1], true);
+    const int bits0 = fix::TOP - first_growth(tb.ax[1], true);   // the last radix's stage has no twiddles
     const int e0 = row_shifts(meta + (size_t)band * Ny, Ny, bits0, shift, sst, red);
     Scale sc{bits0, e0, 0};
     if (e0 != BAD) {
@@ -415,9 +576,13 @@ k_xy_inverse_fix(FixTabs tb, const I2 *__restrict__ buf, const Meta *__restrict_
         lines<true, false>(s_plane, tb.ax[1], tb.tw[1], Nx, nxm, 1, RS, sc, 0, slot);
         lines<true, false>(s_plane, tb.ax[0], tb.tw[0], Ny, tb.ax[1].nmag, RS, 1, sc, 0, slot);
     }
+    bool good = e0 != BAD;
+    if (EPI == FixEpi::Hpsi && good && ab)
+        good = scatter_plane_fix(s_plane, RS, discs, z, Nx, Ny, ab + (size_t)band * discs.ndisc * 3,
+                                 s_plane + (size_t)Ny * RS + (RS > Nx ? 0 : SHIFTS / 16), room, sc, red + 1);
     const double nan = __longlong_as_double(0x7ff8000000000000ll);
     auto at = [&](int i) {
-        if (e0 == BAD) return make_double2(nan, nan);
+        if (!good) return make_double2(nan, nan);
         const I2 v = s_plane[pidx(i, Nx, RS, nxm)];
         return make_double2(value(v.x, sc.e), value(v.y, sc.e));
     };
@@ -430,47 +595,11 @@ k_xy_inverse_fix(FixTabs tb, const I2 *__restrict__ buf, const Meta *__restrict_
     } else {
         const double2 *ps = psi + band * n + off;
         const double *vv = vloc + off;
-        const int np = pt.natom * pt.nproj;
-        const double2 *pb = p + (size_t)band * np;
-        // E_aj <beta_aj|psi> of this band, staged once per CTA after the plane
-        // (when it fits; else read from global memory)
-        double2 *s_pe = reinterpret_cast<double2 *>(s_plane + (size_t)Ny * RS + (RS > Nx ? 0 : SHIFTS / 16));
-        if (stage_pe) {
-            for (int q = threadIdx.x; q < np; q += blockDim.x) {
-                const double2 c = pb[q];
-                const double e = pt.e_kb[q];
-                s_pe[q] = make_double2(e * c.x, e * c.y);
-            }
-            __syncthreads();
-        }
         double2 *o = out + band * n + off;
         for (int i = threadIdx.x; i < plane; i += blockDim.x) {
-            const double2 t = at(i);
-            const double2 y = ps[i];
+            const double2 t = at(i), y = ps[i];
             const double vi = vv[i];
-            double ax = t.x + vi * y.x, ay = t.y + vi * y.y;
-            const int g = (int)off + i;
-            const int e0_ = pt.c_rowptr[g], e1 = pt.c_rowptr[g + 1];
-            for (int e = e0_; e < e1; ++e) {
-                const int a0 = pt.c_atom[e] * pt.nproj;
-                double bt[4];
-                beta4(pt.c_beta + 4 * (size_t)e, bt);
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    if (j >= pt.nproj) break;
-                    double2 q;
-                    if (stage_pe) {
-                        q = s_pe[a0 + j];
-                    } else {
-                        const double2 c = pb[a0 + j];
-                        const double ek = pt.e_kb[a0 + j];
-                        q = make_double2(ek * c.x, ek * c.y);
-                    }
-                    ax += bt[j] * q.x;
-                    ay += bt[j] * q.y;
-                }
-            }
-            o[i] = make_double2(ax, ay);
+            o[i] = make_double2(t.x + vi * y.x, t.y + vi * y.y);
         }
     }
 }
@@ -536,7 +665,7 @@ FixTabs tabs_of(const rsdft_ctx *ctx) {
 }  // namespace
 
 rsdft_status fft_xy_forward(rsdft_ctx *ctx, Src kind, const double2 *src, const double2 *src2, const double *theta,
-                            const int *act, const double *rsrc, double2 *dst, int nb, cudaStream_t st) {
+                            const int *act, const double *rsrc, double2 *dst, int nb, cudaStream_t st, double2 *part) {
     if (nb <= 0) return RSDFT_OK;
     RS_TRY(check_plane(ctx));
     Meta *mp, *ms;
@@ -550,18 +679,23 @@ rsdft_status fft_xy_forward(rsdft_ctx *ctx, Src kind, const double2 *src, const 
     ProfScope ps(ctx, RSDFT_K_FFT_XY_FWD, 5.0 * nxy * std::log2(nxy) * ctx->N[2] * nb, bpp * (double)ctx->n * nb, st);
     const FixTabs tb = tabs_of(ctx);
     I2 *o = reinterpret_cast<I2 *>(dst);
+    int db = 63;   // bits at which the sum over a disc's row cannot overflow
+    while ((1 << (63 - db)) < ctx->discs.wmax) --db;
     switch (kind) {
         case Src::Plain:
             RS_TRY(set_smem(ctx, k_xy_forward_fix<Src::Plain>, sm));
-            k_xy_forward_fix<Src::Plain><<<grid, th, sm, st>>>(tb, src, src2, theta, act, rsrc, RS, o, mp);
+            k_xy_forward_fix<Src::Plain><<<grid, th, sm, st>>>(tb, src, src2, theta, act, rsrc, RS, o, mp, ctx->discs,
+                                                                db, part);
             break;
         case Src::Residual:
             RS_TRY(set_smem(ctx, k_xy_forward_fix<Src::Residual>, sm));
-            k_xy_forward_fix<Src::Residual><<<grid, th, sm, st>>>(tb, src, src2, theta, act, rsrc, RS, o, mp);
+            k_xy_forward_fix<Src::Residual><<<grid, th, sm, st>>>(tb, src, src2, theta, act, rsrc, RS, o, mp, ctx->discs,
+                                                                db, part);
             break;
         case Src::RealField:
             RS_TRY(set_smem(ctx, k_xy_forward_fix<Src::RealField>, sm));
-            k_xy_forward_fix<Src::RealField><<<grid, th, sm, st>>>(tb, src, src2, theta, act, rsrc, RS, o, mp);
+            k_xy_forward_fix<Src::RealField><<<grid, th, sm, st>>>(tb, src, src2, theta, act, rsrc, RS, o, mp, ctx->discs,
+                                                                db, part);
             break;
     }
     RS_LAUNCHED(ctx, "k_xy_forward_fix");
@@ -611,17 +745,20 @@ rsdft_status fft_z_mid(rsdft_ctx *ctx, Mid mid, double2 *buf, const double *tkin
     return RSDFT_OK;
 }
 
-rsdft_status fft_xy_inverse(rsdft_ctx *ctx, const double2 *buf, const double2 *psi, const double2 *p, double2 *out,
+rsdft_status fft_xy_inverse(rsdft_ctx *ctx, const double2 *buf, const double2 *psi, const double2 *ab, double2 *out,
                             double *rout, int nb, cudaStream_t st) {
     if (nb <= 0) return RSDFT_OK;
     RS_TRY(check_plane(ctx));
     Meta *mp, *ms;
     RS_TRY(ensure_meta(ctx, nb, &mp, &ms));
-    // the plane plus, when it fits, the band's E_aj <beta_aj|psi> after it
-    const size_t pe = psi ? (size_t)ctx->pt.natom * ctx->pt.nproj * sizeof(double2) : 0;
     const int RS = plane_stride(ctx);
-    const int stage = psi && plane_smem(ctx) + pe <= MAX_DYN_SMEM ? 1 : 0;
-    const size_t sm = plane_smem(ctx) + (stage ? pe : 0);
+    size_t sm = plane_smem(ctx);
+    int room = 0;
+    if (psi && ab) {   // the scatter table beside the plane
+        const size_t per = 2 * (size_t)ctx->discs.wmax * sizeof(I2);
+        room = disc_room(sm, per, ctx->discs.maxdiscs, MAX_DYN_SMEM);
+        sm += room * per;
+    }
     const dim3 grid(ctx->N[2], nb);
     const int th = threads_for(sm, ctx->N[0] * ctx->N[1]);
     const double nxy = (double)ctx->N[0] * ctx->N[1];
@@ -632,13 +769,16 @@ rsdft_status fft_xy_inverse(rsdft_ctx *ctx, const double2 *buf, const double2 *p
     const I2 *b = reinterpret_cast<const I2 *>(buf);
     if (rout) {
         RS_TRY(set_smem(ctx, k_xy_inverse_fix<FixEpi::Real>, sm));
-        k_xy_inverse_fix<FixEpi::Real><<<grid, th, sm, st>>>(tb, b, ms, psi, ctx->v, ctx->pt, p, RS, out, rout, 0);
+        k_xy_inverse_fix<FixEpi::Real><<<grid, th, sm, st>>>(tb, b, ms, psi, ctx->v, ctx->discs, ab, room, RS, out,
+                                                               rout);
     } else if (psi) {
         RS_TRY(set_smem(ctx, k_xy_inverse_fix<FixEpi::Hpsi>, sm));
-        k_xy_inverse_fix<FixEpi::Hpsi><<<grid, th, sm, st>>>(tb, b, ms, psi, ctx->v, ctx->pt, p, RS, out, rout, stage);
+        k_xy_inverse_fix<FixEpi::Hpsi><<<grid, th, sm, st>>>(tb, b, ms, psi, ctx->v, ctx->discs, ab, room, RS, out,
+                                                               rout);
     } else {
         RS_TRY(set_smem(ctx, k_xy_inverse_fix<FixEpi::Plain>, sm));
-        k_xy_inverse_fix<FixEpi::Plain><<<grid, th, sm, st>>>(tb, b, ms, psi, ctx->v, ctx->pt, p, RS, out, rout, 0);
+        k_xy_inverse_fix<FixEpi::Plain><<<grid, th, sm, st>>>(tb, b, ms, psi, ctx->v, ctx->discs, ab, room, RS, out,
+                                                               rout);
     }
     RS_LAUNCHED(ctx, "k_xy_inverse_fix");
     return RSDFT_OK;

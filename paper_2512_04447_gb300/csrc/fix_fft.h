@@ -4,7 +4,7 @@
 // GB300 issues a warp's FP64 instruction in 64 cycles of its sub-partition and integer
 // instructions in 2 to 4, so a 64-bit integer addition (2 instructions) costs a fifteenth of an
 // FP64 one and a complex product with a twiddle factor (12 multiply-adds of 32 x 32 -> 64 bits)
-// a third.  Values are kept below 2^61.5 in magnitude.  Before every stage the block is shifted to
+// a third.  Values are kept below 2^62.5 in magnitude.  Before every stage the block is shifted to
 // the largest scale at which the stage's sums cannot overflow, by the bits that its values
 // really have, so that a rounding error is one unit of some 2^-58 of the block's largest value at
 // each stage, where the FP64 transform rounds to 2^-53 of each value at each addition.
@@ -30,7 +30,7 @@ struct W4 {          // a factor w of magnitude <= 1: round(w 2^62) = h 2^32 + l
     int rh, rl, ih, il;
 };
 
-constexpr int TOP = 61;   // components are at most 2^TOP
+constexpr int TOP = 62;   // components are at most 2^TOP before the sums of a stage are formed, 2^62.5 after
 
 FIX_HD I2 add(I2 a, I2 b) { return I2{a.x + b.x, a.y + b.y}; }
 FIX_HD I2 sub(I2 a, I2 b) { return I2{a.x - b.x, a.y - b.y}; }
@@ -45,7 +45,9 @@ FIX_HD i64 mw(int a, int b, i64 c) { return (i64)a * b + c; }         // 32 x 32
 FIX_HD i64 rshift(i64 v, int s) { return s > 0 ? (v + ((v >> s) & 1) + (((i64)1 << (s - 1)) - 1)) >> s : v; }
 FIX_HD I2 rshift(I2 v, int s) { return I2{rshift(v.x, s), rshift(v.y, s)}; }
 
-// v w / 4 (CONJ: v conj(w) / 4) for |v| < 2^62; the product of the low words is left out
+// v w / 4 (CONJ: v conj(w) / 4) for |v| < 2^62.5; the product of the low words is left out.  The sums of
+// the mixed products stay below 2^62.8: |xl rh| + |yl ih| <= 2^31 sqrt(2) 2^30 and
+// |xh rl| + |yh il| <= sqrt(2) 2^30.5 2^31.
 template <bool CONJ> FIX_HD I2 mul_w(I2 v, W4 w) {
     const int xl = lo_of(v.x), xh = hi_of(v.x), yl = lo_of(v.y), yh = hi_of(v.y);
     const i64 half = 0x80000000ll;
@@ -55,10 +57,10 @@ template <bool CONJ> FIX_HD I2 mul_w(I2 v, W4 w) {
     return I2{mw(xh, w.rh, 0) - mw(yh, w.ih, 0) + ((a - b) >> 32), mw(xh, w.ih, mw(yh, w.rh, (c + d) >> 32))};
 }
 
-// v c for a constant 0 < c < 1 given as round(c 2^63) = ch 2^32 + cl, signed cl; |v| < 2^61.9
+// v c for a constant 0 < c < 1 given as round(c 2^63) = ch 2^32 + cl, signed cl; |v| < 2^62.5
 FIX_HD i64 mul_c(i64 v, int ch, int cl) {
     const int l = lo_of(v), h = hi_of(v);
-    return mw(2 * h, ch, mw(l, ch, mw(h, cl, 0x40000000ll)) >> 31);
+    return (mw(h, ch, 0) << 1) + (mw(l, ch, mw(h, cl, 0x40000000ll)) >> 31);
 }
 FIX_HD I2 mul_c(I2 v, int ch, int cl) { return I2{mul_c(v.x, ch, cl), mul_c(v.y, ch, cl)}; }
 constexpr i64 split_c(long double c) { return (i64)(c * 9223372036854775808.0L + 0.5L); }

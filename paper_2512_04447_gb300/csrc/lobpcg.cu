@@ -490,11 +490,11 @@ static rsdft_status gram_pair(rsdft_ctx *ctx, const RowBlocksT<V> &Y, const RowB
                               double2 *gs, double2 *gh, int k, bool tc, cudaStream_t st) {
     if constexpr (std::is_same<V, float2>::value) {
         if (tc) return gram_tc_sh(ctx, Y, HY, gs, gh, k, st);
+        RS_TRY(Ops<V>::gram(ctx, Y, Y, gs, k, true, ctx->dV, st));
+        return Ops<V>::gram(ctx, Y, HY, gh, k, true, ctx->dV, st);
     } else {
         return gram_sh(ctx, Y, HY, gs, gh, k, ctx->dV, st);
     }
-    RS_TRY(Ops<V>::gram(ctx, Y, Y, gs, k, true, ctx->dV, st));
-    return Ops<V>::gram(ctx, Y, HY, gh, k, true, ctx->dV, st);
 }
 
 // the double-float cluster tridiagonalisation in the subspace eigensolves

@@ -36,27 +36,40 @@ struct AxisPlan {
 
 struct Fft3Plan {
     AxisPlan ax[3];          // x, y, z
+    AxisPlan ax32[3];        // the FP32 passes' radices
     const double2 *tw64[3];  // [N] exp(-2 pi i k / N), device
     const float2 *tw32[3];
     const double *g2pos[3];  // G_a^2 at each digit-reversed position, device
-    const float *g2pos32[3];
+    const float *g2pos32[3]; // at the positions of ax32
     const double *gpos[3];   // G_a at each digit-reversed position (0 on the
                              // Nyquist plane of an even axis), device
 };
 
-// Device views handed to kernels (T = double for the FP64 form, float for the
-// FP32 data path of the mixed form; the index arrays are shared).
-template <typename T> struct ProjT {
+// Projector data that kernels other than the passes need.
+struct ProjTables {
     int natom, nproj;
-    const int *a_start;      // [natom+1] atom-major entry ranges
-    const int *a_idx;        // [nent] grid index
-    const T *a_beta;         // [nent][4] beta values (unused slots 0)
-    const int *c_rowptr;     // [n+1] point-major CSR
-    const int *c_atom;       // [nent]
-    const T *c_beta;         // [nent][4]
-    const T *e_kb;           // [natom*nproj]
+    const double *e_kb;      // [natom*nproj]
 };
-using ProjTables = ProjT<double>;
+
+// Kleinman-Bylander projectors by plane (proj.h).
+struct DiscMeta { int row0; unsigned packed; };                               // first row; rows | width << 8 | first x << 16
+struct __align__(16) DiscRow { int packed; float g, h; int pad; };            // a row of a disc: gy, dy/rc gy
+struct __align__(16) DiscRowFix { int packed, gh, gl, hh, hl, pad[3]; };      // the same in units of 2^-62
+struct Discs {
+    int natom, nproj, ndisc;
+    int wmax, maxrows, maxdiscs;             // widest disc, most rows of a disc, most discs of a plane
+    const int *plane_start;                  // [Nz + 1] discs of each plane
+    const int *color_ptr, *color_start;      // [Nz + 1] colours of each plane, [colours + 1] their discs: no two
+                                             // discs of a colour share a point
+    const DiscMeta *meta;                    // [ndisc]
+    const DiscRow *row;                      // by disc, in order of y: y | first x offset << 8 | points << 16
+    const DiscRowFix *rowfix;
+    const float2 *gx;                        // [ndisc][wmax] gx, dx/rc gx
+    const int4 *gxfix;                       // the same in units of 2^-62 (high, low words)
+    const int *atom_start, *atom_disc;       // [natom + 1], [ndisc] discs of each atom
+    const double2 *gz;                       // [ndisc] gz, dz/rc gz
+    const double *cnorm, *e_kb;              // [natom][4] norms c; [natom * nproj]
+};
 
 struct Workspace {
     int cap_band = 0;        // bands the buffers are sized for
@@ -159,7 +172,9 @@ struct rsdft_ctx {
     double *v = nullptr;             // [n] potential used by H
     float *v32 = nullptr;            // [n] FP32 copy of v for the mixed form
     rsdft::ProjTables pt{};
-    rsdft::ProjT<float> pt32{};
+    rsdft::Discs discs{};
+    void *discbuf = nullptr;         // [2][bands][ndisc][3]: partial sums, scatter coefficients
+    int disc_cap = 0;                // bands it holds
     long long nent = 0;
     rsdft::Workspace ws;
     rsdft::ScfWork scf;
@@ -223,29 +238,35 @@ enum class Src { Plain, Residual, RealField };
 // Forward xy-plane pass: src -> dst ([nb][n] complex).  Src::Residual reads
 // hx[act[b]] - theta[act[b]] x[act[b]]; Src::RealField reads a real [n] field
 // (nb must be 1).
+// part (with Src::Plain): also the projector gather of src, three sums per disc (proj.h).
 rsdft_status fft_xy_forward(rsdft_ctx *ctx, Src kind, const double2 *src, const double2 *src2,
                             const double *theta, const int *act, const double *rsrc,
-                            double2 *dst, int nb, cudaStream_t st);
+                            double2 *dst, int nb, cudaStream_t st, double2 *part = nullptr);
 // z pass: forward z FFT, multiply by the Mid factor, inverse z FFT (in place).
 rsdft_status fft_z_mid(rsdft_ctx *ctx, Mid mid, double2 *buf, const double *tkin, int nb,
                        cudaStream_t st);
-// Inverse xy pass.  When psi != nullptr: out = T psi + V psi + NL(p) (H psi);
+// Inverse xy pass.  When psi != nullptr: out = T psi + V psi + NL (H psi), the nonlocal part from the
+// disc coefficients ab (disc_finish);
 // else out = buf transformed (plain).  When rout != nullptr (nb == 1) the real
 // part is written to rout instead.
 rsdft_status fft_xy_inverse(rsdft_ctx *ctx, const double2 *buf, const double2 *psi,
-                            const double2 *p, double2 *out, double *rout, int nb,
+                            const double2 *ab, double2 *out, double *rout, int nb,
                             cudaStream_t st);
+// Partial-sum and coefficient buffers of nb bands, and the sums of part joined per atom: p (or null)
+// the projections, ab (or null) the scatter coefficients E <beta|psi> of every disc.
+rsdft_status disc_buffers(rsdft_ctx *ctx, int nb, double2 **part, double2 **ab);
+rsdft_status disc_finish(rsdft_ctx *ctx, const double2 *part, int nb, double2 *p, double2 *ab, cudaStream_t st);
 rsdft_status project(rsdft_ctx *ctx, const double2 *psi, double2 *p, int nb, cudaStream_t st);
 rsdft_status apply_h64(rsdft_ctx *ctx, const double2 *psi, double2 *hpsi, int nb,
                        cudaStream_t st);
 // FP32 data path of the mixed form
 rsdft_status fft_xy_forward32(rsdft_ctx *ctx, Src kind, const float2 *src, const float2 *src2,
                               const double *theta, const int *act, float2 *dst, int nb,
-                              cudaStream_t st);
+                              cudaStream_t st, float2 *part = nullptr);
 rsdft_status fft_z_mid32(rsdft_ctx *ctx, Mid mid, float2 *buf, const double *tkin, int nb,
                          cudaStream_t st);
 rsdft_status fft_xy_inverse32(rsdft_ctx *ctx, const float2 *buf, const float2 *psi,
-                              const float2 *p, float2 *out, int nb, cudaStream_t st);
+                              const float2 *ab, float2 *out, int nb, cudaStream_t st);
 rsdft_status project32(rsdft_ctx *ctx, const float2 *psi, float2 *p, int nb, cudaStream_t st);
 rsdft_status apply_h32(rsdft_ctx *ctx, const float2 *psi, float2 *hpsi, int nb, cudaStream_t st);
 rsdft_status refresh_v32(rsdft_ctx *ctx, cudaStream_t st);
