@@ -722,19 +722,10 @@ rsdft_status fft_xy_inverse_t(rsdft_ctx *ctx, const V *buf, const V *psi, const 
     return RSDFT_OK;
 }
 
-rsdft_status disc_buffers(rsdft_ctx *ctx, int nb, double2 **part, double2 **ab) {
+rsdft_status disc_buffers(rsdft_ctx *ctx, int nb, double2 **part, double2 **ab, cudaStream_t st) {
     const size_t per = (size_t)ctx->discs.ndisc * 3;
-    if (nb > ctx->disc_cap) {
-        if (ctx->discbuf) {
-            cudaFree(ctx->discbuf);
-            ctx->owned.erase(std::remove(ctx->owned.begin(), ctx->owned.end(), ctx->discbuf), ctx->owned.end());
-        }
-        ctx->discbuf = nullptr;
-        ctx->disc_cap = 0;
-        RS_TRY(dev_alloc(ctx, &ctx->discbuf, 2 * per * nb * sizeof(double2)));
-        ctx->disc_cap = nb;
-    }
-    *part = static_cast<double2 *>(ctx->discbuf);
+    RS_TRY(grow(ctx, ctx->discbuf, std::max<size_t>(16, 2 * per * nb * sizeof(double2)), st));
+    *part = static_cast<double2 *>(ctx->discbuf.p);
     *ab = *part + per * nb;
     return RSDFT_OK;
 }
@@ -756,7 +747,7 @@ template <typename V>
 rsdft_status project_t(rsdft_ctx *ctx, const V *psi, V *p, int nb, cudaStream_t st) {
     if (nb <= 0 || ctx->pt.natom == 0) return RSDFT_OK;
     double2 *part, *ab;
-    RS_TRY(disc_buffers(ctx, nb, &part, &ab));
+    RS_TRY(disc_buffers(ctx, nb, &part, &ab, st));
     const double ne = (double)ctx->nent;
     const double e = (double)sizeof(V);
     {
@@ -801,7 +792,7 @@ rsdft_status apply_h64(rsdft_ctx *ctx, const double2 *psi, double2 *hpsi, int nb
     RS_TRY(ensure_workspace(ctx, nb));
     double2 *part = nullptr, *ab = nullptr;
     const bool nl = ctx->discs.ndisc > 0;
-    if (nl) RS_TRY(disc_buffers(ctx, nb, &part, &ab));
+    if (nl) RS_TRY(disc_buffers(ctx, nb, &part, &ab, st));
     RS_TRY(fft_xy_forward(ctx, Src::Plain, psi, nullptr, nullptr, nullptr, nullptr, ctx->ws.T1, nb, st, part));
     if (nl) RS_TRY(disc_finish(ctx, part, nb, nullptr, ab, st));
     RS_TRY(fft_z_mid(ctx, Mid::Kinetic, ctx->ws.T1, nullptr, nb, st));
@@ -815,7 +806,7 @@ rsdft_status apply_h32(rsdft_ctx *ctx, const float2 *psi, float2 *hpsi, int nb, 
     RS_TRY(ensure_workspace(ctx, nb));
     double2 *part = nullptr, *ab = nullptr;
     const bool nl = ctx->discs.ndisc > 0;
-    if (nl) RS_TRY(disc_buffers(ctx, nb, &part, &ab));
+    if (nl) RS_TRY(disc_buffers(ctx, nb, &part, &ab, st));
     float2 *part32 = reinterpret_cast<float2 *>(part), *ab32 = reinterpret_cast<float2 *>(ab);
     float2 *t1 = reinterpret_cast<float2 *>(ctx->ws.T1);
     RS_TRY(fft_xy_forward32(ctx, Src::Plain, psi, nullptr, nullptr, nullptr, t1, nb, st, part32));

@@ -16,8 +16,10 @@
 // points go in chunks that keep the residues within RNS_BYTES.
 //
 // Measured on one GB300 against the FP64 kernels (which run at 97% of the FP64 pipe):
-//   Gram 432 x 432 over 64^3 points   321.8 -> 12.7 ms     rotation 432 -> 144   104.8 -> 6.0 ms
-//   real Gram 285 x 285 over 60^3      30.2 ->  2.8 ms
+//   Gram 432 x 432 over 64^3 points   321.8 -> 8.7 ms     rotation 432 -> 144   104.8 -> 4.9 ms
+//   real Gram 285 x 285 over 60^3      30.2 -> 2.35 ms
+// of the Gram's 8.7 ms the residue planes take 3.4 (81% of DRAM bandwidth, 78% of the issue slots), the
+// statistics 0.6 and the MMAs 4.6 (75% of the BF16 rate).
 // and errors against extended precision (150 x 150 over 5,400 points: relative 2.5e-16 against
 // 1.4e-15; rotation 432 -> 144: 1.6e-16 against 9.8e-16).
 //
@@ -38,6 +40,7 @@ namespace rsdft {
 namespace rns {
 
 using tc::smem_u32;
+typedef long long i64;
 typedef unsigned long long u64;
 typedef unsigned __int128 u128;
 
@@ -51,8 +54,9 @@ struct Consts {
     float p[NM], ip[NM];
     int m[NM];
     int lo[NM], hi[NM];        // 256^j mod p, symmetric, as signed bytes j = 0..3 and 4..7
-    uint32_t w[NM][4];         // frac((P/p)^-1 mod p / p) * 2^128, little-endian limbs
-    u64 P0, P1;                // P
+    // W = floor(frac((P/p)^-1 mod p / p) 2^96) by byte j = 0..11, four moduli a word (the sixteenth is 0)
+    uint32_t w[12][4];
+    u64 Ptop;                  // P / 2^54, rounded
 };
 
 constexpr Consts make_consts() {
@@ -76,18 +80,17 @@ constexpr Consts make_consts() {
         const int q = (int)((P / (u128)p) % (u128)p);
         int inv = 1;
         while ((inv * q) % p != 1) ++inv;
-        // floor(inv 2^128 / p) by long division
+        // floor(inv 2^96 / p) by long division
         u128 w = 0;
         int r = inv;
-        for (int k = 0; k < 128; ++k) {
+        for (int k = 0; k < 96; ++k) {
             r *= 2;
             w <<= 1;
             if (r >= p) { r -= p; w |= 1; }
         }
-        for (int k = 0; k < 4; ++k) c.w[i][k] = (uint32_t)(w >> (32 * k));
+        for (int j = 0; j < 12; ++j) c.w[j][i >> 2] |= (uint32_t)(uint8_t)(w >> (8 * j)) << (8 * (i & 3));
     }
-    c.P0 = (u64)P;
-    c.P1 = (u64)(P >> 64);
+    c.Ptop = (u64)((P + ((u128)1 << 53)) >> 54);
     return c;
 }
 __constant__ Consts K = make_consts();
@@ -376,7 +379,7 @@ __global__ void k_coef_residues(const double2 *__restrict__ c, int ldc, Seg s, i
 // reduced modulo p into 128 registers of each drain thread while the next chunk's MMAs run,
 // so that every FP32 sum stays an exact integer below 2^24.
 //   Gram (ROT = false): A, B K-major [row][point]; tile of conj(A) B^T; residues of the sums
-//     go to out16[split][q][plane][M][N].
+//     go to out16[split][q][plane][M][blocks npad].
 //   Rotation (ROT = true): A = residues of Y read MN-major (points are M), B = coefficients
 //     K-major; residues go to out8[q][segment][plane][N / 4][points], four bands a word.
 constexpr int THREADS = 320;
@@ -394,6 +397,7 @@ template <bool REAL> struct Cfg {
 struct Args {
     int items;
     int mt, nt;                 // tile counts
+    int npad;                   // Gram: columns of a block of out16 (N rounded up to 8)
     int nstep;                  // columns per tile
     int boxn;                   // rows of the B box (its bytes: boxn * 128 per plane)
     int M, N;                   // output rows and columns (Gram: N of one block)
@@ -632,18 +636,35 @@ k_rns(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMa
             if (stop) break;
             const int row = it.m0 + lq * 32 + lane;
             if (!ROT) {
+                // eight residues a store: rows of npad columns a block, npad and the tiles multiples of 8
                 const int plane = REAL ? 0 : half;
-                const int ldn = a.N * a.blocks;
-                short *o = a.out16 + ((((size_t)it.slot * NM + it.q) * PL + plane) * a.M + row) * (size_t)ldn +
-                           it.n0 + (REAL ? half * 128 : 0);
+                const int blk = it.n0 / a.N, col = it.n0 - blk * a.N + (REAL ? half * 128 : 0);
+                int4 *o = reinterpret_cast<int4 *>(a.out16 + ((((size_t)it.slot * NM + it.q) * PL + plane) * a.M + row) *
+                                                                 (size_t)(a.npad * a.blocks) + blk * a.npad + col);
                 if (row < a.M) {
 #pragma unroll
-                    for (int i = 0; i < 128; ++i) {
-                        if (i < ncol) {
-                            float v = acc[i];
-                            if (a.accumulate) v += (float)o[i];
-                            const float k = fmaf(v, ip, MAGIC) - MAGIC;
-                            o[i] = (short)(int)fmaf(-k, p, v);
+                    for (int i = 0; i < 16; ++i) {
+                        if (8 * i < ncol) {
+                            int w[4] = {0, 0, 0, 0};
+                            if (a.accumulate) {
+                                const int4 old = o[i];
+                                w[0] = old.x;
+                                w[1] = old.y;
+                                w[2] = old.z;
+                                w[3] = old.w;
+                            }
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                int r[2];
+#pragma unroll
+                                for (int h = 0; h < 2; ++h) {
+                                    const float v = acc[8 * i + 2 * j + h] + (float)(short)(w[j] >> (16 * h));
+                                    const float k = fmaf(v, ip, MAGIC) - MAGIC;
+                                    r[h] = __float_as_int(fmaf(-k, p, v) + MAGIC);
+                                }
+                                w[j] = (int)__byte_perm(r[0], r[1], 0x5410);
+                            }
+                            o[i] = make_int4(w[0], w[1], w[2], w[3]);
                         }
                     }
                 }
@@ -680,61 +701,66 @@ k_rns(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMa
 }
 
 // ---- Chinese remainder ----------------------------------------------------------------
-// f += r w: 128-bit, 0 <= r < p.  f holds the fraction (integer / P) as 2^-128 f, truncated by
-// at most sum p; a sum that is 0 has zero residues and gives exactly 0.
-__device__ __forceinline__ void crt_add(uint32_t f[4], unsigned r, int q) {
-    asm("mad.lo.cc.u32 %0, %4, %5, %0;\n\t"
-        "madc.lo.cc.u32 %1, %4, %6, %1;\n\t"
-        "madc.lo.cc.u32 %2, %4, %7, %2;\n\t"
-        "madc.lo.u32 %3, %4, %8, %3;\n\t"
-        "mad.hi.cc.u32 %1, %4, %5, %1;\n\t"
-        "madc.hi.cc.u32 %2, %4, %6, %2;\n\t"
-        "madc.hi.u32 %3, %4, %7, %3;"
-        : "+r"(f[0]), "+r"(f[1]), "+r"(f[2]), "+r"(f[3])
-        : "r"(r), "r"(K.w[q][0]), "r"(K.w[q][1]), "r"(K.w[q][2]), "r"(K.w[q][3]));
-}
-
-// x 2^-s of the integer x = P f / 2^128 (f signed), rounded to nearest
-__device__ __forceinline__ double crt_value(const uint32_t f[4], int s) {
-    u64 f0 = ((u64)f[1] << 32) | f[0], f1 = ((u64)f[3] << 32) | f[2];
-    const bool neg = (long long)f1 < 0;
+// x 2^-s of the integer x with the symmetric residues r (bytes, four moduli a word): the fraction
+// x / P is sum r W / 2^96 modulo 1, its bytes' columns summed by dp4a (48 instead of 75 to 105
+// wide multiply-adds), good to 2^-85: 2^-83 of the product of the operands' bounds.  All residues 0
+// give exactly 0.
+__device__ __forceinline__ double crt_value(const int r[4], int s) {
+    i64 limb[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        int c[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            int d = 0;
+#pragma unroll
+            for (int g = 0; g < 4; ++g)
+                asm("dp4a.s32.u32 %0, %1, %2, %0;" : "+r"(d) : "r"(r[g]), "r"(K.w[4 * k + j][g]));
+            c[j] = d;   // |d| < 2^19
+        }
+        limb[k] = (i64)(c[2] + (c[3] << 8)) * 65536 + (c[0] + (c[1] << 8));
+    }
+    const i64 m1 = limb[1] + (limb[0] >> 32), m2 = limb[2] + (m1 >> 32);
+    unsigned f0 = (unsigned)limb[0], f1 = (unsigned)m1, f2 = (unsigned)m2;
+    const bool neg = (int)f2 < 0;
     if (neg) {   // two's complement
         f0 = ~f0 + 1;
         f1 = ~f1 + (f0 == 0);
+        f2 = ~f2 + (f0 == 0 && f1 == 0);
     }
-    // (f1 f0)(P1 P0) / 2^128, rounded: the integer result
-    const u64 a = __umul64hi(f0, K.P0);
-    u64 lo = f0 * K.P1, m = a + lo, hi = __umul64hi(f0, K.P1) + (m < a);
-    lo = f1 * K.P0;
-    m += lo;
-    u64 hi2 = __umul64hi(f1, K.P0) + (m < lo);
-    u64 x0 = f1 * K.P1, x1 = __umul64hi(f1, K.P1);
-    x0 += hi;
-    x1 += x0 < hi;
-    x0 += hi2;
-    x1 += x0 < hi2;
-    x0 += m >> 63;
-    x1 += x0 < (m >> 63);
-    if (!(x0 | x1)) return 0.0;
-    // 64 leading bits (sticky), then to nearest even
-    const int lz = x1 ? __clzll(x1) : 64 + __clzll(x0);
-    u64 t = lz >= 64 ? x0 << (lz - 64) : (lz ? (x1 << lz) | (x0 >> (64 - lz)) : x1);
-    if (lz < 64 && (x0 << lz)) t |= 1;
-    u64 r = t >> 11;
-    const u64 rest = t & 0x7ff;
-    r += rest > 0x400 || (rest == 0x400 && (r & 1));
-    // value = r 2^e with 2^52 <= r <= 2^53
-    const int e = 75 - lz - s, field = e + 1075;
+    int e = 22 - s;   // x = hi 2^(e + s), below
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+        if (f2 == 0) {
+            f2 = f1;
+            f1 = f0;
+            f0 = 0;
+            e -= 32;
+        }
+    if (f2 == 0) return 0.0;
+    const int lz = __clz((int)f2);
+    const u64 m = ((u64)__funnelshift_l(f1, f2, lz) << 32) | __funnelshift_l(f0, f1, lz);   // F = m 2^(32 - lz)
+    u64 hi = __umul64hi(m, K.Ptop);        // x = F P / 2^96 = hi 2^(64 + 32 - lz + 54 - 96)
+    e += 32 - lz;
+    if (!(hi >> 63)) {
+        hi <<= 1;
+        e -= 1;
+    }
+    u64 t = hi >> 11;
+    const u64 rest = hi & 0x7ff;
+    t += rest > 0x400 || (rest == 0x400 && (t & 1));
+    // value = t 2^(11 + e) with 2^52 <= t <= 2^53
+    const int field = e + 11 + 1075;
     double v;
-    if (field >= 1 && field <= 2045) v = __longlong_as_double((long long)r + ((long long)(field - 1) << 52));
-    else v = scalbn((double)r, e);   // beyond the normal range
+    if (field >= 1 && field <= 2045) v = __longlong_as_double((long long)t + ((long long)(field - 1) << 52));
+    else v = scalbn((double)t, e + 11);   // beyond the normal range
     return neg ? -v : v;
 }
 
-// g entries of one or two blocks from the residue sums out16[slot][q][plane][M][N blocks]
+// g entries of one or two blocks from the residue sums out16[slot][q][plane][M][blocks npad]
 // (padded bands in real form).  herm: entries below the diagonal from their mirror, the
 // diagonal real.
-__global__ void k_crt_gram(const short *__restrict__ out16, int slots, int M, int N, int blocks, int real, int a0,
+__global__ void k_crt_gram(const short *__restrict__ out16, int slots, int M, int N, int npad, int blocks, int real, int a0,
                            int a1, int b0, int b1, int na, int nb, int herm, const int *__restrict__ sa,
                            const int *__restrict__ sb, double scale, double2 *__restrict__ g0,
                            double2 *__restrict__ g1, int ldg, const int *flag) {
@@ -757,21 +783,22 @@ __global__ void k_crt_gram(const short *__restrict__ out16, int slots, int M, in
     }
     const bool mirror = herm && I > J;
     const int r = mirror ? J : I, c = mirror ? I : J;
-    const int PL = real ? 1 : 2, ldn = N * blocks;
+    const int PL = real ? 1 : 2, ldn = npad * blocks;
     double v[2] = {0.0, 0.0};
     // scales are per complex row and plane: 2 row + plane is the padded band in real form
     const int s = sa[real ? r : 2 * r] + sb[real ? blk * N + c : 2 * (blk * N + c)];
     for (int pl = 0; pl < PL; ++pl) {
-        uint32_t f[4] = {0, 0, 0, 0};
+        int rr[4] = {0, 0, 0, 0};
+#pragma unroll
         for (int q = 0; q < NM; ++q) {
             int t = 0;
             for (int u = 0; u < slots; ++u)
-                t += out16[((((size_t)u * NM + q) * PL + pl) * M + r) * (size_t)ldn + blk * N + c];
+                t += out16[((((size_t)u * NM + q) * PL + pl) * M + r) * (size_t)ldn + blk * npad + c];
             const float k = fmaf((float)t, K.ip[q], MAGIC) - MAGIC;
-            t -= (int)k * K.m[q];
-            crt_add(f, (unsigned)(t < 0 ? t + K.m[q] : t), q);
+            t -= (int)k * K.m[q];   // symmetric; 128 = -128 modulo 256
+            rr[q >> 2] |= (t & 255) << (8 * (q & 3));
         }
-        v[pl] = crt_value(f, s);
+        v[pl] = crt_value(rr, s);
     }
     if (herm && I == J) v[1] = 0.0;
     if (mirror) v[1] = -v[1];
@@ -793,25 +820,23 @@ k_crt_rot(const unsigned *__restrict__ out8, int segs, int m, long long ldp, lon
     constexpr int PL = REAL ? 1 : 2;
     double sum[4][PL];
     for (int sg = segs - 1; sg >= 0; --sg) {
-        uint32_t f[4][PL][4];
+        int r[PL][4][4];   // [plane][column][word of moduli]
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
+        for (int pl = 0; pl < PL; ++pl)
 #pragma unroll
-            for (int pl = 0; pl < PL; ++pl)
+            for (int g = 0; g < 4; ++g) {
+                unsigned w[4];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) f[j][pl][k] = 0;
-#pragma unroll
-        for (int q = 0; q < NM; ++q) {
-#pragma unroll
-            for (int pl = 0; pl < PL; ++pl) {
-                const unsigned w = __ldg(out8 + (((size_t)(q * segs + sg) * PL + pl) * nquad + quad) * ldp + t);
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int r = (int)(w << (24 - 8 * j)) >> 24;
-                    crt_add(f[j][pl], (unsigned)(r + ((r >> 31) & K.m[q])), q);
-                }
+                for (int i = 0; i < 4; ++i)
+                    w[i] = 4 * g + i < NM ? __ldg(out8 + (((size_t)((4 * g + i) * segs + sg) * PL + pl) * nquad + quad) * ldp + t) : 0u;
+                // four columns of four moduli -> four moduli of each column
+                const unsigned a0 = __byte_perm(w[0], w[1], 0x5140), a1 = __byte_perm(w[2], w[3], 0x5140);
+                const unsigned b0 = __byte_perm(w[0], w[1], 0x7362), b1 = __byte_perm(w[2], w[3], 0x7362);
+                r[pl][0][g] = (int)__byte_perm(a0, a1, 0x5410);
+                r[pl][1][g] = (int)__byte_perm(a0, a1, 0x7632);
+                r[pl][2][g] = (int)__byte_perm(b0, b1, 0x5410);
+                r[pl][3][g] = (int)__byte_perm(b0, b1, 0x7632);
             }
-        }
         const int h = hmax[(size_t)sg * n + p0 + t];
         const int sp = point_scale(h, sg ? bits1 : bits0);
 #pragma unroll
@@ -820,7 +845,7 @@ k_crt_rot(const unsigned *__restrict__ out8, int segs, int m, long long ldp, lon
             const int s = (b < m ? sc[sg * mcols + b] : 0) + sp;
 #pragma unroll
             for (int pl = 0; pl < PL; ++pl) {
-                const double v = crt_value(f[j][pl], s);
+                const double v = crt_value(r[pl][j], s);
                 sum[j][pl] = sg == segs - 1 ? v : sum[j][pl] + v;
             }
         }
@@ -859,22 +884,26 @@ __global__ void k_poison(double2 *out, long long cnt, const int *flag) {
 using namespace rns;
 
 // ---- host side ---------------------------------------------------------------------------
-// Bytes of residues held at a time (the points go in chunks of that size).
-constexpr size_t RNS_BYTES = (size_t)1 << 30;
+// Bytes of residues held at a time (the points go in chunks of that size): a chunk's launches end
+// with a partly filled wave and the residues' way out (432 x 432: 9.0 ms with 2^30, 8.7 with 2^31, 8.5 with
+// 2^32).  Where that does not fit, an eighth of it is tried, then the FP64 kernels run.
+constexpr size_t RNS_BYTES = (size_t)1 << 31;
 
-static rsdft_status rns_buffer(rsdft_ctx *ctx, size_t bytes) {
+// Whether there is room for a call's residues: growing takes at most a quarter of the free memory.
+static bool rns_buffer(rsdft_ctx *ctx, size_t bytes, cudaStream_t st) {
     RnsWork &w = ctx->rns;
-    if (!w.flag) RS_TRY(dev_alloc(ctx, (void **)&w.flag, 64));
-    if (bytes <= w.bytes) return RSDFT_OK;
-    if (w.buf) {
-        cudaFree(w.buf);
-        ctx->owned.erase(std::remove(ctx->owned.begin(), ctx->owned.end(), w.buf), ctx->owned.end());
+    if (bytes > w.buf.bytes) {
+        size_t free_now = 0, total = 0;
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        if (cudaMemGetInfo(&free_now, &total) != cudaSuccess) cudaGetLastError();
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        if (bytes > (free_now + w.buf.bytes) / 4) return false;
     }
-    w.buf = nullptr;
-    w.bytes = 0;
-    RS_TRY(dev_alloc(ctx, &w.buf, bytes));
-    w.bytes = bytes;
-    return RSDFT_OK;
+    const bool ok = grow(ctx, w.fbuf, 64, st) == RSDFT_OK && grow(ctx, w.buf, bytes, st) == RSDFT_OK;
+    if (!ok) ctx->err.clear();
+    w.flag = static_cast<int *>(w.fbuf.p);
+    return ok;
 }
 
 struct Carver {
@@ -905,19 +934,26 @@ static rsdft_status launch_gemm(rsdft_ctx *ctx, const CUtensorMap &mA, const CUt
     return RSDFT_OK;
 }
 
-// Whether the residue path is the faster one: an estimate of both, in seconds.  FP64 kernels:
-// f flops per product at 1.15 TFLOP/s.  Residues: launches, residue planes written and read,
-// MMAs over whole tiles.
-static bool rns_wins(double n, double rows, double mpad, double npad, double entries, bool real, double extra) {
-    const double f = real ? 2.0 : 8.0;
-    const double t64 = f * n * entries / 1.15e12;
-    const double trns = 60e-6 + rows * n * (8.0 * NM + 32.0) / 4.0e12 + NM * f * n * mpad * npad / 0.7e15 + extra;
-    return t64 > 1.25 * trns;
+// Whether the residue path is the faster one.
+//  Gram: the FP64 kernel sums at least 512 points a CTA (all of them below that), a microsecond each and
+//  0.3 in real form, whatever the number of rows; measured on 216 to 262,144 points and 16 to 288 rows a
+//  side, the residue path was the faster one throughout (16 x 16 on 6^3 236 -> 66 us, real 78 -> 64 us;
+//  on 20^3 562 -> 103 us, real 173 -> 89 us).
+static bool gram_wins(long long n) { return n >= 200; }
+//  Rotation, in seconds: the FP64 kernel at 1.15 TFLOP/s over whole tiles of 16 rows and bands (pair rows in
+//  real form) against launches, work items of 128 points (some 2 us each on an SM) and the residue
+//  planes (33 ps a row and point).  Within 25% of the times measured on the sizes above; the line at
+//  1.15 keeps FP64 where the two meet (24 -> 8 bands on 32^3: 136 against 111 us).
+static bool rotation_wins(double n, int rows, int k, int m, bool real, int items_per_tile) {
+    auto up = [real](int c) { return real ? 2.0 * (cdiv((c + 1) / 2, 16) * 16) : (double)(cdiv(c, 16) * 16); };
+    const double t64 = (real ? 2.0 : 8.0) * n * up(k) * up(m) / 1.15e12;
+    const double trns = 50e-6 + n / 128.0 * items_per_tile * 1.4e-8 + rows * n * 3.3e-11;
+    return t64 > 1.15 * trns;
 }
 
-rsdft_status rns_gram(rsdft_ctx *ctx, const RowBlocks &A0, const RowBlocks &B0, const RowBlocks *B1, bool real,
-                      bool herm, double2 *g0, double2 *g1, int ldg, double scale, cudaStream_t st, bool *used) {
-    *used = false;
+static rsdft_status gram_within(rsdft_ctx *ctx, size_t limit, const RowBlocks &A0, const RowBlocks &B0,
+                                const RowBlocks *B1, bool real, bool herm, double2 *g0, double2 *g1, int ldg,
+                                double scale, cudaStream_t st, bool *used) {
     const int na = rows_of(A0), nb = rows_of(B0), blocks = B1 ? 2 : 1;
     const RowBlocks A = real ? pair_rows(A0) : A0, B = real ? pair_rows(B0) : B0;
     const int ra = rows_of(A), rb = rows_of(B);
@@ -927,16 +963,14 @@ rsdft_status rns_gram(rsdft_ctx *ctx, const RowBlocks &A0, const RowBlocks &B0, 
     const int PL = real ? 1 : 2, M = real ? 2 * ra : ra, N = real ? 2 * rb : rb;
     const int NT = real ? 256 : 128;
     const int mt = cdiv(M, 128), nt = cdiv(N, NT);
-    const double part = herm ? 0.5 * (1.0 + 1.0 / mt) : 1.0;
     const double frac = (herm ? 0.5 : 1.0) * blocks;
     const int R = (same ? 0 : ra) + rb * blocks;
-    if (!rns_wins((double)n, R, 128.0 * mt * part * blocks, cdiv(N, 16) * 16.0, frac * na * nb, real, 0.0)) return RSDFT_OK;
     int tiles = 0;
     for (int t = 0; t < mt; ++t) tiles += herm ? nt - t * 128 / NT : nt;
     tiles *= blocks;
     // chunks of points, equal and multiples of 64
     const size_t per_point = (size_t)NM * R * 4;
-    const long long most = std::max<long long>(4096, (long long)(RNS_BYTES / per_point) / 64 * 64);
+    const long long most = std::max<long long>(4096, (long long)(limit / per_point) / 64 * 64);
     const int nchunk = cdiv(n, most);
     const int ld = cdiv(cdiv(n, nchunk), 64) * 64;
     const int kbt = ld / 64;
@@ -949,15 +983,13 @@ rsdft_status rns_gram(rsdft_ctx *ctx, const RowBlocks &A0, const RowBlocks &B0, 
         if (eff > best + 0.02) { best = eff; splits = s; }
     }
     const int S = std::max(1, std::min<int>(64, (int)(n / 4096)));
-    const size_t out_elems = (size_t)splits * NM * PL * M * N * blocks;
+    const int npad = cdiv(N, 8) * 8;
+    const size_t out_elems = (size_t)splits * NM * PL * M * npad * blocks;
     Carver cv{nullptr};
     for (int pass = 0; pass < 2; ++pass) {
         if (pass == 1) {
-            if (rns_buffer(ctx, cv.at) != RSDFT_OK) {   // no room: the FP64 kernels
-                ctx->err.clear();
-                return RSDFT_OK;
-            }
-            cv = Carver{(unsigned char *)ctx->rns.buf};
+            if (!rns_buffer(ctx, cv.at, st)) return RSDFT_OK;
+            cv = Carver{(unsigned char *)ctx->rns.buf.p};
         }
         __nv_bfloat16 *res = cv.take<__nv_bfloat16>((size_t)NM * R * 2 * ld);
         short *out16 = cv.take<short>(out_elems);
@@ -998,6 +1030,7 @@ rsdft_status rns_gram(rsdft_ctx *ctx, const RowBlocks &A0, const RowBlocks &B0, 
         a.boxn = NT;
         a.M = M;
         a.N = N;
+        a.npad = npad;
         a.herm = herm ? 1 : 0;
         a.blocks = blocks;
         a.tiles = tiles;
@@ -1020,7 +1053,7 @@ rsdft_status rns_gram(rsdft_ctx *ctx, const RowBlocks &A0, const RowBlocks &B0, 
             else RS_TRY((launch_gemm<false, false>(ctx, mA, mB, mB, a, st)));
         }
         k_crt_gram<<<dim3(cdiv((long long)na * nb, 128), blocks), 128, 0, st>>>(
-            out16, splits, M, N, blocks, real ? 1 : 0, A0.cnt[0], A0.cnt[1], B0.cnt[0], B0.cnt[1], na, nb, herm ? 1 : 0,
+            out16, splits, M, N, npad, blocks, real ? 1 : 0, A0.cnt[0], A0.cnt[1], B0.cnt[0], B0.cnt[1], na, nb, herm ? 1 : 0,
             scl, scl + 2 * rowB, scale, g0, g1, ldg, flag);
         count_launch(ctx);
         RS_LAUNCHED(ctx, "k_crt_gram");
@@ -1028,13 +1061,21 @@ rsdft_status rns_gram(rsdft_ctx *ctx, const RowBlocks &A0, const RowBlocks &B0, 
     return RSDFT_OK;
 }
 
-rsdft_status rns_rotate(rsdft_ctx *ctx, const RowBlocks &Y0, const double2 *c, int ldc, int m, bool real,
-                        const double2 *base, int sign, double2 *out0, double2 *out1, cudaStream_t st, bool *used) {
+rsdft_status rns_gram(rsdft_ctx *ctx, const RowBlocks &A, const RowBlocks &B0, const RowBlocks *B1, bool real, bool herm,
+                      double2 *g0, double2 *g1, int ldg, double scale, cudaStream_t st, bool *used) {
     *used = false;
+    if (!gram_wins(ctx->n)) return RSDFT_OK;
+    for (size_t limit = RNS_BYTES; limit >= RNS_BYTES / 8 && !*used; limit /= 8)
+        RS_TRY(gram_within(ctx, limit, A, B0, B1, real, herm, g0, g1, ldg, scale, st, used));
+    return RSDFT_OK;
+}
+
+static rsdft_status rotate_within(rsdft_ctx *ctx, size_t limit, const RowBlocks &Y0, const double2 *c, int ldc, int m,
+                                  bool real, const double2 *base, int sign, double2 *out0, double2 *out1,
+                                  cudaStream_t st, bool *used) {
     const RowBlocks Y = real ? pair_rows(Y0) : Y0;
     const int R = rows_of(Y), k = rows_of(Y0);
     const long long n = ctx->n;
-    if (Y0.cnt[0] <= 0) return RSDFT_OK;
     const int segs = Y0.cnt[1] + Y0.cnt[2] > 0 ? 2 : 1;
     const int PL = real ? 1 : 2, NT = real ? 256 : 128;
     const int nt = cdiv(m, NT), nstep = cdiv(cdiv(m, nt), 16) * 16, nbp = nt * nstep, nquad = cdiv(m, 4);
@@ -1043,30 +1084,24 @@ rsdft_status rns_rotate(rsdft_ctx *ctx, const RowBlocks &Y0, const double2 *c, i
     sg[1] = Seg{{Y0.cnt[1], Y0.cnt[2]}, {Y0.cnt[0], Y0.cnt[0] + Y0.cnt[1]},
                 real ? 2 * (Y.cnt[1] + Y.cnt[2]) : Y.cnt[1] + Y.cnt[2]};
     int kb[2], kpad[2], bits[2];
-    double kpads = 0.0;
     for (int s = 0; s < segs; ++s) {
         kb[s] = cdiv(sg[s].k, 64);
         kpad[s] = kb[s] * 64;
-        kpads += kpad[s];
         // |y_r| over the K products of a sum is at most sqrt(K) max|y|
         int h = 0;
         while ((1LL << (2 * h)) < (long long)sg[s].k * PL) ++h;
         bits[s] = T_ROW - h;
     }
     const double out_bytes = (double)NM * segs * PL * nquad * 4;
-    if (!rns_wins((double)n, R, nbp, kpads, (double)k * m, real, (double)n * out_bytes * 4.0 / 4.0e12)) return RSDFT_OK;
     const size_t per_point = (size_t)NM * R * 4 + (size_t)out_bytes;
-    const long long most = std::max<long long>(4096, (long long)(RNS_BYTES / per_point) / 128 * 128);
+    const long long most = std::max<long long>(4096, (long long)(limit / per_point) / 128 * 128);
     const int nchunk = cdiv(n, most);
     const int ld = cdiv(cdiv(n, nchunk), 128) * 128;
     Carver cv{nullptr};
     for (int pass = 0; pass < 2; ++pass) {
         if (pass == 1) {
-            if (rns_buffer(ctx, cv.at) != RSDFT_OK) {
-                ctx->err.clear();
-                return RSDFT_OK;
-            }
-            cv = Carver{(unsigned char *)ctx->rns.buf};
+            if (!rns_buffer(ctx, cv.at, st)) return RSDFT_OK;
+            cv = Carver{(unsigned char *)ctx->rns.buf.p};
         }
         __nv_bfloat16 *res = cv.take<__nv_bfloat16>((size_t)NM * R * 2 * ld);
         unsigned *out8 = cv.take<unsigned>((size_t)NM * segs * PL * nquad * ld);
@@ -1147,6 +1182,18 @@ rsdft_status rns_rotate(rsdft_ctx *ctx, const RowBlocks &Y0, const double2 *c, i
             RS_LAUNCHED(ctx, "k_crt_rot");
         }
     }
+    return RSDFT_OK;
+}
+
+rsdft_status rns_rotate(rsdft_ctx *ctx, const RowBlocks &Y, const double2 *c, int ldc, int m, bool real,
+                        const double2 *base, int sign, double2 *out0, double2 *out1, cudaStream_t st, bool *used) {
+    *used = false;
+    const int segs = Y.cnt[1] + Y.cnt[2] > 0 ? 2 : 1, nt = cdiv(m, real ? 256 : 128);
+    if (Y.cnt[0] <= 0 ||
+        !rotation_wins((double)ctx->n, rows_of(real ? pair_rows(Y) : Y), rows_of(Y), m, real, NM * segs * nt))
+        return RSDFT_OK;
+    for (size_t limit = RNS_BYTES; limit >= RNS_BYTES / 8 && !*used; limit /= 8)
+        RS_TRY(rotate_within(ctx, limit, Y, c, ldc, m, real, base, sign, out0, out1, st, used));
     return RSDFT_OK;
 }
 

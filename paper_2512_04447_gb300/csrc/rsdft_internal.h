@@ -130,6 +130,14 @@ struct NnState {
     float *tr = nullptr;   size_t tr_cap = 0;      // training activations and gradients
 };
 
+// Scratch of a context that grows to the largest call.  A captured graph may be replayed at any time
+// before the context ends, so a buffer that a capture has seen is never freed earlier.
+struct Scratch {
+    void *p = nullptr;
+    size_t bytes = 0;
+    bool captured = false;
+};
+
 // Tables and block exponents of the fixed-point FP64 transforms (fft_fix.cu).
 struct FixFft {
     const void *tw[3] = {};                  // [N] exp(-2 pi i k / N) as fix::W4
@@ -137,15 +145,13 @@ struct FixFft {
     int kexp = 0;
     const double *g2abs[3] = {};             // G_a^2 by |frequency index|
     const unsigned char *fabs[3] = {};       // |frequency index| by position
-    void *meta = nullptr;                    // exponents of the planes and slabs in flight
-    int cap_band = 0;
+    Scratch meta;                            // exponents of the planes and slabs in flight
 };
 
 // Residue-arithmetic products (rns.cu): residue planes and scratch, and the device flag
 // that hands a call back to the FP64 kernels.
 struct RnsWork {
-    void *buf = nullptr;
-    size_t bytes = 0;
+    Scratch buf, fbuf;
     int *flag = nullptr;
 };
 
@@ -173,8 +179,7 @@ struct rsdft_ctx {
     float *v32 = nullptr;            // [n] FP32 copy of v for the mixed form
     rsdft::ProjTables pt{};
     rsdft::Discs discs{};
-    void *discbuf = nullptr;         // [2][bands][ndisc][3]: partial sums, scatter coefficients
-    int disc_cap = 0;                // bands it holds
+    rsdft::Scratch discbuf;                 // [2][bands][ndisc][3]: partial sums, scatter coefficients
     long long nent = 0;
     rsdft::Workspace ws;
     rsdft::ScfWork scf;
@@ -213,6 +218,7 @@ rsdft_status cuda_check(rsdft_ctx *ctx, cudaError_t e, const char *what);
     } while (0)
 
 rsdft_status dev_alloc(rsdft_ctx *ctx, void **p, size_t bytes);
+rsdft_status grow(rsdft_ctx *ctx, Scratch &s, size_t bytes, cudaStream_t st);
 
 // Brackets the launches of one hot kernel with CUDA events when profiling is
 // on; always counts the launches.
@@ -254,7 +260,7 @@ rsdft_status fft_xy_inverse(rsdft_ctx *ctx, const double2 *buf, const double2 *p
                             cudaStream_t st);
 // Partial-sum and coefficient buffers of nb bands, and the sums of part joined per atom: p (or null)
 // the projections, ab (or null) the scatter coefficients E <beta|psi> of every disc.
-rsdft_status disc_buffers(rsdft_ctx *ctx, int nb, double2 **part, double2 **ab);
+rsdft_status disc_buffers(rsdft_ctx *ctx, int nb, double2 **part, double2 **ab, cudaStream_t st);
 rsdft_status disc_finish(rsdft_ctx *ctx, const double2 *part, int nb, double2 *p, double2 *ab, cudaStream_t st);
 rsdft_status project(rsdft_ctx *ctx, const double2 *psi, double2 *p, int nb, cudaStream_t st);
 rsdft_status apply_h64(rsdft_ctx *ctx, const double2 *psi, double2 *hpsi, int nb,

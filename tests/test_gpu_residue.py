@@ -76,6 +76,23 @@ def test_rotation_at_the_edges(N, k, m, base, real):
     ctx.close()
 
 
+@pytest.mark.parametrize("real", [False, True])
+@pytest.mark.parametrize("N,na,nb", [((9, 2, 10), 3, 5), ((5, 5, 8), 3, 5), ((6, 6, 6), 1, 16), ((8, 10, 6), 17, 9),
+                                     ((30, 20, 15), 1, 8)])
+def test_gram_of_few_points_and_rows(N, na, nb, real):
+    ctx = _ctx(N)   # 180 points: the FP64 kernels; from 200 on the residue passes
+    a, b = _draw(7, na, ctx.n, real), _draw(8, nb, ctx.n, real)
+    g = torch.empty((na, nb), dtype=torch.float64 if real else torch.complex128, device="cuda")
+    (ctx.gram_real if real else ctx.gram)(dev(a), dev(b), g)
+    ref = a.conj() @ b.T * ctx.dV
+    assert np.all(np.abs(host(g) - ref) <= TOL * _norm(a, 1)[:, None] * _norm(b, 1)[None] * ctx.dV)
+    y, c = _draw(9, nb + 32, ctx.n, real), _draw(10, nb + 32, na, real)
+    out = torch.empty((na, ctx.n), dtype=g.dtype, device="cuda")
+    (ctx.rotate_real if real else ctx.rotate)(dev(y), dev(c), out)
+    assert np.all(np.abs(host(out) - c.T @ y) <= TOL * _norm(c, 0)[:, None] * _norm(y, 0)[None])
+    ctx.close()
+
+
 @pytest.mark.parametrize("bad", [np.inf, np.nan, 1e200, 1e-200])
 def test_inputs_that_the_fp64_kernels_take(bad):
     ctx = _ctx((30, 30, 30))
