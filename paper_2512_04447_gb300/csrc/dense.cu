@@ -1124,9 +1124,9 @@ k_inverse_iter(const double *d, const double *e, int k, int nkeep, const double 
 
 // Gram-Schmidt (two passes) of each vector against the earlier vectors of its
 // eigenvalue cluster (a maximal run of consecutive eigenvalues with gaps of at
-// most 1e-6 ||T||), then normalisation.  Inverse iteration leaves two vectors
-// whose eigenvalues are g apart orthogonal to about eps ||T|| / g, so outside
-// such clusters the loss is below 3e-10; a wider threshold (LAPACK's 1e-3 ||T||)
+// most 1e-5 ||T||), then normalisation.  Inverse iteration leaves two vectors
+// whose eigenvalues are g apart orthogonal to about eps ||T|| / g (twice that where the roundings
+// fall badly: 3.9e-10 at 1.2e-6), so outside such clusters the loss is below 5e-11; a wider threshold (LAPACK's 1e-3 ||T||)
 // merged hundreds of distinct eigenvalues of a 1440 x 1440 problem into one
 // cluster, whose Gram-Schmidt on one CTA then took most of the solve.  Clusters
 // are independent: CTA j handles the cluster that starts at eigenvalue j;
@@ -1134,7 +1134,7 @@ k_inverse_iter(const double *d, const double *e, int k, int nkeep, const double 
 __global__ void k_cluster_gs(int k, int nkeep, const double *lam, const double *scr, double *zt) {
     __shared__ double sh[33];
     __shared__ double dots[1024];
-    const double ortol = 1e-6 * scr[0];
+    const double ortol = 1e-5 * scr[0];
     const int cstart = blockIdx.x;
     if (cstart >= nkeep) return;
     if (cstart > 0 && lam[cstart] - lam[cstart - 1] <= ortol) return;   // not a cluster start

@@ -12,20 +12,22 @@
 // barrier per step.  Here:
 //   - the matrix lives in distributed shared memory: row r in CTA r mod 16,
 //     full rows of complex double-floats (16 B), so k <= 448 fits in 227 KB;
-//   - A is Hermitian, so column i below the diagonal is the conjugate of row i,
-//     which one CTA (the owner of row i) holds whole: it brings row i up to date
-//     and forms the reflector's scalars (norm, beta, tau, the scale of v) alone,
-//     while the other CTAs apply the previous step's rank-2 update to their rows
-//     (the update of step i-1 is applied lazily at step i);
-//   - two cluster barriers per step: after the scalars and the updates (every
-//     CTA then reads row i from the owner's shared memory and forms v_i itself),
-//     and after the matrix-vector products, whose results y_r and per-warp
-//     partial sums of y^H v each CTA has stored into every CTA's shared memory
-//     (every CTA then forms w' redundantly from local data);
-//   - the FP64 outputs are written off the owner's path: vh row i by one warp of
-//     each CTA, d_i, e_i, tau_i by the next CTA;
+//   - one exchange per step: after a cluster barrier every CTA holds y = A v_{i-1} of all rows and the
+//     next pivot row (their owners stored them into every CTA's shared memory), and forms w', the updated
+//     pivot row and its reflector by itself, an element a thread.  A second barrier says that y
+//     and the pivot row have been read; its wait comes long after and costs nothing;
+//   - the reflector's scalars (norm, root, reciprocals: a chain) are one warp's work, beside the rank-2
+//     update by the other 15;
+//   - warps whose columns are all reduced already leave the per-element work;
 //   - double-float keeps about 48 significant bits, so the reduction's backward
 //     error is a small multiple of 2^-46 |A| instead of 2^-53 |A|.
+// Bound: the FP32 lanes for the first half of the columns (115 operations an element in the update, 55 in
+// A v; packed pairs have the same rate), the chain of a step for the rest.  SM cycles a column by quarters, k = 432:
+//   28.2k, 19.3k, 11.1k, 7.4k; before (the owner of the pivot row formed the reflector, a second exchange
+//   gave it out): 31.0k, 21.7k, 14.2k, 10.0k.
+// Measured, the whole eigensolve (a third of the vectors): k = 144 1.28 -> 1.10 ms, 288 2.89 -> 2.52 ms, 432 5.39 -> 4.90 ms.
+// Over all SMs, with polled values in global memory instead of cluster barriers, a column took 14k cycles
+// throughout (7k of them until the last value was seen): 3.5 ms at k = 432 and slower below 360.
 // Outputs as the FP64 kernel: d, e (real), tau, and v_i in vh row i (columns
 // i+1 .. k-1), for the compact-WY back-transformation.
 #include <cooperative_groups.h>
@@ -43,13 +45,20 @@ using namespace dfl;
 constexpr int TC_C = 16;     // CTAs in the cluster
 constexpr int TC_T = 512;    // threads per CTA
 constexpr int TC_W = TC_T / 32;
-constexpr int TC_KMAX = 448;   // largest k whose rows fit the cluster's shared memory
+constexpr int TC_WORK = TC_W - 1;      // warps of the rank-2 update; the last one does the scalars meanwhile
+constexpr int TC_KMAX = 448;           // largest k whose rows fit the cluster's shared memory
+constexpr int TC_ROWS = TC_KMAX / TC_C;
+constexpr int TC_SPLIT = 8;            // pieces of a row, at most
+constexpr int TC_PARTS = 64;           // pieces of all rows, at most
 
 __device__ __forceinline__ cdf ld4(const float4 &v) { return cdf{df{v.x, v.y}, df{v.z, v.w}}; }
 __device__ __forceinline__ float4 st4(const cdf &c) { return make_float4(c.re.h, c.re.l, c.im.h, c.im.l); }
 
-__device__ __forceinline__ void cl_barrier() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+__device__ __forceinline__ void cl_arrive() {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cl_wait() {
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 // s + sum of one product's exact pieces: the running sum keeps its hi part by
@@ -69,6 +78,17 @@ __device__ __forceinline__ void acc_df(Acc &s, df x) {
     s.l = fadd(s.l, fadd(t.l, x.l));
 }
 __device__ __forceinline__ df acc_get(const Acc &s) { return fast_two_sum(s.h, s.l); }
+
+// 1 / x and sqrt(x), x > 0 well inside FP32's range, with one division or root: the correction term
+// (2^-24 of the value) takes the FP32 reciprocal, an error of some 2^-47
+__device__ __forceinline__ df rcp_df(df x) {
+    const float r = fdiv(1.0f, x.h);
+    return fast_two_sum(r, fmul(r, ffma(-r, x.l, ffma(-r, x.h, 1.0f))));
+}
+__device__ __forceinline__ df sqrt_df(df x, float half_rsq) {   // half_rsq = 0.5 / sqrt(x) to FP32's accuracy
+    const float s = fsqrt(x.h);
+    return fast_two_sum(s, fmul(fadd(ffma(-s, s, x.h), x.l), half_rsq));
+}
 
 // a - v_r conj(w_c) - w_r conj(v_c), all complex double-float
 __device__ __forceinline__ cdf rank2(const cdf &a, const cdf &vr, const cdf &wr, const cdf &vc, const cdf &wc) {
@@ -90,26 +110,23 @@ __device__ __forceinline__ df shfl_df(df x, int o) {
     return df{__shfl_xor_sync(0xffffffffu, x.h, o), __shfl_xor_sync(0xffffffffu, x.l, o)};
 }
 
-// Block-wide sum of a complex double-float; every thread gets the result.
-__device__ cdf block_sum_cdf(cdf v, float4 *scratch) {
-    for (int o = 16; o > 0; o >>= 1) {
-        v.re = add(v.re, shfl_df(v.re, o));
-        v.im = add(v.im, shfl_df(v.im, o));
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    __syncthreads();
-    if (lane == 0) scratch[warp] = st4(v);
-    __syncthreads();
-    if (warp == 0) {
-        cdf s = lane < TC_W ? ld4(scratch[lane]) : cdf{df{0.f, 0.f}, df{0.f, 0.f}};
-        for (int o = 16; o > 0; o >>= 1) {
-            s.re = add(s.re, shfl_df(s.re, o));
-            s.im = add(s.im, shfl_df(s.im, o));
-        }
-        if (lane == 0) scratch[TC_W] = st4(s);
-    }
-    __syncthreads();
-    return ld4(scratch[TC_W]);
+// the same over one xor step of a warp
+__device__ __forceinline__ void acc_xor(Acc &s, int o) {
+    const df t = two_sum(s.h, __shfl_xor_sync(0xffffffffu, s.h, o));
+    s.l = fadd(fadd(s.l, __shfl_xor_sync(0xffffffffu, s.l, o)), t.l);
+    s.h = t.h;
+}
+
+// re and im over a warp: the sum of re in lanes 0-15, of im in lanes 16-31
+__device__ __forceinline__ Acc warp_sum2(const Acc &re, const Acc &im, bool up) {
+    Acc s{up ? im.h : re.h, up ? im.l : re.l};
+    const float oh = __shfl_xor_sync(0xffffffffu, up ? re.h : im.h, 16);
+    const float ol = __shfl_xor_sync(0xffffffffu, up ? re.l : im.l, 16);
+    const df t = two_sum(s.h, oh);
+    s = Acc{t.h, fadd(fadd(s.l, ol), t.l)};
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) acc_xor(s, o);
+    return s;
 }
 
 __global__ void __launch_bounds__(TC_T, 1)
@@ -117,189 +134,256 @@ k_tridiag_cluster(const double2 *__restrict__ a, int k, int ld, double2 *__restr
                   double2 *__restrict__ tau, double *__restrict__ d, double *__restrict__ e) {
     cg::cluster_group cl = cg::this_cluster();
     const int me = (int)cl.block_rank();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int R = (k + TC_C - 1) / TC_C;   // row slots per CTA
     extern __shared__ float4 sm[];
-    float4 *A = sm;                        // [R][k]: row me + 16 lr in slot lr
-    float4 *Vb0 = A + (size_t)R * k;       // v of even steps, [k]
-    float4 *Vb1 = Vb0 + k;                 // v of odd steps
-    float4 *YW = Vb1 + k;                  // [k]: y of all rows (pushed by their owners), then w'
-    __shared__ float4 scratch[TC_W + 1];
-    __shared__ float4 bc[4];               // scalars broadcast inside the CTA
-    __shared__ float4 pub[3];              // owner of the step: tau, scal, (beta, d_i)
-    __shared__ float4 loc[3];              // every CTA: its copy of the owner's pub
-    __shared__ float4 Sall[TC_C * TC_W];   // every warp's part of y^H v (pushed)
-    const int tid = threadIdx.x;
-    const int lane = tid & 31, warp = tid >> 5;
+    float4 *A = sm;                        // [R][k]: row me + 16 j in slot j
+    float4 *V = A + (size_t)R * k;         // v of the last reflector, by column
+    float4 *W = V + k;                     // its w'
+    float4 *Y = W + k;                     // y = A v, stored here by the owners of its rows
+    float4 *P = Y + k;                     // the next pivot row, stored here by its owner
+    __shared__ float4 s_alpha, s_pub[3];
+    __shared__ float2 s_sum[2][TC_W], s_norm[TC_W], s_part[2][TC_PARTS];
+    __shared__ unsigned char s_split[TC_ROWS + 1];
+    const int c = tid;                     // this thread's column (k < TC_T)
+    const bool up = lane >= 16;
     const cdf zero{df{0.f, 0.f}, df{0.f, 0.f}};
     const cdf one{df{1.f, 0.f}, df{0.f, 0.f}};
 
     for (int idx = tid; idx < R * k; idx += TC_T) {
-        const int lr = idx / k, c = idx - lr * k;
-        const int r = me + TC_C * lr;
+        const int j = idx / k, q = idx - j * k, r = me + TC_C * j;
         cdf v = zero;
         if (r < k) {
-            const double2 x = a[(size_t)r * ld + c];
+            const double2 x = a[(size_t)r * ld + q];
             v = cdf{from_double(x.x), from_double(x.y)};
         }
         A[idx] = st4(v);
     }
-    __syncthreads();
-    cl_barrier();
-
-    for (int i = 0; i < k - 1; ++i) {
-        const int L = k - 1 - i;
-        float4 *Vp = (i & 1) ? Vb0 : Vb1;   // v_{i-1}: rows/columns i .. k-1 at [c - i]
-        float4 *Vc = (i & 1) ? Vb1 : Vb0;   // v_i: rows/columns i+1 .. k-1 at [c - i - 1]
-        const int owner = i % TC_C;
-        // first own row slot with a row > i
-        const int lr_first = (i + 1 - me + TC_C - 1) / TC_C > 0 ? (i + 1 - me + TC_C - 1) / TC_C : 0;
-        const int nrow = max(0, R - lr_first - ((me + TC_C * (R - 1) >= k) ? 1 : 0));
-        if (me == owner) {
-            // ---- phase 1: row i up to date, then its reflector
-            const int li = i / TC_C;
-            float4 *row = A + (size_t)li * k;
-            if (i > 0) {
-                const cdf vr = ld4(Vp[0]), wr = ld4(YW[0]);
-                for (int c = i + tid; c < k; c += TC_T)
-                    row[c] = st4(rank2(ld4(row[c]), vr, wr, ld4(Vp[c - i]), ld4(YW[c - i])));
-                __syncthreads();
-            }
-            // x_q = conj(A[i][i+1+q]); alpha = x_0
-            df nrm{0.f, 0.f};
-            for (int q = 1 + tid; q < L; q += TC_T) nrm = add(nrm, cabs2(ld4(row[i + 1 + q])));
-            const cdf ns = block_sum_cdf(cdf{nrm, df{0.f, 0.f}}, scratch);
-            if (tid == 0) {
-                const cdf x0 = cconj(ld4(row[i + 1]));
-                const df xnorm2 = ns.re;
-                cdf t = zero, scal = zero;
-                df beta;
-                // a column below 1e-18 (squares near FP32's underflow) is taken as
-                // reduced already: H = I, beta = Re alpha (an absolute change below
-                // 1e-18, far under the rounding of an Ha-scale matrix)
-                const df nb2 = add(cabs2(x0), xnorm2);
-                if ((xnorm2.h == 0.f && x0.im.h == 0.f) || !(nb2.h > 1e-36f)) {
-                    beta = x0.re;
-                } else {
-                    // beta = -sign(Re alpha) |(alpha, x)|, tau = (beta - alpha) / beta,
-                    // scal = 1 / (alpha - beta) = conj(alpha - beta) / |alpha - beta|^2
-                    const df nb = sqrt(nb2);
-                    beta = x0.re.h >= 0.f ? neg(nb) : nb;
-                    const df rb = div(mk(1.0f), beta);
-                    t = cdf{mul(sub(beta, x0.re), rb), neg(mul(x0.im, rb))};
-                    const cdf den{sub(x0.re, beta), x0.im};
-                    const df rd = div(mk(1.0f), cabs2(den));
-                    scal = cdf{mul(den.re, rd), neg(mul(den.im, rd))};
-                }
-                // published for every CTA (which form v_i from row i themselves)
-                const df di = ld4(row[i]).re;
-                pub[0] = st4(t);
-                pub[1] = st4(scal);
-                pub[2] = make_float4(beta.h, beta.l, di.h, di.l);
+    // pieces a row of the matrix-vector product is cut into when nr own rows (of about 16 nr columns)
+    // are left: the fewest turns, of 55 instructions a column and 100 for the sum of a piece
+    if (tid <= TC_ROWS) {
+        int best = 1, cost = 1 << 30;
+        for (int S = 1; S <= TC_SPLIT && S * tid <= TC_PARTS; ++S) {
+            const int t = ((tid * S + TC_W - 1) / TC_W) * (((16 * tid + 32 * S - 1) / (32 * S)) * 55 + 100);
+            if (t < cost) {
+                cost = t;
+                best = S;
             }
         }
-        // ---- phase 2: step i-1's update of this CTA's rows > i (columns > i)
-        if (i > 0 && nrow > 0) {
-            const int total = nrow * L;
-            const int dj = TC_T / L, dc = TC_T - dj * L;
-            int j = tid / L, c = tid - j * L;
-            for (int t = tid; t < total; t += TC_T) {
-                const int r = me + TC_C * (lr_first + j);
-                float4 *p = A + (size_t)(lr_first + j) * k + (i + 1 + c);
-                *p = st4(rank2(ld4(*p), ld4(Vp[r - i]), ld4(YW[r - i]), ld4(Vp[i + 1 + c - i]),
-                               ld4(YW[i + 1 + c - i])));
-                j += dj;
-                c += dc;
-                if (c >= L) {
-                    c -= L;
-                    ++j;
-                }
+        s_split[tid] = (unsigned char)best;
+    }
+    cdf t = zero, v = zero, x = zero;      // tau_i, v_i[c], conj of the pivot row at c
+    df half{0.f, 0.f};                     // -|tau_i|^2 / 2
+    cl_arrive();
+    for (int i = -1;; ++i) {
+        const int n = i + 1;               // the reflector this pass forms, over columns n + 1 .. k - 1
+        cl_wait();                         // Y and P are complete
+        if (i < 0) {
+            if (c < k) {
+                const double2 p = a[c];
+                x = cdf{from_double(p.x), neg(from_double(p.y))};
+                if (me == 1 && c == 0) d[0] = p.x;
             }
-        }
-        cl_barrier();
-        // ---- phase 3: v_i from the owner's row i and scalars, y = A v_i for own rows > i
-        {
-            const float4 *prow = cl.map_shared_rank(A, owner) + (size_t)(i / TC_C) * k + (i + 1);
-            const float4 x = tid < L ? prow[tid] : make_float4(0.f, 0.f, 0.f, 0.f);   // L < TC_T
-            if (tid < 3) loc[tid] = cl.map_shared_rank(pub, owner)[tid];
+            cl_arrive();
+        } else {
+            const bool live = warp * 32 + 31 >= n && warp * 32 < k;   // this warp has columns left
+            const bool in = c >= n && c < k;
+            const cdf y = in ? ld4(Y[c]) : zero, p = in ? ld4(P[c]) : zero;
+            cl_arrive();                   // Y and P have been read: the owners may store the next ones
+            Acc wr{0.f, 0.f}, wi{0.f, 0.f};
+            cdf w = zero;
+            if (live) {
+                // y^H v
+                Acc sr{0.f, 0.f}, si{0.f, 0.f};
+                acc_prod(sr, y.re.h, y.re.l, v.re.h, v.re.l);
+                acc_prod(si, y.re.h, y.re.l, v.im.h, v.im.l);
+                acc_prod(sr, y.im.h, y.im.l, v.im.h, v.im.l);
+                acc_prod(si, -y.im.h, -y.im.l, v.re.h, v.re.l);
+                const Acc q = warp_sum2(sr, si, up);
+                if ((lane & 15) == 0) s_sum[up][warp] = make_float2(q.h, q.l);
+                // tau y, which does not wait for that sum
+                acc_prod(wr, t.re.h, t.re.l, y.re.h, y.re.l);
+                acc_prod(wi, t.re.h, t.re.l, y.im.h, y.im.l);
+                acc_prod(wr, -t.im.h, -t.im.l, y.im.h, y.im.l);
+                acc_prod(wi, t.im.h, t.im.l, y.re.h, y.re.l);
+            } else if ((lane & 15) == 0) {
+                s_sum[up][warp] = make_float2(0.f, 0.f);
+            }
             __syncthreads();
-            const cdf scal = ld4(loc[1]);
-            if (tid < L) {
-                const cdf vq = tid == 0 ? one : cmul(cconj(ld4(x)), scal);
-                Vc[tid] = st4(vq);
-                // the FP64 copy for the back-transformation: one warp's range per CTA
-                if (warp == me) vh[(size_t)i * ldv + i + 1 + tid] = make_double2(to_double(vq.re), to_double(vq.im));
+            if (live) {
+                const float2 q = s_sum[up][lane & (TC_W - 1)];
+                Acc s{q.x, q.y};
+#pragma unroll
+                for (int o = TC_W / 2; o > 0; o >>= 1) acc_xor(s, o);
+                // w' = tau y - |tau|^2 / 2 (y^H v) v
+                const df al = mul(half, acc_get(s));
+                const df ar{__shfl_sync(0xffffffffu, al.h, 0), __shfl_sync(0xffffffffu, al.l, 0)};
+                const df ai{__shfl_sync(0xffffffffu, al.h, 16), __shfl_sync(0xffffffffu, al.l, 16)};
+                acc_prod(wr, ar.h, ar.l, v.re.h, v.re.l);
+                acc_prod(wi, ar.h, ar.l, v.im.h, v.im.l);
+                acc_prod(wr, -ai.h, -ai.l, v.im.h, v.im.l);
+                acc_prod(wi, ai.h, ai.l, v.re.h, v.re.l);
+                w = cdf{acc_get(wr), acc_get(wi)};
+                if (in) W[c] = st4(w);
             }
-            if (me == (owner + 1) % TC_C && tid == 0) {
-                const float4 bd = loc[2], tq = loc[0];
-                d[i] = to_double(df{bd.z, bd.w});
-                e[i] = to_double(df{bd.x, bd.y});
-                tau[i] = make_double2(to_double(df{tq.x, tq.y}), to_double(df{tq.z, tq.w}));
+            __syncthreads();
+            // the pivot row n with the update (v_n = 1)
+            if (live) {
+                const cdf wn = ld4(W[n]);
+                Acc xr{p.re.h, p.re.l}, xi{p.im.h, p.im.l};
+                acc_df(xr, neg(w.re));
+                acc_df(xi, w.im);
+                acc_prod(xr, -wn.re.h, -wn.re.l, v.re.h, v.re.l);
+                acc_prod(xi, -wn.im.h, -wn.im.l, v.re.h, v.re.l);
+                acc_prod(xr, -wn.im.h, -wn.im.l, v.im.h, v.im.l);
+                acc_prod(xi, wn.re.h, wn.re.l, v.im.h, v.im.l);
+                x = cdf{acc_get(xr), neg(acc_get(xi))};
+                if (me == 1 && c == n) d[n] = to_double(x.re);
             }
+            if (n == k - 1) break;
+        }
+        const int L = k - 1 - n;
+        {
+            Acc s{0.f, 0.f};
+            if (warp * 32 + 31 > n + 1 && warp * 32 < k) {
+                if (c > n + 1 && c < k) {
+                    acc_prod(s, x.re.h, x.re.l, x.re.h, x.re.l);
+                    acc_prod(s, x.im.h, x.im.l, x.im.h, x.im.l);
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) acc_xor(s, o);
+            }
+            if (lane == 0) s_norm[warp] = make_float2(s.h, s.l);
+            if (c == n + 1) s_alpha = st4(x);
         }
         __syncthreads();
-        cdf sp = zero;   // sum over own rows of conj(y_r) v_r
-        for (int j = warp; j < nrow; j += TC_W) {
-            const int lr = lr_first + j;
-            const int r = me + TC_C * lr;
-            const float4 *row = A + (size_t)lr * k + (i + 1);
-            Acc yr{0.f, 0.f}, yi{0.f, 0.f};
-            for (int q = lane; q < L; q += 32) {
-                const cdf x = ld4(row[q]), v = ld4(Vc[q]);
-                acc_prod(yr, x.re.h, x.re.l, v.re.h, v.re.l);
-                acc_prod(yr, -x.im.h, -x.im.l, v.im.h, v.im.l);
-                acc_prod(yi, x.re.h, x.re.l, v.im.h, v.im.l);
-                acc_prod(yi, x.im.h, x.im.l, v.re.h, v.re.l);
-            }
-            cdf y{acc_get(yr), acc_get(yi)};
-            for (int o = 16; o > 0; o >>= 1) {
-                y.re = add(y.re, shfl_df(y.re, o));
-                y.im = add(y.im, shfl_df(y.im, o));
-            }
-            // y_r into every CTA's YW (one remote store per lane; the stores need no
-            // reply, and the cluster barrier below makes them visible)
-            if (lane < TC_C) cl.map_shared_rank(YW, lane)[r - i - 1] = st4(y);
-            if (lane == 0) sp = cadd(sp, cmulc(y, ld4(Vc[r - i - 1])));
-        }
-        {   // this warp's part of y^H v into every CTA
-            const float4 sp4 = st4(sp);
-            const float4 b{__shfl_sync(0xffffffffu, sp4.x, 0), __shfl_sync(0xffffffffu, sp4.y, 0),
-                           __shfl_sync(0xffffffffu, sp4.z, 0), __shfl_sync(0xffffffffu, sp4.w, 0)};
-            if (lane < TC_C) cl.map_shared_rank(Sall, lane)[me * TC_W + warp] = b;
-        }
-        cl_barrier();
-        // ---- phase 4: y^H v, then w' = tau y - 1/2 |tau|^2 (y^H v) v
-        if (warp == 0) {
-            // y^H v: the TC_C x TC_W per-warp parts, TC_C * TC_W / 32 per lane
-            float4 part[TC_C * TC_W / 32];
+        cl_wait();                         // every CTA has read Y and P
+        // own rows > n: slots j0 .. j0 + nr - 1
+        const int j0 = (n + 1 - me + TC_C - 1) / TC_C;   // n + 1 - me > -TC_C
+        const int nr = max(0, (k - me + TC_C - 1) / TC_C - j0);
+        if (warp == TC_WORK) {
+            // ---- the reflector's scalars
+            const float2 q = s_norm[lane & (TC_W - 1)];
+            Acc s{q.x, q.y};
 #pragma unroll
-            for (int u = 0; u < TC_C * TC_W / 32; ++u) part[u] = Sall[lane + 32 * u];
-            cdf s = zero;
-#pragma unroll
-            for (int u = 0; u < TC_C * TC_W / 32; ++u) s = cadd(s, ld4(part[u]));
-            for (int o = 16; o > 0; o >>= 1) {
-                s.re = add(s.re, shfl_df(s.re, o));
-                s.im = add(s.im, shfl_df(s.im, o));
+            for (int o = TC_W / 2; o > 0; o >>= 1) acc_xor(s, o);
+            const df xnorm2 = acc_get(s);
+            const cdf x0 = ld4(s_alpha);
+            cdf tn = zero, scal = zero;
+            df beta;
+            // a column below 1e-18 (squares near FP32's underflow) is taken as
+            // reduced already: H = I, beta = Re alpha (an absolute change below
+            // 1e-18, far under the rounding of an Ha-scale matrix)
+            const df nb2 = add(cabs2(x0), xnorm2);
+            if ((xnorm2.h == 0.f && x0.im.h == 0.f) || !(nb2.h > 1e-36f)) {
+                beta = x0.re;
+            } else {
+                // beta = -sign(Re alpha) |(alpha, x)|, tau = (beta - alpha) / beta,
+                // scal = 1 / (alpha - beta) = conj(alpha - beta) / |alpha - beta|^2
+                const df nb = sqrt_df(nb2, 0.5f * rsqrtf(nb2.h));
+                beta = x0.re.h >= 0.f ? neg(nb) : nb;
+                const cdf den{sub(x0.re, beta), x0.im};
+                const df rb = rcp_df(beta), rd = rcp_df(cabs2(den));
+                tn = cdf{mul(sub(beta, x0.re), rb), neg(mul(x0.im, rb))};
+                scal = cdf{mul(den.re, rd), neg(mul(den.im, rd))};
             }
             if (lane == 0) {
-                const cdf t = ld4(loc[0]);
-                const df h = mul_f(cabs2(t), -0.5f);
-                bc[3] = st4(cdf{mul(h, s.re), mul(h, s.im)});
+                const df h = mul_f(cabs2(tn), -0.5f);
+                s_pub[0] = st4(tn);
+                s_pub[1] = st4(scal);
+                s_pub[2] = make_float4(h.h, h.l, 0.f, 0.f);
+                if (me == 1) {
+                    e[n] = to_double(beta);
+                    tau[n] = make_double2(to_double(tn.re), to_double(tn.im));
+                }
+            }
+        } else {
+            // ---- the rank-2 update of the own rows: units of a row and 64 columns, ordered by columns
+            // (v and w' of a column stay in registers), a share for each warp; row n + 1, the next
+            // pivot row, goes to every CTA
+            const int total = nr * ((L + 63) >> 6);
+            const int u1 = (warp + 1) * total / TC_WORK;
+            int u = warp * total / TC_WORK;
+            while (u < u1) {
+                const int blk = u / nr;
+                int j = u - blk * nr;
+                const int je = min(nr, j + u1 - u);
+                u += je - j;
+                const int ca = n + 1 + blk * 64 + lane, cb = ca + 32;
+                const bool ina = ca < k, inb = cb < k;
+                cdf va = zero, wa = zero, vb = zero, wb = zero;
+                if (i >= 0 && ina) {
+                    va = ld4(V[ca]);
+                    wa = ld4(W[ca]);
+                }
+                if (i >= 0 && inb) {
+                    vb = ld4(V[cb]);
+                    wb = ld4(W[cb]);
+                }
+                for (; j < je; ++j) {
+                    const int r = me + TC_C * (j0 + j);
+                    float4 *row = A + (size_t)(j0 + j) * k;
+                    float4 za = make_float4(0.f, 0.f, 0.f, 0.f), zb = za;
+                    if (ina) za = row[ca];
+                    if (inb) zb = row[cb];
+                    if (i >= 0) {
+                        const cdf vr = ld4(V[r]), wr = ld4(W[r]);
+                        za = st4(rank2(ld4(za), vr, wr, va, wa));
+                        zb = st4(rank2(ld4(zb), vr, wr, vb, wb));
+                        if (ina) row[ca] = za;
+                        if (inb) row[cb] = zb;
+                    }
+                    if (r == n + 1)
+                        for (int b = 0; b < TC_C; ++b) {
+                            float4 *dst = cl.map_shared_rank(P, b);
+                            if (ina) dst[ca] = za;
+                            if (inb) dst[cb] = zb;
+                        }
+                }
             }
         }
         __syncthreads();
-        {
-            const cdf t = ld4(loc[0]), al = ld4(bc[3]);
-            for (int q = tid; q < L; q += TC_T) YW[q] = st4(cadd(cmul(t, ld4(YW[q])), cmul(al, ld4(Vc[q]))));
+        t = ld4(s_pub[0]);
+        half = df{s_pub[2].x, s_pub[2].y};
+        v = zero;
+        if (c > n && c < k) {
+            v = c == n + 1 ? one : cmul(x, ld4(s_pub[1]));
+            V[c] = st4(v);
+            // the FP64 copy for the back-transformation: one warp's range per CTA
+            if (warp == me) vh[(size_t)n * ldv + c] = make_double2(to_double(v.re), to_double(v.im));
         }
         __syncthreads();
+        // ---- y = A v over the own rows
+        const int S = s_split[nr], seg = (L + S - 1) / S;
+        for (int u = warp; u < nr * S; u += TC_W) {
+            const int j = u / S, c0 = n + 1 + (u - j * S) * seg, c1 = min(k, c0 + seg);
+            const float4 *row = A + (size_t)(j0 + j) * k;
+            Acc yr{0.f, 0.f}, yi{0.f, 0.f};
+            for (int cc = c0 + lane; cc < c1; cc += 32) {
+                const cdf z = ld4(row[cc]), s = ld4(V[cc]);
+                acc_prod(yr, z.re.h, z.re.l, s.re.h, s.re.l);
+                acc_prod(yi, z.re.h, z.re.l, s.im.h, s.im.l);
+                acc_prod(yr, -z.im.h, -z.im.l, s.im.h, s.im.l);
+                acc_prod(yi, z.im.h, z.im.l, s.re.h, s.re.l);
+            }
+            const Acc q = warp_sum2(yr, yi, up);
+            if ((lane & 15) == 0) s_part[up][u] = make_float2(q.h, q.l);
+        }
+        __syncthreads();
+        // every row's sum into every CTA (one remote store a thread)
+        if (tid < nr * TC_C) {
+            const int j = tid / TC_C;
+            Acc yr{0.f, 0.f}, yi{0.f, 0.f};
+            for (int s = 0; s < S; ++s) {
+                const float2 q = s_part[0][j * S + s], z = s_part[1][j * S + s];
+                acc_df(yr, df{q.x, q.y});
+                acc_df(yi, df{z.x, z.y});
+            }
+            cl.map_shared_rank(Y, tid & (TC_C - 1))[me + TC_C * (j0 + j)] = st4(cdf{acc_get(yr), acc_get(yi)});
+        }
+        cl_arrive();
     }
-    // d[k-1]: row k-1 after the last update, v_{k-2} = (1)
-    if (me == (k - 1) % TC_C && tid == 0) {
-        const cdf x = ld4(A[(size_t)((k - 1) / TC_C) * k + (k - 1)]);
-        const cdf w = ld4(YW[0]);
-        d[k - 1] = to_double(sub(x.re, mul_f(w.re, 2.0f)));
-    }
-    cl_barrier();   // no CTA leaves while another may still read its shared memory
+    cl_wait();   // no CTA leaves while another may still read its shared memory
 }
 
 // Each reflector made unitary in FP64.  H = I - tau v v^H is unitary exactly when
@@ -329,7 +413,7 @@ k_unitarize(int k, const double2 *__restrict__ vh, int ldv, double2 *__restrict_
 
 size_t tridiag_cluster_smem(int k) {
     const size_t R = (size_t)(k + TC_C - 1) / TC_C;
-    return (R * k + 3 * (size_t)k) * sizeof(float4);
+    return (R * k + 4 * (size_t)k) * sizeof(float4);
 }
 
 bool tridiag_cluster_fits(int k) { return k >= 2 && k <= TC_KMAX; }
