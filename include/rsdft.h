@@ -470,7 +470,7 @@ rsdft_status rsdft_propagate(rsdft_ctx *ctx, void *psi_dev, int nband, double dt
  * events.  Enabling resets the counters.
  */
 typedef enum {
-    RSDFT_K_GRAM = 0,        /* Gram partial tiles (split-K)                    */
+    RSDFT_K_GRAM = 0,        /* Gram (FP64 residue products, or split-K tiles)  */
     RSDFT_K_ROTATE = 1,      /* Ritz rotation / block update                    */
     RSDFT_K_FFT_XY_FWD = 2,  /* xy-plane forward FFT pass                       */
     RSDFT_K_FFT_Z = 3,       /* z pass: forward, per-G factor, inverse          */
@@ -505,7 +505,8 @@ long long rsdft_launch_count(const rsdft_ctx *ctx);
  * CUDA events on the call's stream (the call synchronises), and later calls of
  * that shape on this context use the fastest.  Candidates differ only in the
  * summation order, so results agree to rounding.  on = 0 switches it off and
- * forgets the choices. */
+ * forgets the choices.  FP64 Grams and rotations that run as residue products
+ * on the tensor cores have no candidates. */
 rsdft_status rsdft_set_autotune(rsdft_ctx *ctx, int on);
 
 /* ---------------------------------------------------------------------------
