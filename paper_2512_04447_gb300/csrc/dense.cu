@@ -64,7 +64,9 @@ __device__ double block_sum(double v, double *sh) {
     __syncthreads();
     if (warp == 0) {
         double s = lane < nw ? sh[lane] : 0.0;
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            if (o < nw) s += __shfl_down_sync(0xffffffffu, s, o);   // lanes nw and up hold 0
         if (lane == 0) sh[32] = s;
     }
     __syncthreads();
@@ -687,10 +689,12 @@ __device__ double2 block_sum_c(double2 v, double2 *sh2) {
     if (warp == 0) {
         const int nw = blockDim.x >> 5;
         double2 s = lane < nw ? sh2[lane] : make_double2(0.0, 0.0);
-        for (int o = 16; o > 0; o >>= 1) {
-            s.x += __shfl_down_sync(0xffffffffu, s.x, o);
-            s.y += __shfl_down_sync(0xffffffffu, s.y, o);
-        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            if (o < nw) {   // lanes nw and up hold 0
+                s.x += __shfl_down_sync(0xffffffffu, s.x, o);
+                s.y += __shfl_down_sync(0xffffffffu, s.y, o);
+            }
         if (lane == 0) sh2[32] = s;
     }
     __syncthreads();
@@ -1326,7 +1330,10 @@ rsdft_status eigh_lowest(rsdft_ctx *ctx, double2 *a, int k, int nkeep, double *l
         const bool try_coop = !cluster_done && occ > 0 && k <= MAX_K_COOP;
         if (try_coop) coop_lock = std::unique_lock<std::mutex>(coop_mutex());
         if (try_coop) {
-            int nb = std::max(1, std::min(ctx->num_sms * std::min(occ, 1), cdiv((long long)k * k, 1024)));
+            // a CTA for 256 entries of the matrix: the rows of a step then come in pieces and the FP64 chain of
+            // a piece is short; more CTAs make the barrier dearer.  Whole eigensolve with one for 1,024 entries and
+            // for 256: k = 96 1.41 -> 1.33 ms, 144 2.09 -> 1.96, 192 2.80 -> 2.63, 288 4.44 -> 4.28, from 432 the same.
+            int nb = std::max(1, std::min(ctx->num_sms * std::min(occ, 1), cdiv((long long)k * k, 256)));
             GridSync *gs = reinterpret_cast<GridSync *>(w.gsync);
             RS_CUDA(ctx, cudaMemsetAsync(gs, 0, sizeof(GridSync), st));
             long long limit = 4000000000LL;   // ~2 s of SM clock per barrier wait
