@@ -158,16 +158,6 @@ static rsdft_status ensure_gram_part(rsdft_ctx *ctx, size_t elems) {
 
 rsdft_status ensure_gram_partials(rsdft_ctx *ctx, size_t elems) { return ensure_gram_part(ctx, elems); }
 
-rsdft_status gram_reduce(rsdft_ctx *ctx, int nsplit, int na, int nb, bool hermitian, int te, double scale,
-                         double2 *g, int ldg, cudaStream_t st) {
-    const long long tot = (long long)na * nb;
-    k_gram_reduce<<<cdiv(tot, 256), 256, 0, st>>>(ctx->ws.gram_part, nsplit, na, nb, hermitian ? 1 : 0, te, scale,
-                                                   g, ldg, nullptr);
-    count_launch(ctx);
-    RS_LAUNCHED(ctx, "k_gram_reduce");
-    return RSDFT_OK;
-}
-
 // Resident CTAs of a kernel per SM (queried once per instantiation).
 template <typename K> static int occupancy(K kernel, int threads) {
     int occ = 0;

@@ -370,23 +370,6 @@ __global__ void k_mirror_block(double2 *gs, double2 *gh, int k, int m, int nwp) 
     }
 }
 
-// The m x m leading blocks of gs and gh (ld k) made Hermitian: the upper
-// triangle mirrored into the lower one, real diagonal.
-__global__ void k_herm_block(double2 *gs, double2 *gh, int k, int m) {
-    const int i = blockIdx.x * 32 + threadIdx.x;
-    for (int j = blockIdx.y * 32 + threadIdx.y; j < min(m, (int)(blockIdx.y + 1) * 32); j += blockDim.y) {
-        if (i >= m || j > i) continue;
-        if (j == i) {
-            gs[(size_t)i * k + i].y = 0.0;
-            gh[(size_t)i * k + i].y = 0.0;
-            continue;
-        }
-        const double2 a = gs[(size_t)j * k + i], b = gh[(size_t)j * k + i];
-        gs[(size_t)i * k + j] = make_double2(a.x, -a.y);
-        gh[(size_t)i * k + j] = make_double2(b.x, -b.y);
-    }
-}
-
 // out += in, FP32 values added to an FP64 block
 __global__ void k_add_f32(double2 *out, const float2 *__restrict__ in, long long cnt) {
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < cnt;
@@ -714,8 +697,7 @@ static rsdft_status lobpcg_t(rsdft_ctx *ctx, const V *x_in, V *x_out, int m,
 // FP64 refinement of the mixed form with FP32 corrections.  X and HX are FP64:
 // the residuals and their norms, the X-X blocks of G_S and G_H, the blocks that
 // couple X to the corrections, and the X part of the Ritz rotation are formed
-// to FP64 accuracy (the Grams and rotations on the FP32 pipe with error-free
-// products and compensated sums, gemm_df.cu).  The corrections W = TPA(R), HW = H W and the directions P, HP are FP32,
+// in FP64 (Grams and rotations by residue products, rns.cu).  The corrections W = TPA(R), HW = H W and the directions P, HP are FP32,
 // and only the Gram blocks among them run on the FP32 path (split-BF16 tensor
 // cores when tensor_cores >= 1):
 //  - an error e in a coupling block would move the Ritz vectors by O(e / gap)
@@ -738,6 +720,7 @@ static rsdft_status lobpcg_refine(rsdft_ctx *ctx, double2 *x, int m, const rsdft
                                   int maxit, bool carryP, RunState &rs, double *hres, rsdft_lobpcg_stats *stats,
                                   bool *stalled, cudaStream_t st) {
     using B32 = RowBlocksT<float2>;
+    using B64 = RowBlocks;
     Workspace &w = ctx->ws;
     const long long n = ctx->n;
     const double dV = ctx->dV;
@@ -746,11 +729,6 @@ static rsdft_status lobpcg_refine(rsdft_ctx *ctx, double2 *x, int m, const rsdft
     float2 *W = (float2 *)w.W, *HW = (float2 *)w.HW, *P = (float2 *)w.P, *HP = (float2 *)w.HP;
     float2 *Pn = (float2 *)w.Pn, *HPn = (float2 *)w.HPn, *T1 = (float2 *)w.T1;
     float2 *Xs = w.Xs;
-    // lo parts of X and the pairs of HX in the unused halves of the FP64-sized
-    // buffers that hold FP32 rows here (T1: FFT scratch of at most m bands;
-    // Pn, HPn: at most m P columns)
-    const size_t mn = (size_t)m * ctx->n;
-    float2 *Xl = (float2 *)w.T1 + mn, *HXh = (float2 *)w.Pn + mn, *HXl = (float2 *)w.HPn + mn;
     float2 *proj = (float2 *)w.proj;
     int *hact = reinterpret_cast<int *>(w.hbuf + m);
     int *hactp = reinterpret_cast<int *>(w.hbuf + 3 * m);
@@ -812,11 +790,10 @@ static rsdft_status lobpcg_refine(rsdft_ctx *ctx, double2 *x, int m, const rsdft
         if (stats) RS_CUDA(ctx, cudaEventRecord(pe.ev[0], st));
         const dim3 rowgrid(std::min(cdiv(n, 256), 1024), na);
         const dim3 scalegrid(std::max(1, std::min(cdiv(n, 256 * 8), 256)), na);
-        // X and HX as FP32 hi/lo pairs: the hi part of X is its FP32 copy (for the
-        // TPA T_b and the W orthogonalisation); the pairs feed the FP64-accurate
-        // Grams and rotations on the FP32 pipe (gemm_df.cu)
-        RS_TRY(split_df(ctx, X, cntm, Xs, Xl, st));
-        RS_TRY(split_df(ctx, HX, cntm, HXh, HXl, st));
+        // the FP32 copy of X (for the TPA T_b and the W orthogonalisation)
+        k_convert<double2, float2><<<cgrid, 256, 0, st>>>(X, cntm, Xs);
+        count_launch(ctx);
+        RS_LAUNCHED(ctx, "k_convert");
         // R = HX - X Theta of the active bands in FP64 (into Xn, free until the
         // rotation), rounded to FP32 into W
         k_residual_rows<double2><<<rowgrid, 256, 0, st>>>(HX, X, w.theta, w.act, n, Xn);
@@ -885,16 +862,21 @@ static rsdft_status lobpcg_refine(rsdft_ctx *ctx, double2 *x, int m, const rsdft
             // (1e-5 of max |G|) in these blocks, divided by small gaps of the
             // projected problem, slowed the refinement below 1e-8
             RS_TRY(gram_pair<float2>(ctx, Y, HY, w.GS + (size_t)m * k + m, w.GH + (size_t)m * k + m, k, false, st));
-            const B32 none{{nullptr, nullptr, nullptr}, {0, 0, 0}};
-            const B32 bx{{Xs, nullptr, nullptr}, {m, 0, 0}}, bxl{{Xl, nullptr, nullptr}, {m, 0, 0}};
-            const B32 bhx{{HXh, nullptr, nullptr}, {m, 0, 0}}, bhxl{{HXl, nullptr, nullptr}, {m, 0, 0}};
-            RS_TRY(gram_df(ctx, Xs, Xl, m, bx, bxl, w.GS, k, dV, st));
-            RS_TRY(gram_df(ctx, Xs, Xl, m, bhx, bhxl, w.GH, k, dV, st));
-            RS_TRY(gram_df(ctx, Xs, Xl, m, Y, none, w.GS + m, k, dV, st));
-            RS_TRY(gram_df(ctx, HXh, HXl, m, Y, none, w.GH + m, k, dV, st));
-            k_herm_block<<<dim3(cdiv(m, 32), cdiv(m, 32)), dim3(32, 8), 0, st>>>(w.GS, w.GH, k, m);
+            // The FP64 ones by residue products (rns.cu), W and P widened into Xn and HXn, which are free
+            // until the rotation.  In double-float on the FP32 pipe (12 operations a real product) they bound the
+            // refinement: 144 bands on 64^3 to 1e-6, Grams 1,368 -> 221 ms, rotations 381 -> 175 ms, 2.21 -> 0.85 s in all
+            // (10 of 41 iterations refine); 16 bands on 24^3 to 1e-8, 0.44 -> 0.20 s.
+            const B64 bx{{X, nullptr, nullptr}, {m, 0, 0}}, bhx{{HX, nullptr, nullptr}, {m, 0, 0}};
+            const B64 y64{{Xn, HXn, nullptr}, {na, np_, 0}};
+            k_convert<float2, double2><<<cgrid, 256, 0, st>>>(W, (long long)na * n, Xn);
+            if (np_ > 0) k_convert<float2, double2><<<cgrid, 256, 0, st>>>(Pn, (long long)np_ * n, HXn);
+            count_launch(ctx, np_ > 0 ? 2 : 1);
+            RS_LAUNCHED(ctx, "k_convert");
+            RS_TRY(gram_sh(ctx, bx, bhx, w.GS, w.GH, k, dV, st));
+            RS_TRY(gram(ctx, bx, y64, w.GS + m, k, false, dV, st));
+            RS_TRY(gram(ctx, bhx, y64, w.GH + m, k, false, dV, st));
             k_mirror_block<<<dim3(cdiv(m, 32), cdiv(nwp, 32)), dim3(32, 8), 0, st>>>(w.GS, w.GH, k, m, nwp);
-            count_launch(ctx, 2);
+            count_launch(ctx);
             RS_LAUNCHED(ctx, "k_mirror_block");
         }
         if (stats) RS_CUDA(ctx, cudaEventRecord(pe.ev[4], st));
@@ -909,8 +891,9 @@ static rsdft_status lobpcg_refine(rsdft_ctx *ctx, double2 *x, int m, const rsdft
             B32 HYWP{{HW, HPn, nullptr}, {na, np_, 0}};
             RS_TRY(rotate32(ctx, YWP, cwp, m, m, nullptr, 1, P, nullptr, st));
             RS_TRY(rotate32(ctx, HYWP, cwp, m, m, nullptr, 1, HP, nullptr, st));
-            RS_TRY(rotate_df(ctx, Xs, Xl, m, w.Cfull, m, m, Xn, st));
-            RS_TRY(rotate_df(ctx, HXh, HXl, m, w.Cfull, m, m, HXn, st));
+            const B64 bx{{X, nullptr, nullptr}, {m, 0, 0}}, bhx{{HX, nullptr, nullptr}, {m, 0, 0}};
+            RS_TRY(rotate(ctx, bx, w.Cfull, m, m, nullptr, 1, Xn, nullptr, st));
+            RS_TRY(rotate(ctx, bhx, w.Cfull, m, m, nullptr, 1, HXn, nullptr, st));
             k_add_f32<<<cgrid, 256, 0, st>>>(Xn, P, cntm);
             k_add_f32<<<cgrid, 256, 0, st>>>(HXn, HP, cntm);
             count_launch(ctx, 2);

@@ -312,21 +312,8 @@ rsdft_status rns_poison(rsdft_ctx *ctx, double2 *out, long long cnt, cudaStream_
 // partials reduced in FP64; rotation coefficients rounded to FP32.
 rsdft_status gram32(rsdft_ctx *ctx, const RowBlocksT<float2> &A, const RowBlocksT<float2> &B,
                     double2 *g, int ldg, bool hermitian, double scale, cudaStream_t st);
-// Split-K partial buffer of the Gram kernels (grown when needed) and its FP64
-// reduction into g (hermitian: tiles of edge te below the diagonal mirrored).
+// Split-K partial buffer of the Gram kernels (grown when needed).
 rsdft_status ensure_gram_partials(rsdft_ctx *ctx, size_t elems);
-rsdft_status gram_reduce(rsdft_ctx *ctx, int nsplit, int na, int nb, bool hermitian, int te, double scale,
-                         double2 *g, int ldg, cudaStream_t st);
-// FP64-accurate products on the FP32 pipe (gemm_df.cu): FP64 rows held as
-// FP32 hi/lo pairs (split_df), error-free products, TwoSum accumulation.
-rsdft_status split_df(rsdft_ctx *ctx, const double2 *x, long long cnt, float2 *h, float2 *l, cudaStream_t st);
-// g[i][j] = scale * sum_r conj(A_i) B_j, A = (ah, al) [na][n], B = (bh, bl) row
-// blocks (bl all null: B exact in FP32).
-rsdft_status gram_df(rsdft_ctx *ctx, const float2 *ah, const float2 *al, int na, const RowBlocksT<float2> &bh,
-                     const RowBlocksT<float2> &bl, double2 *g, int ldg, double scale, cudaStream_t st);
-// out[b] = sum_{i < k} c[i][b] Y_i, Y = (yh, yl) [k][n], c [k][ldc] FP64, out [m][n] FP64.
-rsdft_status rotate_df(rsdft_ctx *ctx, const float2 *yh, const float2 *yl, int k, const double2 *c, int ldc, int m,
-                       double2 *out, cudaStream_t st);
 rsdft_status rotate32(rsdft_ctx *ctx, const RowBlocksT<float2> &Y, const double2 *c, int ldc, int m,
                       const float2 *base, int sign, float2 *out0, float2 *out1, cudaStream_t st);
 // Tensor-core (split-BF16, tcgen05) Grams of FP32 blocks (gram_tc.cu).
