@@ -371,8 +371,10 @@ k_xy_forward_fix(FixTabs tb, const double2 *__restrict__ src, const double2 *__r
     if (threadIdx.x < 8) red[threadIdx.x] = 0;
     int hmax = 0;
     auto put = [&](int i, double2 v) {
-        const int hx = __double2hiint(v.x), hy = __double2hiint(v.y);
-        hmax = max(hmax, max(hx & 0x7fffffff, hy & 0x7fffffff));
+        // (subnormal values may have nothing but a low word)
+        const int hx = (__double2hiint(v.x) & 0x7fffffff) | (__double2loint(v.x) != 0);
+        const int hy = (__double2hiint(v.y) & 0x7fffffff) | (__double2loint(v.y) != 0);
+        hmax = max(hmax, max(hx, hy));
         s_plane[pidx(i, Nx, RS, nxm)] = I2{__double_as_longlong(v.x), __double_as_longlong(v.y)};
     };
     const bool gather = SRC == Src::Plain && part;
@@ -392,7 +394,7 @@ k_xy_forward_fix(FixTabs tb, const double2 *__restrict__ src, const double2 *__r
         stage_in<double2>(plane, [&](int i) { return make_double2(in[i], 0.0); }, put);
     }
     __syncthreads();
-    const int top = block_max(hmax, red) >> 20;
+    const int big = block_max(hmax, red), top = big >> 20;
     Meta *m = meta + (size_t)band * Nz + z;
     if (top == 0x7ff) {
         if (threadIdx.x == 0) *m = Meta{BAD, 0};
@@ -405,7 +407,7 @@ k_xy_forward_fix(FixTabs tb, const double2 *__restrict__ src, const double2 *__r
     }
     int bits0 = fix::TOP - first_growth(tb.ax[0], false);
     if (gather) bits0 = min(bits0, disc_bits);
-    const int s0 = bits0 - (top - 1022);
+    const int s0 = bits0 - (top ? top - 1022 : 32 - __clz(big) - 1042);   // subnormal: by its high word's bits
     Scale sc{bits0, -s0, 0};
     if (gather) {
         for (int i = threadIdx.x; i < Ny * RS; i += blockDim.x) {
@@ -423,7 +425,7 @@ k_xy_forward_fix(FixTabs tb, const double2 *__restrict__ src, const double2 *__r
     lines<false, false>(s_plane, tb.ax[1], tb.tw[1], Nx, tb.ax[0].nmag, 1, RS, sc, 0, slot);
     I2 *out = dst + band * n + off;
     for (int i = threadIdx.x; i < plane; i += blockDim.x) out[i] = s_plane[pidx(i, Nx, RS, nxm)];
-    if (threadIdx.x == 0) *m = Meta{top == 0 ? EMPTY : sc.e, sc.bits};
+    if (threadIdx.x == 0) *m = Meta{big == 0 ? EMPTY : sc.e, sc.bits};
 }
 
 // ---- z pass with the per-G factor ------------------------------------------------

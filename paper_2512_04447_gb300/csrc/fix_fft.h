@@ -132,8 +132,13 @@ FIX_HD int bits_of(u64 v) {
 // The double with these words as an integer of units 2^-s (|x| 2^s <= 2^62), rounded
 FIX_HD i64 from_double(int hi, unsigned lo, int s) {
     const int e = (hi >> 20) & 0x7ff;
-    const u64 m = ((u64)(unsigned)((hi & 0xfffff) | (e ? 0x100000 : 0)) << 42) | ((u64)lo << 10);   // 2^62 <= m < 2^63
+    u64 m = ((u64)(unsigned)((hi & 0xfffff) | (e ? 0x100000 : 0)) << 42) | ((u64)lo << 10);   // 2^62 <= m < 2^63
     int r = 1085 - e - s;   // x 2^s = m 2^-r
+    if (e == 0) {           // subnormal: the same with its leading bit brought there
+        const int k = m ? 63 - bits_of(m) : 0;
+        m <<= k;
+        r += k - 1;
+    }
     r = r < 1 ? 1 : (r > 63 ? 63 : r);
     const i64 v = (i64)((m + (1ull << (r - 1))) >> r);
     return hi < 0 ? -v : v;
