@@ -256,6 +256,17 @@ static void split62(double v, int &hi, int &lo) {
     lo = fix::lo_of(q);
 }
 
+// v by the power of two that brings its largest value to [1/2, 1): the norms of the projectors take it back,
+// and the fixed-point forms keep their bits where a projector is narrower than the grid's spacing and
+// even its largest factor is tiny (rc = h / 16: 2^-46 an axis).
+static void to_unit(std::vector<double> &v) {
+    double most = 0.0;
+    for (double x : v) most = std::max(most, std::fabs(x));
+    if (most == 0.0) return;
+    const int e = std::ilogb(most) + 1;
+    for (double &x : v) x = std::ldexp(x, -e);
+}
+
 // The projectors as discs (proj.h): per atom its windows and factors, per plane its rows.
 static rsdft_status build_projectors(rsdft_ctx *ctx, const rsdft_projectors *pj) {
     const int natom = pj->natom, nproj = pj->nproj;
@@ -272,6 +283,8 @@ static rsdft_status build_projectors(rsdft_ctx *ctx, const rsdft_projectors *pj)
                 at[a].g[k].push_back(g);
                 at[a].h[k].push_back(d / rc * g);
             }
+            to_unit(at[a].g[k]);
+            to_unit(at[a].h[k]);
         }
     }
     // per plane its discs with their rows by increasing dy (and the sums of beta^2 per atom), then in the

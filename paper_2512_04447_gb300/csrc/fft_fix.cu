@@ -289,7 +289,7 @@ __device__ __forceinline__ bool scatter_plane_fix(I2 *plane, int RS, const Discs
     for (int i = threadIdx.x; i < 6 * nd; i += blockDim.x) hmax = max(hmax, __double2hiint(a[i]) & 0x7fffffff);
     const int top = block_max(hmax, red) >> 20;
     if (top == 0x7ff) return false;
-    // a point gets at most nd times 2.3 of the largest coefficient: below 2^59 units of 2^e
+    // a point gets at most nd times 3 of the largest coefficient: below 2^59 units of 2^e
     const int e = max(sc.e, top - 1022 + 3 + (32 - __clz(nd)) - 60);
     if (e > sc.e) {
         const int sh = min(e - sc.e, 63);
