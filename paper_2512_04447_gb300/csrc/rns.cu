@@ -1,6 +1,6 @@
 // FP64 Gram matrices and rotations on the tensor cores by residue arithmetic.
 //
-// GB300 issues FP64 at 4 flop/clk/SM and BF16 MMAs at some 16,000, so an FP64 product
+// GB300 issues FP64 at 4 flop/clk/SM and BF16 MMAs at some 8,200, so an FP64 product
 // of matrices is cheapest as exact integer arithmetic on the tensor cores (the
 // residue-number form of the Ozaki scheme: Ozaki, Uchino, Imamura, "Ozaki scheme II",
 // 2025).  Every operand row is scaled by a power of two and rounded to integers; their
@@ -8,8 +8,9 @@
 // residues (|r| <= 128) are exact in BF16 and whose sums over CHUNK terms stay below
 // 2^24, exact in the FP32 accumulators of tcgen05; the sums modulo the p give the
 // integer result by the Chinese remainder theorem, which is rounded to FP64 once.
-// Nothing is rounded but the operands (2^-59 of their row's norm) and the result:
-//   |error| <= about 2^-58 |a| |b|  per entry,  against some 2^-54 of an FP64 sum.
+// Nothing is rounded but the operands (2^-62 of their row's norm, at most) and the result:
+//   |error| <= 2^-61 sqrt(n) |a| |b|  per entry of n points, where every value rounds the same way, and
+//   some 2^-61 |a| |b| where they do not,  against some 2^-54 to 2^-50 of an FP64 sum.
 //
 // The passes: row statistics (power-of-two scales) -> residues (one bf16 plane per
 // modulus and per real or imaginary part) -> k_rns (one GEMM per modulus) -> CRT.  The
@@ -45,18 +46,22 @@ typedef unsigned long long u64;
 typedef unsigned __int128 u128;
 
 // ---- moduli and their constants ---------------------------------------------------
-constexpr int NM = 15;
-constexpr int MODS[NM] = {256, 255, 253, 251, 247, 241, 239, 233, 229, 227, 223, 217, 211, 199, 197};
-// P = prod MODS = 2^117.78: twice the largest |sum| must stay below it
-constexpr int T_ROW = 58;      // |row|_2 <= 2^58 after scaling (both operands: 2^117 < P)
+// T_ROW is set by the operands' own accuracy, not by the result's: a row of n points that is equally large
+// everywhere has values 2^-(log2(n)/2) of its norm, and a plane wave rounds every one of them the same
+// way, so that the errors add up.  At 62 such a row of 64^3 points keeps 53 bits (and is exact), one of
+// 128^3 51.  With 15 moduli and 58 bits a uniform row's <a|a> was off by 2.2e-15 on 64^3, 3.6e-15 on 96^3.
+constexpr int NM = 16;
+constexpr int MODS[NM] = {256, 255, 253, 251, 247, 241, 239, 233, 229, 227, 223, 217, 211, 199, 197, 193};
+// P = prod MODS = 2^125.37: twice the largest |sum| must stay below it
+constexpr int T_ROW = 62;      // |row|_2 < 2^62 after scaling (both operands: 2^125 < P)
 
 struct Consts {
     float p[NM], ip[NM];
     int m[NM];
     int lo[NM], hi[NM];        // 256^j mod p, symmetric, as signed bytes j = 0..3 and 4..7
-    // W = floor(frac((P/p)^-1 mod p / p) 2^96) by byte j = 0..11, four moduli a word (the sixteenth is 0)
+    // W = floor(frac((P/p)^-1 mod p / p) 2^96) by byte j = 0..11, four moduli a word
     uint32_t w[12][4];
-    u64 Ptop;                  // P / 2^54, rounded
+    u64 Ptop;                  // P / 2^62, rounded
 };
 
 constexpr Consts make_consts() {
@@ -90,7 +95,7 @@ constexpr Consts make_consts() {
         }
         for (int j = 0; j < 12; ++j) c.w[j][i >> 2] |= (uint32_t)(uint8_t)(w >> (8 * j)) << (8 * (i & 3));
     }
-    c.Ptop = (u64)((P + ((u128)1 << 53)) >> 54);
+    c.Ptop = (u64)((P + ((u128)1 << 61)) >> 62);
     return c;
 }
 __constant__ Consts K = make_consts();
@@ -233,11 +238,11 @@ __device__ __forceinline__ int point_scale(int h, int bits) {
 }
 
 // ---- residues ---------------------------------------------------------------------
-// |x| 2^s rounded to an integer below 2^59, by integer shifts
+// |x| 2^s < 2^62 rounded to an integer, by integer shifts
 __device__ __forceinline__ u64 fix(int hi, unsigned lo, int s) {
     const int e = (hi >> 20) & 0x7ff;
-    const u64 m = ((u64)(unsigned)((hi & 0xfffff) | (e ? 0x100000 : 0)) << 40) | ((u64)lo << 8);
-    const int r = min(max(1083 - e - s, 1), 63);   // mantissa was shifted by 8; r >= 2 by the choice of s
+    const u64 m = ((u64)(unsigned)((hi & 0xfffff) | (e ? 0x100000 : 0)) << 42) | ((u64)lo << 10);
+    const int r = min(max(1085 - e - s, 1), 63);   // mantissa was shifted by 10; r >= 1 by the choice of s
     return (m + (1ull << (r - 1))) >> r;
 }
 
@@ -703,7 +708,7 @@ k_rns(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMa
 // ---- Chinese remainder ----------------------------------------------------------------
 // x 2^-s of the integer x with the symmetric residues r (bytes, four moduli a word): the fraction
 // x / P is sum r W / 2^96 modulo 1, its bytes' columns summed by dp4a (48 instead of 75 to 105
-// wide multiply-adds), good to 2^-85: 2^-83 of the product of the operands' bounds.  All residues 0
+// wide multiply-adds), good to 2^-85: 2^-83 of the product of the operands' bounds (2^124).  All residues 0
 // give exactly 0.
 __device__ __forceinline__ double crt_value(const int r[4], int s) {
     i64 limb[3];
@@ -728,7 +733,7 @@ __device__ __forceinline__ double crt_value(const int r[4], int s) {
         f1 = ~f1 + (f0 == 0);
         f2 = ~f2 + (f0 == 0 && f1 == 0);
     }
-    int e = 22 - s;   // x = hi 2^(e + s), below
+    int e = 30 - s;   // x = hi 2^(e + s), below
 #pragma unroll
     for (int k = 0; k < 2; ++k)
         if (f2 == 0) {
@@ -740,7 +745,7 @@ __device__ __forceinline__ double crt_value(const int r[4], int s) {
     if (f2 == 0) return 0.0;
     const int lz = __clz((int)f2);
     const u64 m = ((u64)__funnelshift_l(f1, f2, lz) << 32) | __funnelshift_l(f0, f1, lz);   // F = m 2^(32 - lz)
-    u64 hi = __umul64hi(m, K.Ptop);        // x = F P / 2^96 = hi 2^(64 + 32 - lz + 54 - 96)
+    u64 hi = __umul64hi(m, K.Ptop);        // x = F P / 2^96 = hi 2^(64 + 32 - lz + 62 - 96)
     e += 32 - lz;
     if (!(hi >> 63)) {
         hi <<= 1;
