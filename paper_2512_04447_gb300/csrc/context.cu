@@ -339,7 +339,7 @@ static rsdft_status build_projectors(rsdft_ctx *ctx, const rsdft_projectors *pj)
     std::vector<DiscRowFix> rowfix;
     std::vector<float2> gx;
     std::vector<int4> gxfix;
-    std::vector<double2> gz;
+    std::vector<double2> rowd, gxd, gz;
     for (int z = 0; z < Nz; ++z) {
         // greedy colouring: a disc takes the first colour none of whose points (bits of the plane) it has
         std::vector<std::vector<int>> colors;
@@ -368,7 +368,7 @@ static rsdft_status build_projectors(rsdft_ctx *ctx, const rsdft_projectors *pj)
                 const Disc &D = planes[z][k];
                 const Atom &A = at[D.atom];
                 meta.push_back(DiscMeta{(int)row.size(), (unsigned)D.rows.size() | (unsigned)D.xn << 8 |
-                                                             (unsigned)((A.i[0][0] + D.xa) % Nx) << 16});
+                                                             (unsigned)((A.i[0][0] + D.xa) % Nx) << 16 | (unsigned)z << 24});
                 datom.push_back(D.atom);
                 gz.push_back(make_double2(A.g[2][D.tz], A.h[2][D.tz]));
                 for (const Row &r : D.rows) {
@@ -379,10 +379,12 @@ static rsdft_status build_projectors(rsdft_ctx *ctx, const rsdft_projectors *pj)
                     split62(r.g, f.gh, f.gl);
                     split62(r.h, f.hh, f.hl);
                     rowfix.push_back(f);
+                    rowd.push_back(make_double2(r.g, r.h));
                 }
                 for (int t = 0; t < wmax; ++t) {
                     const double g = t < D.xn ? A.g[0][D.xa + t] : 0.0, h = t < D.xn ? A.h[0][D.xa + t] : 0.0;
                     gx.push_back(make_float2((float)g, (float)h));
+                    gxd.push_back(make_double2(g, h));
                     int4 f;
                     split62(g, f.x, f.y);
                     split62(h, f.z, f.w);
@@ -411,7 +413,7 @@ static rsdft_status build_projectors(rsdft_ctx *ctx, const rsdft_projectors *pj)
     DiscRowFix *d_rowf;
     float2 *d_gx;
     int4 *d_gxf;
-    double2 *d_gz;
+    double2 *d_rowd, *d_gxd, *d_gz;
     double *d_cn, *d_ek;
     RS_TRY(upload(ctx, &d_ps, plane_start.data(), plane_start.size()));
     RS_TRY(upload(ctx, &d_as, atom_start.data(), atom_start.size()));
@@ -423,12 +425,14 @@ static rsdft_status build_projectors(rsdft_ctx *ctx, const rsdft_projectors *pj)
     RS_TRY(upload(ctx, &d_cs, color_start.data(), color_start.size()));
     RS_TRY(upload(ctx, &d_gx, gx.data(), gx.size()));
     RS_TRY(upload(ctx, &d_gxf, gxfix.data(), gxfix.size()));
+    RS_TRY(upload(ctx, &d_rowd, rowd.data(), rowd.size()));
+    RS_TRY(upload(ctx, &d_gxd, gxd.data(), gxd.size()));
     RS_TRY(upload(ctx, &d_gz, gz.data(), gz.size()));
     RS_TRY(upload(ctx, &d_cn, cnorm.data(), cnorm.size()));
     RS_TRY(upload(ctx, &d_ek, ekb.data(), ekb.size()));
     ctx->pt = ProjTables{natom, nproj, d_ek};
     ctx->discs = Discs{natom, nproj, (int)datom.size(), wmax, mrows, mdiscs, d_ps, d_cp, d_cs, d_meta, d_row, d_rowf,
-                       d_gx, d_gxf, d_as, d_ad, d_gz, d_cn, d_ek};
+                       d_rowd, d_gx, d_gxf, d_gxd, d_as, d_ad, d_gz, d_cn, d_ek};
     ctx->nent = nent;
     return RSDFT_OK;
 }

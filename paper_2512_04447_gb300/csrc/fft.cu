@@ -493,86 +493,111 @@ k_xy_inverse(FftTabs<V> tb, const V *__restrict__ buf, const V *__restrict__ psi
 }
 
 // ---- projectors --------------------------------------------------------------------------
-// The gather alone, on planes in global memory (lane = x; FP64 takes the fixed-point factors).
 constexpr int PROJ_THREADS = 256;
 
-__device__ __forceinline__ double unfix(int h, int l) { return ((double)h * 4294967296.0 + (double)l) * 0x1p-62; }
-
+// p[band][atom nproj + j] = <beta_j|psi>: a block per (band, atom), a warp per disc of the atom, joined
+// in the block, so that the call needs no memory but the caller's.  lane = x; discs of at most 16 or 8
+// points across take two or four rows at a time.  A point costs four multiply-adds (a warp's FP64 ones 64 cycles each,
+// which bounds the FP64 form) and the factors of a row are loaded.  One GB300, FP64, against partial sums
+// per plane in scratch with the factors converted from fixed point: 144 bands on 64^3, 64 atoms 5,033 -> 1,443 us (a table
+// of every point's values 1,734), one band 127 -> 40 (51), 64 bands on 24^3, 8 atoms 106 -> 31 (31).
 template <typename V>
 __global__ void __launch_bounds__(PROJ_THREADS)
-k_gather(Discs t, const V *__restrict__ psi, int Nx, int Ny, long long n, V *__restrict__ part) {
+k_project(Discs t, const V *__restrict__ psi, int Nx, int Ny, long long n, typename Sc<V>::T dV, V *__restrict__ p) {
     using T = typename Sc<V>::T;
-    const int z = blockIdx.x, band = blockIdx.y;
-    const V *plane = psi + (size_t)band * n + (size_t)z * Nx * Ny;
-    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    const int d1 = t.plane_start[z + 1];
-    for (int d = t.plane_start[z] + (threadIdx.x >> 5); d < d1; d += nw) {
-        const DiscMeta m = t.meta[d];
-        const int rows = disc_rows(m.packed), w = disc_width(m.packed);
-        T s[6] = {(T)0, (T)0, (T)0, (T)0, (T)0, (T)0};
-        for (int c = 0; c < w; c += 32) {
-            const int l = c + lane;
-            int x = disc_x0(m.packed) + l;
+    const int band = blockIdx.x / t.natom, a = blockIdx.x - band * t.natom;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int i1 = t.atom_start[a + 1];
+    T s[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s[k] = (T)0;
+    for (int i = t.atom_start[a] + warp; i < i1; i += PROJ_THREADS / 32) {
+        const int d = t.atom_disc[i];
+        const int2 m = __ldg(reinterpret_cast<const int2 *>(t.meta + d));
+        const int rows = disc_rows(m.y), w = disc_width(m.y);
+        const V *plane = psi + (size_t)band * n + (size_t)disc_z(m.y) * Nx * Ny;
+        T v[6] = {(T)0, (T)0, (T)0, (T)0, (T)0, (T)0};   // sums of gx gy, hx gy and gx hy times psi
+        const int W = w <= 8 ? 8 : (w <= 16 ? 16 : 32);   // lanes a row
+        for (int c = 0; c < w; c += W) {
+            const int l = c + (lane & (W - 1));
+            int x = disc_x0(m.y) + l;
             if (x >= Nx) x -= Nx;
             T ax = (T)0, ay = (T)0, bx = (T)0, by = (T)0;
 #pragma unroll 4
-            for (int r = 0; r < rows; ++r) {
-                int pk;
-                T g, h;
-                if constexpr (sizeof(T) == 4) {
-                    const int4 k = __ldg(reinterpret_cast<const int4 *>(t.row + m.row0 + r));
-                    pk = k.x;
-                    g = __int_as_float(k.y);
-                    h = __int_as_float(k.z);
-                } else {
-                    const int4 k = __ldg(reinterpret_cast<const int4 *>(t.rowfix + m.row0 + r));
-                    pk = k.x;
-                    g = unfix(k.y, k.z);
-                    h = unfix(k.w, __ldg(&t.rowfix[m.row0 + r].hl));
-                }
-                if (in_row(pk, l)) {
-                    const V v = plane[(pk & 255) * Nx + x];
-                    ax += g * v.x;
-                    ay += g * v.y;
-                    bx += h * v.x;
-                    by += h * v.y;
+            for (int r = lane / W; r < rows; r += 32 / W) {
+                const int4 k = __ldg(reinterpret_cast<const int4 *>(t.row + m.x + r));
+                if (in_row(k.x, l)) {
+                    const V u = plane[(k.x & 255) * Nx + x];
+                    T g, h;
+                    if constexpr (sizeof(T) == 4) {
+                        g = __int_as_float(k.y);
+                        h = __int_as_float(k.z);
+                    } else {
+                        const double2 f = __ldg(t.rowd + m.x + r);
+                        g = f.x;
+                        h = f.y;
+                    }
+                    ax += g * u.x;
+                    ay += g * u.y;
+                    bx += h * u.x;
+                    by += h * u.y;
                 }
             }
-            T gx = (T)0, hx = (T)0;
             if (l < w) {
+                T gx, hx;
                 if constexpr (sizeof(T) == 4) {
-                    const float2 k = __ldg(t.gx + (size_t)d * t.wmax + l);
-                    gx = k.x;
-                    hx = k.y;
+                    const float2 f = __ldg(t.gx + (size_t)d * t.wmax + l);
+                    gx = f.x;
+                    hx = f.y;
                 } else {
-                    const int4 k = __ldg(t.gxfix + (size_t)d * t.wmax + l);
-                    gx = unfix(k.x, k.y);
-                    hx = unfix(k.z, k.w);
+                    const double2 f = __ldg(t.gxd + (size_t)d * t.wmax + l);
+                    gx = f.x;
+                    hx = f.y;
                 }
+                v[0] += gx * ax;
+                v[1] += gx * ay;
+                v[2] += hx * ax;
+                v[3] += hx * ay;
+                v[4] += gx * bx;
+                v[5] += gx * by;
             }
-            s[0] += gx * ax;
-            s[1] += gx * ay;
-            s[2] += hx * ax;
-            s[3] += hx * ay;
-            s[4] += gx * bx;
-            s[5] += gx * by;
         }
+        const double2 gd = t.gz[d];
+        const T gz = (T)gd.x, hz = (T)gd.y;
 #pragma unroll
-        for (int k = 0; k < 6; ++k)
-            for (int o = 16; o > 0; o >>= 1) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
-        if (lane < 3)
-            part[((size_t)band * t.ndisc + d) * 3 + lane] = mk<V>(lane == 0 ? s[0] : (lane == 1 ? s[2] : s[4]),
-                                                                 lane == 0 ? s[1] : (lane == 1 ? s[3] : s[5]));
+        for (int k = 0; k < 6; ++k) s[k] += gz * v[k];
+        s[6] += hz * v[0];
+        s[7] += hz * v[1];
+    }
+    // the eight sums over the warp, half of them going to each half of the lanes at every step: 9 additions instead of 40
+#pragma unroll
+    for (int o = 16, m = 4; m > 0; o >>= 1, m >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int k = 0; k < m; ++k) {
+            const T give = up ? s[k] : s[k + m];
+            s[k] = (up ? s[k + m] : s[k]) + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    }
+    s[0] += __shfl_xor_sync(0xffffffffu, s[0], 2);
+    s[0] += __shfl_xor_sync(0xffffffffu, s[0], 1);
+    __shared__ T red[PROJ_THREADS / 32][8];
+    if ((lane & 3) == 0) red[warp][lane >> 2] = s[0];   // bits 4, 3, 2 of the lane: those of the sum's number
+    __syncthreads();
+    const int j = threadIdx.x >> 1, part = threadIdx.x & 1;
+    if (j < t.nproj) {
+        T q = (T)0;
+        for (int k = 0; k < PROJ_THREADS / 32; ++k) q += red[k][threadIdx.x];
+        T *o = reinterpret_cast<T *>(p + (size_t)blockIdx.x * t.nproj + j);
+        o[part] = (T)t.cnorm[4 * a + j] * dV * q;
     }
 }
 
-// One warp per (band, atom): the disc sums joined with their z factors, p[band][atom nproj + j] =
-// <beta_j|psi> (p may be null) and the scatter coefficients of every disc, ab[band][disc] =
-// (gz q_s + hz q_z, gz q_x, gz q_y) with q_j = c_j E_j <beta_j|psi> (ab may be null).
+// One warp per (band, atom): the disc sums joined with their z factors, and the scatter coefficients of
+// every disc, ab[band][disc] = (gz q_s + hz q_z, gz q_x, gz q_y) with q_j = c_j E_j <beta_j|psi>.
 template <typename V>
 __global__ void __launch_bounds__(PROJ_THREADS)
-k_disc_fin(Discs t, const V *__restrict__ part, int nb, typename Sc<V>::T dV, V *__restrict__ p,
-           V *__restrict__ ab) {
+k_disc_fin(Discs t, const V *__restrict__ part, int nb, typename Sc<V>::T dV, V *__restrict__ ab) {
     using T = typename Sc<V>::T;
     const int w = (blockIdx.x * PROJ_THREADS + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     const int band = w / t.natom, a = w - band * t.natom;
@@ -603,11 +628,9 @@ k_disc_fin(Discs t, const V *__restrict__ part, int nb, typename Sc<V>::T dV, V 
     for (int j = 0; j < 4; ++j) {
         const T c = (T)t.cnorm[4 * a + j];   // 0 for projectors that are not there
         q[j] = mk<V>(c * dV * s[2 * j], c * dV * s[2 * j + 1]);
-        if (p && lane == 0 && j < t.nproj) p[(size_t)band * t.natom * t.nproj + a * t.nproj + j] = q[j];
         const T e = j < t.nproj ? c * (T)t.e_kb[a * t.nproj + j] : (T)0;
         q[j] = mk<V>(e * q[j].x, e * q[j].y);
     }
-    if (!ab) return;
     V *ob = ab + (size_t)band * t.ndisc * 3;
     for (int i = i0 + lane; i < i1; i += 32) {
         const int d = t.atom_disc[i];
@@ -722,7 +745,9 @@ rsdft_status fft_xy_inverse_t(rsdft_ctx *ctx, const V *buf, const V *psi, const 
     return RSDFT_OK;
 }
 
-rsdft_status disc_buffers(rsdft_ctx *ctx, int nb, double2 **part, double2 **ab, cudaStream_t st) {
+// Partial-sum and coefficient buffers of nb bands, and the scatter coefficients E <beta|psi> of every disc
+// from the sums.
+static rsdft_status disc_buffers(rsdft_ctx *ctx, int nb, double2 **part, double2 **ab, cudaStream_t st) {
     const size_t per = (size_t)ctx->discs.ndisc * 3;
     RS_TRY(grow(ctx, ctx->discbuf, std::max<size_t>(16, 2 * per * nb * sizeof(double2)), st));
     *part = static_cast<double2 *>(ctx->discbuf.p);
@@ -731,32 +756,24 @@ rsdft_status disc_buffers(rsdft_ctx *ctx, int nb, double2 **part, double2 **ab, 
 }
 
 template <typename V>
-static rsdft_status disc_finish_t(rsdft_ctx *ctx, const V *part, int nb, V *p, V *ab, cudaStream_t st) {
+static rsdft_status disc_finish(rsdft_ctx *ctx, const V *part, int nb, V *ab, cudaStream_t st) {
     using T = typename Sc<V>::T;
     k_disc_fin<V><<<cdiv((long long)nb * ctx->pt.natom * 32, PROJ_THREADS), PROJ_THREADS, 0, st>>>(
-        ctx->discs, part, nb, (T)ctx->dV, p, ab);
+        ctx->discs, part, nb, (T)ctx->dV, ab);
     count_launch(ctx);
     RS_LAUNCHED(ctx, "k_disc_fin");
     return RSDFT_OK;
-}
-rsdft_status disc_finish(rsdft_ctx *ctx, const double2 *part, int nb, double2 *p, double2 *ab, cudaStream_t st) {
-    return disc_finish_t<double2>(ctx, part, nb, p, ab, st);
 }
 
 template <typename V>
 rsdft_status project_t(rsdft_ctx *ctx, const V *psi, V *p, int nb, cudaStream_t st) {
     if (nb <= 0 || ctx->pt.natom == 0) return RSDFT_OK;
-    double2 *part, *ab;
-    RS_TRY(disc_buffers(ctx, nb, &part, &ab, st));
+    using T = typename Sc<V>::T;
     const double ne = (double)ctx->nent;
-    const double e = (double)sizeof(V);
-    {
-        ProfScope ps(ctx, RSDFT_K_PROJECT, 4.0 * ctx->pt.nproj * ne * nb, e * ne * nb, st);
-        k_gather<V><<<dim3(ctx->N[2], nb), PROJ_THREADS, 0, st>>>(ctx->discs, psi, ctx->N[0], ctx->N[1], ctx->n,
-                                                                reinterpret_cast<V *>(part));
-    }
-    RS_LAUNCHED(ctx, "k_gather");
-    return disc_finish_t<V>(ctx, reinterpret_cast<const V *>(part), nb, p, (V *)nullptr, st);
+    ProfScope ps(ctx, RSDFT_K_PROJECT, 4.0 * ctx->pt.nproj * ne * nb, (double)sizeof(V) * ne * nb, st);
+    k_project<V><<<nb * ctx->pt.natom, PROJ_THREADS, 0, st>>>(ctx->discs, psi, ctx->N[0], ctx->N[1], ctx->n, (T)ctx->dV, p);
+    RS_LAUNCHED(ctx, "k_project");
+    return RSDFT_OK;
 }
 
 rsdft_status fft_xy_forward32(rsdft_ctx *ctx, Src kind, const float2 *src, const float2 *src2,
@@ -794,7 +811,7 @@ rsdft_status apply_h64(rsdft_ctx *ctx, const double2 *psi, double2 *hpsi, int nb
     const bool nl = ctx->discs.ndisc > 0;
     if (nl) RS_TRY(disc_buffers(ctx, nb, &part, &ab, st));
     RS_TRY(fft_xy_forward(ctx, Src::Plain, psi, nullptr, nullptr, nullptr, nullptr, ctx->ws.T1, nb, st, part));
-    if (nl) RS_TRY(disc_finish(ctx, part, nb, nullptr, ab, st));
+    if (nl) RS_TRY(disc_finish<double2>(ctx, part, nb, ab, st));
     RS_TRY(fft_z_mid(ctx, Mid::Kinetic, ctx->ws.T1, nullptr, nb, st));
     RS_TRY(fft_xy_inverse(ctx, ctx->ws.T1, psi, ab, hpsi, nullptr, nb, st));
     return RSDFT_OK;
@@ -810,7 +827,7 @@ rsdft_status apply_h32(rsdft_ctx *ctx, const float2 *psi, float2 *hpsi, int nb, 
     float2 *part32 = reinterpret_cast<float2 *>(part), *ab32 = reinterpret_cast<float2 *>(ab);
     float2 *t1 = reinterpret_cast<float2 *>(ctx->ws.T1);
     RS_TRY(fft_xy_forward32(ctx, Src::Plain, psi, nullptr, nullptr, nullptr, t1, nb, st, part32));
-    if (nl) RS_TRY(disc_finish_t<float2>(ctx, part32, nb, nullptr, ab32, st));
+    if (nl) RS_TRY(disc_finish<float2>(ctx, part32, nb, ab32, st));
     RS_TRY(fft_z_mid32(ctx, Mid::Kinetic, t1, nullptr, nb, st));
     RS_TRY(fft_xy_inverse32(ctx, t1, psi, ab32, hpsi, nb, st));
     return RSDFT_OK;

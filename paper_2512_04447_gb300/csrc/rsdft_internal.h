@@ -52,7 +52,7 @@ struct ProjTables {
 };
 
 // Kleinman-Bylander projectors by plane (proj.h).
-struct DiscMeta { int row0; unsigned packed; };                               // first row; rows | width << 8 | first x << 16
+struct DiscMeta { int row0; unsigned packed; };                               // first row; rows | width << 8 | first x << 16 | z << 24
 struct __align__(16) DiscRow { int packed; float g, h; int pad; };            // a row of a disc: gy, dy/rc gy
 struct __align__(16) DiscRowFix { int packed, gh, gl, hh, hl, pad[3]; };      // the same in units of 2^-62
 struct Discs {
@@ -64,8 +64,10 @@ struct Discs {
     const DiscMeta *meta;                    // [ndisc]
     const DiscRow *row;                      // by disc, in order of y: y | first x offset << 8 | points << 16
     const DiscRowFix *rowfix;
+    const double2 *rowd;                     // gy, dy/rc gy of a row
     const float2 *gx;                        // [ndisc][wmax] gx, dx/rc gx
     const int4 *gxfix;                       // the same in units of 2^-62 (high, low words)
+    const double2 *gxd;
     const int *atom_start, *atom_disc;       // [natom + 1], [ndisc] discs of each atom
     const double2 *gz;                       // [ndisc] gz, dz/rc gz
     const double *cnorm, *e_kb;              // [natom][4] norms c; [natom * nproj]
@@ -258,10 +260,6 @@ rsdft_status fft_z_mid(rsdft_ctx *ctx, Mid mid, double2 *buf, const double *tkin
 rsdft_status fft_xy_inverse(rsdft_ctx *ctx, const double2 *buf, const double2 *psi,
                             const double2 *ab, double2 *out, double *rout, int nb,
                             cudaStream_t st);
-// Partial-sum and coefficient buffers of nb bands, and the sums of part joined per atom: p (or null)
-// the projections, ab (or null) the scatter coefficients E <beta|psi> of every disc.
-rsdft_status disc_buffers(rsdft_ctx *ctx, int nb, double2 **part, double2 **ab, cudaStream_t st);
-rsdft_status disc_finish(rsdft_ctx *ctx, const double2 *part, int nb, double2 *p, double2 *ab, cudaStream_t st);
 rsdft_status project(rsdft_ctx *ctx, const double2 *psi, double2 *p, int nb, cudaStream_t st);
 rsdft_status apply_h64(rsdft_ctx *ctx, const double2 *psi, double2 *hpsi, int nb,
                        cudaStream_t st);
