@@ -196,7 +196,7 @@ static rsdft_status build_fix_tables(rsdft_ctx *ctx) {
         const AxisPlan &p = ctx->fft.ax[a];
         const int N = p.N;
         std::vector<fix::W4> tw(N);
-        std::vector<long long> kin(N);
+        std::vector<longlong2> kin(N);
         std::vector<double> g2abs(N / 2 + 1);
         std::vector<unsigned char> fabs(N);
         const double gunit = 2.0 * M_PI / ctx->L[a];
@@ -210,10 +210,12 @@ static rsdft_status build_fix_tables(rsdft_ctx *ctx) {
             const double g = gunit * ka;
             fabs[pos] = (unsigned char)ka;
             g2abs[ka] = g * g;
-            kin[pos] = llroundl(ldexpl(0.5L * (long double)(g * g) / (long double)ctx->n, f.kexp));
+            const long double v = ldexpl(0.5L * (long double)(g * g) / (long double)ctx->n, f.kexp);
+            kin[pos].x = (long long)floorl(v);
+            kin[pos].y = (long long)floorl(ldexpl(v - (long double)kin[pos].x, 32));
         }
         fix::W4 *d_tw;
-        long long *d_kin;
+        longlong2 *d_kin;
         double *d_g2;
         unsigned char *d_f;
         RS_TRY(upload(ctx, &d_tw, tw.data(), N));

@@ -4,8 +4,9 @@
 // epilogue; digit-reversed spectrum in between), FP64 in and out.  A block (an xy plane, or the
 // slab of one y) is scaled to integers by its largest value; between the passes the buffer
 // holds integers, and (exponent, bits) of every block says what they are worth, so that the
-// next pass brings its rows to one exponent.  The per-G factor keeps full precision: products
-// are formed with a normalised factor and shifted to the largest one of the slab.
+// next pass brings its rows to one exponent.  The per-G factor keeps its relative precision (53
+// bits, the kinetic one 61): products are formed with a normalised factor and its exponent and shifted to the
+// largest one of the slab.
 //
 // What bounds it: the FP64 passes ran at some 80% of the FP64 pipe; the integer instructions on
 // 64-bit values bound these.  144 bands on 64^3, one GB300: forward 3.23 -> 0.68 ms (1.46 with
@@ -42,13 +43,12 @@ constexpr int SHIFTS = MAX_N * 4;      // row shifts behind it (xy planes with p
 struct FixTabs {
     AxisPlan ax[3];
     const W4 *tw[3];
-    const i64 *kin[3];                 // G_a^2 / (2 n) in units of 2^-kexp, by position
+    const longlong2 *kin[3];           // G_a^2 / (2 n) in units of 2^-kexp, by position: whole part, 2^32 times the rest
     int kexp;
     const double *g2[3], *g1[3];       // by position
     const double *g2abs[3];            // G_a^2 by |frequency index|
     const unsigned char *fabs[3];      // |frequency index| by position
     double inv_n;
-    int fexp;                          // other factors: |f| < 2^(61 - fexp)
 };
 
 struct Meta { int e, bits; };          // block values are integers below 2^bits times 2^e
@@ -58,6 +58,7 @@ __device__ __forceinline__ unsigned mag_hi(I2 v) {
     return (unsigned)(hx ^ (hx >> 31)) | (unsigned)(hy ^ (hy >> 31));
 }
 __device__ __forceinline__ int bits_hi(unsigned m) { return 64 - __clz((int)m); }   // 32 for m = 0
+__device__ __forceinline__ int bits_of(I2 v) { return fix::bits_of((u64)(v.x ^ (v.x >> 63)) | (u64)(v.y ^ (v.y >> 63))); }
 
 // Every thread's word joined over the block (or / max); red: a zeroed word of shared memory
 __device__ __forceinline__ unsigned block_or(unsigned v, unsigned *red) {
@@ -436,12 +437,29 @@ template <Mid MID> __device__ __forceinline__ double factor(const FixTabs &tb, i
     const double g2 = tb.g2[0][x] + tb.g2[1][y] + tb.g2[2][z];   // Hartree
     return g2 > 0.0 ? 4.0 * M_PI / g2 * tb.inv_n : 0.0;
 }
-__device__ __forceinline__ double tpa_factor(double x) {
+__device__ __forceinline__ double tpa_factor(double x, double c) {
     const double num = 27.0 + x * (18.0 + x * (12.0 + 8.0 * x));
-    return num / (num + 16.0 * x * x * x * x);
+    return c * num / (num + 16.0 * x * x * x * x);
 }
-__device__ __forceinline__ i64 fixed_factor(double f, int s) {
-    return fix::from_double(__double2hiint(f), (unsigned)__double2loint(f), s);
+struct Fac { i64 w; int nf; };   // a factor w 2^-nf, 2^61 <= w < 2^62 (0 for factors of zero)
+__device__ __forceinline__ Fac fac_of(double f) {   // |f|
+    const int hi = __double2hiint(f), e = (hi >> 20) & 0x7ff;
+    if (e == 0) return Fac{0, 0};
+    return Fac{((i64)((hi & 0xfffff) | 0x100000) << 41) | ((i64)(unsigned)__double2loint(f) << 9), 1084 - e};
+}
+__device__ __forceinline__ Fac fac_of(longlong2 a, longlong2 b, longlong2 c) {   // their sum, below 2^60
+    const u64 rest = (u64)(a.y + b.y + c.y);
+    u64 h = (u64)(a.x + b.x + c.x) + (rest >> 32);
+    unsigned l = (unsigned)rest;
+    int nf = 0;
+    if (h == 0) {
+        if (l == 0) return Fac{0, 0};
+        h = l;
+        l = 0;
+        nf = 32;
+    }
+    const int k = __clzll((i64)h) - 2;
+    return Fac{(i64)((h << k) | (k < 32 ? (u64)(l >> (32 - k)) : (u64)l << (k - 32))), nf + k};
 }
 
 // tab: TPA's factor depends on |k| of each axis only, so a slab evaluates it once per (|kz|, |kx|),
@@ -461,7 +479,7 @@ k_z_mid_fix(FixTabs tb, I2 *__restrict__ buf, const double *__restrict__ tkin, c
     const int tot = Nx * Nz;
     const unsigned nxm = tb.ax[0].nmag;
     int *shift = reinterpret_cast<int *>(s_slab + tot);
-    i64 *tab = reinterpret_cast<i64 *>(shift + SHIFTS / 4);
+    double *tab = reinterpret_cast<double *>(shift + SHIFTS / 4);
     const int hx = Nx / 2 + 1, hz = Nz / 2 + 1;
     double tk = 1.0;
     if (MID == Mid::Tpa) {
@@ -489,46 +507,45 @@ k_z_mid_fix(FixTabs tb, I2 *__restrict__ buf, const double *__restrict__ tkin, c
         for (int i = threadIdx.x; i < hx * hz; i += blockDim.x) {
             const int z = i / hx, x = i - z * hx;
             const double g2 = tb.g2abs[0][x] + gy + tb.g2abs[2][z];
-            tab[i] = fixed_factor(tpa_factor(0.5 * g2 / tk) * tb.inv_n, tb.fexp);
+            tab[i] = tpa_factor(0.5 * g2 / tk, tb.inv_n);
         }
     }
     __syncthreads();
     Scale sc{bits0, e0, 0};
     lines<false, false>(s_slab, tb.ax[2], tb.tw[2], Nx, nxm, 1, Nx, sc, 0, slot);
-    const i64 ky = MID == Mid::Kinetic ? tb.kin[1][y] : 0;
-    auto f_of = [&](int i, bool &neg) -> i64 {
+    const longlong2 ky = MID == Mid::Kinetic ? tb.kin[1][y] : make_longlong2(0, 0);
+    auto f_of = [&](int i, bool &neg) -> Fac {
         const int z = qdiv(i, nxm), x = i - z * Nx;
         if constexpr (MID == Mid::Kinetic) {
-            return tb.kin[0][x] + ky + tb.kin[2][z];
+            return fac_of(tb.kin[0][x], ky, tb.kin[2][z]);
         } else if constexpr (MID == Mid::Tpa) {
-            if (table) return tab[(int)tb.fabs[2][z] * hx + tb.fabs[0][x]];
+            if (table) return fac_of(tab[(int)tb.fabs[2][z] * hx + tb.fabs[0][x]]);
             const double g2 = tb.g2[0][x] + tb.g2[1][y] + tb.g2[2][z];
-            return fixed_factor(tpa_factor(0.5 * g2 / tk) * tb.inv_n, tb.fexp);
+            return fac_of(tpa_factor(0.5 * g2 / tk, tb.inv_n));
         } else {
             const double f = factor<MID>(tb, x, y, z);
             neg = f < 0.0;
-            return fixed_factor(fabs(f), tb.fexp);
+            return fac_of(f);
         }
     };
-    // bits of the largest product v F 2^-62, then the products shifted to it
+    // bits of the largest product, then the products shifted to it (all bits count: a value that rounds to nothing may
+    // meet the largest factor)
     int big = EMPTY;
     bool neg = false;
     for (int i = threadIdx.x; i < tot; i += blockDim.x) {
-        const i64 f = f_of(i, neg);
-        if (f) big = max(big, bits_hi(mag_hi(s_slab[i])) - __clzll(f));
+        const Fac f = f_of(i, neg);
+        if (f.w) big = max(big, bits_of(s_slab[i]) - f.nf - 2);
     }
     big = block_max(big, red + 1);
-    const int g = big <= EMPTY / 2 ? 0 : fix::TOP - big;   // normalising by clz - 2 gives the 2 of pr's bound back
+    const int g = big <= EMPTY / 2 ? 0 : fix::TOP - big;   // v w 2^-64 has two bits less than v
     constexpr bool GRAD = MID == Mid::GradX || MID == Mid::GradY || MID == Mid::GradZ;
     for (int i = threadIdx.x; i < tot; i += blockDim.x) {
         bool ng = false;
-        const i64 f = f_of(i, ng);
+        const Fac f = f_of(i, ng);
         I2 v{0, 0};
-        if (f) {
-            const int nf = __clzll(f) - 2;
-            const i64 w = f << nf;                                // in [2^61, 2^62)
-            v = fix::mul_w<false>(s_slab[i], W4{fix::hi_of(w), fix::lo_of(w), 0, 0});   // v w 2^-64
-            const int d = g - nf;
+        if (f.w) {
+            v = fix::mul_w<false>(s_slab[i], W4{fix::hi_of(f.w), fix::lo_of(f.w), 0, 0});   // v w 2^-64
+            const int d = ::min(g - f.nf, 63);
             v = I2{shifted(v.x, -d), shifted(v.y, -d)};
             if (GRAD) v = ng ? fix::rot<false>(v) : fix::rot<true>(v);   // i f v
         }
@@ -536,7 +553,7 @@ k_z_mid_fix(FixTabs tb, I2 *__restrict__ buf, const double *__restrict__ tkin, c
     }
     __syncthreads();
     sc.bits = fix::TOP;
-    sc.e += 64 - (MID == Mid::Kinetic ? tb.kexp : tb.fexp) - g;
+    sc.e += 64 - (MID == Mid::Kinetic ? tb.kexp : 0) - g;
     lines<true, false>(s_slab, tb.ax[2], tb.tw[2], Nx, nxm, 1, Nx, sc, 0, slot);
     for (int i = threadIdx.x; i < tot; i += blockDim.x) {
         const int z = qdiv(i, nxm), x = i - z * Nx;
@@ -650,7 +667,6 @@ FixTabs tabs_of(const rsdft_ctx *ctx) {
     }
     t.kexp = ctx->fix.kexp;
     t.inv_n = 1.0 / (double)ctx->n;
-    t.fexp = 0;
     return t;
 }
 
@@ -700,7 +716,7 @@ rsdft_status fft_z_mid(rsdft_ctx *ctx, Mid mid, double2 *buf, const double *tkin
     Meta *mp, *ms;
     RS_TRY(ensure_meta(ctx, nb, &mp, &ms, st));
     size_t sm = HEAD + (size_t)ctx->N[0] * ctx->N[2] * sizeof(I2) + SHIFTS;
-    const size_t tabb = (size_t)(ctx->N[0] / 2 + 1) * (ctx->N[2] / 2 + 1) * sizeof(i64);
+    const size_t tabb = (size_t)(ctx->N[0] / 2 + 1) * (ctx->N[2] / 2 + 1) * sizeof(double);
     int table = 0;
     if (mid == Mid::Tpa && sm + tabb <= MAX_DYN_SMEM) {
         table = 1;
@@ -709,15 +725,7 @@ rsdft_status fft_z_mid(rsdft_ctx *ctx, Mid mid, double2 *buf, const double *tkin
     const dim3 grid(ctx->N[1], nb);
     const int th = threads_for(sm, ctx->N[0] * ctx->N[2]);
     ProfScope ps(ctx, RSDFT_K_FFT_Z, 10.0 * (double)ctx->n * std::log2((double)ctx->N[2]) * nb, 32.0 * (double)ctx->n * nb, st);
-    FixTabs tb = tabs_of(ctx);
-    // bound of the factor: 1 (TPA), 4 pi / min G^2, max |G|; all divided by n
-    double fmax = 1.0;
-    const double gmin = 2.0 * M_PI / std::max(ctx->L[0], std::max(ctx->L[1], ctx->L[2]));
-    if (mid == Mid::Hartree) fmax = 4.0 * M_PI / (gmin * gmin);
-    else if (mid == Mid::GradX) fmax = M_PI * ctx->N[0] / ctx->L[0];
-    else if (mid == Mid::GradY) fmax = M_PI * ctx->N[1] / ctx->L[1];
-    else if (mid == Mid::GradZ) fmax = M_PI * ctx->N[2] / ctx->L[2];
-    tb.fexp = 59 - std::ilogb(fmax * tb.inv_n);   // |f| 2^fexp < 2^60
+    const FixTabs tb = tabs_of(ctx);
     I2 *b = reinterpret_cast<I2 *>(buf);
 #define RS_Z(M)                                                              \
     case M:                                                                  \

@@ -143,7 +143,7 @@ struct Scratch {
 // Tables and block exponents of the fixed-point FP64 transforms (fft_fix.cu).
 struct FixFft {
     const void *tw[3] = {};                  // [N] exp(-2 pi i k / N) as fix::W4
-    const long long *kin[3] = {};            // G_a^2 / (2 n) 2^kexp by position
+    const longlong2 *kin[3] = {};            // G_a^2 / (2 n) 2^kexp by position: whole part, 2^32 times the rest
     int kexp = 0;
     const double *g2abs[3] = {};             // G_a^2 by |frequency index|
     const unsigned char *fabs[3] = {};       // |frequency index| by position

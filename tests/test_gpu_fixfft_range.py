@@ -40,3 +40,34 @@ def test_subnormal_orbitals(bits, natom):
     ref = ham.apply(x).view(np.float64)
     assert np.max(np.abs(got - ref)) <= 2.0 + 5.0 * natom + 1e-12 * np.max(np.abs(ref))
     ctx.close()
+
+
+@pytest.mark.parametrize("axis", [0, 1, 2])
+def test_factors_far_below_the_largest(axis):
+    """A plane wave of alternating signs along one axis of a cell of very unequal grid spacings: its transform is
+    exact, so the result is the input times one factor, and that keeps FP64's relative precision
+    however small it is (the largest kinetic factor is 2^41 times the smallest here).  Roundings of 2^-53: G^2
+    from G 3, the kinetic and the Hartree factor 4, the rational TPA function twice those of x and 14, the
+    result and its product with 1/n 2."""
+    need_gpu()
+    N, L = (16, 24, 12), (30000.0, 100.0, 3.0)
+    ctx = R.Context(L, N, np.zeros(N[0] * N[1] * N[2]))
+    i = np.meshgrid(*[np.arange(m) for m in N[::-1]], indexing="ij")[2 - axis]
+    x = (1.0 - 2.0 * (i % 2)).reshape(-1)
+    g2 = (np.longdouble(np.pi) * N[axis] / np.longdouble(L[axis])) ** 2
+    h = torch.empty(1, ctx.n, dtype=torch.complex128, device="cuda")
+
+    def close(got, factor, roundings):
+        return np.all(np.abs(got - x * float(factor)) <= roundings * 2.0 ** -53 * float(factor))
+
+    ctx.apply_h(dev(x[None] + 0j), h)
+    assert close(host(h)[0], g2 / 2, 10)
+    v = torch.empty(ctx.n, dtype=torch.float64, device="cuda")
+    ctx.hartree(dev(x), v)
+    assert close(host(v), 4 * np.longdouble(np.pi) / g2, 10)
+    for t in (1.0, 1e-3, 1e-6, 1e-9, 1e-12):
+        ctx.precondition_tpa(dev(x[None] + 0j), h, dev(np.array([t])))
+        q = g2 / 2 / np.longdouble(t)
+        p = 27 + q * (18 + q * (12 + 8 * q))
+        assert close(host(h)[0], p / (p + 16 * q ** 4), 24), t
+    ctx.close()
