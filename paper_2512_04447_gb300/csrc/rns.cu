@@ -12,6 +12,11 @@
 //   |error| <= 2^-61 sqrt(n) |a| |b|  per entry of n points, where every value rounds the same way, and
 //   some 2^-61 |a| |b| where they do not,  against some 2^-54 to 2^-50 of an FP64 sum.
 //
+// Rotations multiply rows that need not be alike in size by coefficients of any size: rows are first
+// scaled to equal norms and the coefficients by what that took away, both by powers of two, so that the result does
+// not depend on how a program scales its rows.  Then one scale per point and one per column of coefficients serve
+// all rows: |error| <= some 2^-57 max_i |y_i(p)| / |y_i| times the norm of |c_i| |y_i|.
+//
 // The passes: row statistics (power-of-two scales) -> residues (one bf16 plane per
 // modulus and per real or imaginary part) -> k_rns (one GEMM per modulus) -> CRT.  The
 // points go in chunks that keep the residues within RNS_BYTES.
@@ -204,10 +209,16 @@ __global__ void k_row_scale(const Stat *__restrict__ part, int S, int rows, int 
     }
 }
 
-// Largest high word |x| per point over rows [r0, r0 + nr) of the block list (any of the two
-// parts), for the rotation's per-point scales.
+// Largest exponent per point of the scaled rows |x| 2^scale over rows [r0, r0 + nr) of the block list
+// (any of the two parts), offset by PT_BIAS (0: a point of zeros), for the rotation's per-point scales.
+constexpr int PT_BIAS = 4096;   // scales lie within +-1,200
+__device__ __forceinline__ int point_exp(int hi, int lo, int s) {
+    const int h = hi & 0x7fffffff;
+    return (h | lo) ? max(h >> 20, 1) + s + PT_BIAS : 0;
+}
 __global__ void __launch_bounds__(256)
-k_point_max(RowBlocks src, int r0, int nr, long long n, int rows_per_cta, int *__restrict__ hmax, int *flag) {
+k_point_max(RowBlocks src, int r0, int nr, long long n, int rows_per_cta, const int *__restrict__ scale,
+            int *__restrict__ pmax) {
     const long long q = (long long)blockIdx.x * 256 + threadIdx.x;
     if (q >= n) return;
     const int a = r0 + blockIdx.y * rows_per_cta, b = min(r0 + nr, a + rows_per_cta);
@@ -224,25 +235,24 @@ k_point_max(RowBlocks src, int r0, int nr, long long n, int rows_per_cta, int *_
             }
         }
 #pragma unroll
-        for (int u = 0; u < 8; ++u) m = max(m, max(v[u].y & 0x7fffffff, v[u].w & 0x7fffffff));
+        for (int u = 0; u < 8; ++u)
+            if (row + u < b) {
+                const int2 s = __ldg(reinterpret_cast<const int2 *>(scale) + row + u);
+                m = max(m, max(point_exp(v[u].y, v[u].x, s.x), point_exp(v[u].w, v[u].z, s.y)));
+            }
     }
-    const int e = m >> 20;
-    if (e > EXP_HI || (m > 0 && e == 0)) atomicExch(flag, 1);
-    atomicMax(hmax + q, m);
+    atomicMax(pmax + q, m);
 }
 
-// s with |x| 2^s <= 2^bits for every |x| whose high word is at most h (a column of zeros: any)
-__device__ __forceinline__ int point_scale(int h, int bits) {
-    const int e = h >> 20;
-    return e == 0 ? 0 : bits - (e - 1022);
-}
+// s with |x| 2^s <= 2^bits for every scaled |x| of a point whose largest exponent is e
+__device__ __forceinline__ int point_scale(int e, int bits) { return e == 0 ? 0 : bits - (e - PT_BIAS - 1022); }
 
 // ---- residues ---------------------------------------------------------------------
 // |x| 2^s < 2^62 rounded to an integer, by integer shifts
 __device__ __forceinline__ u64 fix(int hi, unsigned lo, int s) {
     const int e = (hi >> 20) & 0x7ff;
     const u64 m = ((u64)(unsigned)((hi & 0xfffff) | (e ? 0x100000 : 0)) << 42) | ((u64)lo << 10);
-    const int r = min(max(1085 - e - s, 1), 63);   // mantissa was shifted by 10; r >= 1 by the choice of s
+    const int r = min(max(1085 - max(e, 1) - s, 1), 63);   // mantissa was shifted by 10; r >= 1 by the choice of s
     return (m + (1ull << (r - 1))) >> r;
 }
 
@@ -261,13 +271,13 @@ __device__ __forceinline__ unsigned pack(float a, float b, unsigned neg) {
 }
 
 // Residue planes of rows of FP64 complex values: res[q][row][plane][ld], points p0 .. p0 + ld
-// (zero beyond n).  Scales per row and plane (per_point 0) or per point and segment: rows
-// below seg1 use hmax[0][..], the others hmax[1][..].  Four points a thread; all integer and
+// (zero beyond n).  Scales per row and plane; per_point: on top of them per point and segment, rows
+// below seg1 by pmax[0][..], the others by pmax[1][..].  Four points a thread; all integer and
 // FP32 arithmetic, about 7 instructions a residue: this pass is bound by its instructions
 // and by the 4 NM bytes that it writes for every 16 read.
 __global__ void __launch_bounds__(256)
 k_residues(RowBlocks src, long long n, long long p0, int ld, int R, int row0, int per_point,
-           const int *__restrict__ scale, const int *__restrict__ hmax, int seg1, int bits0, int bits1,
+           const int *__restrict__ scale, const int *__restrict__ pmax, int seg1, int bits0, int bits1,
            __nv_bfloat16 *__restrict__ res, const int *flag) {
     if (*flag) return;
     const int row = blockIdx.y;
@@ -287,8 +297,9 @@ k_residues(RowBlocks src, long long n, long long p0, int ld, int R, int row0, in
         int sr = 0, si = 0;
         if (p < n) {
             w = __ldg(x + p);
-            if (per_point) sr = si = point_scale(hmax[seg * n + p], seg ? bits1 : bits0);
-            else { sr = scale[2 * (row0 + row)]; si = scale[2 * (row0 + row) + 1]; }
+            const int sp = per_point ? point_scale(pmax[seg * n + p], seg ? bits1 : bits0) : 0;
+            sr = scale[2 * (row0 + row)] + sp;
+            si = scale[2 * (row0 + row) + 1] + sp;
         }
         v[u] = fix(w.y, (unsigned)w.x, sr);
         v[4 + u] = fix(w.w, (unsigned)w.z, si);
@@ -321,35 +332,41 @@ __device__ __forceinline__ int coef_row(const Seg &s, int t, bool real) {
     return t < s.cnt[1] ? s.crow[1] + t : -1;
 }
 
-// scale of column b of a segment's coefficients: |c_b|_2 2^s <= 2^T_ROW
-__global__ void k_coef_scale(const double2 *__restrict__ c, int ldc, Seg s, int real, int *__restrict__ sc, int *flag) {
+// scale of column b of a segment's coefficients c 2^-ys (ys: the scales of their rows of Y, from the
+// segment's first row on): |c_b 2^-ys|_2 2^s < 2^T_ROW
+__global__ void k_coef_scale(const double2 *__restrict__ c, int ldc, Seg s, int real, const int *__restrict__ ys,
+                             int *__restrict__ sc, int *flag) {
     const int b = blockIdx.x;
-    double sum = 0.0, big = 0.0;
-    for (int t = threadIdx.x; t < s.k; t += 32) {
+    auto value = [&](int t) {
         const int r = coef_row(s, t, real);
-        if (r < 0) continue;
-        double2 v = c[(size_t)r * ldc + b];
+        double2 v = make_double2(0.0, 0.0);
+        if (r >= 0) v = c[(size_t)r * ldc + b];
         if (real) v.y = 0.0;
-        sum = fma(v.x, v.x, fma(v.y, v.y, sum));
-        big = fmax(big, fmax(fabs(v.x), fabs(v.y)));
+        return v;
+    };
+    int top = -(1 << 20);
+    for (int t = threadIdx.x; t < s.k; t += 32) {
+        const double2 v = value(t);
+        const double m = fmax(fabs(v.x), fabs(v.y));
         if (!isfinite(v.x) || !isfinite(v.y)) atomicExch(flag, 1);
+        else if (m > 0x1p400 || (m > 0.0 && m < 0x1p-400)) atomicExch(flag, 1);
+        if (m > 0.0) top = max(top, ((__double2hiint(m) >> 20) & 0x7ff) - 1023 - ys[real ? t : 2 * t]);
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        sum += __shfl_xor_sync(0xffffffffu, sum, o);
-        big = fmax(big, __shfl_xor_sync(0xffffffffu, big, o));
+    top = __reduce_max_sync(0xffffffffu, top);
+    double sum = 0.0;
+    for (int t = threadIdx.x; t < s.k; t += 32) {
+        const double2 v = value(t);
+        const int e = -ys[real ? t : 2 * t] - top;
+        const double x = scalbn(v.x, e), y = scalbn(v.y, e);
+        sum = fma(x, x, fma(y, y, sum));
     }
-    if (threadIdx.x) return;
-    int e = 0;
-    if (big > 0.0) {
-        if (big > 0x1p400 || big < 0x1p-400) atomicExch(flag, 1);
-        e = ilogb(sum * (1.0 + 1e-12));
-    }
-    sc[b] = big > 0.0 ? T_ROW - ((e + 2) >> 1) : 0;
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (threadIdx.x == 0) sc[b] = sum > 0.0 ? T_ROW - top - ((ilogb(sum * (1.0 + 1e-12)) + 2) >> 1) : 0;
 }
 
 // res[q][plane][nbp][kpad] of a segment's coefficients (zero outside)
 __global__ void k_coef_residues(const double2 *__restrict__ c, int ldc, Seg s, int real, int m, int nbp, int kpad,
-                                const int *__restrict__ sc, __nv_bfloat16 *__restrict__ res, const int *flag) {
+                                const int *__restrict__ ys, const int *__restrict__ sc, __nv_bfloat16 *__restrict__ res, const int *flag) {
     if (*flag) return;
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (long long)nbp * (kpad / 2)) return;
@@ -361,7 +378,7 @@ __global__ void k_coef_residues(const double2 *__restrict__ c, int ldc, Seg s, i
     for (int u = 0; u < 2; ++u) {
         const int r = b < m && t + u < s.k ? coef_row(s, t + u, real) : -1;
         const double2 z = r >= 0 ? c[(size_t)r * ldc + b] : make_double2(0.0, 0.0);
-        const int e = r >= 0 ? sc[b] : 0;
+        const int e = r >= 0 ? sc[b] - ys[real ? t + u : 2 * (t + u)] : 0;
         v[u] = fix(__double2hiint(z.x), __double2loint(z.x), e);
         v[2 + u] = fix(__double2hiint(z.y), __double2loint(z.y), e);
         neg[0] |= (__double2hiint(z.x) & 0x80000000u) >> (u ? 0 : 16);
@@ -816,7 +833,7 @@ __global__ void k_crt_gram(const short *__restrict__ out16, int slots, int M, in
 template <bool REAL>
 __global__ void __launch_bounds__(256)
 k_crt_rot(const unsigned *__restrict__ out8, int segs, int m, long long ldp, long long n, long long p0, int np,
-          const int *__restrict__ hmax, int bits0, int bits1, const int *__restrict__ sc, int mcols,
+          const int *__restrict__ pmax, int bits0, int bits1, const int *__restrict__ sc, int mcols,
           const double2 *base, int sign, double2 *out0, double2 *out1, const int *flag) {
     if (*flag) return;
     const int t = blockIdx.x * 256 + threadIdx.x;
@@ -842,8 +859,7 @@ k_crt_rot(const unsigned *__restrict__ out8, int segs, int m, long long ldp, lon
                 r[pl][2][g] = (int)__byte_perm(b0, b1, 0x5410);
                 r[pl][3][g] = (int)__byte_perm(b0, b1, 0x7632);
             }
-        const int h = hmax[(size_t)sg * n + p0 + t];
-        const int sp = point_scale(h, sg ? bits1 : bits0);
+        const int sp = point_scale(pmax[(size_t)sg * n + p0 + t], sg ? bits1 : bits0);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int b = 4 * quad + j;
@@ -1092,7 +1108,7 @@ static rsdft_status rotate_within(rsdft_ctx *ctx, size_t limit, const RowBlocks 
     for (int s = 0; s < segs; ++s) {
         kb[s] = cdiv(sg[s].k, 64);
         kpad[s] = kb[s] * 64;
-        // |y_r| over the K products of a sum is at most sqrt(K) max|y|
+        // |y| over the K products of a sum is at most sqrt(K) times the largest
         int h = 0;
         while ((1LL << (2 * h)) < (long long)sg[s].k * PL) ++h;
         bits[s] = T_ROW - h;
@@ -1102,6 +1118,7 @@ static rsdft_status rotate_within(rsdft_ctx *ctx, size_t limit, const RowBlocks 
     const long long most = std::max<long long>(4096, (long long)(limit / per_point) / 128 * 128);
     const int nchunk = cdiv(n, most);
     const int ld = cdiv(cdiv(n, nchunk), 128) * 128;
+    const int S = std::max(1, std::min<int>(64, (int)(n / 4096)));
     Carver cv{nullptr};
     for (int pass = 0; pass < 2; ++pass) {
         if (pass == 1) {
@@ -1110,8 +1127,10 @@ static rsdft_status rotate_within(rsdft_ctx *ctx, size_t limit, const RowBlocks 
         }
         __nv_bfloat16 *res = cv.take<__nv_bfloat16>((size_t)NM * R * 2 * ld);
         unsigned *out8 = cv.take<unsigned>((size_t)NM * segs * PL * nquad * ld);
-        int *hmax = cv.take<int>((size_t)segs * n);
+        int *pmax = cv.take<int>((size_t)segs * n);
         int *sc = cv.take<int>((size_t)segs * m);
+        Stat *stat = cv.take<Stat>((size_t)R * S * 2);
+        int *scl = cv.take<int>(2 * (size_t)R);
         __nv_bfloat16 *cres[2];
         for (int s = 0; s < segs; ++s) cres[s] = cv.take<__nv_bfloat16>((size_t)NM * PL * nbp * kpad[s]);
         if (pass == 0) continue;
@@ -1121,20 +1140,24 @@ static rsdft_status rotate_within(rsdft_ctx *ctx, size_t limit, const RowBlocks 
         ProfScope ps(ctx, RSDFT_K_ROTATE, (real ? 2.0 : 8.0) * (double)n * k * m,
                      16.0 * (double)n * (R + mrows * (1 + (out1 ? 1 : 0) + (base ? 1 : 0))), st, 0);
         RS_CUDA(ctx, cudaMemsetAsync(flag, 0, sizeof(int), st));
-        RS_CUDA(ctx, cudaMemsetAsync(hmax, 0, (size_t)segs * n * sizeof(int), st));
+        RS_CUDA(ctx, cudaMemsetAsync(pmax, 0, (size_t)segs * n * sizeof(int), st));
+        k_row_stat<<<dim3(S, R), 256, 0, st>>>(Y, n, S, stat);
+        k_row_scale<<<cdiv(R, 128), 128, 0, st>>>(stat, S, R, real ? 0 : 1, scl, flag);
+        count_launch(ctx, 2);
+        RS_LAUNCHED(ctx, "k_row_scale");
         CUtensorMap mA, mB[2];
         for (int s = 0; s < segs; ++s) {
             const int r0 = s ? Y.cnt[0] : 0, nr = s ? Y.cnt[1] + Y.cnt[2] : Y.cnt[0];
             // enough CTAs for small grids: at least 8 per SM, at least 16 rows each
             const int want = std::max(1, std::min(cdiv(nr, 16), cdiv(8LL * ctx->num_sms, cdiv(n, 256))));
             const int per = cdiv(cdiv(nr, want), 8) * 8;
-            k_point_max<<<dim3(cdiv(n, 256), cdiv(nr, per)), 256, 0, st>>>(Y, r0, nr, n, per, hmax + (size_t)s * n, flag);
-            k_coef_scale<<<m, 32, 0, st>>>(c, ldc, sg[s], real ? 1 : 0, sc + (size_t)s * m, flag);
+            k_point_max<<<dim3(cdiv(n, 256), cdiv(nr, per)), 256, 0, st>>>(Y, r0, nr, n, per, scl, pmax + (size_t)s * n);
+            k_coef_scale<<<m, 32, 0, st>>>(c, ldc, sg[s], real ? 1 : 0, scl + 2 * r0, sc + (size_t)s * m, flag);
             count_launch(ctx, 2);
         }
         for (int s = 0; s < segs; ++s) {
             k_coef_residues<<<cdiv((long long)nbp * kpad[s] / 2, 256), 256, 0, st>>>(c, ldc, sg[s], real ? 1 : 0, m, nbp, kpad[s],
-                                                                          sc + (size_t)s * m, cres[s], flag);
+                                                                          scl + 2 * (s ? Y.cnt[0] : 0), sc + (size_t)s * m, cres[s], flag);
             count_launch(ctx);
             const long long dims[4] = {kpad[s], nbp, PL, NM};
             const long long str[3] = {2LL * kpad[s], 2LL * kpad[s] * nbp, 2LL * kpad[s] * nbp * PL};
@@ -1167,7 +1190,7 @@ static rsdft_status rotate_within(rsdft_ctx *ctx, size_t limit, const RowBlocks 
             const long long p0 = (long long)ch * ld;
             const int np = (int)std::min<long long>(ld, n - p0);
             if (np <= 0) break;
-            k_residues<<<dim3(cdiv(ld, 1024), R), 256, 0, st>>>(Y, n, p0, ld, R, 0, 1, nullptr, hmax, Y.cnt[0], bits[0],
+            k_residues<<<dim3(cdiv(ld, 1024), R), 256, 0, st>>>(Y, n, p0, ld, R, 0, 1, scl, pmax, Y.cnt[0], bits[0],
                                                                 bits[segs - 1], res, flag);
             count_launch(ctx);
             RS_LAUNCHED(ctx, "k_residues");
@@ -1178,10 +1201,10 @@ static rsdft_status rotate_within(rsdft_ctx *ctx, size_t limit, const RowBlocks 
             else RS_TRY((launch_gemm<false, true>(ctx, mA, mB[0], mB[1], a, st)));
             const dim3 g(cdiv(np, 256), nquad);
             if (real)
-                k_crt_rot<true><<<g, 256, 0, st>>>(out8, segs, m, ld, n, p0, np, hmax, bits[0], bits[segs - 1], sc, m, base,
+                k_crt_rot<true><<<g, 256, 0, st>>>(out8, segs, m, ld, n, p0, np, pmax, bits[0], bits[segs - 1], sc, m, base,
                                                    sign, out0, out1, flag);
             else
-                k_crt_rot<false><<<g, 256, 0, st>>>(out8, segs, m, ld, n, p0, np, hmax, bits[0], bits[segs - 1], sc, m, base,
+                k_crt_rot<false><<<g, 256, 0, st>>>(out8, segs, m, ld, n, p0, np, pmax, bits[0], bits[segs - 1], sc, m, base,
                                                     sign, out0, out1, flag);
             count_launch(ctx);
             RS_LAUNCHED(ctx, "k_crt_rot");

@@ -3,7 +3,10 @@ cost bits."""
 import numpy as np
 import pytest
 
-from tests.gpu_common import R, dev, host, need_gpu, torch
+from oracle.gamma import lobpcg_gamma
+from oracle.lobpcg import lobpcg
+from tests.gpu_common import R, dev, host, need_gpu, pair, torch
+from workloads import draw_x0, draw_x0_real, small_cell
 
 pytestmark = pytest.mark.gpu
 EPS = 2.0 ** -53
@@ -33,4 +36,51 @@ def test_gram_of_uniform_rows(N, real):
     assert ctx.launch_count() - before > 5          # the residue passes ran
     ref = np.outer(v.conj(), v) * ctx.n * ctx.dV
     assert np.all(np.abs(host(g) - ref) <= 12 * EPS * np.abs(ref))
+    ctx.close()
+
+
+def _draw(seed, rows, n, real):
+    return (draw_x0_real if real else draw_x0)(seed, rows, n)
+
+
+@pytest.mark.parametrize("real", [False, True])
+@pytest.mark.parametrize("N,k,m", [((32, 32, 32), 128, 128), ((27, 25, 15), 193, 65)])
+def test_rotation_of_rows_of_any_size(N, k, m, real):
+    """Rows 2^-120 to 2^60 apart.  The scaled rows are rounded to 2^-bits of the largest one of a point, with
+    bits = 62 - h and 2^h < 2 sqrt(2 k): in the norm of an output row at most 4 k 2^-62 (1.5 x 2^-53 for 193), the
+    result to another 2^-53.  Rows and coefficients whose powers of two cancel give the same bits; an FP64 sum is good to
+    some 2^-53 of sum |c| |y|, and eight of them cover both sides."""
+    ctx = _ctx(N)
+    y, s = _draw(3, k, ctx.n, real), 2.0 ** np.random.default_rng(11).integers(-120, 60, k)
+    rotate, out = (ctx.rotate_real if real else ctx.rotate), _empty(real, m, ctx.n)
+    before = ctx.launch_count()
+    rotate(dev(y * s[:, None]), dev(np.eye(k, m).astype(y.dtype)), out)
+    assert ctx.launch_count() - before > 5          # the residue passes ran
+    off = np.linalg.norm(host(out) / s[:m, None] - y[:m], axis=1)
+    assert np.all(off <= 4 * EPS * np.linalg.norm(y[:m], axis=1))
+    c = _draw(4, k, m, real)
+    rotate(dev(y), dev(c), out)
+    plain = host(out).copy()
+    assert np.all(np.abs(plain - c.T @ y) <= 8 * EPS * (np.abs(c).T @ np.abs(y)))
+    rotate(dev(y * s[:, None]), dev(c / s[:, None]), out)
+    assert np.array_equal(plain, host(out))
+    ctx.close()
+
+
+@pytest.mark.parametrize("real", [False, True])
+def test_rotation_of_two_segments(real):
+    """The solvers' rotations of X and [W P] as two sums (45 rows each, no multiple of a K-block) at a size where
+    they run as residues: four iterations against the oracle's, to the LOBPCG tests' bars."""
+    need_gpu()
+    wl = small_cell(N=(32, 30, 32), L=(8.0, 7.5, 8.0), natom=4, nband=45, rcut=2.5)
+    ctx, ham, _ = pair(wl)
+    x0 = wl.x0_real(45) if real else wl.x0()
+    x = dev(x0)
+    eig, res, stats, _ = (ctx.lobpcg_real if real else ctx.lobpcg)(x, ctx.lobpcg_opts(maxit=4, tol=0.0))
+    o = (lobpcg_gamma if real else lobpcg)(ham, x0, maxit=4, tol=0.0)
+    assert stats.iterations == o.iterations
+    assert np.max(np.abs(eig - o.eig)) < 1e-9
+    assert np.max(np.abs(res - o.resnorm)) < 1e-7
+    charge = np.abs(host(x)) ** 2
+    assert np.max(np.abs(charge - np.abs(o.X) ** 2)) < 1e-7 * np.max(charge)
     ctx.close()
