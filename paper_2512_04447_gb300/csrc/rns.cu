@@ -29,7 +29,7 @@
 // and errors against extended precision (150 x 150 over 5,400 points: relative 2.5e-16 against
 // 1.4e-15; rotation 432 -> 144: 1.6e-16 against 9.8e-16).
 //
-// Non-finite values, and magnitudes outside 2^+-400, raise a device flag; then the
+// Non-finite values, and rows of nothing but subnormal ones, raise a device flag; then the
 // kernels here leave their outputs alone and the FP64 kernels launched behind them
 // (which return at once otherwise) do the work, so such inputs give what they gave.
 #include <cuda.h>
@@ -108,8 +108,6 @@ __constant__ Consts K = make_consts();
 constexpr float MAGIC = 12582912.0f;   // 1.5 * 2^23: adding it rounds to an integer
 
 // ---- scales -----------------------------------------------------------------------
-constexpr int EXP_HI = 1023 + 400, EXP_LO = 1023 - 400;   // double exponent fields taken of a row's largest value
-
 // Part of one row: the largest exponent field and the sum of squares in units of 4^(that
 // field - 1023), from the leading 21 bits of each value (integer and FP32 instructions:
 // the FP64 pipe would bound this pass).
@@ -124,7 +122,10 @@ __device__ __forceinline__ void stat_rebase(Stat &a, int e) {
     }
 }
 __device__ __forceinline__ void stat_add(Stat &a, int habs) {
-    if (a.e == 0) return;   // nothing but zeros (or subnormal values) so far
+    if (a.e == 0) {   // nothing but zeros and subnormal values so far
+        if (habs) a.s = 1.0f;
+        return;
+    }
     const int u = habs - ((a.e - 127) << 20);
     const float f = __int_as_float(max(u, 0) << 3);
     a.s = fmaf(f, f, a.s);
@@ -152,8 +153,8 @@ k_row_stat(RowBlocks src, long long n, int S, Stat *__restrict__ part) {
             const long long r = q + u * 256;
             int4 v = make_int4(0, 0, 0, 0);
             if (r < i1) v = __ldg(x + r);
-            hx[u] = v.y & 0x7fffffff;
-            hy[u] = v.w & 0x7fffffff;
+            hx[u] = (v.y & 0x7fffffff) | (v.x != 0);   // (a subnormal value may have nothing but a low word)
+            hy[u] = (v.w & 0x7fffffff) | (v.z != 0);
             mx = max(mx, hx[u]);
             my = max(my, hy[u]);
         }
@@ -184,7 +185,7 @@ k_row_stat(RowBlocks src, long long n, int S, Stat *__restrict__ part) {
 }
 
 // scale[2 row + plane] = s with |row|_2 2^s <= 2^T_ROW; both planes of a complex row (joint)
-// share it.  Raises the flag where the row is not finite or out of range.
+// share it.  Raises the flag where the row is not finite or has no normal number (its values' bits are not known).
 __global__ void k_row_scale(const Stat *__restrict__ part, int S, int rows, int joint, int *__restrict__ scale,
                             int *flag) {
     const int row = blockIdx.x * blockDim.x + threadIdx.x;
@@ -198,12 +199,10 @@ __global__ void k_row_scale(const Stat *__restrict__ part, int S, int rows, int 
     for (int pl = 0; pl < 2; ++pl) {
         int s = 0;
         if (t[pl].s > 0.0f) {
-            if (t[pl].e > EXP_HI || t[pl].e < EXP_LO) atomicExch(flag, 1);
+            if (t[pl].e == 0x7ff || t[pl].e == 0) atomicExch(flag, 1);
             // |row|^2 < 2^(g + 1) 4^(e - 1023) with the truncated bits counted in
             const int g = ilogbf(t[pl].s * 1.001f);
             s = T_ROW - (t[pl].e - 1023) - ((g + 2) >> 1);
-        } else if (t[pl].e > 0) {
-            atomicExch(flag, 1);   // a non-zero row whose statistics underflowed
         }
         scale[2 * row + pl] = s;
     }
@@ -349,7 +348,6 @@ __global__ void k_coef_scale(const double2 *__restrict__ c, int ldc, Seg s, int 
         const double2 v = value(t);
         const double m = fmax(fabs(v.x), fabs(v.y));
         if (!isfinite(v.x) || !isfinite(v.y)) atomicExch(flag, 1);
-        else if (m > 0x1p400 || (m > 0.0 && m < 0x1p-400)) atomicExch(flag, 1);
         if (m > 0.0) top = max(top, ((__double2hiint(m) >> 20) & 0x7ff) - 1023 - ys[real ? t : 2 * t]);
     }
     top = __reduce_max_sync(0xffffffffu, top);

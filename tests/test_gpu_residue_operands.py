@@ -84,3 +84,45 @@ def test_rotation_of_two_segments(real):
     charge = np.abs(host(x)) ** 2
     assert np.max(np.abs(charge - np.abs(o.X) ** 2)) < 1e-7 * np.max(charge)
     ctx.close()
+
+
+@pytest.mark.parametrize("real", [False, True])
+def test_rows_anywhere_in_the_range(real):
+    """Powers of two of rows cancel to the bit wherever in the range they lie, and values without a normal number count:
+    a row of them against numpy's product of the scaled rows, to 8 x 2^-53 of their norms' product."""
+    ctx = _ctx((20, 20, 20))
+    x = _draw(1, 20, ctx.n, real)
+    gram = ctx.gram_real if real else ctx.gram
+    ref, g = _empty(real, 20, 20), _empty(real, 20, 20)
+    gram(dev(x), dev(x), ref)
+    gram(dev(x * 2.0 ** -450), dev(x * 2.0 ** 450), g)
+    assert np.array_equal(host(ref), host(g))
+    gram(dev(x * 2.0 ** 900), dev(x * 2.0 ** -900), g)
+    assert np.array_equal(host(ref), host(g))
+    for bits in (3, 20, 40):
+        a = x.copy()
+        a[4] = np.round(x[4].real * 2.0 ** bits)
+        b = a.copy()
+        b[4] = np.ldexp(a[4].real, -1074)
+        gram(dev(b), dev(x * 2.0 ** 390), g)
+        got = host(g) * np.where(np.arange(20) == 4, 2.0 ** (1074 - 390), 2.0 ** -390)[:, None]
+        bound = np.linalg.norm(a, axis=1)[:, None] * np.linalg.norm(x, axis=1)[None] * ctx.dV
+        assert np.all(np.abs(got - a.conj() @ x.T * ctx.dV) <= 8 * EPS * bound), bits
+    ctx.close()
+
+
+@pytest.mark.parametrize("real", [False, True])
+def test_a_point_of_subnormal_values_leaves_the_others(real):
+    ctx = _ctx((24, 24, 24))
+    y, c = _draw(5, 128, ctx.n, real), _draw(6, 128, 128, real)
+    rotate, one, two = (ctx.rotate_real if real else ctx.rotate), _empty(real, 128, ctx.n), _empty(real, 128, ctx.n)
+    rotate(dev(y), dev(c), one)
+    k = np.arange(1.0, 129.0)
+    y[:, 5] = np.ldexp(k, -1074)
+    rotate(dev(y), dev(c), two)
+    rest = np.arange(ctx.n) != 5
+    one, two = host(one), host(two)
+    assert np.array_equal(one[:, rest], two[:, rest])
+    got = np.ldexp(two[:, 5].real, 1074)
+    assert np.all(np.abs(got - (c.T @ k).real) <= 1.0)          # whole numbers of 2^-1074, rounded twice
+    ctx.close()
