@@ -633,6 +633,8 @@ void rsdft_destroy(rsdft_ctx *ctx) {
     cudaDeviceSynchronize();
     for (auto &r : ctx->prof.pending) { cudaEventDestroy(r.a); cudaEventDestroy(r.b); }
     for (auto e : ctx->prof.pool) cudaEventDestroy(e);
+    for (auto &r : ctx->rns.slots)
+        if (r->done) cudaEventDestroy(r->done);
     for (void *p : ctx->owned) cudaFree(p);
     if (ctx->ws.hbuf) cudaFreeHost(ctx->ws.hbuf);
     cudaGetLastError();

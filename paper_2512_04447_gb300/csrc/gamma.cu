@@ -483,19 +483,18 @@ rsdft_status gram_pair(rsdft_ctx *ctx, const RowBlocks &A, const RowBlocks &B, d
     const int nb = B.cnt[0] + B.cnt[1] + B.cnt[2];
     if (na <= 0 || nb <= 0) return RSDFT_OK;
     if (sym && na != nb) return fail(ctx, RSDFT_E_INVALID, "symmetric gram needs na == nb");
-    bool used = false;
-    RS_TRY(rns_gram(ctx, A, B, nullptr, true, sym, g, nullptr, ldg, scale, st, &used));
-    return gram_pair_fp64(ctx, A, B, na, nb, g, ldg, sym, scale, used ? ctx->rns.flag : nullptr, st);
+    RnsLease lease(ctx, st);
+    RS_TRY(rns_gram(ctx, A, B, nullptr, true, sym, g, nullptr, ldg, scale, st, lease));
+    return gram_pair_fp64(ctx, A, B, na, nb, g, ldg, sym, scale, lease.guard(), st);
 }
 
 // g_s = <Y|Y> and g_h = <Y|HY>, both symmetric
 static rsdft_status gram_pair_sh(rsdft_ctx *ctx, const RowBlocks &Y, const RowBlocks &HY, double2 *gs, double2 *gh, int k,
                                  cudaStream_t st) {
-    bool used = false;
-    RS_TRY(rns_gram(ctx, Y, Y, &HY, true, true, gs, gh, k, ctx->dV, st, &used));
-    const int *guard = used ? ctx->rns.flag : nullptr;
-    RS_TRY(gram_pair_fp64(ctx, Y, Y, k, k, gs, k, true, ctx->dV, guard, st));
-    return gram_pair_fp64(ctx, Y, HY, k, k, gh, k, true, ctx->dV, guard, st);
+    RnsLease lease(ctx, st);
+    RS_TRY(rns_gram(ctx, Y, Y, &HY, true, true, gs, gh, k, ctx->dV, st, lease));
+    RS_TRY(gram_pair_fp64(ctx, Y, Y, k, k, gs, k, true, ctx->dV, lease.guard(), st));
+    return gram_pair_fp64(ctx, Y, HY, k, k, gh, k, true, ctx->dV, lease.guard(), st);
 }
 // ---- Ritz rotation on pair rows ---------------------------------------------------------
 // out0[b] = base[b] + sign sum_i Re c[i][b] y_i over the real bands y_i of the
@@ -616,9 +615,9 @@ rsdft_status rotate_pair(rsdft_ctx *ctx, const RowBlocks &Y, const double2 *c, i
     const int k = Y.cnt[0] + Y.cnt[1] + Y.cnt[2];
     const int kp = pairs_of(Y.cnt[0]) + pairs_of(Y.cnt[1]) + pairs_of(Y.cnt[2]);
     const int mp = pairs_of(m);
-    bool used = false;
-    RS_TRY(rns_rotate(ctx, Y, c, ldc, m, true, base, sign, out0, out1, st, &used));
-    const int *guard = used ? ctx->rns.flag : nullptr;
+    RnsLease lease(ctx, st);
+    RS_TRY(rns_rotate(ctx, Y, c, ldc, m, true, base, sign, out0, out1, st, lease));
+    const int *guard = lease.guard();
     ProfScope ps(ctx, RSDFT_K_ROTATE, guard ? 0.0 : 2.0 * (double)ctx->n * k * m,
                  guard ? 0.0 : (double)sizeof(double2) * (double)ctx->n * (kp + mp + (out1 ? mp : 0) + (base ? mp : 0)), st);
     // output tile of 16 or 32 pair rows, the one with less padding (ties: 32)
@@ -629,7 +628,7 @@ rsdft_status rotate_pair(rsdft_ctx *ctx, const RowBlocks &Y, const double2 *c, i
         k_rotate_pair<2><<<dim3(cdiv(mp, 32), cdiv(ctx->n, GRPTS)), GR_THREADS, 0, st>>>(Y, c, ldc, m, ctx->n, base,
                                                                                         sign, out0, out1, guard);
     RS_LAUNCHED(ctx, "k_rotate_pair");
-    if (used && base == out0) return rns_poison(ctx, out0, (long long)mp * ctx->n, st);
+    if (lease.used && base == out0) return rns_poison(ctx, out0, (long long)mp * ctx->n, st, lease);
     return RSDFT_OK;
 }
 

@@ -258,17 +258,16 @@ rsdft_status gram_t(rsdft_ctx *ctx, const RowBlocksT<V> &A, const RowBlocksT<V> 
 
 rsdft_status gram(rsdft_ctx *ctx, const RowBlocks &A, const RowBlocks &B, double2 *g, int ldg,
                   bool hermitian, double scale, cudaStream_t st) {
-    bool used = false;
-    RS_TRY(rns_gram(ctx, A, B, nullptr, false, hermitian, g, nullptr, ldg, scale, st, &used));
-    return gram_t<double2>(ctx, A, B, g, ldg, hermitian, scale, used ? ctx->rns.flag : nullptr, st);
+    RnsLease lease(ctx, st);
+    RS_TRY(rns_gram(ctx, A, B, nullptr, false, hermitian, g, nullptr, ldg, scale, st, lease));
+    return gram_t<double2>(ctx, A, B, g, ldg, hermitian, scale, lease.guard(), st);
 }
 rsdft_status gram_sh(rsdft_ctx *ctx, const RowBlocks &Y, const RowBlocks &HY, double2 *gs, double2 *gh, int ldg,
                      double scale, cudaStream_t st) {
-    bool used = false;
-    RS_TRY(rns_gram(ctx, Y, Y, &HY, false, true, gs, gh, ldg, scale, st, &used));
-    const int *guard = used ? ctx->rns.flag : nullptr;
-    RS_TRY(gram_t<double2>(ctx, Y, Y, gs, ldg, true, scale, guard, st));
-    return gram_t<double2>(ctx, Y, HY, gh, ldg, true, scale, guard, st);
+    RnsLease lease(ctx, st);
+    RS_TRY(rns_gram(ctx, Y, Y, &HY, false, true, gs, gh, ldg, scale, st, lease));
+    RS_TRY(gram_t<double2>(ctx, Y, Y, gs, ldg, true, scale, lease.guard(), st));
+    return gram_t<double2>(ctx, Y, HY, gh, ldg, true, scale, lease.guard(), st);
 }
 rsdft_status gram32(rsdft_ctx *ctx, const RowBlocksT<float2> &A, const RowBlocksT<float2> &B,
                     double2 *g, int ldg, bool hermitian, double scale, cudaStream_t st) {
@@ -427,10 +426,10 @@ rsdft_status rotate(rsdft_ctx *ctx, const RowBlocks &Y, const double2 *c, int ld
                     const double2 *base, int sign, double2 *out0, double2 *out1,
                     cudaStream_t st) {
     if (m <= 0) return RSDFT_OK;
-    bool used = false;
-    RS_TRY(rns_rotate(ctx, Y, c, ldc, m, false, base, sign, out0, out1, st, &used));
-    RS_TRY(rotate_t<double2>(ctx, Y, c, ldc, m, base, sign, out0, out1, used ? ctx->rns.flag : nullptr, st));
-    return used && base == out0 ? rns_poison(ctx, out0, (long long)m * ctx->n, st) : RSDFT_OK;
+    RnsLease lease(ctx, st);
+    RS_TRY(rns_rotate(ctx, Y, c, ldc, m, false, base, sign, out0, out1, st, lease));
+    RS_TRY(rotate_t<double2>(ctx, Y, c, ldc, m, base, sign, out0, out1, lease.guard(), st));
+    return lease.used && base == out0 ? rns_poison(ctx, out0, (long long)m * ctx->n, st, lease) : RSDFT_OK;
 }
 rsdft_status rotate32(rsdft_ctx *ctx, const RowBlocksT<float2> &Y, const double2 *c, int ldc, int m,
                       const float2 *base, int sign, float2 *out0, float2 *out1, cudaStream_t st) {

@@ -908,20 +908,100 @@ using namespace rns;
 // 2^32).  Where that does not fit, an eighth of it is tried, then the FP64 kernels run.
 constexpr size_t RNS_BYTES = (size_t)1 << 31;
 
-// Whether there is room for a call's residues: growing takes at most a quarter of the free memory.
-static bool rns_buffer(rsdft_ctx *ctx, size_t bytes, cudaStream_t st) {
-    RnsWork &w = ctx->rns;
-    if (bytes > w.buf.bytes) {
-        size_t free_now = 0, total = 0;
-        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-        cudaThreadExchangeStreamCaptureMode(&mode);
-        if (cudaMemGetInfo(&free_now, &total) != cudaSuccess) cudaGetLastError();
-        cudaThreadExchangeStreamCaptureMode(&mode);
-        if (bytes > (free_now + w.buf.bytes) / 4) return false;
+// The end of a capture's last graph
+static void graphs_gone(void *p) {
+    auto *alive = static_cast<std::shared_ptr<std::atomic<bool>> *>(p);
+    (*alive)->store(false);
+    delete alive;
+}
+
+// Whether nothing that was or may be launched uses the slot any more
+static bool slot_free(const RnsSlot &s) {
+    if (s.capture) return !s.graphs->load();
+    const bool done = s.done && cudaEventQuery(s.done) == cudaSuccess;
+    cudaGetLastError();
+    return done;
+}
+
+// A slot for the lease's stream, of `bytes` already if there is one to choose from (RnsSlot)
+static rsdft_status take_slot(RnsLease &l, size_t bytes) {
+    if (l.slot) return RSDFT_OK;
+    RnsWork &w = l.ctx->rns;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    unsigned long long capture = 0, stream = 0;
+    cudaGraph_t graph = nullptr;
+    if (l.st && l.st != cudaStreamLegacy) RS_CUDA(l.ctx, cudaStreamGetCaptureInfo(l.st, &cs, &capture, &graph));
+    l.capturing = cs != cudaStreamCaptureStatusNone;
+    if (l.capturing) {
+        stream = reinterpret_cast<uintptr_t>(l.st);   // (the id of a capturing stream cannot be asked for)
+    } else {
+        capture = 0;
+        RS_CUDA(l.ctx, cudaStreamGetId(l.st, &stream));
     }
-    const bool ok = grow(ctx, w.fbuf, 64, st) == RSDFT_OK && grow(ctx, w.buf, bytes, st) == RSDFT_OK;
+    RnsSlot *own = nullptr, *idle = nullptr, *oldest = nullptr;
+    int eager = 0;
+    for (auto &p : w.slots) {
+        RnsSlot &s = *p;
+        if (s.capture == capture && s.stream == stream) own = &s;
+        else if (slot_free(s) && (!idle || (idle->buf.bytes < bytes && s.buf.bytes > idle->buf.bytes))) idle = &s;
+        if (!s.capture) {
+            ++eager;
+            if (!oldest || s.use < oldest->use) oldest = &s;
+        }
+    }
+    // (a capture cannot give back a smaller buffer for a larger one)
+    if (l.capturing && idle && idle->buf.bytes < bytes) idle = nullptr;
+    RnsSlot *s = own ? own : idle;
+    if (!s && !l.capturing && eager >= RNS_SLOTS) {
+        s = oldest;
+        RS_CUDA(l.ctx, cudaStreamWaitEvent(l.st, s->done, 0));
+    }
+    if (!s) {
+        w.slots.emplace_back(new RnsSlot);
+        s = w.slots.back().get();
+    }
+    if (s != own) {
+        s->stream = stream;
+        s->capture = capture;
+        s->graphs.reset();
+        s->buf.captured = s->fbuf.captured = false;
+        if (l.capturing) {
+            s->graphs = std::make_shared<std::atomic<bool>>(true);
+            auto *alive = new std::shared_ptr<std::atomic<bool>>(s->graphs);
+            cudaUserObject_t obj = nullptr;
+            cudaError_t e = cudaUserObjectCreate(&obj, alive, graphs_gone, 1, cudaUserObjectNoDestructorSync);
+            if (e != cudaSuccess) delete alive;
+            else e = cudaGraphRetainUserObject(graph, obj, 1, cudaGraphUserObjectMove);
+            RS_CUDA(l.ctx, e);
+        }
+    }
+    if (!l.capturing && !s->done) RS_CUDA(l.ctx, cudaEventCreateWithFlags(&s->done, cudaEventDisableTiming));
+    s->use = ++w.uses;
+    l.slot = s;
+    return RSDFT_OK;
+}
+
+RnsLease::~RnsLease() {
+    if (slot && !capturing && cudaEventRecord(slot->done, st) != cudaSuccess) {
+        cudaGetLastError();
+        cudaStreamSynchronize(st);
+    }
+}
+
+// Whether there is room for a call's residues: growing takes at most a quarter of the free memory.
+static bool rns_buffer(rsdft_ctx *ctx, size_t bytes, cudaStream_t st, RnsLease &lease) {
+    // this or another thread may be capturing: nothing here is work of a stream
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    bool ok = take_slot(lease, bytes) == RSDFT_OK;
+    if (ok && bytes > lease.slot->buf.bytes) {
+        size_t free_now = 0, total = 0;
+        if (cudaMemGetInfo(&free_now, &total) != cudaSuccess) cudaGetLastError();
+        if (bytes > (free_now + lease.slot->buf.bytes) / 4) ok = false;
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    ok = ok && grow(ctx, lease.slot->fbuf, 64, st) == RSDFT_OK && grow(ctx, lease.slot->buf, bytes, st) == RSDFT_OK;
     if (!ok) ctx->err.clear();
-    w.flag = static_cast<int *>(w.fbuf.p);
     return ok;
 }
 
@@ -972,7 +1052,7 @@ static bool rotation_wins(double n, int rows, int k, int m, bool real, int items
 
 static rsdft_status gram_within(rsdft_ctx *ctx, size_t limit, const RowBlocks &A0, const RowBlocks &B0,
                                 const RowBlocks *B1, bool real, bool herm, double2 *g0, double2 *g1, int ldg,
-                                double scale, cudaStream_t st, bool *used) {
+                                double scale, cudaStream_t st, RnsLease &lease) {
     const int na = rows_of(A0), nb = rows_of(B0), blocks = B1 ? 2 : 1;
     const RowBlocks A = real ? pair_rows(A0) : A0, B = real ? pair_rows(B0) : B0;
     const int ra = rows_of(A), rb = rows_of(B);
@@ -1007,17 +1087,17 @@ static rsdft_status gram_within(rsdft_ctx *ctx, size_t limit, const RowBlocks &A
     Carver cv{nullptr};
     for (int pass = 0; pass < 2; ++pass) {
         if (pass == 1) {
-            if (!rns_buffer(ctx, cv.at, st)) return RSDFT_OK;
-            cv = Carver{(unsigned char *)ctx->rns.buf.p};
+            if (!rns_buffer(ctx, cv.at, st, lease)) return RSDFT_OK;
+            cv = Carver{(unsigned char *)lease.slot->buf.p};
         }
         __nv_bfloat16 *res = cv.take<__nv_bfloat16>((size_t)NM * R * 2 * ld);
         short *out16 = cv.take<short>(out_elems);
         Stat *stat = cv.take<Stat>((size_t)R * S * 2);
         int *scl = cv.take<int>(2 * (size_t)R);
         if (pass == 0) continue;
-        int *flag = ctx->rns.flag;
+        int *flag = lease.flag();
         const int rowB = same ? 0 : ra;
-        *used = true;
+        lease.used = true;
         ProfScope ps(ctx, RSDFT_K_GRAM, (real ? 2.0 : 8.0) * (double)n * frac * na * (herm ? na + 1.0 : (double)nb),
                      16.0 * (double)n * R, st, 0);
         RS_CUDA(ctx, cudaMemsetAsync(flag, 0, sizeof(int), st));
@@ -1081,17 +1161,16 @@ static rsdft_status gram_within(rsdft_ctx *ctx, size_t limit, const RowBlocks &A
 }
 
 rsdft_status rns_gram(rsdft_ctx *ctx, const RowBlocks &A, const RowBlocks &B0, const RowBlocks *B1, bool real, bool herm,
-                      double2 *g0, double2 *g1, int ldg, double scale, cudaStream_t st, bool *used) {
-    *used = false;
+                      double2 *g0, double2 *g1, int ldg, double scale, cudaStream_t st, RnsLease &lease) {
     if (!gram_wins(ctx->n)) return RSDFT_OK;
-    for (size_t limit = RNS_BYTES; limit >= RNS_BYTES / 8 && !*used; limit /= 8)
-        RS_TRY(gram_within(ctx, limit, A, B0, B1, real, herm, g0, g1, ldg, scale, st, used));
+    for (size_t limit = RNS_BYTES; limit >= RNS_BYTES / 8 && !lease.used; limit /= 8)
+        RS_TRY(gram_within(ctx, limit, A, B0, B1, real, herm, g0, g1, ldg, scale, st, lease));
     return RSDFT_OK;
 }
 
 static rsdft_status rotate_within(rsdft_ctx *ctx, size_t limit, const RowBlocks &Y0, const double2 *c, int ldc, int m,
                                   bool real, const double2 *base, int sign, double2 *out0, double2 *out1,
-                                  cudaStream_t st, bool *used) {
+                                  cudaStream_t st, RnsLease &lease) {
     const RowBlocks Y = real ? pair_rows(Y0) : Y0;
     const int R = rows_of(Y), k = rows_of(Y0);
     const long long n = ctx->n;
@@ -1120,8 +1199,8 @@ static rsdft_status rotate_within(rsdft_ctx *ctx, size_t limit, const RowBlocks 
     Carver cv{nullptr};
     for (int pass = 0; pass < 2; ++pass) {
         if (pass == 1) {
-            if (!rns_buffer(ctx, cv.at, st)) return RSDFT_OK;
-            cv = Carver{(unsigned char *)ctx->rns.buf.p};
+            if (!rns_buffer(ctx, cv.at, st, lease)) return RSDFT_OK;
+            cv = Carver{(unsigned char *)lease.slot->buf.p};
         }
         __nv_bfloat16 *res = cv.take<__nv_bfloat16>((size_t)NM * R * 2 * ld);
         unsigned *out8 = cv.take<unsigned>((size_t)NM * segs * PL * nquad * ld);
@@ -1132,8 +1211,8 @@ static rsdft_status rotate_within(rsdft_ctx *ctx, size_t limit, const RowBlocks 
         __nv_bfloat16 *cres[2];
         for (int s = 0; s < segs; ++s) cres[s] = cv.take<__nv_bfloat16>((size_t)NM * PL * nbp * kpad[s]);
         if (pass == 0) continue;
-        int *flag = ctx->rns.flag;
-        *used = true;
+        int *flag = lease.flag();
+        lease.used = true;
         const int mrows = real ? pairs_up(m) : m;
         ProfScope ps(ctx, RSDFT_K_ROTATE, (real ? 2.0 : 8.0) * (double)n * k * m,
                      16.0 * (double)n * (R + mrows * (1 + (out1 ? 1 : 0) + (base ? 1 : 0))), st, 0);
@@ -1212,19 +1291,18 @@ static rsdft_status rotate_within(rsdft_ctx *ctx, size_t limit, const RowBlocks 
 }
 
 rsdft_status rns_rotate(rsdft_ctx *ctx, const RowBlocks &Y, const double2 *c, int ldc, int m, bool real,
-                        const double2 *base, int sign, double2 *out0, double2 *out1, cudaStream_t st, bool *used) {
-    *used = false;
+                        const double2 *base, int sign, double2 *out0, double2 *out1, cudaStream_t st, RnsLease &lease) {
     const int segs = Y.cnt[1] + Y.cnt[2] > 0 ? 2 : 1, nt = cdiv(m, real ? 256 : 128);
     if (Y.cnt[0] <= 0 ||
         !rotation_wins((double)ctx->n, rows_of(real ? pair_rows(Y) : Y), rows_of(Y), m, real, NM * segs * nt))
         return RSDFT_OK;
-    for (size_t limit = RNS_BYTES; limit >= RNS_BYTES / 8 && !*used; limit /= 8)
-        RS_TRY(rotate_within(ctx, limit, Y, c, ldc, m, real, base, sign, out0, out1, st, used));
+    for (size_t limit = RNS_BYTES; limit >= RNS_BYTES / 8 && !lease.used; limit /= 8)
+        RS_TRY(rotate_within(ctx, limit, Y, c, ldc, m, real, base, sign, out0, out1, st, lease));
     return RSDFT_OK;
 }
 
-rsdft_status rns_poison(rsdft_ctx *ctx, double2 *out, long long cnt, cudaStream_t st) {
-    k_poison<<<std::min(cdiv(cnt, 256), 4 * ctx->num_sms), 256, 0, st>>>(out, cnt, ctx->rns.flag);
+rsdft_status rns_poison(rsdft_ctx *ctx, double2 *out, long long cnt, cudaStream_t st, const RnsLease &lease) {
+    k_poison<<<std::min(cdiv(cnt, 256), 4 * ctx->num_sms), 256, 0, st>>>(out, cnt, lease.flag());
     count_launch(ctx);
     RS_LAUNCHED(ctx, "k_poison");
     return RSDFT_OK;

@@ -2,11 +2,13 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <atomic>
 #include <cstdio>
 #include <cstring>
 #include <string>
 #include <functional>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <vector>
 
@@ -150,11 +152,21 @@ struct FixFft {
     Scratch meta;                            // exponents of the planes and slabs in flight
 };
 
-// Residue-arithmetic products (rns.cu): residue planes and scratch, and the device flag
-// that hands a call back to the FP64 kernels.
-struct RnsWork {
+// Memory of a residue product (rns.cu): residue planes and sums, and the device flag that hands
+// a call back to the FP64 kernels.  Calls on one stream share a slot; a call on another one gets a slot whose last
+// work is done, or one of its own (at most RNS_SLOTS outside captures, then it waits for the one used longest ago).  A
+// slot that a capture has used belongs to that stream and capture until the last graph made of it is gone.
+constexpr int RNS_SLOTS = 4;
+struct RnsSlot {
     Scratch buf, fbuf;
-    int *flag = nullptr;
+    unsigned long long stream = 0, capture = 0;     // ids of the stream that used it last, of its capture (0: none)
+    long long use = 0;                              // counts uses
+    cudaEvent_t done = nullptr;                     // end of the last use outside captures
+    std::shared_ptr<std::atomic<bool>> graphs;      // whether a graph that uses it may still be launched
+};
+struct RnsWork {
+    std::vector<std::unique_ptr<RnsSlot>> slots;
+    long long uses = 0;
 };
 
 struct Profiler {
@@ -294,18 +306,30 @@ rsdft_status gram_sh(rsdft_ctx *ctx, const RowBlocks &Y, const RowBlocks &HY, do
 rsdft_status rotate(rsdft_ctx *ctx, const RowBlocks &Y, const double2 *c, int ldc, int m,
                     const double2 *base, int sign, double2 *out0, double2 *out1,
                     cudaStream_t st);
+// A call's hold on a slot, from the product's first launch to the last one that reads its flag.
+struct RnsLease {
+    rsdft_ctx *ctx;
+    cudaStream_t st;
+    RnsSlot *slot = nullptr;
+    bool capturing = false, used = false;
+    RnsLease(rsdft_ctx *c, cudaStream_t s) : ctx(c), st(s) {}
+    RnsLease(const RnsLease &) = delete;
+    ~RnsLease();
+    int *flag() const { return static_cast<int *>(slot->fbuf.p); }
+    const int *guard() const { return used ? flag() : nullptr; }
+};
 // The same on the tensor cores by residue arithmetic (rns.cu), exact to the rounding of the
-// operands; *used = false and nothing launched where the FP64 kernels are faster or the
+// operands; lease.used stays false and nothing is launched where the FP64 kernels are faster or the
 // scratch does not fit.  When used, the caller launches its FP64 kernels behind them guarded
-// by ctx->rns.flag: they return at once unless the flag asks for them.  Blocks hold complex
+// by lease.guard(): they return at once unless the flag asks for them.  Blocks hold complex
 // rows (real: counts are real bands, rows are pair rows).  B1 (optional): g1 = <A|B1>, its
 // rows like B0's.
 rsdft_status rns_gram(rsdft_ctx *ctx, const RowBlocks &A, const RowBlocks &B0, const RowBlocks *B1, bool real,
-                      bool herm, double2 *g0, double2 *g1, int ldg, double scale, cudaStream_t st, bool *used);
+                      bool herm, double2 *g0, double2 *g1, int ldg, double scale, cudaStream_t st, RnsLease &lease);
 rsdft_status rns_rotate(rsdft_ctx *ctx, const RowBlocks &Y, const double2 *c, int ldc, int m, bool real,
-                        const double2 *base, int sign, double2 *out0, double2 *out1, cudaStream_t st, bool *used);
+                        const double2 *base, int sign, double2 *out0, double2 *out1, cudaStream_t st, RnsLease &lease);
 // After the guarded FP64 rotation of an in-place update (base == out0).
-rsdft_status rns_poison(rsdft_ctx *ctx, double2 *out, long long cnt, cudaStream_t st);
+rsdft_status rns_poison(rsdft_ctx *ctx, double2 *out, long long cnt, cudaStream_t st, const RnsLease &lease);
 // FP32 operands (mixed form): products and CTA-level sums in FP32, Gram
 // partials reduced in FP64; rotation coefficients rounded to FP32.
 rsdft_status gram32(rsdft_ctx *ctx, const RowBlocksT<float2> &A, const RowBlocksT<float2> &B,
