@@ -647,9 +647,11 @@ int threads_for(size_t smem, int points) {
     return smem <= 113 * 1024 ? 384 : 768;
 }
 
-rsdft_status ensure_meta(rsdft_ctx *ctx, int nb, Meta **planes, Meta **slabs, cudaStream_t st) {
-    RS_TRY(grow(ctx, ctx->fix.meta, (size_t)nb * (ctx->N[1] + ctx->N[2]) * sizeof(Meta), st));
-    *planes = static_cast<Meta *>(ctx->fix.meta.p);
+// buf: the buffer between the passes, which says whose exponents
+rsdft_status ensure_meta(rsdft_ctx *ctx, const double2 *buf, int nb, Meta **planes, Meta **slabs, cudaStream_t st) {
+    Scratch &m = buf == ctx->scf.cbuf ? ctx->fix.field_meta : ctx->fix.meta;
+    RS_TRY(grow(ctx, m, (size_t)nb * (ctx->N[1] + ctx->N[2]) * sizeof(Meta), st));
+    *planes = static_cast<Meta *>(m.p);
     *slabs = *planes + (size_t)nb * ctx->N[2];
     return RSDFT_OK;
 }
@@ -677,7 +679,7 @@ rsdft_status fft_xy_forward(rsdft_ctx *ctx, Src kind, const double2 *src, const 
     if (nb <= 0) return RSDFT_OK;
     RS_TRY(check_plane(ctx));
     Meta *mp, *ms;
-    RS_TRY(ensure_meta(ctx, nb, &mp, &ms, st));
+    RS_TRY(ensure_meta(ctx, dst, nb, &mp, &ms, st));
     const int RS = plane_stride(ctx);
     const size_t sm = HEAD + (size_t)RS * ctx->N[1] * sizeof(I2);
     const dim3 grid(ctx->N[2], nb);
@@ -714,7 +716,7 @@ rsdft_status fft_z_mid(rsdft_ctx *ctx, Mid mid, double2 *buf, const double *tkin
     if (nb <= 0) return RSDFT_OK;
     RS_TRY(check_plane(ctx));
     Meta *mp, *ms;
-    RS_TRY(ensure_meta(ctx, nb, &mp, &ms, st));
+    RS_TRY(ensure_meta(ctx, buf, nb, &mp, &ms, st));
     size_t sm = HEAD + (size_t)ctx->N[0] * ctx->N[2] * sizeof(I2) + SHIFTS;
     const size_t tabb = (size_t)(ctx->N[0] / 2 + 1) * (ctx->N[2] / 2 + 1) * sizeof(double);
     int table = 0;
@@ -750,7 +752,7 @@ rsdft_status fft_xy_inverse(rsdft_ctx *ctx, const double2 *buf, const double2 *p
     if (nb <= 0) return RSDFT_OK;
     RS_TRY(check_plane(ctx));
     Meta *mp, *ms;
-    RS_TRY(ensure_meta(ctx, nb, &mp, &ms, st));
+    RS_TRY(ensure_meta(ctx, buf, nb, &mp, &ms, st));
     const int RS = plane_stride(ctx);
     size_t sm = plane_smem(ctx);
     int room = 0;

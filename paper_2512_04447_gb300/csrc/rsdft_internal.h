@@ -149,7 +149,8 @@ struct FixFft {
     int kexp = 0;
     const double *g2abs[3] = {};             // G_a^2 by |frequency index|
     const unsigned char *fabs[3] = {};       // |frequency index| by position
-    Scratch meta;                            // exponents of the planes and slabs in flight
+    Scratch meta, field_meta;                // exponents of the planes and slabs in flight: of orbitals (ws.T1),
+                                             // of the field solvers' buffer (scf.cbuf)
 };
 
 // Memory of a residue product (rns.cu): residue planes and sums, and the device flag that hands
@@ -254,7 +255,8 @@ inline int cdiv(long long a, long long b) { return (int)((a + b - 1) / b); }
 enum class Mid { Kinetic, Tpa, Hartree, GradX, GradY, GradZ };   // FP32: Kinetic and Tpa
 enum class Src { Plain, Residual, RealField };
 // FP64 passes (fft_fix.cu).  Between them the buffer holds fixed-point values whose exponents are kept
-// in the context, so the three passes of a transform follow one another on one stream.
+// in the context, for the orbitals' buffer and the field solvers' one each, so the three passes of a transform
+// follow one another on one stream.
 // Forward xy-plane pass: src -> dst ([nb][n] complex).  Src::Residual reads
 // hx[act[b]] - theta[act[b]] x[act[b]]; Src::RealField reads a real [n] field
 // (nb must be 1).

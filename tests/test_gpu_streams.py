@@ -126,3 +126,25 @@ def test_memory_of_captured_calls_is_used_again():
     torch.cuda.empty_cache()
     assert before - torch.cuda.mem_get_info()[0] < 8 * planes
     ctx.close()
+
+
+def test_field_solvers_beside_h_psi():
+    need_gpu()
+    ctx, _, _ = pair(diamond8_24())
+    x = dev(draw_x0(1, 64, ctx.n))
+    rho = dev(np.random.default_rng(2).uniform(0.1, 1.0, ctx.n))
+    h, v, e, u = _empty(64, ctx.n), *(torch.zeros_like(rho) for _ in range(3))
+    ctx.apply_h(x, h)
+    ctx.hartree(rho, v)
+    ctx.xc_pbe(rho, e, u)
+    ref = [host(t).copy() for t in (h, v, e, u)]
+    for t in (h, v, e, u):
+        t.zero_()
+
+    def fields():
+        ctx.hartree(rho, v)
+        ctx.xc_pbe(rho, e, u)
+
+    _beside(lambda: ctx.apply_h(x, h), fields)
+    assert all(np.array_equal(host(t), r) for t, r in zip((h, v, e, u), ref))
+    ctx.close()
