@@ -905,7 +905,8 @@ using namespace rns;
 // ---- host side ---------------------------------------------------------------------------
 // Bytes of residues held at a time (the points go in chunks of that size): a chunk's launches end
 // with a partly filled wave and the residues' way out (432 x 432: 9.0 ms with 2^30, 8.7 with 2^31, 8.5 with
-// 2^32).  Where that does not fit, an eighth of it is tried, then the FP64 kernels run.
+// 2^32).  Where that does not fit, an eighth and a 64th of it are tried (4,096 points at least: 0.1 GB for 432
+// rows), and the FP64 kernels run only where even that does not: chunks change no bit of a result.
 constexpr size_t RNS_BYTES = (size_t)1 << 31;
 
 // The end of a capture's last graph
@@ -1163,7 +1164,7 @@ static rsdft_status gram_within(rsdft_ctx *ctx, size_t limit, const RowBlocks &A
 rsdft_status rns_gram(rsdft_ctx *ctx, const RowBlocks &A, const RowBlocks &B0, const RowBlocks *B1, bool real, bool herm,
                       double2 *g0, double2 *g1, int ldg, double scale, cudaStream_t st, RnsLease &lease) {
     if (!gram_wins(ctx->n)) return RSDFT_OK;
-    for (size_t limit = RNS_BYTES; limit >= RNS_BYTES / 8 && !lease.used; limit /= 8)
+    for (size_t limit = RNS_BYTES; limit >= RNS_BYTES / 64 && !lease.used; limit /= 8)
         RS_TRY(gram_within(ctx, limit, A, B0, B1, real, herm, g0, g1, ldg, scale, st, lease));
     return RSDFT_OK;
 }
@@ -1296,7 +1297,7 @@ rsdft_status rns_rotate(rsdft_ctx *ctx, const RowBlocks &Y, const double2 *c, in
     if (Y.cnt[0] <= 0 ||
         !rotation_wins((double)ctx->n, rows_of(real ? pair_rows(Y) : Y), rows_of(Y), m, real, NM * segs * nt))
         return RSDFT_OK;
-    for (size_t limit = RNS_BYTES; limit >= RNS_BYTES / 8 && !lease.used; limit /= 8)
+    for (size_t limit = RNS_BYTES; limit >= RNS_BYTES / 64 && !lease.used; limit /= 8)
         RS_TRY(rotate_within(ctx, limit, Y, c, ldc, m, real, base, sign, out0, out1, st, lease));
     return RSDFT_OK;
 }

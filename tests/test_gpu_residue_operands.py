@@ -126,3 +126,27 @@ def test_a_point_of_subnormal_values_leaves_the_others(real):
     got = np.ldexp(two[:, 5].real, 1074)
     assert np.all(np.abs(got - (c.T @ k).real) <= 1.0)          # whole numbers of 2^-1074, rounded twice
     ctx.close()
+
+
+@pytest.mark.parametrize("real", [False, True])
+def test_short_memory_changes_no_bit(real):
+    """Chunks of points as small as 4,096 where the device's memory is nearly all taken."""
+    N = (64, 64, 64)
+    ctx, short = _ctx(N), _ctx(N)
+    a, b, c = (dev(_draw(i, k, ctx.n if i < 3 else 96, real)) for i, k in ((1, 160), (2, 160), (3, 160)))
+    rows = {}
+    for name, x in (("all", ctx), ("short", short)):
+        g, o = _empty(real, 160, 160), _empty(real, 96, ctx.n)
+        if name == "short":
+            if real:                                # the packed rows' workspace, before there is no room for it
+                x.apply_h_real(a, torch.empty_like(a))
+            torch.cuda.empty_cache()
+            held = torch.empty(torch.cuda.mem_get_info()[0] - 700_000_000, dtype=torch.uint8, device="cuda")
+        (x.gram_real if real else x.gram)(a, b, g)
+        (x.rotate_real if real else x.rotate)(a, c, o)
+        rows[name] = host(g).copy(), host(o).copy()
+    del held
+    torch.cuda.empty_cache()
+    assert all(np.array_equal(p, q) for p, q in zip(rows["all"], rows["short"]))
+    ctx.close()
+    short.close()
