@@ -1051,6 +1051,9 @@ static bool rotation_wins(double n, int rows, int k, int m, bool real, int items
     return t64 > 1.15 * trns;
 }
 
+// The passes have a row of blocks for every row (65,535 at most); more rows than that stay with the FP64 kernels.
+constexpr int MAX_ROWS = 65535;
+
 static rsdft_status gram_within(rsdft_ctx *ctx, size_t limit, const RowBlocks &A0, const RowBlocks &B0,
                                 const RowBlocks *B1, bool real, bool herm, double2 *g0, double2 *g1, int ldg,
                                 double scale, cudaStream_t st, RnsLease &lease) {
@@ -1163,7 +1166,8 @@ static rsdft_status gram_within(rsdft_ctx *ctx, size_t limit, const RowBlocks &A
 
 rsdft_status rns_gram(rsdft_ctx *ctx, const RowBlocks &A, const RowBlocks &B0, const RowBlocks *B1, bool real, bool herm,
                       double2 *g0, double2 *g1, int ldg, double scale, cudaStream_t st, RnsLease &lease) {
-    if (!gram_wins(ctx->n)) return RSDFT_OK;
+    const int rows = std::max(rows_of(real ? pair_rows(A) : A), rows_of(real ? pair_rows(B0) : B0));
+    if (rows > MAX_ROWS || !gram_wins(ctx->n)) return RSDFT_OK;
     for (size_t limit = RNS_BYTES; limit >= RNS_BYTES / 64 && !lease.used; limit /= 8)
         RS_TRY(gram_within(ctx, limit, A, B0, B1, real, herm, g0, g1, ldg, scale, st, lease));
     return RSDFT_OK;
@@ -1294,8 +1298,9 @@ static rsdft_status rotate_within(rsdft_ctx *ctx, size_t limit, const RowBlocks 
 rsdft_status rns_rotate(rsdft_ctx *ctx, const RowBlocks &Y, const double2 *c, int ldc, int m, bool real,
                         const double2 *base, int sign, double2 *out0, double2 *out1, cudaStream_t st, RnsLease &lease) {
     const int segs = Y.cnt[1] + Y.cnt[2] > 0 ? 2 : 1, nt = cdiv(m, real ? 256 : 128);
-    if (Y.cnt[0] <= 0 ||
-        !rotation_wins((double)ctx->n, rows_of(real ? pair_rows(Y) : Y), rows_of(Y), m, real, NM * segs * nt))
+    const int rows = rows_of(real ? pair_rows(Y) : Y);
+    if (Y.cnt[0] <= 0 || rows > MAX_ROWS || cdiv(m, 4) > MAX_ROWS ||
+        !rotation_wins((double)ctx->n, rows, rows_of(Y), m, real, NM * segs * nt))
         return RSDFT_OK;
     for (size_t limit = RNS_BYTES; limit >= RNS_BYTES / 64 && !lease.used; limit /= 8)
         RS_TRY(rotate_within(ctx, limit, Y, c, ldc, m, real, base, sign, out0, out1, st, lease));

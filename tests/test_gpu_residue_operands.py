@@ -150,3 +150,16 @@ def test_short_memory_changes_no_bit(real):
     assert all(np.array_equal(p, q) for p, q in zip(rows["all"], rows["short"]))
     ctx.close()
     short.close()
+
+
+def test_more_rows_than_a_grid_has_blocks():
+    """70,000 rows: the FP64 kernels, one after the other.  Sums of n products err by some sqrt(n) 2^-53 of the sum of the
+    magnitudes, 15 and 265 here; four times that is allowed."""
+    ctx = _ctx((6, 6, 6))
+    a, b, c = draw_x0(1, 70000, ctx.n), draw_x0(2, 1, ctx.n), draw_x0(3, 70000, 1)
+    g, o = _empty(False, 70000, 1), _empty(False, 1, ctx.n)
+    ctx.gram(dev(a), dev(b), g)
+    assert np.all(np.abs(host(g) - a.conj() @ b.T * ctx.dV) <= 60 * EPS * (np.abs(a) @ np.abs(b).T * ctx.dV))
+    ctx.rotate(dev(a), dev(c), o)
+    assert np.all(np.abs(host(o) - c.T @ a) <= 1060 * EPS * (np.abs(c).T @ np.abs(a)))
+    ctx.close()
