@@ -1,8 +1,9 @@
-// Pieces shared by the FP32 passes (fft.cu) and the fixed-point passes (fft_fix.cu).
+// Pieces shared by the FP32 passes (fft.cu), the fixed-point passes (fft_fix.cu) and the residue products (rns.cu).
 #pragma once
 
 #include <algorithm>
 #include <mutex>
+#include <utility>
 #include <vector>
 
 #include "rsdft_internal.h"
@@ -43,18 +44,20 @@ __device__ __forceinline__ void stage_in(int tot, SrcF src, DstF dst) {
 
 constexpr size_t MAX_DYN_SMEM = 227 * 1024;   // largest dynamic shared memory of one CTA
 
-// The attribute is per function and process-wide, so it is raised once to the
-// largest size (occupancy follows each launch's own dynamic size); lowering it
+// The attribute belongs to a function on a device, for the whole process, so it is raised once for each to the
+// largest size, `most` (occupancy follows each launch's own dynamic size); lowering it
 // per launch would race with launches of other contexts on other threads.
-template <typename K> static rsdft_status set_smem(rsdft_ctx *ctx, K kernel, size_t bytes) {
+template <typename K> static rsdft_status set_smem(rsdft_ctx *ctx, K kernel, size_t bytes, size_t most = MAX_DYN_SMEM) {
     if (bytes <= 48 * 1024) return RSDFT_OK;
-    if (bytes > MAX_DYN_SMEM) return fail(ctx, RSDFT_E_INVALID, "plane needs %zu B of shared memory", bytes);
+    if (bytes > most) return fail(ctx, RSDFT_E_INVALID, "plane needs %zu B of shared memory", bytes);
+    int dev = 0;
+    RS_CUDA(ctx, cudaGetDevice(&dev));
     static std::mutex mu;
-    static std::vector<const void *> done;
+    static std::vector<std::pair<int, const void *>> done;
     std::lock_guard<std::mutex> g(mu);
-    const void *key = reinterpret_cast<const void *>(kernel);
+    const std::pair<int, const void *> key(dev, reinterpret_cast<const void *>(kernel));
     if (std::find(done.begin(), done.end(), key) == done.end()) {
-        RS_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MAX_DYN_SMEM));
+        RS_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
         done.push_back(key);
     }
     return RSDFT_OK;

@@ -39,6 +39,7 @@
 #include <cmath>
 #include <mutex>
 
+#include "fft_common.h"
 #include "rsdft_internal.h"
 #include "tc_ptx.h"
 
@@ -1025,9 +1026,7 @@ static RowBlocks pair_rows(const RowBlocks &b) {
 template <bool REAL, bool ROT>
 static rsdft_status launch_gemm(rsdft_ctx *ctx, const CUtensorMap &mA, const CUtensorMap &mB0, const CUtensorMap &mB1,
                                 const Args &a, cudaStream_t st) {
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(k_rns<REAL, ROT>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
-    RS_CUDA(ctx, attr);
+    RS_TRY(set_smem(ctx, k_rns<REAL, ROT>, SMEM, SMEM));
     k_rns<REAL, ROT><<<std::min(a.items, ctx->num_sms), THREADS, SMEM, st>>>(mA, mB0, mB1, a);
     count_launch(ctx);
     RS_LAUNCHED(ctx, "k_rns");
