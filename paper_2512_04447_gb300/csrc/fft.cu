@@ -652,10 +652,8 @@ __global__ void k_to_float(const double *__restrict__ in, long long n, float *__
 template <typename V> static size_t plane_bytes(const rsdft_ctx *ctx) {
     return (size_t)(ctx->N[0] | 1) * ctx->N[1] * sizeof(V);   // odd row stride
 }
-// 256 threads where three CTAs share an SM (fewer for small planes), else enough to fill it
-static int fft_threads(size_t smem, int points) {
-    if (smem <= 75 * 1024) return std::max(64, std::min(256, cdiv(points, 256) * 32));
-    return smem <= 113 * 1024 ? 384 : 768;
+static int fft_threads(const rsdft_ctx *ctx, size_t smem, int points, const dim3 &grid) {
+    return pass_threads(smem, points, (long long)grid.x * grid.y, ctx->num_sms, 64);
 }
 template <typename V> static size_t slab_bytes(const rsdft_ctx *ctx) {
     return (size_t)ctx->N[0] * ctx->N[2] * sizeof(V);
@@ -687,10 +685,10 @@ rsdft_status fft_xy_forward_t(rsdft_ctx *ctx, Src kind, const V *src, const V *s
     const Discs &discs = ctx->discs;
     if (kind == Src::Plain) {
         RS_TRY(set_smem(ctx, k_xy_forward<V, Src::Plain>, sm));
-        k_xy_forward<V, Src::Plain><<<grid, fft_threads(sm, pts), sm, st>>>(tb, src, src2, theta, act, dst, discs, part);
+        k_xy_forward<V, Src::Plain><<<grid, fft_threads(ctx, sm, pts, grid), sm, st>>>(tb, src, src2, theta, act, dst, discs, part);
     } else {
         RS_TRY(set_smem(ctx, k_xy_forward<V, Src::Residual>, sm));
-        k_xy_forward<V, Src::Residual><<<grid, fft_threads(sm, pts), sm, st>>>(tb, src, src2, theta, act, dst, discs, part);
+        k_xy_forward<V, Src::Residual><<<grid, fft_threads(ctx, sm, pts, grid), sm, st>>>(tb, src, src2, theta, act, dst, discs, part);
     }
     RS_LAUNCHED(ctx, "k_xy_forward");
     return RSDFT_OK;
@@ -708,10 +706,10 @@ rsdft_status fft_z_mid_t(rsdft_ctx *ctx, Mid mid, V *buf, const double *tkin, in
     const FftTabs<V> tb = tabs_of(ctx, (V *)nullptr);
     if (mid == Mid::Kinetic) {
         RS_TRY(set_smem(ctx, k_z_mid<V, Mid::Kinetic>, sm));
-        k_z_mid<V, Mid::Kinetic><<<grid, fft_threads(sm, pts), sm, st>>>(tb, buf, tkin);
+        k_z_mid<V, Mid::Kinetic><<<grid, fft_threads(ctx, sm, pts, grid), sm, st>>>(tb, buf, tkin);
     } else {
         RS_TRY(set_smem(ctx, k_z_mid<V, Mid::Tpa>, sm));
-        k_z_mid<V, Mid::Tpa><<<grid, fft_threads(sm, pts), sm, st>>>(tb, buf, tkin);
+        k_z_mid<V, Mid::Tpa><<<grid, fft_threads(ctx, sm, pts, grid), sm, st>>>(tb, buf, tkin);
     }
     RS_LAUNCHED(ctx, "k_z_mid");
     return RSDFT_OK;
@@ -736,10 +734,10 @@ rsdft_status fft_xy_inverse_t(rsdft_ctx *ctx, const V *buf, const V *psi, const 
     const auto *v = v_of(ctx, (V *)nullptr);
     if (psi) {
         RS_TRY(set_smem(ctx, k_xy_inverse<V, Epi::Hpsi>, sm));
-        k_xy_inverse<V, Epi::Hpsi><<<grid, fft_threads(sm, pts), sm, st>>>(tb, buf, psi, v, discs, room, ab, out);
+        k_xy_inverse<V, Epi::Hpsi><<<grid, fft_threads(ctx, sm, pts, grid), sm, st>>>(tb, buf, psi, v, discs, room, ab, out);
     } else {
         RS_TRY(set_smem(ctx, k_xy_inverse<V, Epi::Plain>, sm));
-        k_xy_inverse<V, Epi::Plain><<<grid, fft_threads(sm, pts), sm, st>>>(tb, buf, psi, v, discs, room, ab, out);
+        k_xy_inverse<V, Epi::Plain><<<grid, fft_threads(ctx, sm, pts, grid), sm, st>>>(tb, buf, psi, v, discs, room, ab, out);
     }
     RS_LAUNCHED(ctx, "k_xy_inverse");
     return RSDFT_OK;

@@ -63,4 +63,17 @@ template <typename K> static rsdft_status set_smem(rsdft_ctx *ctx, K kernel, siz
     return RSDFT_OK;
 }
 
+// Threads of a pass of `ctas` blocks, `smem` bytes and `points` points each.  With blocks for more than
+// three on an SM: 256 where three share it (fewer for small planes), else enough to fill it alone or in pairs.  With fewer
+// blocks the chain of a block is what counts, and more threads shorten it: one band on 24^3, 8 atoms, FP64 H psi 68 -> 62
+// us, FP32 41 -> 35, TPA 48 -> 41; on 64^3, 64 atoms 155 -> 139, 72 -> 62, 89 -> 78; 16 bands on 24^3 78 -> 72, 42 -> 39.  From
+// three blocks an SM on (24 bands on 24^3) both sides are the same or fewer threads the faster.
+inline int pass_threads(size_t smem, int points, long long ctas, int sms, int least) {
+    if (smem <= 75 * 1024) {
+        if (ctas > 3LL * sms) return std::max(least, std::min(256, cdiv(points, 256) * 32));
+        return std::max(least, std::min(ctas <= sms ? 512 : (ctas <= 2LL * sms ? 384 : 256), cdiv(points, 64) * 32));
+    }
+    return smem <= 113 * 1024 ? 384 : 768;
+}
+
 }  // namespace rsdft

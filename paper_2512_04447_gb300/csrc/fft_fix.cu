@@ -640,11 +640,9 @@ rsdft_status check_plane(rsdft_ctx *ctx) {
     return RSDFT_OK;
 }
 
-// A radix-8 butterfly a thread, 256 threads where three CTAs share an SM, else enough to fill it
-// alone or in pairs (and at least one thread a row)
-int threads_for(size_t smem, int points) {
-    if (smem <= 75 * 1024) return std::max(128, std::min(256, cdiv(points, 256) * 32));
-    return smem <= 113 * 1024 ? 384 : 768;
+// (at least one thread a row)
+int threads_for(const rsdft_ctx *ctx, size_t smem, int points, const dim3 &grid) {
+    return pass_threads(smem, points, (long long)grid.x * grid.y, ctx->num_sms, 128);
 }
 
 // buf: the buffer between the passes, which says whose exponents
@@ -683,7 +681,7 @@ rsdft_status fft_xy_forward(rsdft_ctx *ctx, Src kind, const double2 *src, const 
     const int RS = plane_stride(ctx);
     const size_t sm = HEAD + (size_t)RS * ctx->N[1] * sizeof(I2);
     const dim3 grid(ctx->N[2], nb);
-    const int th = threads_for(sm, ctx->N[0] * ctx->N[1]);
+    const int th = threads_for(ctx, sm, ctx->N[0] * ctx->N[1], grid);
     const double nxy = (double)ctx->N[0] * ctx->N[1];
     const double bpp = kind == Src::Plain ? 32.0 : (kind == Src::Residual ? 48.0 : 24.0);
     ProfScope ps(ctx, RSDFT_K_FFT_XY_FWD, 5.0 * nxy * std::log2(nxy) * ctx->N[2] * nb, bpp * (double)ctx->n * nb, st);
@@ -725,7 +723,7 @@ rsdft_status fft_z_mid(rsdft_ctx *ctx, Mid mid, double2 *buf, const double *tkin
         sm += tabb;
     }
     const dim3 grid(ctx->N[1], nb);
-    const int th = threads_for(sm, ctx->N[0] * ctx->N[2]);
+    const int th = threads_for(ctx, sm, ctx->N[0] * ctx->N[2], grid);
     ProfScope ps(ctx, RSDFT_K_FFT_Z, 10.0 * (double)ctx->n * std::log2((double)ctx->N[2]) * nb, 32.0 * (double)ctx->n * nb, st);
     const FixTabs tb = tabs_of(ctx);
     I2 *b = reinterpret_cast<I2 *>(buf);
@@ -762,7 +760,7 @@ rsdft_status fft_xy_inverse(rsdft_ctx *ctx, const double2 *buf, const double2 *p
         sm += room * per;
     }
     const dim3 grid(ctx->N[2], nb);
-    const int th = threads_for(sm, ctx->N[0] * ctx->N[1]);
+    const int th = threads_for(ctx, sm, ctx->N[0] * ctx->N[1], grid);
     const double nxy = (double)ctx->N[0] * ctx->N[1];
     const double bpp = rout ? 24.0 : (psi ? 48.0 : 32.0);
     ProfScope ps(ctx, RSDFT_K_FFT_XY_INV, 5.0 * nxy * std::log2(nxy) * ctx->N[2] * nb,
