@@ -370,7 +370,7 @@ static rsdft_status build_projectors(rsdft_ctx *ctx, const rsdft_projectors *pj)
                 const Disc &D = planes[z][k];
                 const Atom &A = at[D.atom];
                 meta.push_back(DiscMeta{(int)row.size(), (unsigned)D.rows.size() | (unsigned)D.xn << 8 |
-                                                             (unsigned)((A.i[0][0] + D.xa) % Nx) << 16 | (unsigned)z << 24});
+                                                             (unsigned)((A.i[0][0] + D.xa) % Nx) << 16});
                 datom.push_back(D.atom);
                 gz.push_back(make_double2(A.g[2][D.tz], A.h[2][D.tz]));
                 for (const Row &r : D.rows) {
@@ -404,12 +404,14 @@ static rsdft_status build_projectors(rsdft_ctx *ctx, const rsdft_projectors *pj)
     for (int a = 0; a < natom; ++a)
         for (int j = 0; j < nproj; ++j)
             if (sq[4 * a + j] > 0.0) cnorm[4 * a + j] = 1.0 / std::sqrt(sq[4 * a + j] * ctx->dV);
-    std::vector<int> atom_start(natom + 1, 0), atom_disc(datom.size());
+    std::vector<int> atom_start(natom + 1, 0), atom_disc(datom.size()), disc_plane(datom.size());
     for (int a : datom) atom_start[a + 1]++;
     for (int a = 0; a < natom; ++a) atom_start[a + 1] += atom_start[a];
     std::vector<int> at_fill(atom_start.begin(), atom_start.end() - 1);
     for (size_t d = 0; d < datom.size(); ++d) atom_disc[at_fill[datom[d]]++] = (int)d;
-    int *d_ps, *d_as, *d_ad, *d_cp, *d_cs;
+    for (int z = 0; z < Nz; ++z)
+        for (int d = plane_start[z]; d < plane_start[z + 1]; ++d) disc_plane[d] = z;
+    int *d_ps, *d_as, *d_ad, *d_cp, *d_cs, *d_pl;
     DiscMeta *d_meta;
     DiscRow *d_row;
     DiscRowFix *d_rowf;
@@ -427,14 +429,15 @@ static rsdft_status build_projectors(rsdft_ctx *ctx, const rsdft_projectors *pj)
     RS_TRY(upload(ctx, &d_cs, color_start.data(), color_start.size()));
     RS_TRY(upload(ctx, &d_gx, gx.data(), gx.size()));
     RS_TRY(upload(ctx, &d_gxf, gxfix.data(), gxfix.size()));
-    RS_TRY(upload(ctx, &d_rowd, rowd.data(), rowd.size()));
-    RS_TRY(upload(ctx, &d_gxd, gxd.data(), gxd.size()));
     RS_TRY(upload(ctx, &d_gz, gz.data(), gz.size()));
     RS_TRY(upload(ctx, &d_cn, cnorm.data(), cnorm.size()));
     RS_TRY(upload(ctx, &d_ek, ekb.data(), ekb.size()));
-    ctx->pt = ProjTables{natom, nproj, d_ek};
+    RS_TRY(upload(ctx, &d_pl, disc_plane.data(), disc_plane.size()));
+    RS_TRY(upload(ctx, &d_rowd, rowd.data(), rowd.size()));
+    RS_TRY(upload(ctx, &d_gxd, gxd.data(), gxd.size()));
+    ctx->pt = ProjTables{natom, nproj, d_ek, d_pl, d_rowd, d_gxd};
     ctx->discs = Discs{natom, nproj, (int)datom.size(), wmax, mrows, mdiscs, d_ps, d_cp, d_cs, d_meta, d_row, d_rowf,
-                       d_rowd, d_gx, d_gxf, d_gxd, d_as, d_ad, d_gz, d_cn, d_ek};
+                       d_gx, d_gxf, d_as, d_ad, d_gz, d_cn, d_ek};
     ctx->nent = nent;
     return RSDFT_OK;
 }

@@ -495,79 +495,57 @@ k_xy_inverse(FftTabs<V> tb, const V *__restrict__ buf, const V *__restrict__ psi
 // ---- projectors --------------------------------------------------------------------------
 constexpr int PROJ_THREADS = 256;
 
-// p[band][atom nproj + j] = <beta_j|psi>: a block per (band, atom), a warp per disc of the atom, joined
+// p[band][atom nproj + j] = <beta_j|psi> in FP64: a block per (band, atom), a warp per disc of the atom, joined
 // in the block, so that the call needs no memory but the caller's.  lane = x; discs of at most 16 or 8
-// points across take two or four rows at a time.  A point costs four multiply-adds (a warp's FP64 ones 64 cycles each,
-// which bounds the FP64 form) and the factors of a row are loaded.  One GB300, FP64, against partial sums
-// per plane in scratch with the factors converted from fixed point: 144 bands on 64^3, 64 atoms 5,033 -> 1,443 us (a table
+// points across take two or four rows at a time.  A point costs four multiply-adds (a warp's 64 cycles each, which
+// bounds the kernel) and the factors of a row are loaded.  One GB300, against partial sums per
+// plane in scratch with the factors converted from fixed point: 144 bands on 64^3, 64 atoms 5,033 -> 1,443 us (a table
 // of every point's values 1,734), one band 127 -> 40 (51), 64 bands on 24^3, 8 atoms 106 -> 31 (31).
-template <typename V>
 __global__ void __launch_bounds__(PROJ_THREADS)
-k_project(Discs t, const V *__restrict__ psi, int Nx, int Ny, long long n, typename Sc<V>::T dV, V *__restrict__ p) {
-    using T = typename Sc<V>::T;
+k_project(Discs t, ProjTables pt, const double2 *__restrict__ psi, int Nx, int Ny, long long n, double dV,
+          double2 *__restrict__ p) {
     const int band = blockIdx.x / t.natom, a = blockIdx.x - band * t.natom;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int i1 = t.atom_start[a + 1];
-    T s[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) s[k] = (T)0;
+    double s[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
     for (int i = t.atom_start[a] + warp; i < i1; i += PROJ_THREADS / 32) {
         const int d = t.atom_disc[i];
         const int2 m = __ldg(reinterpret_cast<const int2 *>(t.meta + d));
         const int rows = disc_rows(m.y), w = disc_width(m.y);
-        const V *plane = psi + (size_t)band * n + (size_t)disc_z(m.y) * Nx * Ny;
-        T v[6] = {(T)0, (T)0, (T)0, (T)0, (T)0, (T)0};   // sums of gx gy, hx gy and gx hy times psi
+        const double2 *plane = psi + (size_t)band * n + (size_t)pt.plane[d] * Nx * Ny;
+        double v[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};   // sums of gx gy, hx gy and gx hy times psi
         const int W = w <= 8 ? 8 : (w <= 16 ? 16 : 32);   // lanes a row
         for (int c = 0; c < w; c += W) {
             const int l = c + (lane & (W - 1));
             int x = disc_x0(m.y) + l;
             if (x >= Nx) x -= Nx;
-            T ax = (T)0, ay = (T)0, bx = (T)0, by = (T)0;
+            double ax = 0.0, ay = 0.0, bx = 0.0, by = 0.0;
 #pragma unroll 4
             for (int r = lane / W; r < rows; r += 32 / W) {
-                const int4 k = __ldg(reinterpret_cast<const int4 *>(t.row + m.x + r));
-                if (in_row(k.x, l)) {
-                    const V u = plane[(k.x & 255) * Nx + x];
-                    T g, h;
-                    if constexpr (sizeof(T) == 4) {
-                        g = __int_as_float(k.y);
-                        h = __int_as_float(k.z);
-                    } else {
-                        const double2 f = __ldg(t.rowd + m.x + r);
-                        g = f.x;
-                        h = f.y;
-                    }
-                    ax += g * u.x;
-                    ay += g * u.y;
-                    bx += h * u.x;
-                    by += h * u.y;
+                const int k = __ldg(&t.row[m.x + r].packed);
+                if (in_row(k, l)) {
+                    const double2 u = plane[(k & 255) * Nx + x], f = __ldg(pt.row + m.x + r);
+                    ax += f.x * u.x;
+                    ay += f.x * u.y;
+                    bx += f.y * u.x;
+                    by += f.y * u.y;
                 }
             }
             if (l < w) {
-                T gx, hx;
-                if constexpr (sizeof(T) == 4) {
-                    const float2 f = __ldg(t.gx + (size_t)d * t.wmax + l);
-                    gx = f.x;
-                    hx = f.y;
-                } else {
-                    const double2 f = __ldg(t.gxd + (size_t)d * t.wmax + l);
-                    gx = f.x;
-                    hx = f.y;
-                }
-                v[0] += gx * ax;
-                v[1] += gx * ay;
-                v[2] += hx * ax;
-                v[3] += hx * ay;
-                v[4] += gx * bx;
-                v[5] += gx * by;
+                const double2 f = __ldg(pt.gx + (size_t)d * t.wmax + l);
+                v[0] += f.x * ax;
+                v[1] += f.x * ay;
+                v[2] += f.y * ax;
+                v[3] += f.y * ay;
+                v[4] += f.x * bx;
+                v[5] += f.x * by;
             }
         }
         const double2 gd = t.gz[d];
-        const T gz = (T)gd.x, hz = (T)gd.y;
 #pragma unroll
-        for (int k = 0; k < 6; ++k) s[k] += gz * v[k];
-        s[6] += hz * v[0];
-        s[7] += hz * v[1];
+        for (int k = 0; k < 6; ++k) s[k] += gd.x * v[k];
+        s[6] += gd.y * v[0];
+        s[7] += gd.y * v[1];
     }
     // the eight sums over the warp, half of them going to each half of the lanes at every step: 9 additions instead of 40
 #pragma unroll
@@ -575,29 +553,77 @@ k_project(Discs t, const V *__restrict__ psi, int Nx, int Ny, long long n, typen
         const bool up = lane & o;
 #pragma unroll
         for (int k = 0; k < m; ++k) {
-            const T give = up ? s[k] : s[k + m];
+            const double give = up ? s[k] : s[k + m];
             s[k] = (up ? s[k + m] : s[k]) + __shfl_xor_sync(0xffffffffu, give, o);
         }
     }
     s[0] += __shfl_xor_sync(0xffffffffu, s[0], 2);
     s[0] += __shfl_xor_sync(0xffffffffu, s[0], 1);
-    __shared__ T red[PROJ_THREADS / 32][8];
+    __shared__ double red[PROJ_THREADS / 32][8];
     if ((lane & 3) == 0) red[warp][lane >> 2] = s[0];   // bits 4, 3, 2 of the lane: those of the sum's number
     __syncthreads();
     const int j = threadIdx.x >> 1, part = threadIdx.x & 1;
     if (j < t.nproj) {
-        T q = (T)0;
+        double q = 0.0;
         for (int k = 0; k < PROJ_THREADS / 32; ++k) q += red[k][threadIdx.x];
-        T *o = reinterpret_cast<T *>(p + (size_t)blockIdx.x * t.nproj + j);
-        o[part] = (T)t.cnorm[4 * a + j] * dV * q;
+        double *o = reinterpret_cast<double *>(p + (size_t)blockIdx.x * t.nproj + j);
+        o[part] = t.cnorm[4 * a + j] * dV * q;
     }
 }
 
-// One warp per (band, atom): the disc sums joined with their z factors, and the scatter coefficients of
-// every disc, ab[band][disc] = (gz q_s + hz q_z, gz q_x, gz q_y) with q_j = c_j E_j <beta_j|psi>.
+// The gather alone on FP32 planes in global memory (lane = x), for the solvers: a CTA's discs are those of one
+// plane, whose rows it reads from L1 again (144 bands on 64^3 0.30 ms; a block per atom, as above, 0.51).
+__global__ void __launch_bounds__(PROJ_THREADS)
+k_gather(Discs t, const float2 *__restrict__ psi, int Nx, int Ny, long long n, float2 *__restrict__ part) {
+    const int z = blockIdx.x, band = blockIdx.y;
+    const float2 *plane = psi + (size_t)band * n + (size_t)z * Nx * Ny;
+    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    const int d1 = t.plane_start[z + 1];
+    for (int d = t.plane_start[z] + (threadIdx.x >> 5); d < d1; d += nw) {
+        const DiscMeta m = t.meta[d];
+        const int rows = disc_rows(m.packed), w = disc_width(m.packed);
+        float s[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        for (int c = 0; c < w; c += 32) {
+            const int l = c + lane;
+            int x = disc_x0(m.packed) + l;
+            if (x >= Nx) x -= Nx;
+            float ax = 0.f, ay = 0.f, bx = 0.f, by = 0.f;
+#pragma unroll 4
+            for (int r = 0; r < rows; ++r) {
+                const int4 k = __ldg(reinterpret_cast<const int4 *>(t.row + m.row0 + r));
+                const float g = __int_as_float(k.y), h = __int_as_float(k.z);
+                if (in_row(k.x, l)) {
+                    const float2 v = plane[(k.x & 255) * Nx + x];
+                    ax += g * v.x;
+                    ay += g * v.y;
+                    bx += h * v.x;
+                    by += h * v.y;
+                }
+            }
+            const float2 k = l < w ? __ldg(t.gx + (size_t)d * t.wmax + l) : make_float2(0.f, 0.f);
+            s[0] += k.x * ax;
+            s[1] += k.x * ay;
+            s[2] += k.y * ax;
+            s[3] += k.y * ay;
+            s[4] += k.x * bx;
+            s[5] += k.x * by;
+        }
+#pragma unroll
+        for (int k = 0; k < 6; ++k)
+            for (int o = 16; o > 0; o >>= 1) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
+        if (lane < 3)
+            part[((size_t)band * t.ndisc + d) * 3 + lane] = make_float2(lane == 0 ? s[0] : (lane == 1 ? s[2] : s[4]),
+                                                                       lane == 0 ? s[1] : (lane == 1 ? s[3] : s[5]));
+    }
+}
+
+// One warp per (band, atom): the disc sums joined with their z factors, p[band][atom nproj + j] =
+// <beta_j|psi> (p may be null) and the scatter coefficients of every disc, ab[band][disc] =
+// (gz q_s + hz q_z, gz q_x, gz q_y) with q_j = c_j E_j <beta_j|psi> (ab may be null).
 template <typename V>
 __global__ void __launch_bounds__(PROJ_THREADS)
-k_disc_fin(Discs t, const V *__restrict__ part, int nb, typename Sc<V>::T dV, V *__restrict__ ab) {
+k_disc_fin(Discs t, const V *__restrict__ part, int nb, typename Sc<V>::T dV, V *__restrict__ p,
+           V *__restrict__ ab) {
     using T = typename Sc<V>::T;
     const int w = (blockIdx.x * PROJ_THREADS + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     const int band = w / t.natom, a = w - band * t.natom;
@@ -628,9 +654,11 @@ k_disc_fin(Discs t, const V *__restrict__ part, int nb, typename Sc<V>::T dV, V 
     for (int j = 0; j < 4; ++j) {
         const T c = (T)t.cnorm[4 * a + j];   // 0 for projectors that are not there
         q[j] = mk<V>(c * dV * s[2 * j], c * dV * s[2 * j + 1]);
+        if (p && lane == 0 && j < t.nproj) p[(size_t)band * t.natom * t.nproj + a * t.nproj + j] = q[j];
         const T e = j < t.nproj ? c * (T)t.e_kb[a * t.nproj + j] : (T)0;
         q[j] = mk<V>(e * q[j].x, e * q[j].y);
     }
+    if (!ab) return;
     V *ob = ab + (size_t)band * t.ndisc * 3;
     for (int i = i0 + lane; i < i1; i += 32) {
         const int d = t.atom_disc[i];
@@ -743,8 +771,8 @@ rsdft_status fft_xy_inverse_t(rsdft_ctx *ctx, const V *buf, const V *psi, const 
     return RSDFT_OK;
 }
 
-// Partial-sum and coefficient buffers of nb bands, and the scatter coefficients E <beta|psi> of every disc
-// from the sums.
+// Partial-sum and coefficient buffers of nb bands (of the calls that work in the orbitals' workspace), and the sums
+// joined per atom: p (or null) the projections, ab (or null) the scatter coefficients E <beta|psi> of every disc.
 static rsdft_status disc_buffers(rsdft_ctx *ctx, int nb, double2 **part, double2 **ab, cudaStream_t st) {
     const size_t per = (size_t)ctx->discs.ndisc * 3;
     RS_TRY(grow(ctx, ctx->discbuf, std::max<size_t>(16, 2 * per * nb * sizeof(double2)), st));
@@ -754,24 +782,36 @@ static rsdft_status disc_buffers(rsdft_ctx *ctx, int nb, double2 **part, double2
 }
 
 template <typename V>
-static rsdft_status disc_finish(rsdft_ctx *ctx, const V *part, int nb, V *ab, cudaStream_t st) {
+static rsdft_status disc_finish(rsdft_ctx *ctx, const V *part, int nb, V *p, V *ab, cudaStream_t st) {
     using T = typename Sc<V>::T;
     k_disc_fin<V><<<cdiv((long long)nb * ctx->pt.natom * 32, PROJ_THREADS), PROJ_THREADS, 0, st>>>(
-        ctx->discs, part, nb, (T)ctx->dV, ab);
+        ctx->discs, part, nb, (T)ctx->dV, p, ab);
     count_launch(ctx);
     RS_LAUNCHED(ctx, "k_disc_fin");
     return RSDFT_OK;
 }
 
-template <typename V>
-rsdft_status project_t(rsdft_ctx *ctx, const V *psi, V *p, int nb, cudaStream_t st) {
+rsdft_status project(rsdft_ctx *ctx, const double2 *psi, double2 *p, int nb, cudaStream_t st) {
     if (nb <= 0 || ctx->pt.natom == 0) return RSDFT_OK;
-    using T = typename Sc<V>::T;
     const double ne = (double)ctx->nent;
-    ProfScope ps(ctx, RSDFT_K_PROJECT, 4.0 * ctx->pt.nproj * ne * nb, (double)sizeof(V) * ne * nb, st);
-    k_project<V><<<nb * ctx->pt.natom, PROJ_THREADS, 0, st>>>(ctx->discs, psi, ctx->N[0], ctx->N[1], ctx->n, (T)ctx->dV, p);
+    ProfScope ps(ctx, RSDFT_K_PROJECT, 4.0 * ctx->pt.nproj * ne * nb, 16.0 * ne * nb, st);
+    k_project<<<nb * ctx->pt.natom, PROJ_THREADS, 0, st>>>(ctx->discs, ctx->pt, psi, ctx->N[0], ctx->N[1], ctx->n, ctx->dV,
+                                                            p);
     RS_LAUNCHED(ctx, "k_project");
     return RSDFT_OK;
+}
+rsdft_status project32(rsdft_ctx *ctx, const float2 *psi, float2 *p, int nb, cudaStream_t st) {
+    if (nb <= 0 || ctx->pt.natom == 0) return RSDFT_OK;
+    double2 *buf, *ab;
+    RS_TRY(disc_buffers(ctx, nb, &buf, &ab, st));
+    float2 *part = reinterpret_cast<float2 *>(buf);
+    const double ne = (double)ctx->nent;
+    {
+        ProfScope ps(ctx, RSDFT_K_PROJECT, 4.0 * ctx->pt.nproj * ne * nb, 8.0 * ne * nb, st);
+        k_gather<<<dim3(ctx->N[2], nb), PROJ_THREADS, 0, st>>>(ctx->discs, psi, ctx->N[0], ctx->N[1], ctx->n, part);
+    }
+    RS_LAUNCHED(ctx, "k_gather");
+    return disc_finish<float2>(ctx, part, nb, p, nullptr, st);
 }
 
 rsdft_status fft_xy_forward32(rsdft_ctx *ctx, Src kind, const float2 *src, const float2 *src2,
@@ -787,13 +827,6 @@ rsdft_status fft_xy_inverse32(rsdft_ctx *ctx, const float2 *buf, const float2 *p
                               const float2 *ab, float2 *out, int nb, cudaStream_t st) {
     return fft_xy_inverse_t<float2>(ctx, buf, psi, ab, out, nb, st);
 }
-rsdft_status project(rsdft_ctx *ctx, const double2 *psi, double2 *p, int nb, cudaStream_t st) {
-    return project_t<double2>(ctx, psi, p, nb, st);
-}
-rsdft_status project32(rsdft_ctx *ctx, const float2 *psi, float2 *p, int nb, cudaStream_t st) {
-    return project_t<float2>(ctx, psi, p, nb, st);
-}
-
 rsdft_status refresh_v32(rsdft_ctx *ctx, cudaStream_t st) {
     k_to_float<<<std::max(1, std::min(cdiv(ctx->n, 256), 608)), 256, 0, st>>>(ctx->v, ctx->n, ctx->v32);
     count_launch(ctx);
@@ -809,7 +842,7 @@ rsdft_status apply_h64(rsdft_ctx *ctx, const double2 *psi, double2 *hpsi, int nb
     const bool nl = ctx->discs.ndisc > 0;
     if (nl) RS_TRY(disc_buffers(ctx, nb, &part, &ab, st));
     RS_TRY(fft_xy_forward(ctx, Src::Plain, psi, nullptr, nullptr, nullptr, nullptr, ctx->ws.T1, nb, st, part));
-    if (nl) RS_TRY(disc_finish<double2>(ctx, part, nb, ab, st));
+    if (nl) RS_TRY(disc_finish<double2>(ctx, part, nb, nullptr, ab, st));
     RS_TRY(fft_z_mid(ctx, Mid::Kinetic, ctx->ws.T1, nullptr, nb, st));
     RS_TRY(fft_xy_inverse(ctx, ctx->ws.T1, psi, ab, hpsi, nullptr, nb, st));
     return RSDFT_OK;
@@ -825,7 +858,7 @@ rsdft_status apply_h32(rsdft_ctx *ctx, const float2 *psi, float2 *hpsi, int nb, 
     float2 *part32 = reinterpret_cast<float2 *>(part), *ab32 = reinterpret_cast<float2 *>(ab);
     float2 *t1 = reinterpret_cast<float2 *>(ctx->ws.T1);
     RS_TRY(fft_xy_forward32(ctx, Src::Plain, psi, nullptr, nullptr, nullptr, t1, nb, st, part32));
-    if (nl) RS_TRY(disc_finish<float2>(ctx, part32, nb, ab32, st));
+    if (nl) RS_TRY(disc_finish<float2>(ctx, part32, nb, nullptr, ab32, st));
     RS_TRY(fft_z_mid32(ctx, Mid::Kinetic, t1, nullptr, nb, st));
     RS_TRY(fft_xy_inverse32(ctx, t1, psi, ab32, hpsi, nb, st));
     return RSDFT_OK;

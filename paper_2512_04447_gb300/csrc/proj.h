@@ -26,8 +26,7 @@ template <> struct Sc<float2> { using T = float; };
 // DiscMeta::packed and DiscRow::packed (rsdft_internal.h)
 __device__ __forceinline__ int disc_rows(unsigned p) { return p & 255; }
 __device__ __forceinline__ int disc_width(unsigned p) { return (p >> 8) & 255; }
-__device__ __forceinline__ int disc_x0(unsigned p) { return (p >> 16) & 255; }
-__device__ __forceinline__ int disc_z(unsigned p) { return p >> 24; }
+__device__ __forceinline__ int disc_x0(unsigned p) { return p >> 16; }
 __device__ __forceinline__ bool in_row(int packed, int l) {
     return (unsigned)(l - ((packed >> 8) & 255)) < (unsigned)(packed >> 16);
 }

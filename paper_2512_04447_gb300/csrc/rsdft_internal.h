@@ -50,11 +50,13 @@ struct Fft3Plan {
 // Projector data that kernels other than the passes need.
 struct ProjTables {
     int natom, nproj;
-    const double *e_kb;      // [natom*nproj]
+    const double *e_kb;          // [natom*nproj]
+    const int *plane;            // plane of each disc
+    const double2 *row, *gx;     // Discs::row and Discs::gx in FP64
 };
 
 // Kleinman-Bylander projectors by plane (proj.h).
-struct DiscMeta { int row0; unsigned packed; };                               // first row; rows | width << 8 | first x << 16 | z << 24
+struct DiscMeta { int row0; unsigned packed; };                               // first row; rows | width << 8 | first x << 16
 struct __align__(16) DiscRow { int packed; float g, h; int pad; };            // a row of a disc: gy, dy/rc gy
 struct __align__(16) DiscRowFix { int packed, gh, gl, hh, hl, pad[3]; };      // the same in units of 2^-62
 struct Discs {
@@ -66,10 +68,8 @@ struct Discs {
     const DiscMeta *meta;                    // [ndisc]
     const DiscRow *row;                      // by disc, in order of y: y | first x offset << 8 | points << 16
     const DiscRowFix *rowfix;
-    const double2 *rowd;                     // gy, dy/rc gy of a row
     const float2 *gx;                        // [ndisc][wmax] gx, dx/rc gx
     const int4 *gxfix;                       // the same in units of 2^-62 (high, low words)
-    const double2 *gxd;
     const int *atom_start, *atom_disc;       // [natom + 1], [ndisc] discs of each atom
     const double2 *gz;                       // [ndisc] gz, dz/rc gz
     const double *cnorm, *e_kb;              // [natom][4] norms c; [natom * nproj]
