@@ -209,7 +209,7 @@ def traffic_for(name):
 
 def kernel_roofline(name, d, precision, sm_mhz, hbm_gbs):
     """Bound, achieved and peak of one profiled kernel id.  The FP64 Grams and rotations
-    run as 15 residue products on the tensor cores (BF16 MMAs); the FP32 ones are bound by
+    run as 16 residue products on the tensor cores (BF16 MMAs); the FP32 ones are bound by
     the FP32 CUDA cores; FFT passes (FP64 ones in 64-bit fixed point) and the projector
     gather are compared with HBM."""
     s = d["ms"] / 1e3
@@ -262,13 +262,13 @@ def kernel_roofline(name, d, precision, sm_mhz, hbm_gbs):
                 "peak_source": f"FP64 ALU: {NUM_SM} SMs x {FP64_FLOP_PER_CLK_PER_SM:g} flop/clk x {sm_mhz:g} MHz "
                                "(unit counts and max clock; no measured FP64 peak is recorded)"}
     if name in ("gram", "rotate") and not fp32:
-        # 15 moduli: 15 BF16 flops for one FP64 flop of the product
+        # 16 moduli: 16 BF16 flops for one FP64 flop of the product
         peak = float(_peaks().get("bf16_tflops", 1955.4))
-        ach = 15.0 * d["flops"] / s / 1e12
+        ach = 16.0 * d["flops"] / s / 1e12
         return {"kernel": name, "bound": "tensor", "achieved": ach, "peak": peak, "unit": "TFLOP/s",
                 "frac": ach / peak, "avg_launch_ms": per_launch_s * 1e3,
                 "algorithmic_flops_per_launch": d["flops"] / d["launches"],
-                "arithmetic": "FP64 operands as residues modulo 15 numbers, exact BF16 products",
+                "arithmetic": "FP64 operands as residues modulo 16 numbers, exact BF16 products",
                 "peak_source": "MEASURED_PEAKS.json bf16_tflops (cuBLAS BF16 GEMM, burst)"}
     if name in ("gram", "rotate"):
         per = FP32_FLOP_PER_CLK_PER_SM

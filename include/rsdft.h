@@ -31,6 +31,11 @@
  *    in their last valid state.  A context is used by one host thread at a
  *    time; work is issued on the CUDA stream passed in (NULL = legacy stream),
  *    and calls that return host values synchronise that stream first.
+ *  - Memory of a context grows to its largest calls and is freed by rsdft_destroy.
+ *    FP64 Grams and rotations take up to 2 GB for each stream that runs them at a
+ *    time (four at most: a call on a fifth waits for one) and for each capture
+ *    whose graphs are still there, never more than a quarter of what is free; less
+ *    memory makes them slower, not different.
  */
 #ifndef RSDFT_H
 #define RSDFT_H
@@ -135,6 +140,9 @@ rsdft_status rsdft_precondition_tpa(rsdft_ctx *ctx, const void *r_dev, void *w_d
  *
  * Gram matrix G[i][j] = <a_i|b_j> = dV sum_r conj(a_i(r)) b_j(r).
  * a_dev: [na][n], b_dev: [nb][n], g_dev: [na][nb] row-major, complex128.
+ * Rows may have any size: entries are good to some 2^-53 of |G[i][j]| and, beside
+ * that, 2^-61 sqrt(n) |a_i| |b_j| dV at most (2^-61 |a_i| |b_j| dV where the values
+ * of the rows do not all round alike).
  */
 rsdft_status rsdft_gram(rsdft_ctx *ctx, const void *a_dev, int na, const void *b_dev, int nb,
                         void *g_dev, void *stream);
@@ -194,7 +202,10 @@ rsdft_status rsdft_rotate_bf16x3(rsdft_ctx *ctx, const void *y_dev, int k, const
 
 /* Rotation out[b] = sum_i c[i][b] y[i] (+ base[b] when base_dev != NULL;
  * base may alias out).  y_dev: [k][n]; c_dev: [k][m] row-major;
- * out_dev, base_dev: [m][n]; complex128.  sign = +1 adds, -1 subtracts the sum. */
+ * out_dev, base_dev: [m][n]; complex128.  sign = +1 adds, -1 subtracts the sum.
+ * Rows and coefficients may have any size: out[b] is good to some 2^-53 of its
+ * value and, beside that, to some 2^-56 of the norm over i of |c[i][b]| |y[i]|
+ * times the largest |y[j](r)| / |y[j]| at its point. */
 rsdft_status rsdft_rotate(rsdft_ctx *ctx, const void *y_dev, int k, const void *c_dev, int m,
                           const void *base_dev, int sign, void *out_dev, void *stream);
 

@@ -12,7 +12,7 @@
 //   z-mid       (one CTA per (band, y) slab: z DIF, multiply by a function of
 //                |G|^2 at the digit-reversed position, z DIT)
 //   xy-inverse  (one CTA per (band, z) plane: y and x DIT, then the epilogue:
-//                + V psi and the point-major projector scatter for H psi)
+//                + V psi and the projector scatter by discs for H psi)
 // Forward stages leave the spectrum in mixed-radix digit-reversed order and
 // the inverse stages take it back to natural order, so the per-G factor is
 // applied through position-indexed |G|^2 tables and no permutation pass exists.
