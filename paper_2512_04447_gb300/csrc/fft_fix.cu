@@ -9,10 +9,10 @@
 // largest one of the slab.
 //
 // What bounds it: the FP64 passes ran at some 80% of the FP64 pipe; the integer instructions on
-// 64-bit values bound these.  144 bands on 64^3, one GB300: forward 3.23 -> 0.68 ms (1.46 with
-// the projector gather, then 1.77 on its own), z 3.66 -> 0.81 ms, inverse 5.9 -> 2.1 ms with the
+// 64-bit values bound these.  144 bands on 64^3, one GB300: forward 3.23 -> 0.68 ms (1.49 with
+// the projector gather, then 1.77 on its own), z 3.66 -> 0.87 ms, inverse 5.9 -> 2.2 ms with the
 // projector scatter; TPA of 53
-// bands on 45^3 1.94 -> 0.55 ms.  Errors against 64-bit FFTs are those of the reference itself:
+// bands on 45^3 1.94 -> 0.54 ms.  Errors against 64-bit FFTs are those of the reference itself:
 // relative 4.4e-16 (FP64 passes 4.8e-16) for TPA, 7.1e-16 (8.4e-16) for H psi.
 //
 // Non-finite values make a block's exponent BAD, which every following pass hands on, and the

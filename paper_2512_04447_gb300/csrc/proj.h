@@ -10,7 +10,7 @@
 //            colour after colour, so that no two warps write a point at a time and the order
 //            of the sums is fixed
 // What bounds both is the number of instructions.  One GB300, before and after: H psi of 144 bands on
-// 64^3 (64 atoms, FP64, after the fixed-point transforms) 6.73 -> 4.48 ms, its gather 1.77 -> 0.8
+// 64^3 (64 atoms, FP64, after the fixed-point transforms) 6.73 -> 4.58 ms, its gather 1.77 -> 0.8
 // and scatter 2.8 -> 1.3 ms; of 160 bands on 96^3 (216 atoms, FP32) gather 1.16 -> 0.6 ms, scatter 1.9 ->
 // 1.6 ms.
 #pragma once

@@ -22,12 +22,14 @@
 // points go in chunks that keep the residues within RNS_BYTES.
 //
 // Measured on one GB300 against the FP64 kernels (which run at 97% of the FP64 pipe):
-//   Gram 432 x 432 over 64^3 points   321.8 -> 8.7 ms     rotation 432 -> 144   104.8 -> 4.9 ms
-//   real Gram 285 x 285 over 60^3      30.2 -> 2.35 ms
-// of the Gram's 8.7 ms the residue planes take 3.4 (81% of DRAM bandwidth, 78% of the issue slots), the
-// statistics 0.6 and the MMAs 4.6 (75% of the BF16 rate).
-// and errors against extended precision (150 x 150 over 5,400 points: relative 2.5e-16 against
-// 1.4e-15; rotation 432 -> 144: 1.6e-16 against 9.8e-16).
+//   Gram 432 x 432 over 64^3 points   321.8 -> 9.3 ms     rotation 432 -> 144   104.8 -> 5.7 ms
+//   real Gram 285 x 285 over 60^3      30.2 -> 2.5 ms
+// of the Gram's 9.3 ms the residue planes take 3.6 (80% of DRAM bandwidth, 78% of the issue slots), the
+// statistics 0.6 and the MMAs 5.1 (60% of the tensor pipe's cycles, the rest waits for shared memory); of the
+// rotation's 5.7 the statistics of rows and points 0.75, residues 1.5, MMAs 2.5 and remainders 0.8;
+// and errors against extended precision (150 x 150 over 5,400 points: relative 7.1e-17 against
+// 1.1e-15; rotation 432 -> 144: 4.7e-17 against 9.8e-16; <a|a> of uniform rows on 64^3, 96^3, 120^3: 0, 3.0e-16,
+// 6.4e-16 against 4.3e-14, 1.5e-13, 3.2e-13).
 //
 // Non-finite values, and rows of nothing but subnormal ones, raise a device flag; then the
 // kernels here leave their outputs alone and the FP64 kernels launched behind them
@@ -905,8 +907,8 @@ using namespace rns;
 
 // ---- host side ---------------------------------------------------------------------------
 // Bytes of residues held at a time (the points go in chunks of that size): a chunk's launches end
-// with a partly filled wave and the residues' way out (432 x 432: 9.0 ms with 2^30, 8.7 with 2^31, 8.5 with
-// 2^32).  Where that does not fit, an eighth and a 64th of it are tried (4,096 points at least: 0.1 GB for 432
+// with a partly filled wave and the residues' way out (432 x 432, with 15 moduli: 9.0 ms with 2^30, 8.7 with 2^31, 8.5
+// with 2^32).  Where that does not fit, an eighth and a 64th of it are tried (4,096 points at least: 0.1 GB for 432
 // rows), and the FP64 kernels run only where even that does not: chunks change no bit of a result.
 constexpr size_t RNS_BYTES = (size_t)1 << 31;
 
@@ -1035,14 +1037,15 @@ static rsdft_status launch_gemm(rsdft_ctx *ctx, const CUtensorMap &mA, const CUt
 
 // Whether the residue path is the faster one.
 //  Gram: the FP64 kernel sums at least 512 points a CTA (all of them below that), a microsecond each and
-//  0.3 in real form, whatever the number of rows; measured on 216 to 262,144 points and 16 to 288 rows a
+//  0.3 in real form, whatever the number of rows; measured on 216 to 884,736 points and 1 to 288 rows a
 //  side, the residue path was the faster one throughout (16 x 16 on 6^3 236 -> 66 us, real 78 -> 64 us;
-//  on 20^3 562 -> 103 us, real 173 -> 89 us).
+//  on 20^3 562 -> 103 us, real 173 -> 89 us; 1 x 1 on 6^3 235 -> 64 us, on 96^3 7.0 -> 1.1 ms, real 1.94 -> 0.58).
 static bool gram_wins(long long n) { return n >= 200; }
 //  Rotation, in seconds: the FP64 kernel at 1.15 TFLOP/s over whole tiles of 16 rows and bands (pair rows in
 //  real form) against launches, work items of 128 points (some 2 us each on an SM) and the residue
 //  planes (33 ps a row and point).  Within 25% of the times measured on the sizes above; the line at
-//  1.15 keeps FP64 where the two meet (24 -> 8 bands on 32^3: 136 against 111 us).
+//  1.15 keeps FP64 where the two meet (24 -> 8 bands on 32^3: 134 against 125 us; 96 -> 32 real on 32^3: 225
+//  against 167).  Of 52 shapes from 8 -> 8 on 8^3 to 432 -> 144 on 64^3 none runs slower than the FP64 kernel.
 static bool rotation_wins(double n, int rows, int k, int m, bool real, int items_per_tile) {
     auto up = [real](int c) { return real ? 2.0 * (cdiv((c + 1) / 2, 16) * 16) : (double)(cdiv(c, 16) * 16); };
     const double t64 = (real ? 2.0 : 8.0) * n * up(k) * up(m) / 1.15e12;
