@@ -39,22 +39,22 @@ rsdft_status dev_alloc(rsdft_ctx *ctx, void **p, size_t bytes) {
     return RSDFT_OK;
 }
 
-// At least `bytes` in s for work on st, also while st is being captured (the allocation itself is
-// no work of the stream: it is made in the relaxed mode and not captured).
+// At least `bytes` in s for work on st, also while st or another stream of this or another thread is being
+// captured (an allocation is no work of a stream: it is made in the relaxed mode and not captured).
 rsdft_status grow(rsdft_ctx *ctx, Scratch &s, size_t bytes, cudaStream_t st) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (st && st != cudaStreamLegacy) RS_CUDA(ctx, cudaStreamIsCapturing(st, &cs));
     const bool capturing = cs != cudaStreamCaptureStatusNone;
     if (bytes > s.bytes) {
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        RS_CUDA(ctx, cudaThreadExchangeStreamCaptureMode(&mode));
         if (s.p && !s.captured && !capturing) {
             cudaFree(s.p);
             ctx->owned.erase(std::remove(ctx->owned.begin(), ctx->owned.end(), s.p), ctx->owned.end());
         }
         s = Scratch{};
-        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-        if (capturing) RS_CUDA(ctx, cudaThreadExchangeStreamCaptureMode(&mode));
         const rsdft_status a = dev_alloc(ctx, &s.p, bytes);
-        if (capturing) RS_CUDA(ctx, cudaThreadExchangeStreamCaptureMode(&mode));
+        RS_CUDA(ctx, cudaThreadExchangeStreamCaptureMode(&mode));
         RS_TRY(a);
         s.bytes = bytes;
     }

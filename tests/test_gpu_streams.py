@@ -148,3 +148,23 @@ def test_field_solvers_beside_h_psi():
     _beside(lambda: ctx.apply_h(x, h), fields)
     assert all(np.array_equal(host(t), r) for t, r in zip((h, v, e, u), ref))
     ctx.close()
+
+
+def test_first_call_while_another_stream_is_captured():
+    """A rotation that needs its memory allocated, on a stream of its own, in the middle of a capture on another one."""
+    need_gpu()
+    one, two = pair(diamond8_24())[0], pair(diamond8_24())[0]
+    y, c = dev(draw_x0(1, 96, one.n)), dev(draw_x0(2, 96, 64))
+    a, b = _empty(64, one.n), _empty(64, one.n)
+    other, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        one.rotate(y, c, a)
+        with torch.cuda.stream(other):
+            two.rotate(y, c, b)
+    other.synchronize()
+    graph.replay()
+    assert np.any(host(b)) and np.array_equal(host(a), host(b))
+    del graph
+    one.close()
+    two.close()
